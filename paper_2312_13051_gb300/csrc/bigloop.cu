@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(DET_THREADS) k_det_phase(z64* A, long long sA,
         const z64 t = prow[cc];
         for (int r = c + 1; r < p; ++r) {
           z64* e = M + (long long)perm[r] * p + cc;
-          *e = *e - mult[r] * t;
+          cfms(*e, mult[r], t);
         }
       }
       __syncthreads();

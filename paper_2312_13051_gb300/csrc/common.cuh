@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace bw {
@@ -42,17 +43,31 @@ template <typename T>
 __host__ __device__ __forceinline__ T abs2(cx<T> a) {
   return a.re * a.re + a.im * a.im;
 }
-// acc += conj(a) * b
+// acc += conj(a) * b and acc += a * b as four fused multiply-adds each.  Written as
+// acc.re += a.re * b.re - a.im * b.im the compiler must keep the inner difference (a
+// product, a fused multiply-add and an addition per part, six instructions): GB300's FP64
+// pipe issues one warp instruction in ~19 clocks per SM, so the count is the time.
 template <typename T>
 __host__ __device__ __forceinline__ void cfma_conj(cx<T>& acc, cx<T> a, cx<T> b) {
-  acc.re += a.re * b.re + a.im * b.im;
-  acc.im += a.re * b.im - a.im * b.re;
+  acc.re = fma(a.re, b.re, acc.re);
+  acc.im = fma(a.re, b.im, acc.im);
+  acc.re = fma(a.im, b.im, acc.re);
+  acc.im = fma(-a.im, b.re, acc.im);
 }
-// acc += a * b
 template <typename T>
 __host__ __device__ __forceinline__ void cfma(cx<T>& acc, cx<T> a, cx<T> b) {
-  acc.re += a.re * b.re - a.im * b.im;
-  acc.im += a.re * b.im + a.im * b.re;
+  acc.re = fma(a.re, b.re, acc.re);
+  acc.im = fma(a.re, b.im, acc.im);
+  acc.re = fma(-a.im, b.im, acc.re);
+  acc.im = fma(a.im, b.re, acc.im);
+}
+// acc -= a * b
+template <typename T>
+__host__ __device__ __forceinline__ void cfms(cx<T>& acc, cx<T> a, cx<T> b) {
+  acc.re = fma(-a.re, b.re, acc.re);
+  acc.im = fma(-a.re, b.im, acc.im);
+  acc.re = fma(a.im, b.im, acc.re);
+  acc.im = fma(-a.im, b.re, acc.im);
 }
 template <typename To, typename Ti>
 __host__ __device__ __forceinline__ cx<To> ccast(cx<Ti> a) {
@@ -193,7 +208,7 @@ __device__ inline void chol_lower_warp(z64* G, int p, int* flag) {
       const double d = sqrt(fmax(d2, 1e-300));
       for (int i = j + 1 + lane; i < p; i += 32) {
         z64 v = G[i * p + j];
-        for (int k = 0; k < j; ++k) v = v - G[i * p + k] * conj(G[j * p + k]);
+        for (int k = 0; k < j; ++k) cfms(v, G[i * p + k], conj(G[j * p + k]));
         G[i * p + j] = (1.0 / d) * v;
       }
       __syncwarp();

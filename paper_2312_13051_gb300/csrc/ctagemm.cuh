@@ -252,7 +252,7 @@ __device__ void cta_reflect_pw(const cx<TA>* A, int n, cx<TX>* X, int ncol, long
       __syncthreads();
       for (int e = (c + 1) * PW + tid; e < n * PW; e += nt) {
         const int r = e / PW, j = e - r * PW;
-        P[e] = P[e] - us[r] * part[j];
+        cfms(P[e], us[r], part[j]);
       }
       __syncthreads();
     }

@@ -147,7 +147,8 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
     for (int col = c + 1 + tid; col < p; col += nt) {
       z64 w(0.0, 0.0);
       for (int r = c + 1; r < p; ++r) cfma_conj(w, vec[r], H[r * ld + col]);
-      for (int r = c + 1; r < p; ++r) H[r * ld + col] = H[r * ld + col] - 2.0 * (vec[r] * w);
+      const z64 w2 = 2.0 * w;
+      for (int r = c + 1; r < p; ++r) cfms(H[r * ld + col], vec[r], w2);
     }
     __syncthreads();
     // right: H <- H (I - 2 v v^dagger) on columns c+1..; Z likewise
@@ -159,7 +160,8 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         w.re += __shfl_xor_sync(0xffffffffu, w.re, o);
         w.im += __shfl_xor_sync(0xffffffffu, w.im, o);
       }
-      for (int k = c + 1 + lane; k < p; k += 32) hr[k] = hr[k] - 2.0 * (w * conj(vec[k]));
+      w = 2.0 * w;
+      for (int k = c + 1 + lane; k < p; k += 32) cfms(hr[k], w, conj(vec[k]));
       if (want_vec) {
         z64* zr = Z + row * ld;
         z64 wz(0.0, 0.0);
@@ -168,7 +170,8 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
           wz.re += __shfl_xor_sync(0xffffffffu, wz.re, o);
           wz.im += __shfl_xor_sync(0xffffffffu, wz.im, o);
         }
-        for (int k = c + 1 + lane; k < p; k += 32) zr[k] = zr[k] - 2.0 * (wz * conj(vec[k]));
+        wz = 2.0 * wz;
+        for (int k = c + 1 + lane; k < p; k += 32) cfms(zr[k], wz, conj(vec[k]));
       }
     }
     __syncthreads();

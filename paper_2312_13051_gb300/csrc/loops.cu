@@ -400,7 +400,7 @@ __device__ void cholqr_par(z64* nu, z64* G, int p, int m, int* ok) {
     z64* q = nu + r * m;
     for (int j = 0; j < m; ++j) {
       z64 y = conj(q[j]);
-      for (int k = 0; k < j; ++k) y = y - G[j * m + k] * conj(q[k]);
+      for (int k = 0; k < j; ++k) cfms(y, G[j * m + k], conj(q[k]));
       q[j] = conj((1.0 / G[j * m + j].re) * y);
     }
   }
@@ -1477,7 +1477,7 @@ __global__ void k_plaquette_links(const z64* U, int n, int p, int N, int Nt, z64
         const int w = p - c - 1;
         for (int e = tid; e < w * w; e += nt) {
           const int r = c + 1 + e / w, cc = c + 1 + e % w;
-          A[r * p + cc] = A[r * p + cc] - A[r * p + c] * A[c * p + cc];
+          cfms(A[r * p + cc], A[r * p + c], A[c * p + cc]);
         }
         __syncthreads();
       }

@@ -119,7 +119,7 @@ __device__ bool cholqr(z64* Q, z64* G, int n, int p, int* flag) {
     z64* q = Q + r * p;
     for (int j = 0; j < p; ++j) {
       z64 y = conj(q[j]);
-      for (int k = 0; k < j; ++k) y = y - G[j * p + k] * conj(q[k]);
+      for (int k = 0; k < j; ++k) cfms(y, G[j * p + k], conj(q[k]));
       q[j] = conj((1.0 / G[j * p + j].re) * y);
     }
   }
@@ -200,7 +200,7 @@ __device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const
     for (int e = tid; e < n * p; e += nt) {
       const int r = e / p, c = e - r * p;
       z64 acc = HQ[e];
-      for (int q = 0; q < p; ++q) acc = acc - Q[r * p + q] * G[q * p + c];
+      for (int q = 0; q < p; ++q) cfms(acc, Q[r * p + q], G[q * p + c]);
       C[e] = acc;  // residual, kept in C
     }
     __syncthreads();
