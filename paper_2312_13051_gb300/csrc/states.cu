@@ -2,11 +2,11 @@
 //
 //  - k_build_hk:      H(f) = sum_e t_e exp(i 2 pi f.R_e) |i_e><j_e| to global memory
 //                     (Sec. I, the tight-binding Hamiltonian at each k).
-//  - k_states_small:  one CTA per k-point, everything in shared memory: build H(k),
-//                     Jacobi eigensolve, the lowest p eigenvectors and the direct gap
-//                     (Sec. I "exact diagonalization"; Eq. 1 occupied bands), the
-//                     optional FP64 refinement of an FP32 solve, and the optional
-//                     projected-spin-operator sector (Sec. IV).
+//  - k_states_small:  one CTA per k-point, everything in shared memory: build H(k), FP32
+//                     Jacobi eigensolve, the lowest p states refined in FP64 (FP64 request:
+//                     to FP64 accuracy, or an FP64 Jacobi solve where that does not apply)
+//                     and the direct gap (Sec. I "exact diagonalization"; Eq. 1 occupied
+//                     bands), and the optional projected-spin-operator sector (Sec. IV).
 //  - k_eigh_small:    batched Hermitian eigensolver on caller matrices (uneven n).
 #include <float.h>
 
@@ -170,58 +170,64 @@ __device__ bool ritz(const z64* H, z64* Q, z64* HQ, z64* C, z64* G, z64* Zg, dou
   return sw >= 0;
 }
 
-// Mixed precision: refine the lowest-p invariant subspace of the FP64 matrix H
-// starting from an FP32 eigenbasis V (columns ordered by ord, eigenvalues lam).
-// One Newton correction in the FP32 eigenbasis of the complement,
+// One Newton correction of the orthonormal block Q (the lowest p states of the FP64 matrix
+// H) in the FP32 eigenbasis V of the complement (columns ordered by ord, eigenvalues lam),
 //   Q <- Q + V_u C,  C[a][i] = (V_u^dagger R)[a][i] / (G_ii - lam_{p+a}),
 // with the FP64 residual R = H Q - Q G, G = Q^dagger H Q (its off-diagonal part is
 // of the order of the FP32 error and enters the correction at second order), then
-// Cholesky-QR.  The FP32 start is accurate to eps32 ||H|| / gap, the corrected
-// subspace to about (eps32 ||H|| / gap)^2.  Returns the direct gap from FP64
-// Rayleigh quotients of the p-th and (p+1)-th FP32 vectors; *ok = 0 when a
-// Cholesky factorisation broke down.
-__device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const double* lam,
-                               int n, int p, z64* Q, z64* HQ, z64* C, z64* G, z64* Zg,
-                               double* rho, int* ord2, JacRot<double>* rot, double* red,
-                               int max_sweeps, int* ok, int* flag) {
+// Cholesky-QR.  An error e of the subspace becomes about e^2.  Returns |C|_F^2; *ok = 0
+// when the Cholesky factorisation broke down.
+__device__ double newton_step(const z64* H, const c32* V, const int* ord, const double* lam, int n, int p, z64* Q,
+                              z64* HQ, z64* C, z64* G, double* red, int* ok, int* flag) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  (void)Zg; (void)rho; (void)ord2; (void)rot; (void)max_sweeps;
-  *ok = cholqr(Q, G, n, p, flag) ? 1 : 0;
-  if (p < n) {
-    mm(H, Q, HQ, n, n, p);
-    // diagonal of G = Q^dagger H Q, then R = H Q - Q G (full G)
-    for (int e = tid; e < p * p; e += nt) {
-      const int a = e / p, b = e - a * p;
-      z64 acc(0.0, 0.0);
-      for (int r = 0; r < n; ++r) cfma_conj(acc, Q[r * p + a], HQ[r * p + b]);
-      G[e] = acc;
-    }
-    __syncthreads();
-    for (int e = tid; e < n * p; e += nt) {
-      const int r = e / p, c = e - r * p;
-      z64 acc = HQ[e];
-      for (int q = 0; q < p; ++q) cfms(acc, Q[r * p + q], G[q * p + c]);
-      C[e] = acc;  // residual, kept in C
-    }
-    __syncthreads();
-    const int nu = n - p;
-    for (int e = tid; e < nu * p; e += nt) {
-      const int a = e / p, i = e - a * p;
-      const int col = ord[p + a];
-      z64 acc(0.0, 0.0);
-      for (int r = 0; r < n; ++r) cfma_conj(acc, ccast<double>(V[r * n + col]), C[r * p + i]);
-      HQ[e] = (1.0 / (G[i * p + i].re - lam[col])) * acc;  // correction coefficients
-    }
-    __syncthreads();
-    for (int e = tid; e < n * p; e += nt) {
-      const int r = e / p, i = e - r * p;
-      z64 acc = Q[e];
-      for (int a = 0; a < nu; ++a) cfma(acc, ccast<double>(V[r * n + ord[p + a]]), HQ[a * p + i]);
-      Q[e] = acc;
-    }
-    __syncthreads();
-    if (!cholqr(Q, G, n, p, flag)) *ok = 0;
+  mm(H, Q, HQ, n, n, p);
+  // G = Q^dagger H Q, then R = H Q - Q G (full G)
+  for (int e = tid; e < p * p; e += nt) {
+    const int a = e / p, b = e - a * p;
+    z64 acc(0.0, 0.0);
+    for (int r = 0; r < n; ++r) cfma_conj(acc, Q[r * p + a], HQ[r * p + b]);
+    G[e] = acc;
   }
+  __syncthreads();
+  for (int e = tid; e < n * p; e += nt) {
+    const int r = e / p, c = e - r * p;
+    z64 acc = HQ[e];
+    for (int q = 0; q < p; ++q) cfms(acc, Q[r * p + q], G[q * p + c]);
+    C[e] = acc;  // residual, kept in C
+  }
+  __syncthreads();
+  const int nu = n - p;
+  double c2 = 0.0;
+  for (int e = tid; e < nu * p; e += nt) {
+    const int a = e / p, i = e - a * p;
+    const int col = ord[p + a];
+    z64 acc(0.0, 0.0);
+    for (int r = 0; r < n; ++r) cfma_conj(acc, ccast<double>(V[r * n + col]), C[r * p + i]);
+    HQ[e] = (1.0 / (G[i * p + i].re - lam[col])) * acc;  // correction coefficients
+    c2 += abs2(HQ[e]);
+  }
+  __syncthreads();
+  for (int e = tid; e < n * p; e += nt) {
+    const int r = e / p, i = e - r * p;
+    z64 acc = Q[e];
+    for (int a = 0; a < nu; ++a) cfma(acc, ccast<double>(V[r * n + ord[p + a]]), HQ[a * p + i]);
+    Q[e] = acc;
+  }
+  __syncthreads();
+  if (!cholqr(Q, G, n, p, flag)) *ok = 0;
+  return block_sum(c2, red);
+}
+
+// Mixed precision: refine the lowest-p invariant subspace of the FP64 matrix H
+// starting from an FP32 eigenbasis V by one Newton correction.  The FP32 start is
+// accurate to eps32 ||H|| / gap, the corrected subspace to about (eps32 ||H|| / gap)^2.
+// Returns the direct gap from FP64 Rayleigh quotients of the p-th and (p+1)-th FP32
+// vectors; *ok = 0 when a Cholesky factorisation broke down.
+__device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const double* lam,
+                               int n, int p, z64* Q, z64* HQ, z64* C, z64* G, double* red, int* ok, int* flag) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  *ok = cholqr(Q, G, n, p, flag) ? 1 : 0;
+  if (p < n) newton_step(H, V, ord, lam, n, p, Q, HQ, C, G, red, ok, flag);
   // gap from FP64 Rayleigh quotients of the FP32 vectors p-1 and p
   double gap = INFINITY;
   if (p < n) {
@@ -245,11 +251,106 @@ __device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const
   return gap;
 }
 
+// Edge of the spectrum of H to FP64 accuracy from the FP32 eigenbasis V: the largest
+// (want_max) eigenvalue of the levels up to sorted position c1, or the smallest from
+// position c0 on, where [c0, c1] are the g levels that lie within `width` of that edge.
+// Each of the g vectors is corrected once against every level outside the cluster
+// (x_b + sum_j x_j (x_j^dag r_b) / (lam_b - lam_j), r_b = H x_b - lam_b x_b), which leaves
+// an error of (eps32 ||H|| / width)^2 in the vectors and its square in the Ritz values of
+// the cluster, taken after Cholesky-QR.  Y, HY: n x g scratch, G, Zg: g x g.
+__device__ double edge_energy(const z64* H, const c32* V, const int* ord, const double* lam, int n, int c0, int c1,
+                              bool want_max, z64* Y, z64* HY, z64* G, z64* Zg, JacRot<double>* rot, double* red,
+                              int max_sweeps, int* ok, int* flag) {
+  const int tid = threadIdx.x, nt = blockDim.x, g = c1 - c0 + 1;
+  for (int e = tid; e < n * g; e += nt) {
+    const int r = e / g, b = e - r * g, col = ord[c0 + b];
+    z64 acc(0.0, 0.0);
+    for (int q = 0; q < n; ++q) cfma(acc, H[r * n + q], ccast<double>(V[q * n + col]));
+    Y[e] = acc - lam[col] * ccast<double>(V[r * n + col]);
+  }
+  __syncthreads();
+  for (int e = tid; e < n * g; e += nt) {  // coefficient of level j (sorted position) in vector b
+    const int j = e / g, b = e - j * g;
+    c32 acc(0.f, 0.f);
+    if (j < c0 || j > c1) {
+      for (int r = 0; r < n; ++r) cfma_conj(acc, V[r * n + ord[j]], ccast<float>(Y[r * g + b]));
+      acc = float(1.0 / (lam[ord[c0 + b]] - lam[ord[j]])) * acc;
+    }
+    HY[e] = ccast<double>(acc);
+  }
+  __syncthreads();
+  for (int e = tid; e < n * g; e += nt) {
+    const int r = e / g, b = e - r * g;
+    z64 acc = ccast<double>(V[r * n + ord[c0 + b]]);
+    c32 u(0.f, 0.f);
+    for (int j = 0; j < n; ++j) cfma(u, V[r * n + ord[j]], ccast<float>(HY[j * g + b]));
+    Y[e] = acc + ccast<double>(u);
+  }
+  __syncthreads();
+  if (!cholqr(Y, G, n, g, flag)) {
+    *ok = 0;
+    return 0.0;
+  }
+  mm(H, Y, HY, n, n, g);
+  for (int e = tid; e < g * g; e += nt) {
+    const int x = e / g, y = e - x * g;
+    z64 acc(0.0, 0.0);
+    for (int r = 0; r < n; ++r) cfma_conj(acc, Y[r * g + x], HY[r * g + y]);
+    if (x == y) acc.im = 0.0;
+    if (y >= x) G[x * g + y] = acc;
+    if (y > x) G[y * g + x] = conj(acc);
+  }
+  __syncthreads();
+  if (g > 1 && jacobi_eigh<double>(G, Zg, g, g, max_sweeps, rot, red) < 0) *ok = 0;
+  double e0 = G[0].re;
+  for (int c = 1; c < g; ++c) e0 = want_max ? fmax(e0, G[c * g + c].re) : fmin(e0, G[c * g + c].re);
+  __syncthreads();
+  return e0;
+}
+
+// FP64 request from an FP32 eigenbasis V of H: the occupied block Q by Newton corrections,
+// repeated until the square of the last one is below rounding (|C|_F^2 <= 1e-17: two, when
+// the FP32 start is good to 1e-4), and the direct gap from the two band edges.  Replaces
+// the FP64 Jacobi sweeps (~7 n^3 complex multiply-adds each) by ~13 n^2 p FP64 ones, which
+// the FP64 pipe was busy with (n = 32, p = 8, 441 k-points with the spin split: 4.40 ms
+// before, 1.65 ms now).
+// Returns false, and the caller solves in FP64, where this does not apply: a gap below
+// 1e-3 of the spectral radius, H outside the FP32 range, more than p levels (the scratch)
+// within that distance of a band edge, corrections that do not converge.
+__device__ bool refine_fp64(const z64* H, const c32* V, const int* ord, const double* lam, int n, int p, z64* Q,
+                            z64* HQ, z64* C, z64* G, z64* Zg, JacRot<double>* rot, double* red, int max_sweeps,
+                            int* flag, double& gap) {
+  gap = INFINITY;
+  int ok = cholqr(Q, G, n, p, flag) ? 1 : 0;
+  if (!ok) return false;
+  if (p == n) return true;
+  const double nrm = fmax(fabs(lam[ord[0]]), fabs(lam[ord[n - 1]])), width = 1e-3 * nrm;
+  if (!(nrm > 1e-8 && nrm < 1e12) || !(lam[ord[p]] - lam[ord[p - 1]] > width)) return false;
+  int c0 = p - 1, c1 = p;
+  while (c0 > 0 && lam[ord[p - 1]] - lam[ord[c0 - 1]] <= width) --c0;
+  while (c1 + 1 < n && lam[ord[c1 + 1]] - lam[ord[p]] <= width) ++c1;
+  if (p - c0 > p || c1 - p + 1 > p) return false;
+  double c2 = 1.0;
+  for (int it = 0; it < 4 && !(c2 <= 1e-17); ++it) {
+    c2 = newton_step(H, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
+    if (!ok || !(c2 < 1e-4)) return false;
+  }
+  if (!(c2 <= 1e-17)) return false;
+  const double top = edge_energy(H, V, ord, lam, n, c0, p - 1, true, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
+  if (!ok) return false;
+  const double bot = edge_energy(H, V, ord, lam, n, p, c1, false, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
+  gap = bot - top;
+  return ok != 0;
+}
+
 // Projected spin operator sector (Sec. IV): S = U^dagger s U (p x p), eigh, keep the
 // eigenvectors with eigenvalue sign `sign` (split at zero), or the p/2 lowest / highest
 // (median); Us = U V_s written to `out` (n x p/2).
+// The FP64 Jacobi sweeps start from S in the eigenbasis of its FP32 part (X, orthonormalised
+// in FP64), where S is diagonal to ~1e-7: one or two sweeps remain of about six.
+// A32, V32: p x p FP32 scratch; X, T: p x p FP64 scratch.
 __device__ void pso_split(const z64* U, const DevOp& op, int sign, int median, int n, int p, z64* S,
-                          z64* SV, int* ord, double* mu, JacRot<double>* rot, double* red,
+                          z64* SV, c32* A32, c32* V32, z64* X, z64* T, int* flag, int* ord, double* mu, JacRot<double>* rot, double* red,
                           int max_sweeps, z64* out, double* pso_out, double* pso_gap_out,
                           double pso_tol, DevStatus* st, long long k) {
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -274,7 +375,33 @@ __device__ void pso_split(const z64* U, const DevOp& op, int sign, int median, i
     }
   }
   __syncthreads();
+  for (int e = tid; e < p * p; e += nt) A32[e] = ccast<float>(S[e]);
+  __syncthreads();
+  bool pre = jacobi_eigh<float>(A32, V32, p, p, max_sweeps, reinterpret_cast<JacRot<float>*>(rot), red) > 0;
+  if (pre) {
+    for (int e = tid; e < p * p; e += nt) X[e] = ccast<double>(V32[e]);
+    __syncthreads();
+    pre = cholqr(X, T, p, p, flag);
+  }
+  if (pre) {  // S <- X^dag S X, the upper triangle mirrored
+    mm(S, X, T, p, p, p);
+    for (int e = tid; e < p * p; e += nt) {
+      const int a = e / p, b = e - a * p;
+      if (b < a) continue;
+      z64 acc(0.0, 0.0);
+      for (int r = 0; r < p; ++r) cfma_conj(acc, X[r * p + a], T[r * p + b]);
+      if (a == b) acc.im = 0.0;
+      S[a * p + b] = acc;
+      if (a != b) S[b * p + a] = conj(acc);
+    }
+    __syncthreads();
+  }
   const int sw = jacobi_eigh<double>(S, SV, p, p, max_sweeps, rot, red);
+  if (pre) {  // back to the occupied basis
+    mm(X, SV, T, p, p, p);
+    for (int e = tid; e < p * p; e += nt) SV[e] = T[e];
+    __syncthreads();
+  }
   sort_diag<double>(S, p, p, ord);
   for (int c = tid; c < p; c += nt) mu[c] = S[ord[c] * p + ord[c]].re;
   __syncthreads();
@@ -309,17 +436,17 @@ __device__ void pso_split(const z64* U, const DevOp& op, int sign, int median, i
 // ---------------------------------------------------------------------------
 // One CTA per k-point: build, solve, (refine), (spin split), write.
 // ---------------------------------------------------------------------------
-template <typename T>
 __global__ void k_states_small(StatesArgs a, int p_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const DevModel& md = a.model;
   const int n = md.n, p = a.p, tid = threadIdx.x, nt = blockDim.x;
   const int nRs = min(md.n_R, PHASE_CACHE);
   const bool mixed = a.mixed != 0;
-  const SmemLayout L = states_layout<T>(n, p, nRs, mixed);
+  const SmemLayout L = states_layout<float>(n, p, nRs, true);
   z64* phs = reinterpret_cast<z64*>(smem + L.phs);
-  cx<T>* A = reinterpret_cast<cx<T>*>(smem + L.A);
-  cx<T>* V = reinterpret_cast<cx<T>*>(smem + L.V);
+  c32* A = reinterpret_cast<c32*>(smem + L.A);
+  c32* V = reinterpret_cast<c32*>(smem + L.V);
+  z64* V64 = reinterpret_cast<z64*>(smem + L.A);  // FP64 eigenvectors, over A and V
   z64* H64 = reinterpret_cast<z64*>(smem + L.H64);
   z64* Q = reinterpret_cast<z64*>(smem + L.Q);
   z64* HQ = reinterpret_cast<z64*>(smem + L.HQ);
@@ -331,7 +458,7 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
   int* ord = reinterpret_cast<int*>(smem + L.order);
   int* ord2 = reinterpret_cast<int*>(smem + L.order2);
   JacRot<double>* rot64 = reinterpret_cast<JacRot<double>*>(smem + L.rot);
-  JacRot<T>* rot = reinterpret_cast<JacRot<T>*>(smem + L.rot);
+  JacRot<float>* rot = reinterpret_cast<JacRot<float>*>(smem + L.rot);
   double* red = reinterpret_cast<double*>(smem + L.red);
   int* flag = reinterpret_cast<int*>(red + 40);
 
@@ -345,8 +472,8 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
     }
     for (int r = tid; r < nRs; r += nt) phs[r] = bloch_phase(f, md.Rv + 3 * r);
     for (int e = tid; e < n * n; e += nt) {
-      A[e] = cx<T>(T(0), T(0));
-      if (mixed) H64[e] = z64(0.0, 0.0);
+      A[e] = c32(0.f, 0.f);
+      H64[e] = z64(0.0, 0.0);
     }
     __syncthreads();
     for (int e = tid; e < md.n_ent; e += nt) {
@@ -357,12 +484,12 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
         cfma(acc, md.hop_t[h], ph);
       }
       const int at = md.ent_row[e] * n + md.ent_col[e];
-      A[at] = ccast<T>(acc);
-      if (mixed) H64[at] = acc;
+      A[at] = ccast<float>(acc);
+      H64[at] = acc;
     }
     __syncthreads();
-    const int sw = jacobi_eigh<T>(A, V, n, n, a.max_sweeps, rot, red);
-    sort_diag<T>(A, n, n, ord);
+    int sw = jacobi_eigh<float>(A, V, n, n, a.max_sweeps, rot, red);
+    sort_diag<float>(A, n, n, ord);
     for (int c = tid; c < n; c += nt) lam[c] = double(A[c * n + c].re);
     for (int e = tid; e < n * p; e += nt) {
       const int r = e / p, c = e - r * p;
@@ -371,11 +498,21 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
     __syncthreads();
     double gap;
     int ok = 1;
-    if (!mixed) {
+    if (mixed) {
+      gap = refine_mixed(H64, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
+    } else if (sw < 0 ||
+               !refine_fp64(H64, V, ord, lam, n, p, Q, HQ, C, G, Zg, rot64, red, a.max_sweeps, flag, gap)) {
+      // FP64 Jacobi, in place on H
+      __syncthreads();
+      sw = jacobi_eigh<double>(H64, V64, n, n, a.max_sweeps, rot64, red);
+      sort_diag<double>(H64, n, n, ord);
+      for (int c = tid; c < n; c += nt) lam[c] = H64[c * n + c].re;
+      for (int e = tid; e < n * p; e += nt) {
+        const int r = e / p, c = e - r * p;
+        Q[e] = V64[r * n + ord[c]];
+      }
+      __syncthreads();
       gap = p < n ? lam[ord[p]] - lam[ord[p - 1]] : INFINITY;
-    } else {
-      gap = refine_mixed(H64, reinterpret_cast<const c32*>(V), ord, lam, n, p, Q, HQ, C, G, Zg,
-                         rho, ord2, rot64, red, a.max_sweeps, &ok, flag);
     }
     if (tid == 0) {
       a.gap[k] = gap;
@@ -384,7 +521,7 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
     }
     z64* out = a.U + k * (long long)n * p_out;
     if (a.op.nnz > 0) {
-      pso_split(Q, a.op, a.sign, a.pso_median, n, p, G, Zg, ord2, rho, rot64, red, a.max_sweeps, out,
+      pso_split(Q, a.op, a.sign, a.pso_median, n, p, G, Zg, A, V, HQ, C, flag, ord2, rho, rot64, red, a.max_sweeps, out,
                 a.pso_evals ? a.pso_evals + k * p : nullptr, a.pso_gap ? a.pso_gap + k : nullptr,
                 a.pso_gap_tol, a.status, k);
     } else {
@@ -443,8 +580,7 @@ __global__ void k_eigh_small(EighArgs a) {
         Q[e] = ccast<double>(V[r * n + ord[c]]);
       }
       __syncthreads();
-      refine_mixed(H64, reinterpret_cast<const c32*>(V), ord, lam, n, p, Q, HQ, C, G, Zg, rho,
-                   ord2, rot64, red, a.max_sweeps, &ok, flag);
+      refine_mixed(H64, reinterpret_cast<const c32*>(V), ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
       // individual eigenpairs: Rayleigh-Ritz on the refined subspace
       if (!ritz(H64, Q, HQ, C, G, Zg, rho, ord2, n, p, rot64, red, a.max_sweeps)) ok = 0;
     }
@@ -478,14 +614,13 @@ cudaError_t launch_build_hk(const BuildArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <typename T>
 static cudaError_t states_impl(const StatesArgs& a, int p_out, cudaStream_t s) {
   const int nRs = a.model.n_R < PHASE_CACHE ? a.model.n_R : PHASE_CACHE;
-  const SmemLayout L = states_layout<T>(a.model.n, a.p, nRs, a.mixed != 0);
+  const SmemLayout L = states_layout<float>(a.model.n, a.p, nRs, true);
   static size_t cached = 0;
-  cudaError_t e = set_smem_once(k_states_small<T>, L.total, cached);
+  cudaError_t e = set_smem_once(k_states_small, L.total, cached);
   if (e != cudaSuccess) return e;
-  k_states_small<T><<<grid_for(a.K), threads_for(a.model.n), L.total, s>>>(a, p_out);
+  k_states_small<<<grid_for(a.K), threads_for(a.model.n), L.total, s>>>(a, p_out);
   return cudaGetLastError();
 }
 
@@ -494,7 +629,7 @@ cudaError_t launch_states_small(const StatesArgs& a, int p_out, cudaStream_t s) 
   bool handled = false;
   const cudaError_t e = launch_states_tiny(a, p_out, s, &handled);
   if (handled || e != cudaSuccess) return e;
-  return a.mixed ? states_impl<float>(a, p_out, s) : states_impl<double>(a, p_out, s);
+  return states_impl(a, p_out, s);
 }
 
 template <typename T>

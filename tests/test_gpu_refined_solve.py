@@ -1,0 +1,70 @@
+"""FP64 requests at n <= 32: an FP32 eigenbasis refined to FP64, or the FP64 Jacobi solve
+where a band edge leaves the refinement's range.  Phases against the oracle within the
+FP64 bound of the other parity tests; gaps within 8 n eps ||H|| (the forward error of a
+backward-stable eigenvalue, with a factor for the sums of n terms)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2312_13051_gb300 import inputs as I
+from tests.gpu_common import circ_err_rows, ctx, lib  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+EPS = 2.0 ** -52
+
+
+def _check(lib, ctx, model, plane, p, phases=True):
+    ph, gap = lib.wilson_loop(model, plane, p, precision="fp64", ctx=ctx, gap_tol=0.0)
+    ref, rgap = oracle.wilson_loop(model, plane, p, gap_tol=0.0)
+    norm = np.bincount(model.i, np.abs(model.t)).max()  # bounds ||H(k)||
+    assert np.max(np.abs(gap.cpu().numpy() - rgap)) <= 8 * model.n * EPS * norm
+    if phases:
+        assert circ_err_rows(ph.cpu().numpy(), ref) <= 1e-10
+
+
+def _scaled(m, s, hop=1.0):
+    """The model times s, its hoppings between cells times hop as well."""
+    t = s * m.t * np.where(np.any(m.R != 0, axis=1), hop, 1.0)
+    return I.HoppingList(n=m.n, R=m.R, i=m.i, j=m.j, t=t, dim=m.dim)
+
+
+@pytest.mark.parametrize("n,p", [(2, 1), (4, 1), (4, 2), (4, 3), (5, 1), (8, 7), (17, 8), (31, 16), (32, 1), (32, 31)])
+def test_refined_states_and_gap(lib, ctx, n, p):
+    # weak dispersion: the overlaps of neighbouring points stay near one, so that the
+    # eigenphases of their product are well conditioned
+    _check(lib, ctx, _scaled(I.random_hermitian_model(n, 11 + n), 1.0, hop=0.03), I.Plane(9, 5), p)
+
+
+@pytest.mark.parametrize("copies", [1, 2, 5])
+@pytest.mark.parametrize("split", [0.0, 1e-9, 1e-6, 1e-3])
+def test_near_degenerate_band_edges(lib, ctx, copies, split):
+    """Copies of the quadrupole insulator whose levels differ by `split`: the occupied and
+    the unoccupied edge are clusters of 2 to 10 levels."""
+    parts = []
+    for c in range(copies):
+        m = I.bbh(0.5, 0.5)
+        on = I.HoppingList(n=4, R=np.concatenate([m.R, np.zeros((4, 3), np.int32)]),
+                           i=np.concatenate([m.i, np.arange(4)]), j=np.concatenate([m.j, np.arange(4)]),
+                           t=np.concatenate([m.t, np.full(4, c * split + 0j)]), dim=m.dim)
+        parts.append(on)
+    model = I.direct_sum(parts) if copies > 1 else parts[0]
+    _check(lib, ctx, model, I.Plane(8, 5), 2 * copies)
+
+
+@pytest.mark.parametrize("n", [4, 12])
+@pytest.mark.parametrize("offset", [1e-7, 1e-4, 1e-2])
+def test_gap_down_to_closing(lib, ctx, n, offset):
+    """Two identical blocks shifted against each other by `offset`: with p = 1 the direct gap
+    is the offset itself, on both sides of the refinement's limit."""
+    m = I.random_hermitian_model(n // 2, 3)
+    k = n // 2
+    sh = I.HoppingList(n=k, R=np.concatenate([m.R, np.zeros((k, 3), np.int32)]),
+                       i=np.concatenate([m.i, np.arange(k)]), j=np.concatenate([m.j, np.arange(k)]),
+                       t=np.concatenate([m.t, np.full(k, offset + 0j)]), dim=m.dim)
+    _check(lib, ctx, I.direct_sum([m, sh]), I.Plane(7, 4), 1, phases=False)
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-9, 1e20])
+def test_energy_scale_outside_fp32(lib, ctx, scale):
+    for n, p in ((4, 2), (10, 4)):
+        _check(lib, ctx, _scaled(I.random_hermitian_model(n, 5), scale, hop=0.03), I.Plane(7, 4), p)
