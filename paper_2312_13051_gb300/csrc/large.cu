@@ -806,8 +806,8 @@ __host__ __device__ inline size_t refine_work_offset(int p) {
 //   R = H Q - Q rho in FP64; the complement's coefficients
 //   C[a][c] = z_a^T D^dag Q_h^dag R_c / (rho_c - lam_a) and the update
 //   Q_h D Z_u C in FP32 through the reflectors (R is small, FP32 keeps it to ~1e-7
-//   relative); Q64 = Q + update.  Then one first-order Lowdin step,
-//   Q <- Q - Q (Q^dag Q - I) / 2, with Q32^dag Q32 - I compensated and the small
+//   relative); Q64 = Q + update.  Then one second-order Lowdin step,
+//   Q <- Q - Q (E / 2 - 3 E^2 / 8), E = Q^dag Q - I, with Q32^dag Q32 - I compensated and the small
 //   terms in FP32.  The gap comes from FP64 Rayleigh quotients of the (p-1)-th
 //   and p-th FP32 vectors.  The off-diagonal part of Q^dag H Q is of the order of
 //   the FP32 error; its projection on the complement enters at second order.
@@ -931,10 +931,18 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
         },
         [&](int x, int y, c32 v) { E[(long long)x * p + y] = E[(long long)x * p + y] + v; }, work, ts);
     __syncthreads();
-    // Q = (Q32 + C) - (Q32 + C) E / 2, the correction in FP32
+    // second order of (I + E)^{-1/2}: F = E - 3/4 E^2 (E reaches ~3e-5 where inverse iteration
+    // leaves neighbouring vectors short of orthogonal, and E^2 would stay as the error)
+    c32* F = E + (long long)p * p;
+    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+        p, p, p, [&](int x, int q) { return E[(long long)x * p + q]; },
+        [&](int q, int y) { return E[(long long)q * p + y]; },
+        [&](int x, int y, c32 v) { F[(long long)x * p + y] = E[(long long)x * p + y] - 0.75f * v; }, work, ts);
+    __syncthreads();
+    // Q = (Q32 + C) - (Q32 + C) F / 2, the correction in FP32
     tc_ok = tc_ok && cta_cgemm_tc<true, true>(
         n, p, p, [&](int r, int q) { return X[(long long)r * nbt + q] + C[(long long)r * p + q]; },
-        [&](int q, int c) { return E[(long long)q * p + c]; },
+        [&](int q, int c) { return F[(long long)q * p + c]; },
         [&](int r, int c, c32 v) {
           const c32 x32 = X[(long long)r * nbt + c], dc = C[(long long)r * p + c];
           Q[(long long)r * p + c] = z64(double(x32.re) + double(dc.re) - 0.5 * double(v.re),
