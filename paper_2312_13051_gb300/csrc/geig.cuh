@@ -2,8 +2,9 @@
 //
 // The Wilson matrix of Eq. 2 is a product of raw overlaps and is not unitary, so
 // its eigenvalues need a general (non-Hermitian) solver: Householder reduction to
-// upper Hessenberg form, then single-shift implicit QR sweeps with Givens
-// rotations, Wilkinson shifts and deflation on small subdiagonals.  With vectors
+// upper Hessenberg form, then implicit QR sweeps with Givens rotations and deflation on
+// small subdiagonals, several sweeps chasing each other through the matrix two rows apart,
+// with the eigenvalues of the trailing block as their shifts.  With vectors
 // requested the rotations are applied to whole rows/columns, leaving the Schur
 // form T = Z^dagger W Z; right eigenvectors are x = Z y with T y = lambda y solved
 // by back substitution.
@@ -13,12 +14,21 @@
 
 namespace bw {
 
+// Sweeps in flight.  A rotation is a chain of ~20 dependent FP64 operations (64 clocks each
+// on GB300) and three block barriers, whatever the number of entries it moves, so the sweeps
+// of several shifts share the steps: NB sweeps over an active block of s rows take
+// s + 2 NB steps instead of NB s.  Measured (one CTA per loop): p = 64, 27 loops, product
+// included, 19.5 -> 12.9 ms; p = 32 FP64, 17 loops, 5.1 -> 3.5 ms; p = 12 with vectors 1.46 ->
+// 1.16 ms.  A step at p = 64 takes ~7000 clocks: 2100 the rotations, the rest FP64 throughput.
+constexpr int GEIG_NB = 8;
+
 struct GeigShared {
-  z64 c0;        // Givens: G = [[c, s], [-conj(s), c]], c real (stored in c0.re)
-  z64 s;
+  double c[GEIG_NB];    // Givens of each sweep: G = [[c, s], [-conj(s), c]], c real
+  z64 s[GEIG_NB];
+  z64 shift[GEIG_NB];
+  c32 B[GEIG_NB * GEIG_NB];  // trailing block (shift selection)
   z64 mu;
-  int l, hi, active, fail, k;
-  double scale;
+  int l, hi, nb, active, fail;
 };
 
 __device__ __forceinline__ double zabs(z64 a) { return hypot(a.re, a.im); }
@@ -50,15 +60,18 @@ __device__ __forceinline__ void givens(z64 x, z64 y, double& c, z64& s) {
 // Whether the subdiagonal entry H[l][l-1] is negligible: against the neighbouring
 // diagonal entries, or by the product test of Ahues and Tisseur (its product with
 // the superdiagonal small against the local separation of the diagonal entries).
+// Magnitudes are |re| + |im| (within a factor sqrt(2) of the modulus, a hypot each otherwise).
+__device__ __forceinline__ double zabs1(z64 a) { return fabs(a.re) + fabs(a.im); }
+
 __device__ __forceinline__ bool geig_negligible_v(z64 h11, z64 h12, z64 h21, z64 h22, double eps) {
-  const double sub = zabs(h21);
-  const double dia = zabs(h22) + zabs(h11);
+  const double sub = zabs1(h21);
+  const double dia = zabs1(h22) + zabs1(h11);
   bool small = sub <= eps * dia || sub < 1e-300;
   if (!small && sub <= dia) {
-    const double x = zabs(h12);
+    const double x = zabs1(h12);
     const double ab = fmax(sub, x), ba = fmin(sub, x);
-    const double y = zabs(h11 - h22);
-    const double aa = fmax(zabs(h22), y), bb = fmin(zabs(h22), y);
+    const double y = zabs1(h11 - h22);
+    const double aa = fmax(zabs1(h22), y), bb = fmin(zabs1(h22), y);
     const double sc = aa + ab;
     small = ba * (ab / sc) <= fmax(1e-300, eps * (bb * (aa / sc)));
   }
@@ -93,6 +106,75 @@ __device__ __forceinline__ z64 geig_shift(z64 a, z64 b, z64 c, z64 d, int iter, 
   return (abs2(m1 - d) <= abs2(m2 - d)) ? m1 : m2;
 }
 
+// Shifts of nb simultaneous sweeps: the eigenvalues of the trailing nb x nb block of the
+// active window (last row hi) by single-shift QR in FP32 (a shift decides how fast the
+// sweeps converge, not what they converge to), in the order in which they separate from
+// the bottom.  At its cap of sweeps the diagonal entries left over serve.  The first warp
+// calls it, all lanes.
+__device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, z64* shift) {
+  const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
+  for (int e = lane; e < nb * nb; e += 32) {
+    const int r = e / nb, c = e - r * nb;
+    B[e] = r <= c + 1 ? ccast<float>(H[(h0 + r) * ld + h0 + c]) : c32(0.f, 0.f);
+  }
+  __syncwarp();
+  int top = nb - 1, out = 0;
+  for (int it = 0; it < 8 * GEIG_NB && top > 0; ++it) {
+    // split point: the largest l whose subdiagonal entry is negligible
+    const bool small = lane >= 1 && lane <= top &&
+                       abs2(B[lane * nb + lane - 1]) <=
+                           1e-12f * (abs2(B[lane * nb + lane]) + abs2(B[(lane - 1) * nb + lane - 1]));
+    const unsigned m = __ballot_sync(0xffffffffu, small);
+    const int l = m ? 31 - __clz(m) : 0;
+    if (l == top) {
+      if (lane == 0) shift[out] = ccast<double>(B[top * nb + top]);
+      ++out;
+      --top;
+      continue;
+    }
+    // Wilkinson shift: the eigenvalue of the last 2 x 2 block [[a, b], [c, d]] closest to d,
+    // d - b c / (g +- sqrt(g^2 + b c)) with g = (a - d) / 2 and the larger denominator
+    const c32 a = B[(top - 1) * nb + top - 1], d = B[top * nb + top];
+    const c32 bc = B[(top - 1) * nb + top] * B[top * nb + top - 1], g = 0.5f * (a - d), q = g * g + bc;
+    const float aq = sqrtf(abs2(q)), sr = sqrtf(fmaxf(0.5f * (aq + fabsf(q.re)), 1e-38f));
+    c32 sq = q.re >= 0.f ? c32(sr, 0.5f * q.im / sr) : c32(0.5f * fabsf(q.im) / sr, copysignf(sr, q.im));
+    if (g.re * sq.re + g.im * sq.im < 0.f) sq = -sq;
+    const c32 den = g + sq;
+    const float d2 = abs2(den);
+    const c32 mu = d2 > 0.f ? d - (1.f / d2) * (bc * conj(den)) : d;
+    for (int k = l; k < top; ++k) {
+      const c32 x = k == l ? B[l * nb + l] - mu : B[k * nb + k - 1];
+      const c32 y = k == l ? B[(l + 1) * nb + l] : B[(k + 1) * nb + k - 1];
+      const float ax2 = abs2(x), r2 = ax2 + abs2(y);
+      float c = 1.f;
+      c32 s(0.f, 0.f);
+      if (r2 > 0.f) {
+        const float ir = rsqrtf(r2), iax = ax2 > 0.f ? rsqrtf(ax2) : 0.f;
+        c = ax2 * iax * ir;
+        s = ax2 > 0.f ? (ir * iax) * (x * conj(y)) : ir * conj(y);
+      }
+      __syncwarp();
+      const int cb = k > l ? k - 1 : l;
+      if (lane >= cb && lane <= top) {
+        const c32 u = B[k * nb + lane], v = B[(k + 1) * nb + lane];
+        B[k * nb + lane] = c * u + s * v;
+        B[(k + 1) * nb + lane] = c * v - conj(s) * u;
+      }
+      __syncwarp();
+      if (lane >= l && lane <= min(k + 2, top)) {
+        const c32 u = B[lane * nb + k], v = B[lane * nb + k + 1];
+        B[lane * nb + k] = c * u + v * conj(s);
+        B[lane * nb + k + 1] = c * v - u * s;
+      }
+      __syncwarp();
+      if (lane == 0 && k > l) B[(k + 1) * nb + k - 1] = c32(0.f, 0.f);
+      __syncwarp();
+    }
+  }
+  if (lane <= top) shift[out + lane] = ccast<double>(B[(top - lane) * nb + top - lane]);
+  __syncwarp();
+}
+
 // Largest l in [1, hi] whose subdiagonal entry is negligible, or 0: the first warp
 // tests 32 subdiagonals at a time from hi down.  Every lane of the warp calls it.
 __device__ __forceinline__ int geig_split_point(const z64* H, int ld, int hi, double eps) {
@@ -124,7 +206,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
   // reductions; the left update runs one thread per column and the right update one
   // warp per row, so that consecutive threads touch consecutive entries.
   __shared__ double hred[32];
-  const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
+  const int lane = tid & 31, warp = tid >> 5, nwarp = (nt + 31) >> 5;
   for (int c = 0; c + 2 < p; ++c) {
     double nrm2 = 0.0;
     for (int r = c + 1 + tid; r < p; r += nt) nrm2 += abs2(H[r * ld + c]);
@@ -187,16 +269,15 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
   int iter = 0, total = 0;
   const int cap = 120 * p + 120;
   while (true) {
-    if (tid < 32) {  // the first warp finds the active block; its lane 0 sets the shift
-      int hi = sh->hi;
-      if (tid == 0) sh->active = 0;
+    if (tid < 32) {  // the first warp finds the active block and the shifts
+      int hi = sh->hi, l = 0, nb = 0;
       while (hi >= 0) {
         if (hi == 0) {
           if (tid == 0) lam[0] = H[0];
           hi = -1;
           break;
         }
-        const int l = geig_split_point(H, ld, hi, eps);
+        l = geig_split_point(H, ld, hi, eps);
         __syncwarp();
         if (tid == 0 && l > 0) H[l * ld + l - 1] = z64(0.0, 0.0);
         if (l == hi) {
@@ -205,72 +286,87 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
           iter = 0;
           continue;
         }
-        if (tid != 0) break;
-        // shift from the trailing 2x2 of the active window
-        const z64 mu = geig_shift(H[(hi - 1) * ld + hi - 1], H[(hi - 1) * ld + hi], H[hi * ld + hi - 1],
-                                  H[hi * ld + hi], iter, hi >= 2 ? zabs(H[(hi - 1) * ld + hi - 2]) : 0.0);
-        sh->mu = mu;
-        sh->l = l;
-        sh->active = 1;
+        const int size = hi - l + 1;
+        // one sweep with the 2 x 2 block's shift on short blocks, and now and then when
+        // nothing deflates (exceptional shifts)
+        nb = size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
+        if (nb > 1) {
+          geig_shifts(H, ld, hi, nb, sh->B, sh->shift);
+        } else if (tid == 0) {
+          sh->shift[0] =
+              geig_shift(H[(hi - 1) * ld + hi - 1], H[(hi - 1) * ld + hi], H[hi * ld + hi - 1], H[hi * ld + hi],
+                         iter, hi >= 2 ? zabs(H[(hi - 1) * ld + hi - 2]) : 0.0);
+        }
         break;
       }
+      ++iter;
+      total += nb;
       if (tid == 0) {
         sh->hi = hi;
-        ++iter;
-        ++total;
+        sh->l = l;
+        sh->nb = nb;
+        sh->active = nb > 0;
         if (total > cap) {
           sh->fail = 1;
           sh->active = 0;
-          sh->hi = -1;
         }
       }
     }
     __syncthreads();
     if (!sh->active) break;
-    const int l = sh->l, hi = sh->hi;
+    const int l = sh->l, hi = sh->hi, nb = sh->nb;
     const int col_end = want_vec ? p - 1 : hi;
     const int row_beg = want_vec ? 0 : l;
-    for (int k = l; k < hi; ++k) {
-      if (tid == 0) {
-        z64 x, y;
-        if (k == l) {
-          x = H[l * ld + l] - sh->mu;
-          y = H[(l + 1) * ld + l];
-        } else {
-          x = H[k * ld + k - 1];
-          y = H[(k + 1) * ld + k - 1];
+    // Sweep b is at row k_b = l + t - 2 b in step t.  The sweeps of a step act on disjoint
+    // row pairs and disjoint column pairs, and left and right rotations commute, so all row
+    // rotations and then all column rotations give what the sweeps give one after another.
+    const int steps = hi - l + 2 * (nb - 1);
+    const int ncb = (col_end - l) / 32 + 1, nrb = (hi - row_beg) / 32 + 1, nzb = want_vec ? (p - 1) / 32 + 1 : 0;
+    for (int t = 0; t < steps; ++t) {
+      if (tid < nb) {
+        const int k = l + t - 2 * tid;
+        if (k >= l && k < hi) {
+          z64 x, y;
+          if (k == l) {
+            x = H[l * ld + l] - sh->shift[tid];
+            y = H[(l + 1) * ld + l];
+          } else {
+            x = H[k * ld + k - 1];
+            y = H[(k + 1) * ld + k - 1];
+          }
+          double c;
+          z64 s;
+          givens(x, y, c, s);
+          sh->c[tid] = c;
+          sh->s[tid] = s;
         }
-        double c;
-        z64 s;
-        givens(x, y, c, s);
-        sh->c0 = z64(c, 0.0);
-        sh->s = s;
       }
       __syncthreads();
-      const double c = sh->c0.re;
-      const z64 s = sh->s;
-      // rows k, k+1: [rk; rk1] <- G [rk; rk1]
-      const int cb = (k > l) ? k - 1 : l;
-      for (int col = cb + tid; col <= col_end; col += nt) {
-        const z64 x = H[k * ld + col], y = H[(k + 1) * ld + col];
+      // rows k, k+1: [rk; rk1] <- G [rk; rk1], the annihilated entry set to zero
+      for (int w = warp; w < nb * ncb; w += nwarp) {
+        const int b = w / ncb, k = l + t - 2 * b, col = l + 32 * (w - b * ncb) + lane;
+        if (k < l || k >= hi || col > col_end || col < k - 1) continue;
+        const double c = sh->c[b];
+        const z64 s = sh->s[b], x = H[k * ld + col], y = H[(k + 1) * ld + col];
         H[k * ld + col] = c * x + s * y;
-        H[(k + 1) * ld + col] = c * y - conj(s) * x;
+        H[(k + 1) * ld + col] = k > l && col == k - 1 ? z64(0.0, 0.0) : c * y - conj(s) * x;
       }
       __syncthreads();
-      if (tid == 0 && k > l) H[(k + 1) * ld + k - 1] = z64(0.0, 0.0);
-      // columns k, k+1: H <- H G^dagger ; Z <- Z G^dagger
-      const int re = min(k + 2, hi);
-      for (int row = row_beg + tid; row <= re; row += nt) {
-        const z64 x = H[row * ld + k], y = H[row * ld + k + 1];
-        H[row * ld + k] = c * x + y * conj(s);
-        H[row * ld + k + 1] = c * y - x * s;
+      // columns k, k+1: H <- H G^dagger; Z <- Z G^dagger
+      for (int w = warp; w < nb * (nrb + nzb); w += nwarp) {
+        const int b = w / (nrb + nzb), k = l + t - 2 * b;
+        if (k < l || k >= hi) continue;
+        int q = w - b * (nrb + nzb);
+        const bool zr = q >= nrb;
+        if (zr) q -= nrb;
+        const int row = (zr ? 0 : row_beg) + 32 * q + lane;
+        if (row > (zr ? p - 1 : min(k + 2, hi))) continue;
+        z64* M = (zr ? Z : H) + row * ld;
+        const double c = sh->c[b];
+        const z64 s = sh->s[b], x = M[k], y = M[k + 1];
+        M[k] = c * x + y * conj(s);
+        M[k + 1] = c * y - x * s;
       }
-      if (want_vec)
-        for (int row = tid; row < p; row += nt) {
-          const z64 x = Z[row * ld + k], y = Z[row * ld + k + 1];
-          Z[row * ld + k] = c * x + y * conj(s);
-          Z[row * ld + k + 1] = c * y - x * s;
-        }
       __syncthreads();
     }
   }

@@ -180,18 +180,19 @@ __global__ void __launch_bounds__(OVL_THREADS, 1) k_overlaps_df(LoopArgs a) {
 // Per-loop product, eigenphases and (nested) Wannier states
 // ---------------------------------------------------------------------------
 struct LoopSmem {
-  size_t X, Y, Ms, G, lam, vec, th, key, ord, sh, red, total;
+  size_t X, Y, Ms, lam, vec, th, key, ord, sh, red, total;
 };
 
 // df: room for one overlap matrix in double-float (the mixed request's product)
-__host__ __device__ inline LoopSmem loop_layout(int p, int m, bool df = false) {
+__host__ __device__ inline LoopSmem loop_layout(int p, bool df = false) {
   auto al = [](size_t x) { return (x + 15) & ~size_t(15); };
   LoopSmem L;
   size_t o = 0;
-  L.X = o; o = al(o + size_t(p) * p * sizeof(z64));
-  L.Y = o; o = al(o + size_t(p) * p * sizeof(z64));
+  // p x p with a row length of p + 1 for the eigensolver, whose column rotations walk down a
+  // column (a row length of p would put p = 32 or 64 rows in one bank)
+  L.X = o; o = al(o + size_t(p) * (p + 1) * sizeof(z64));
+  L.Y = o; o = al(o + size_t(p) * (p + 1) * sizeof(z64));
   L.Ms = o; o = al(o + (df ? size_t(p) * p * sizeof(cdf) : 0));
-  L.G = o; o = al(o + size_t(m) * m * sizeof(z64));
   L.lam = o; o = al(o + size_t(p) * sizeof(z64));
   L.vec = o; o = al(o + size_t(p) * sizeof(z64));
   L.th = o; o = al(o + size_t(p) * sizeof(double));
@@ -207,7 +208,7 @@ __global__ void k_loops(LoopArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = a.n, p = a.p, N = a.N, tid = threadIdx.x, nt = blockDim.x;
   const int m = a.nested ? a.m : 1;
-  const LoopSmem L = loop_layout(p, m, a.df_overlaps != 0);
+  const LoopSmem L = loop_layout(p, a.df_overlaps != 0);
   z64* X = reinterpret_cast<z64*>(smem + L.X);
   z64* Y = reinterpret_cast<z64*>(smem + L.Y);
   z64* lam = reinterpret_cast<z64*>(smem + L.lam);
@@ -298,8 +299,15 @@ __global__ void k_loops(LoopArgs a) {
         z64* t = W; W = T; T = t;
       }
     }
-    // eigen-decomposition (vectors for the nested loop); Z goes to T
-    const int rc = geig(W, T, p, p, a.nested != 0, lam, vec, sh);
+    // eigen-decomposition (vectors for the nested loop): W moves to T with padded rows, the
+    // vectors take its place
+    const int ldp = p + 1;
+    for (int e = tid; e < p * p; e += nt) {
+      const int r = e / p;
+      T[e + r] = W[e];
+    }
+    __syncthreads();
+    const int rc = geig(T, W, p, ldp, a.nested != 0, lam, vec, sh);
     if (rc != 0 && tid == 0) report(a.status, ST_ENOCONV, k0, 0.0);
     for (int c = tid; c < p; c += nt) th[c] = phase_of(lam[c]);
     __syncthreads();
@@ -337,12 +345,12 @@ __global__ void k_loops(LoopArgs a) {
       if (a.min_wannier_gap) a.min_wannier_gap[i] = wg;
       if (!(wg > a.wannier_gap_tol)) report(a.status, ST_EWANGAP, k0, wg);
     }
-    // nu_0 = Z[:, sector] -> X (W no longer needed), transport with Y as scratch
-    z64* nu = (W == X) ? X : Y;
-    z64* Zm = (W == X) ? Y : X;
+    // nu_0 = Z[:, sector] -> T (no longer needed), transport with W as scratch
+    z64* nu = T;
+    z64* Zm = W;
     for (int e = tid; e < p * m; e += nt) {
       const int r = e / m, c = e - r * m;
-      nu[e] = Zm[r * p + ord[a.first + c]];
+      nu[e] = Zm[r * ldp + ord[a.first + c]];
     }
     __syncthreads();
     z64* nx = Zm;  // scratch for nu_{j+1}
@@ -453,7 +461,7 @@ cudaError_t launch_wannier(const LoopArgs& a, cudaStream_t s) {
 __global__ void k_nested(LoopArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = a.n, m = a.m, Ns = n_planes(a), Nt = a.N_t / Ns, tid = threadIdx.x, nt = blockDim.x;
-  const LoopSmem L = loop_layout(m, 1);
+  const LoopSmem L = loop_layout(m);
   z64* W = reinterpret_cast<z64*>(smem + L.X);
   z64* T = reinterpret_cast<z64*>(smem + L.Y);
   z64* lam = reinterpret_cast<z64*>(smem + L.lam);
@@ -489,7 +497,12 @@ __global__ void k_nested(LoopArgs a) {
       __syncthreads();
       z64* t = W; W = T; T = t;
     }
-    const int rc = geig(W, T, m, m, false, lam, vec, sh);
+    for (int e = tid; e < m * m; e += nt) {
+      const int r = e / m;
+      T[e + r] = W[e];  // rows of m + 1
+    }
+    __syncthreads();
+    const int rc = geig(T, nullptr, m, m + 1, false, lam, vec, sh);
     if (rc != 0 && tid == 0) report(a.status, ST_ENOCONV, b, 0.0);
     for (int c = tid; c < m; c += nt) th[c] = phase_of(lam[c]);
     __syncthreads();
@@ -1308,7 +1321,10 @@ static bool scan_nested_fit(const LoopArgs& a) {
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-static int loop_threads(int p) { return p <= 4 ? 32 : (p <= 16 ? 64 : 128); }
+static int overlap_threads(int p) { return p <= 4 ? 32 : (p <= 16 ? 64 : 128); }
+
+// Loop kernels: the sweeps of the eigensolver rotate up to GEIG_NB row pairs at once.
+static int loop_threads(int p) { return p <= 8 ? 64 : (p <= 16 ? 128 : 256); }
 
 bool loops_form_overlaps(const LoopArgs& a) { return !a.unitarise && scan_loops_fit(a); }
 
@@ -1338,7 +1354,7 @@ cudaError_t launch_overlaps(const LoopArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long cap = 152LL * 32;
   const int grid = int(K < cap ? K : cap);
-  k_overlaps<<<grid, loop_threads(a.p), sm, s>>>(a);
+  k_overlaps<<<grid, overlap_threads(a.p), sm, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1362,9 +1378,9 @@ cudaError_t launch_loops(const LoopArgs& a, cudaStream_t s) {
   // the double-float product stages one more p x p matrix; without room for it the
   // product stays in FP64
   LoopArgs b = a;
-  if (b.df_overlaps && loop_layout(b.p, b.nested ? b.m : 1, true).total > size_t(227) * 1024)
+  if (b.df_overlaps && loop_layout(b.p, true).total > size_t(227) * 1024)
     b.df_overlaps = 0;
-  const LoopSmem L = loop_layout(b.p, b.nested ? b.m : 1, b.df_overlaps != 0);
+  const LoopSmem L = loop_layout(b.p, b.df_overlaps != 0);
   static size_t cached = 0;
   cudaError_t e = set_smem_once(k_loops, L.total, cached);
   if (e != cudaSuccess) return e;
@@ -1562,7 +1578,7 @@ cudaError_t launch_nested(const LoopArgs& a, cudaStream_t s) {
     k_nested_scan<z64><<<grid, 128, Z.total, s>>>(a);
     return cudaGetLastError();
   }
-  const LoopSmem L = loop_layout(a.m, 1);
+  const LoopSmem L = loop_layout(a.m);
   const size_t sm = L.total + size_t(a.m) * a.m * sizeof(z64);
   static size_t cached = 0;
   cudaError_t e = set_smem_once(k_nested, sm, cached);
