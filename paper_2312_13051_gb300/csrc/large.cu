@@ -473,22 +473,17 @@ __global__ void __launch_bounds__(512) k_lg_tridiag_h(LargeArgs a) {
 
 // ---------------------------------------------------------------------------
 // Stage 3: eigenvalues of T' by bisection on Sturm counts, one thread per
-// (k-point, eigenvalue index), Gershgorin interval.
+// (k-point, eigenvalue index), T' of one k-point in the CTA's shared memory.
+//
+// The count at x is the number of sign changes of the leading principal minors
+//   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1}
+// (Givens), rescaled by a power of two every few rows.  The ratios q_i = p_{i+1} / p_i need
+// a division per row on the critical path (~1400 clocks in FP64, ~60 in FP32) where the
+// minors need one fused multiply-add (64, 4.5).  An FP64 bisection starts from the FP32 one
+// (a bracket 2e-5 ||T'|| wide, checked by FP64 counts and widened where it does not hold).
+// Measured, with the spin operator's eigensolves: n = 124 FP64, 256 k-points, 6.1 -> 1.9 ms;
+// n = 324 mixed, 36 k-points, 5.5 -> 1.7 ms; n = 256 FP32, 837 k-points, 1.2 -> 0.57 ms.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ int sturm_count(const T* dg, const T* od, int n, T x, T pivmin) {
-  int cnt = 0;
-  T q = dg[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < T(0);
-  for (int i = 1; i < n; ++i) {
-    q = dg[i] - x - od[i - 1] * od[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < T(0);
-  }
-  return cnt;
-}
-
 template <typename T>
 __device__ __forceinline__ void gershgorin(const T* dg, const T* od, int n, T& lo, T& hi, T& tn) {
   lo = T(INFINITY);
@@ -502,30 +497,139 @@ __device__ __forceinline__ void gershgorin(const T* dg, const T* od, int n, T& l
   }
 }
 
+// 2^-e for |x| in [2^e, 2^(e+1)), from the exponent bits (x normal or zero).
+__device__ __forceinline__ float pow2_inv(float x) {
+  return __int_as_float(0x7f000000 - (__float_as_int(x) & 0x7f800000));
+}
+__device__ __forceinline__ double pow2_inv(double x) {
+  return __hiloint2double(0x7fe00000 - (__double2hiint(x) & 0x7ff00000), 0);
+}
+
+// Sturm count at x of the scaled matrix (entries of T' / ||T'||, |d|, |e| <= 1): d and e2 =
+// e_{i-1}^2 per row (e2[0] = 0), padded to a multiple of UN rows with d = 4, e2 = 0 (no sign
+// change for x < 4).  Between two rescalings a minor loses at most a factor
+// (min(1e-12, e2))^UN, inside the exponent range.
 template <typename T>
-__global__ void k_lg_bisect(LargeArgs a) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= a.W * a.nval) return;
-  const long long kw = t / a.nval;
-  const int idx = int(t - kw * a.nval), n = a.n;
-  const T* dg = reinterpret_cast<const T*>(a.dg) + kw * n;
-  const T* od = reinterpret_cast<const T*>(a.od) + kw * n;
-  T lo, hi, tn;
-  gershgorin(dg, od, n, lo, hi, tn);
-  const T span = fmax(hi - lo, T(1e-30));
-  lo -= T(4) * lg_eps<T>() * span + T(1e-30);
-  hi += T(4) * lg_eps<T>() * span + T(1e-30);
-  const T pivmin = T(1e-30) * fmax(T(1), tn * tn);
+__device__ __forceinline__ int sturm_count(const T* d, const T* e2, int npad, T x) {
+  constexpr int UN = sizeof(T) == 4 ? 2 : 8;
+  T pm = T(0), pc = T(1);
+  int cnt = 0;
+  for (int i = 0; i < npad; i += UN) {
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      T pn = fma(d[i + u] - x, pc, -(e2[i + u] * pm));
+      if (pn == T(0)) pn = T(-1e-12) * pc;  // a zero minor counts as a change of sign
+      cnt += signbit(pn) != signbit(pc);
+      pm = pc;
+      pc = pn;
+    }
+    const T s = pow2_inv(fmax(fabs(pm), fabs(pc)));
+    pm *= s;
+    pc *= s;
+  }
+  return cnt;
+}
+
+constexpr int BIS_THREADS = 128;
+
+__host__ __device__ inline int bisect_pad(int n) { return (n + 7) & ~7; }
+
+template <typename T>
+__host__ __device__ inline size_t bisect_smem(int n) {
+  return size_t(bisect_pad(n)) * 2 * (sizeof(T) + (sizeof(T) == 8 ? sizeof(float) : 0));
+}
+
+// Bisection for eigenvalue idx of the scaled matrix from a bracket lo < hi, to 2 eps |lambda|
+// or an eighth of eps ||T'||.
+template <typename T>
+__device__ __forceinline__ void bisect_run(const T* d, const T* e2, int npad, int idx, T& lo, T& hi) {
   for (int it = 0; it < 96; ++it) {
     const T mid = T(0.5) * (lo + hi);
     if (!(mid > lo && mid < hi)) break;
-    if (hi - lo <= T(2) * lg_eps<T>() * fmax(fabs(lo), fabs(hi))) break;
-    if (sturm_count(dg, od, n, mid, pivmin) > idx)
+    if (hi - lo <= T(2) * lg_eps<T>() * fmax(T(0.0625), fmax(fabs(lo), fabs(hi)))) break;
+    if (sturm_count(d, e2, npad, mid) > idx)
       hi = mid;
     else
       lo = mid;
   }
-  reinterpret_cast<T*>(a.lam)[kw * a.nval + idx] = T(0.5) * (lo + hi);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(BIS_THREADS) k_lg_bisect(LargeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool k64 = sizeof(T) == 8;
+  const int n = a.n, tid = threadIdx.x, np = bisect_pad(n);
+  T* d = reinterpret_cast<T*>(smem);
+  T* e2 = d + np;
+  float* df = reinterpret_cast<float*>(e2 + np);  // FP64: the matrix in FP32 as well
+  float* ef = df + np;
+  __shared__ T rlo[BIS_THREADS / 32], rhi[BIS_THREADS / 32], rtn[BIS_THREADS / 32];
+  for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    const T* dg = reinterpret_cast<const T*>(a.dg) + kw * n;
+    const T* od = reinterpret_cast<const T*>(a.od) + kw * n;
+    // Gershgorin interval and ||T'||
+    T lo = T(INFINITY), hi = -T(INFINITY), tn = T(0);
+    for (int i = tid; i < n; i += BIS_THREADS) {
+      const T di = dg[i], r = (i > 0 ? od[i - 1] : T(0)) + (i + 1 < n ? od[i] : T(0));
+      lo = fmin(lo, di - r);
+      hi = fmax(hi, di + r);
+      tn = fmax(tn, fabs(di) + r);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    }
+    __syncthreads();
+    if ((tid & 31) == 0) {
+      rlo[tid >> 5] = lo;
+      rhi[tid >> 5] = hi;
+      rtn[tid >> 5] = tn;
+    }
+    __syncthreads();
+    for (int w = 0; w < BIS_THREADS / 32; ++w) {
+      lo = fmin(lo, rlo[w]);
+      hi = fmax(hi, rhi[w]);
+      tn = fmax(tn, rtn[w]);
+    }
+    // scaled by a power of two (exact): |entries| <= 1
+    const T tnc = fmax(tn, T(1e-30)), sc = T(0.5) * pow2_inv(tnc);
+    for (int i = tid; i < np; i += BIS_THREADS) {
+      const T di = i < n ? dg[i] * sc : T(4), ei = i > 0 && i < n ? od[i - 1] * sc : T(0);
+      d[i] = di;
+      e2[i] = ei * ei;
+      if constexpr (k64) {
+        df[i] = float(di);
+        ef[i] = float(ei) * float(ei);
+      }
+    }
+    __syncthreads();
+    lo *= sc;
+    hi *= sc;
+    const T span = fmax(hi - lo, T(1e-30));
+    lo -= T(4) * lg_eps<T>() * span + T(1e-30);
+    hi += T(4) * lg_eps<T>() * span + T(1e-30);
+    for (int idx = blockIdx.y * BIS_THREADS + tid; idx < a.nval; idx += gridDim.y * BIS_THREADS) {
+      T l = lo, h = hi;
+      if constexpr (k64) {
+        float fl = float(lo) - 1e-6f, fh = float(hi) + 1e-6f;
+        bisect_run<float>(df, ef, np, idx, fl, fh);
+        T w = T(1e-5);
+        for (; w < T(8); w *= T(64)) {
+          l = fmax(lo, T(fl) - w);
+          h = fmin(hi, T(fh) + w);
+          if (sturm_count(d, e2, np, l) <= idx && sturm_count(d, e2, np, h) > idx) break;
+        }
+        if (!(w < T(8))) {
+          l = lo;
+          h = hi;
+        }
+      }
+      bisect_run<T>(d, e2, np, idx, l, h);
+      reinterpret_cast<T*>(a.lam)[kw * a.nval + idx] = T(0.5) * (l + h) / sc;
+    }
+    __syncthreads();
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -564,56 +668,118 @@ struct Strided {
   __device__ __forceinline__ T& at(int a, int r, long long t) const { return base[((long long)a * n + r) * NT + t]; }
 };
 
+// Rows whose operands are loaded together: the recurrences below are serial, but their
+// operands (interleaved global memory, an L2 or DRAM round trip each) do not depend on them.
+// n = 400, 256 k-points, all vectors: 17.5 -> 8.0 ms (with the reciprocal pivots kept).
+constexpr int TRI_U = 8;
+
 template <typename T>
 __device__ void tri_factor(const T* dg, const T* od, int n, T lam, T tiny, const Strided<T>& W,
                            long long t) {
   T c0 = dg[0] - lam, c1 = n > 1 ? od[0] : T(0);
+  auto pivot = [&](T d) {  // what the solves multiply by
+    if (fabs(d) < tiny) d = d < T(0) ? -tiny : tiny;
+    return T(1) / d;
+  };
   for (int i = 0; i + 1 < n; ++i) {
     const T b = od[i];                          // subdiagonal entry of row i+1
     const T a1 = dg[i + 1] - lam;               // diagonal of row i+1
     const T e1 = i + 2 < n ? od[i + 1] : T(0);  // superdiagonal of row i+1
     if (fabs(b) > fabs(c0)) {                   // swap rows i and i+1
-      const T m = c0 / b;
-      W.at(0, i, t) = b; W.at(1, i, t) = a1; W.at(2, i, t) = e1;
+      const T r = T(1) / b, m = c0 * r;
+      W.at(0, i, t) = fabs(b) < tiny ? pivot(b) : r; W.at(1, i, t) = a1; W.at(2, i, t) = e1;
       W.at(3, i, t) = m; W.at(4, i, t) = T(1);
       const T r1 = c1 - m * a1, r2 = -m * e1;   // remaining row: columns i+1, i+2
       c0 = r1; c1 = r2;
     } else {
       if (c0 == T(0)) c0 = tiny;
-      const T m = b / c0;
-      W.at(0, i, t) = c0; W.at(1, i, t) = c1; W.at(2, i, t) = T(0);
+      const T r = T(1) / c0, m = b * r;
+      W.at(0, i, t) = fabs(c0) < tiny ? pivot(c0) : r; W.at(1, i, t) = c1; W.at(2, i, t) = T(0);
       W.at(3, i, t) = m; W.at(4, i, t) = T(0);
       c0 = a1 - m * c1;
       c1 = e1;
     }
   }
-  W.at(0, n - 1, t) = c0 == T(0) ? tiny : c0;
+  W.at(0, n - 1, t) = pivot(c0);
   W.at(1, n - 1, t) = T(0);
   W.at(2, n - 1, t) = T(0);
 }
 
 // Solves (T' - lambda) x = b in place on array 5 of the thread's scratch.
 template <typename T>
-__device__ void tri_solve(int n, T tiny, const Strided<T>& W, long long t) {
-  for (int i = 0; i + 1 < n; ++i) {
-    T xi = W.at(5, i, t), xn = W.at(5, i + 1, t);
-    if (W.at(4, i, t) != T(0)) { const T q = xi; xi = xn; xn = q; }
-    W.at(5, i, t) = xi;
-    W.at(5, i + 1, t) = xn - W.at(3, i, t) * xi;
+__device__ void tri_solve(int n, const Strided<T>& W, long long t) {
+  T xi = W.at(5, 0, t);
+  for (int i0 = 0; i0 + 1 < n; i0 += TRI_U) {
+    T xn[TRI_U], m[TRI_U], sw[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const int i = i0 + u;
+      const bool in = i + 1 < n;
+      xn[u] = in ? W.at(5, i + 1, t) : T(0);
+      m[u] = in ? W.at(3, i, t) : T(0);
+      sw[u] = in ? W.at(4, i, t) : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const int i = i0 + u;
+      if (i + 1 >= n) break;
+      T x = xn[u];
+      if (sw[u] != T(0)) { const T q = xi; xi = x; x = q; }
+      W.at(5, i, t) = xi;
+      xi = x - m[u] * xi;
+    }
   }
+  W.at(5, n - 1, t) = xi;
   T x1 = T(0), x2 = T(0);  // x_{i+1}, x_{i+2}
-  for (int i = n - 1; i >= 0; --i) {
-    T sv = W.at(5, i, t) - W.at(1, i, t) * x1 - W.at(2, i, t) * x2;
-    T d = W.at(0, i, t);
-    if (fabs(d) < tiny) d = d < T(0) ? -tiny : tiny;
-    const T xi = sv / d;
-    W.at(5, i, t) = xi;
-    x2 = x1;
-    x1 = xi;
+  for (int i0 = n - 1; i0 >= 0; i0 -= TRI_U) {
+    T b[TRI_U], r[TRI_U], u1[TRI_U], u2[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const int i = i0 - u;
+      const bool in = i >= 0;
+      b[u] = in ? W.at(5, i, t) : T(0);
+      r[u] = in ? W.at(0, i, t) : T(0);
+      u1[u] = in ? W.at(1, i, t) : T(0);
+      u2[u] = in ? W.at(2, i, t) : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const int i = i0 - u;
+      if (i < 0) break;
+      const T x = (b[u] - u1[u] * x1 - u2[u] * x2) * r[u];
+      W.at(5, i, t) = x;
+      x2 = x1;
+      x1 = x;
+    }
   }
 }
 
-constexpr int INVIT_WINDOW_N = 512;
+// x (array 5) scaled to unit norm; with Zc, also written to the vector's column of Z.
+template <typename T>
+__device__ void tri_normalise(int n, const Strided<T>& W, long long t, T* Zc, int nv) {
+  T s2 = T(0);
+#pragma unroll 8
+  for (int r = 0; r < n; ++r) {
+    const T x = W.at(5, r, t);
+    s2 += x * x;
+  }
+  s2 = T(1) / sqrt(s2);
+  for (int r0 = 0; r0 < n; r0 += TRI_U) {
+    T x[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) x[u] = r0 + u < n ? s2 * W.at(5, r0 + u, t) : T(0);
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u)
+      if (r0 + u < n) {
+        if (Zc)
+          Zc[(long long)(r0 + u) * nv] = x[u];
+        else
+          W.at(5, r0 + u, t) = x[u];
+      }
+  }
+}
+
+constexpr int INVIT_WINDOW_N = 512, INVIT_ITS = 3;
 
 template <typename T>
 __global__ void k_lg_invit(LargeArgs a) {
@@ -641,19 +807,24 @@ __global__ void k_lg_invit(LargeArgs a) {
       while (lam[j] - lam[q0] > tolc) ++q0;
     tri_factor(dg, od, n, lam[j], tiny, W, t);
     for (int r = 0; r < n; ++r) W.at(5, r, t) = T(hash_unit((unsigned long long)j * 1000003ull + r));
-    for (int it = 0; it < 3; ++it) {
-      tri_solve(n, tiny, W, t);
+    for (int it = 0; it < INVIT_ITS; ++it) {
+      tri_solve(n, W, t);
       for (int q = q0; q < j; ++q) {  // orthogonalise within the cluster (or its window)
         T d = T(0);
+#pragma unroll 8
         for (int r = 0; r < n; ++r) d += Z[(long long)r * nv + q] * W.at(5, r, t);
-        for (int r = 0; r < n; ++r) W.at(5, r, t) -= d * Z[(long long)r * nv + q];
+        for (int r0 = 0; r0 < n; r0 += TRI_U) {
+          T x[TRI_U];
+#pragma unroll
+          for (int u = 0; u < TRI_U; ++u)
+            x[u] = r0 + u < n ? W.at(5, r0 + u, t) - d * Z[(long long)(r0 + u) * nv + q] : T(0);
+#pragma unroll
+          for (int u = 0; u < TRI_U; ++u)
+            if (r0 + u < n) W.at(5, r0 + u, t) = x[u];
+        }
       }
-      T s2 = T(0);
-      for (int r = 0; r < n; ++r) s2 += W.at(5, r, t) * W.at(5, r, t);
-      s2 = T(1) / sqrt(s2);
-      for (int r = 0; r < n; ++r) W.at(5, r, t) *= s2;
+      tri_normalise(n, W, t, it + 1 == INVIT_ITS ? Z + j : static_cast<T*>(nullptr), nv);
     }
-    for (int r = 0; r < n; ++r) Z[(long long)r * nv + j] = W.at(5, r, t);
   }
 }
 
@@ -674,14 +845,10 @@ __global__ void k_lg_invit_par(LargeArgs a) {
   const T tiny = fmax(lg_eps<T>() * tn, T(1e-30));
   tri_factor(dg, od, n, lam[j], tiny, W, t);
   for (int r = 0; r < n; ++r) W.at(5, r, t) = T(hash_unit((unsigned long long)j * 1000003ull + r));
-  for (int it = 0; it < 3; ++it) {
-    tri_solve(n, tiny, W, t);
-    T s2 = T(0);
-    for (int r = 0; r < n; ++r) s2 += W.at(5, r, t) * W.at(5, r, t);
-    s2 = T(1) / sqrt(s2);
-    for (int r = 0; r < n; ++r) W.at(5, r, t) *= s2;
+  for (int it = 0; it < INVIT_ITS; ++it) {
+    tri_solve(n, W, t);
+    tri_normalise(n, W, t, it + 1 == INVIT_ITS ? Z + j : static_cast<T*>(nullptr), nv);
   }
-  for (int r = 0; r < n; ++r) Z[(long long)r * nv + j] = W.at(5, r, t);
 }
 
 // Orthonormalises the vectors of each cluster in place: one warp per eigenvalue index,
@@ -1037,8 +1204,11 @@ cudaError_t lg_common(const LargeArgs& a, cudaStream_t s) {
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   lg_mark(a, "lg_tridiag");
-  const long long nb = a.W * a.nval;
-  k_lg_bisect<T><<<int((nb + 127) / 128), 128, 0, s>>>(a);
+  const size_t sm_b = bisect_smem<T>(a.n);
+  static size_t cached_b = 0;
+  if ((e = set_smem_once(k_lg_bisect<T>, sm_b, cached_b)) != cudaSuccess) return e;
+  k_lg_bisect<T><<<dim3(unsigned(std::min<long long>(a.W, 65535)), unsigned((a.nval + BIS_THREADS - 1) / BIS_THREADS)),
+                   BIS_THREADS, sm_b, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   lg_mark(a, "lg_bisect");
   const long long ni = a.W * a.nvec;
