@@ -62,7 +62,7 @@ struct GemmPlainT {  // C = A B in the precision of T
   using TA = cx<T>;
   using TB = cx<T>;
   using Acc = cx<T>;
-  static constexpr bool kPrefetch = true;
+  static constexpr bool kPrefetch = sizeof(T) == 4;  // FP64: the pipe is busy for far longer than a load
   static __device__ __forceinline__ TA zero_a() { return TA(T(0), T(0)); }
   static __device__ __forceinline__ Acc zero() { return Acc(T(0), T(0)); }
   static __device__ __forceinline__ void mac(Acc& c, const TA& a, const TB& b) { cfma(c, a, b); }
@@ -102,13 +102,13 @@ __host__ __device__ constexpr size_t cg_smem() {
 constexpr size_t CG_SMEM = CG_K * CG_LD * (sizeof(SplitC) + sizeof(c32));  // the largest policy
 
 // C(m, c) = sum_k A(m, k) B(k, c) (the policy's product and accumulator) for m < M,
-// c < Ncol, k < K, computed by all blockDim.x == 256 threads of the CTA in 64 x 64
-// output tiles (thread (ty, tx) owns rows ty + 16 i and columns tx + 16 j).
+// c < Ncol, k < K, computed by all blockDim.x == 256 threads of the CTA in 64 x TN output
+// tiles (thread (ty, tx) owns rows ty + 16 i and columns tx + 16 j; TN = 32 or 64).
 // la(m, k) and lb(k, c) return the operands (out-of-range indices are never
 // requested); st(m, c, acc) consumes each result once.  A_K_CONTIG / B_C_CONTIG say
 // which index of the operand is contiguous in memory, so that the staging loads
 // are coalesced.  sm: cg_smem<Pol>() bytes.
-template <class Pol, bool A_K_CONTIG, bool B_C_CONTIG, class LA, class LB, class ST>
+template <class Pol, bool A_K_CONTIG, bool B_C_CONTIG, int TN = CG_TILE, class LA, class LB, class ST>
 __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned char* sm) {
   using TA = typename Pol::TA;
   using TB = typename Pol::TB;
@@ -116,23 +116,23 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
   TB(*Bs)[CG_LD] = reinterpret_cast<TB(*)[CG_LD]>(sm + CG_K * CG_LD * sizeof(TA));
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += CG_TILE)
-    for (int c0 = 0; c0 < Ncol; c0 += CG_TILE) {
-      typename Pol::Acc acc[4][4];
+    for (int c0 = 0; c0 < Ncol; c0 += TN) {
+      typename Pol::Acc acc[4][TN / 16];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = Pol::zero();
+        for (int j = 0; j < TN / 16; ++j) acc[i][j] = Pol::zero();
       // each thread moves PER elements of each operand per k-step; with Pol::kPrefetch
       // the next step's elements are loaded into registers before this step's products,
       // so that their global-memory latency overlaps the arithmetic
-      constexpr int PER = CG_K * CG_TILE / 256;
+      constexpr int PER = CG_K * CG_TILE / 256, PERB = CG_K * TN / 256;
       TA ra[PER];
-      TB rb[PER];
+      TB rb[PERB];
       auto fetch = [&](int k0) {
 #pragma unroll
         for (int s = 0; s < PER; ++s) {
           const int e = tid + 256 * s;
-          int kk, mm, cc;
+          int kk, mm;
           if (A_K_CONTIG) {
             mm = e / CG_K;
             kk = e - mm * CG_K;
@@ -141,9 +141,14 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
             mm = e - kk * CG_TILE;
           }
           ra[s] = (m0 + mm < M && k0 + kk < K) ? la(m0 + mm, k0 + kk) : Pol::zero_a();
+        }
+#pragma unroll
+        for (int s = 0; s < PERB; ++s) {
+          const int e = tid + 256 * s;
+          int kk, cc;
           if (B_C_CONTIG) {
-            kk = e / CG_TILE;
-            cc = e - kk * CG_TILE;
+            kk = e / TN;
+            cc = e - kk * TN;
           } else {
             cc = e / CG_K;
             kk = e - cc * CG_K;
@@ -155,7 +160,7 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
 #pragma unroll
         for (int s = 0; s < PER; ++s) {
           const int e = tid + 256 * s;
-          int kk, mm, cc;
+          int kk, mm;
           if (A_K_CONTIG) {
             mm = e / CG_K;
             kk = e - mm * CG_K;
@@ -164,9 +169,14 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
             mm = e - kk * CG_TILE;
           }
           As[kk][mm] = ra[s];
+        }
+#pragma unroll
+        for (int s = 0; s < PERB; ++s) {
+          const int e = tid + 256 * s;
+          int kk, cc;
           if (B_C_CONTIG) {
-            kk = e / CG_TILE;
-            cc = e - kk * CG_TILE;
+            kk = e / TN;
+            cc = e - kk * TN;
           } else {
             cc = e / CG_K;
             kk = e - cc * CG_K;
@@ -183,22 +193,22 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
 #pragma unroll 2
         for (int kk = 0; kk < CG_K; ++kk) {
           TA av[4];
-          TB bv[4];
+          TB bv[TN / 16];
 #pragma unroll
           for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx + 16 * j];
+          for (int j = 0; j < TN / 16; ++j) bv[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) Pol::mac(acc[i][j], av[i], bv[j]);
+            for (int j = 0; j < TN / 16; ++j) Pol::mac(acc[i][j], av[i], bv[j]);
         }
         __syncthreads();
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TN / 16; ++j) {
           const int gm = m0 + ty + 16 * i, gc = c0 + tx + 16 * j;
           if (gm < M && gc < Ncol) st(gm, gc, acc[i][j]);
         }

@@ -66,6 +66,7 @@ __global__ void k_lg_build(LargeArgs a) {
   const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
   const int nRs = min(md.n_R, PHASE_CACHE);
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (std::is_same<T, double>::value && a.need && !a.need[kw]) continue;
     if (a.Hin) {  // explicit matrix: lower triangle mirrored, FP64 entries kept for the refinement
       const z64* Hm = a.Hin + a.h_off[a.idx[a.k0 + kw]];
       cx<T>* A = reinterpret_cast<cx<T>*>(a.A) + kw * (long long)n * n;
@@ -94,7 +95,7 @@ __global__ void k_lg_build(LargeArgs a) {
     lg_kpoint(a, k, f);
     cx<T>* A = reinterpret_cast<cx<T>*>(a.A) + kw * (long long)n * n;
     for (long long e = tid; e < (long long)n * n; e += nt) A[e] = cx<T>(T(0), T(0));
-    if (a.Hent && md.hop_tdf) {
+    if (a.Hent && md.hop_tdf && !a.polish) {
       // mixed path: entries in double-float on the FP32 pipe (FP64-grade for the
       // refinement's residual, the FP32 matrix is the high part)
       cdf* phd = reinterpret_cast<cdf*>(phs);
@@ -131,6 +132,7 @@ __global__ void k_lg_build(LargeArgs a) {
         c32* dst = reinterpret_cast<c32*>(a.Hent + kw * (long long)md.n_ent + e);
         dst[0] = hi;
         dst[1] = lo;
+        if (a.polish) a.H64[kw * (long long)md.n_ent + e] = acc;
       }
     }
     __syncthreads();
@@ -157,6 +159,7 @@ __global__ void k_lg_tridiag(LargeArgs a) {
   __shared__ double s_nrm2, s_x0re, s_x0im;
   __shared__ int s_skip;
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (std::is_same<T, double>::value && a.need && !a.need[kw]) continue;
     cx<T>* A = reinterpret_cast<cx<T>*>(a.A) + kw * (long long)n * n;
     T* dg = reinterpret_cast<T*>(a.dg) + kw * n;
     T* od = reinterpret_cast<T*>(a.od) + kw * n;
@@ -409,6 +412,7 @@ __global__ void __launch_bounds__(512) k_lg_tridiag_h(LargeArgs a) {
   cx<T>* pw = al + n;                         // (blockDim / 32) x n per-warp accumulators
   double* red = reinterpret_cast<double*>(pw + (nt >> 5) * n);
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (std::is_same<T, double>::value && a.need && !a.need[kw]) continue;
     cx<T>* A = reinterpret_cast<cx<T>*>(a.A) + kw * (long long)n * n;
     T* dg = reinterpret_cast<T*>(a.dg) + kw * n;
     T* od = reinterpret_cast<T*>(a.od) + kw * n;
@@ -565,6 +569,7 @@ __global__ void __launch_bounds__(BIS_THREADS) k_lg_bisect(LargeArgs a) {
   float* ef = df + np;
   __shared__ T rlo[BIS_THREADS / 32], rhi[BIS_THREADS / 32], rtn[BIS_THREADS / 32];
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (std::is_same<T, double>::value && a.need && !a.need[kw]) continue;
     const T* dg = reinterpret_cast<const T*>(a.dg) + kw * n;
     const T* od = reinterpret_cast<const T*>(a.od) + kw * n;
     // Gershgorin interval and ||T'||
@@ -787,6 +792,7 @@ __global__ void k_lg_invit(LargeArgs a) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= NT) return;
   const long long kw = t / a.nvec;
+  if (std::is_same<T, double>::value && a.need && !a.need[kw]) return;
   const int idx = int(t - kw * a.nvec), n = a.n, nv = a.nvec;
   const T* dg = reinterpret_cast<const T*>(a.dg) + kw * n;
   const T* od = reinterpret_cast<const T*>(a.od) + kw * n;
@@ -888,6 +894,23 @@ __global__ void k_lg_invit_orth(LargeArgs a) {
   }
 }
 
+// Levels of T' within 1e-3 of the spectral radius of the upper edge p (lam ascending, all n).
+__device__ __forceinline__ float polish_width(const float* lam, int n) {
+  return 1e-3f * fmaxf(fabsf(lam[0]), fabsf(lam[n - 1]));
+}
+__device__ __forceinline__ int polish_upper(const float* lam, int n, int p) {
+  const float w = polish_width(lam, n);
+  int c = p;
+  while (c + 1 < n && c - p < POLISH_G && lam[c + 1] - lam[p] <= w) ++c;
+  return c - p + 1;
+}
+__device__ __forceinline__ int polish_lower(const float* lam, int n, int p) {
+  const float w = polish_width(lam, n);
+  int c = p - 1;
+  while (c > 0 && p - c <= POLISH_G && lam[p - 1] - lam[c - 1] <= w) --c;
+  return p - c;
+}
+
 // ---------------------------------------------------------------------------
 // Stage 5: back-transform x = Q D z for the first ncol eigenvectors, Q = P_0 ... P_{n-3}:
 // X = D Z, then X <- P_c X for c = n-3 down to 0 (P_c = I - 2 u_c u_c^dagger): one
@@ -906,13 +929,18 @@ __global__ void __launch_bounds__(256, 2) k_lg_backtransform(LargeArgs a, cx<To>
   if constexpr (kTc) ts = tc::setup(&tmem_slot, &tc_bar);
   const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (!kTc && a.need && !a.need[kw]) continue;
     const cx<T>* A = reinterpret_cast<const cx<T>*>(a.A) + kw * (long long)n * n;
     const cx<T>* Dp = reinterpret_cast<const cx<T>*>(a.Dp) + kw * n;
     const T* Z = reinterpret_cast<const T*>(a.Z) + kw * (long long)a.nvec * n;
     cx<To>* X = out + kw * out_stride;
+    int nc = ncol;  // columns of this k-point (the polish: the occupied ones and the upper edge's)
+    if constexpr (kTc)
+      if (a.polish)
+        nc = min(ncol, a.p + polish_upper(reinterpret_cast<const float*>(a.lam) + kw * a.nval, n, a.p));
     for (int r = tid >> 5; r < n; r += nt >> 5) {
       const cx<T> d = Dp[r];
-      for (int col = tid & 31; col < ncol; col += 32) {
+      for (int col = tid & 31; col < nc; col += 32) {
         const T z = Z[(long long)r * a.nvec + col];
         X[(long long)r * ncol + col] = cx<To>(To(d.re * z), To(d.im * z));
       }
@@ -921,7 +949,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_backtransform(LargeArgs a, cx<To>
     if constexpr (!kTc) {
       cta_reflect<T, To>(A, n, X, ncol, ncol, true, smem, pw);   // FP64-pipe bound: fewest flops
     } else if (!ts.failed) {                                     // blocked, tensor-core GEMMs
-      if (!cta_reflect_wy(A, n, X, ncol, ncol, true, smem, ts) && tid == 0)
+      if (!cta_reflect_wy(A, n, X, nc, ncol, true, smem, ts) && tid == 0)
         report(a.status, ST_ETIMEOUT, a.k0 + kw, 0.0);
     }
   }
@@ -935,6 +963,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_backtransform_wy64(LargeArgs a, z
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (a.need && !a.need[kw]) continue;
     const z64* A = reinterpret_cast<const z64*>(a.A) + kw * (long long)n * n;
     const z64* Dp = reinterpret_cast<const z64*>(a.Dp) + kw * n;
     const double* Z = reinterpret_cast<const double*>(a.Z) + kw * (long long)a.nvec * n;
@@ -954,7 +983,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_backtransform_wy64(LargeArgs a, z
 // FP64 path: direct gap from the bisection eigenvalues.
 __global__ void k_lg_gap64(LargeArgs a) {
   const long long kw = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (kw >= a.W) return;
+  if (kw >= a.W || (a.need && !a.need[kw])) return;
   const double* lam = reinterpret_cast<const double*>(a.lam) + kw * a.nval;
   const double g = a.p < a.n ? lam[a.p] - lam[a.p - 1] : INFINITY;
   const long long k = a.k0 + kw * (a.kstride > 0 ? a.kstride : 1);
@@ -1121,7 +1150,9 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
     // gap from FP64 Rayleigh quotients of the FP32 vectors p-1 and p: rho[p-1] is
     // already q^dag H q of vector p-1; H x_p by one warp per row (lanes along the row,
     // coalesced), in FP64
-    if (p < n) {
+    if (a.polish) {
+      // the polish takes the gap
+    } else if (p < n) {
       double num = 0.0, den = 0.0, den1 = 0.0;
       for (int r = warp; r < n; r += nwarp) {
         z64 hv(0.0, 0.0);
@@ -1152,6 +1183,356 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
       }
     } else if (tid == 0) {
       a.gap[k] = INFINITY;
+    }
+    __syncthreads();
+  }
+  tc::teardown(ts);
+}
+
+// ---------------------------------------------------------------------------
+// Stage 7 (FP64 request from the FP32 solve): one more Newton correction of the refined
+// block Q, now to FP64 accuracy.
+//   R = H Q - Q G, G = Q^dag H Q, and the Gram matrix in FP64; the complement's coefficients
+//   and the correction C = Q_h D Z_u [Z_u^T D^dag Q_h^dag R / (rho - lam)] in FP32 (C is the
+//   error that the first correction left, ~1e-12: FP32 keeps it to 1e-19); Q <- Q + C, then
+//   Q <- Q - Q E / 2.
+// The band edges: the largest eigenvalue of G, whose off-diagonal part is ~1e-6 ||H||, by
+// three diagonally preconditioned corrections of its edge vectors (each takes a factor
+// 1e-3 or more from their error) and their Ritz values; the smallest of the complement from
+// the FP32 vectors of the upper edge, corrected like Q but against every level outside
+// their cluster, made orthogonal to Q, by their Ritz values (error of the vectors
+// (1e-6 ||H|| / width)^2, of the values its square).
+// A k-point is left to the FP64 solve (need = 1) where this is not enough: a gap or an
+// isolation of the edge clusters below 1e-3 of the spectral radius, |C|^2 above 1e-17 (its
+// square is the error that stays), entries outside the FP32 range.
+//
+// FP64 products bound it: four n p^2 (three of them on a sparse H) of the ~16/3 n^3 + 4 n^2 p
+// that the FP64 tridiagonal solve takes, as tiled GEMMs instead of matrix-vector products.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ z64 block_csum(z64 v, double* red) {
+  const double re = block_sum(v.re, red);
+  return z64(re, block_sum(v.im, red));
+}
+
+// Y (n x g, leading dimension POLISH_G) = H X for a few columns (X, Y row-major), one warp
+// per row.
+template <class LX>
+__device__ void polish_apply(const LargeArgs& a, const z64* He, int n, int g, LX x, z64* Y) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  for (int r = warp; r < n; r += nwarp) {
+    const int q0 = a.row_ptr[r], q1 = a.row_ptr[r + 1];
+    for (int b = 0; b < g; ++b) {
+      z64 acc(0.0, 0.0);
+      for (int q = q0 + lane; q < q1; q += 32) cfma(acc, He[q], x(a.model.ent_col[q], b));
+      acc = warp_csum(acc);
+      if (lane == 0) Y[r * POLISH_G + b] = acc;
+    }
+  }
+}
+
+// Orthonormal columns: modified Gram-Schmidt, twice, on g columns of length m.
+__device__ void polish_mgs(z64* X, int m, int g, double* red) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int b = 0; b < g; ++b)
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int q = 0; q < b; ++q) {
+        z64 d(0.0, 0.0);
+        for (int r = tid; r < m; r += nt) cfma_conj(d, X[r * POLISH_G + q], X[r * POLISH_G + b]);
+        d = block_csum(d, red);
+        for (int r = tid; r < m; r += nt) cfms(X[r * POLISH_G + b], X[r * POLISH_G + q], d);
+      }
+      double s = 0.0;
+      for (int r = tid; r < m; r += nt) s += abs2(X[r * POLISH_G + b]);
+      s = 1.0 / sqrt(block_sum(s, red));
+      for (int r = tid; r < m; r += nt) X[r * POLISH_G + b] = s * X[r * POLISH_G + b];
+      __syncthreads();
+    }
+}
+
+// Extreme Ritz value of orthonormal columns X (m x g) with Y = (operator) X; E (g x g,
+// leading dimension lde, <= 1e-8) the deviation of the metric from I, S - (E S + S E) / 2.
+__device__ double polish_ritz(const z64* X, const z64* Y, int m, int g, bool want_max, const c32* E, int lde, z64* S,
+                              z64* V, JacRot<double>* rot, double* red) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int x = 0; x < g; ++x)
+    for (int y = x; y < g; ++y) {
+      z64 d(0.0, 0.0);
+      for (int r = tid; r < m; r += nt) cfma_conj(d, X[r * POLISH_G + x], Y[r * POLISH_G + y]);
+      d = block_csum(d, red);
+      if (tid == 0) {
+        S[x * g + y] = x == y ? z64(d.re, 0.0) : d;
+        if (x != y) S[y * g + x] = conj(d);
+      }
+    }
+  __syncthreads();
+  if (E) {
+    z64 d(0.0, 0.0);
+    const int x = tid / g, y = tid - x * g;
+    if (x < g)
+      for (int q = 0; q < g; ++q) {
+        cfma(d, ccast<double>(E[x * lde + q]), S[q * g + y]);
+        cfma(d, S[x * g + q], ccast<double>(E[q * lde + y]));
+      }
+    __syncthreads();
+    if (x < g) S[x * g + y] = z64(S[x * g + y].re - 0.5 * d.re, x == y ? 0.0 : S[x * g + y].im - 0.5 * d.im);
+    __syncthreads();
+  }
+  if (g > 1) jacobi_eigh<double>(S, V, g, g, 60, rot, red);
+  double e = S[0].re;
+  for (int c = 1; c < g; ++c) e = want_max ? fmax(e, S[c * g + c].re) : fmin(e, S[c * g + c].re);
+  __syncthreads();
+  return e;
+}
+
+template <int TN>
+__global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int n = a.n, p = a.p, nbt = a.nbt, nvec = a.nvec, tid = threadIdx.x, nt = blockDim.x;
+  const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
+  const DevModel& md = a.model;
+  __shared__ double red[64];
+  __shared__ z64 S[POLISH_G * POLISH_G], V[POLISH_G * POLISH_G];
+  __shared__ JacRot<double> rot[POLISH_G];
+  __shared__ double rhox[POLISH_G];
+  __shared__ uint32_t tmem_slot;
+  __shared__ __align__(8) uint64_t tc_bar;
+  tc::State ts = tc::setup(&tmem_slot, &tc_bar);
+  const int ldr = p + 4 * POLISH_G, ldc = p + POLISH_G;
+  for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    const long long k = a.k0 + kw * (a.kstride > 0 ? a.kstride : 1);
+    const c32* A = reinterpret_cast<const c32*>(a.A) + kw * (long long)n * n;
+    const c32* Dp = reinterpret_cast<const c32*>(a.Dp) + kw * n;
+    const float* Z = reinterpret_cast<const float*>(a.Z) + kw * (long long)nvec * n;
+    const float* lam = reinterpret_cast<const float*>(a.lam) + kw * a.nval;
+    const c32* X = reinterpret_cast<const c32*>(a.X) + kw * (long long)n * nbt;
+    const z64* He = a.H64 + kw * (long long)md.n_ent;
+    z64* Q = a.U + kw * (long long)n * p;
+    z64* R = a.R64 + kw * (long long)n * ldr;          // H Q, later small blocks
+    c32* C = a.C32 + kw * (long long)n * ldc;          // corrections: occupied, then upper edge
+    z64* G = a.G64 + kw * ((long long)p * p + ((long long)p * p + 1) / 2);  // Q^dag H Q
+    c32* E = reinterpret_cast<c32*>(G + (long long)p * p);  // Q^dag Q - I
+    const float width = polish_width(lam, n), nrm = 1e3f * width;
+    const int g = polish_upper(lam, n, p), gl = polish_lower(lam, n, p);
+    const bool fit = nrm > 1e-8f && nrm < 1e12f && lam[p] - lam[p - 1] > width && g <= POLISH_G && gl <= POLISH_G &&
+                     p + g <= nbt;
+    if (!fit) {  // uniform over the CTA
+      if (tid == 0) a.need[kw] = 1;
+      continue;
+    }
+    // R = H Q
+    if (md.n_ent == n * n) {
+      cta_gemm<GemmPlainT<double>, true, true, TN>(
+          n, p, n, [&](int r, int q) { return He[(long long)r * n + q]; },
+          [&](int q, int c) { return Q[(long long)q * p + c]; },
+          [&](int r, int c, const z64& v) { R[(long long)r * ldr + c] = v; }, smem);
+    } else {
+      for (int r = warp; r < n; r += nwarp) {
+        const int q0 = a.row_ptr[r], q1 = a.row_ptr[r + 1];
+        for (int c = lane; c < p; c += 32) {
+          z64 acc(0.0, 0.0);
+          for (int q = q0; q < q1; ++q) cfma(acc, He[q], Q[(long long)md.ent_col[q] * p + c]);
+          R[(long long)r * ldr + c] = acc;
+        }
+      }
+    }
+    __syncthreads();
+    cta_gemm<GemmPlainT<double>, false, true, TN>(
+        p, p, n, [&](int x, int r) { return conj(Q[(long long)r * p + x]); },
+        [&](int r, int y) { return R[(long long)r * ldr + y]; },
+        [&](int x, int y, const z64& v) { G[(long long)x * p + y] = x == y ? z64(v.re, 0.0) : v; }, smem);
+    __syncthreads();
+    cta_gemm<GemmPlainT<double>, true, true, TN>(
+        n, p, p, [&](int r, int q) { return Q[(long long)r * p + q]; },
+        [&](int q, int c) { return G[(long long)q * p + c]; },
+        [&](int r, int c, const z64& v) { C[(long long)r * ldc + c] = ccast<float>(R[(long long)r * ldr + c] - v); },
+        smem);
+    __syncthreads();
+    // residuals of the upper edge's FP32 vectors x_b
+    z64* XU = R;                            // n x POLISH_G blocks in the R workspace
+    z64* YU = XU + (long long)n * POLISH_G;
+    z64* XL = YU + (long long)n * POLISH_G; // p x POLISH_G
+    z64* YL = XL + (long long)n * POLISH_G;
+    polish_apply(a, He, n, g, [&](int q, int b) { return ccast<double>(X[(long long)q * nbt + p + b]); }, YU);
+    __syncthreads();
+    for (int b = 0; b < g; ++b) {
+      double num = 0.0, den = 0.0;
+      for (int r = tid; r < n; r += nt) {
+        const z64 x = ccast<double>(X[(long long)r * nbt + p + b]), h = YU[r * POLISH_G + b];
+        num += x.re * h.re + x.im * h.im;
+        den += abs2(x);
+      }
+      num = block_sum(num, red);
+      den = block_sum(den, red);
+      const double rho = num / den;
+      if (tid == 0) rhox[b] = rho;
+      for (int r = tid; r < n; r += nt)
+        C[(long long)r * ldc + p + b] =
+            ccast<float>(YU[r * POLISH_G + b] - rho * ccast<double>(X[(long long)r * nbt + p + b]));
+    }
+    __syncthreads();
+    // C <- D^dag Q_h^dag C
+    bool tc_ok = cta_reflect_wy(A, n, C, p + g, ldc, false, smem, ts);
+    for (int r = warp; r < n; r += nwarp) {
+      const c32 d = conj(Dp[r]);
+      for (int c = lane; c < p + g; c += 32) C[(long long)r * ldc + c] = d * C[(long long)r * ldc + c];
+    }
+    __syncthreads();
+    // coefficients: occupied columns over the levels from p on, edge columns over every level
+    // outside their cluster
+    c32* coef = reinterpret_cast<c32*>(YL + (long long)n * POLISH_G);  // (n - p) x p, then n x POLISH_G
+    c32* coefx = reinterpret_cast<c32*>(XL);
+    const int nu = n - p;
+    tc_ok = tc_ok && cta_cgemm_tc<false, true>(
+        nu, p, n, [&](int ua, int r) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
+        [&](int r, int c) { return C[(long long)r * ldc + c]; },
+        [&](int ua, int c, c32 v) {
+          coef[(long long)ua * p + c] = float(1.0 / (G[(long long)c * p + c].re - double(lam[p + ua]))) * v;
+        },
+        smem, ts);
+    for (int q = tid; q < n * g; q += nt) {
+      const int b = q / n, l = q - b * n;
+      c32 acc(0.f, 0.f);
+      if (l < p || l >= p + g) {
+        for (int r = 0; r < n; ++r) {
+          const float z = Z[(long long)r * nvec + l];
+          const c32 c = C[(long long)r * ldc + p + b];
+          acc.re = fmaf(z, c.re, acc.re);
+          acc.im = fmaf(z, c.im, acc.im);
+        }
+        // (a level just outside the cluster may come close to a far member of it; the edge
+        // itself is a width away)
+        const double dl = rhox[b] - double(lam[l]);
+        acc = fabs(dl) > 0.1 * double(width) ? float(1.0 / dl) * acc : c32(0.f, 0.f);
+      }
+      coefx[l * POLISH_G + b] = acc;
+    }
+    __syncthreads();
+    // C = Q_h D Z coef
+    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+        n, p, nu, [&](int r, int ua) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
+        [&](int ua, int c) { return coef[(long long)ua * p + c]; },
+        [&](int r, int c, c32 v) { C[(long long)r * ldc + c] = Dp[r] * v; }, smem, ts);
+    for (int r = warp; r < n; r += nwarp)
+      for (int b = 0; b < g; ++b) {
+        c32 acc(0.f, 0.f);
+        for (int l = lane; l < n; l += 32) {
+          const float z = Z[(long long)r * nvec + l];
+          const c32 c = coefx[l * POLISH_G + b];
+          acc.re = fmaf(z, c.re, acc.re);
+          acc.im = fmaf(z, c.im, acc.im);
+        }
+        acc = warp_csum(acc);
+        if (lane == 0) C[(long long)r * ldc + p + b] = Dp[r] * acc;
+      }
+    __syncthreads();
+    tc_ok = tc_ok && cta_reflect_wy(A, n, C, p + g, ldc, true, smem, ts);
+    __syncthreads();
+    // Q <- Q + C; |C|^2
+    double c2 = 0.0;
+    for (int r = warp; r < n; r += nwarp)
+      for (int c = lane; c < p; c += 32) {
+        const c32 d = C[(long long)r * ldc + c];
+        z64& q = Q[(long long)r * p + c];
+        q = z64(q.re + double(d.re), q.im + double(d.im));
+        c2 += double(abs2(d));
+      }
+    c2 = block_sum(c2, red);
+    // E = Q^dag Q - I
+    double emax = 0.0;
+    cta_gemm<GemmPlainT<double>, false, true, TN>(
+        p, p, n, [&](int x, int r) { return conj(Q[(long long)r * p + x]); },
+        [&](int r, int y) { return Q[(long long)r * p + y]; },
+        [&](int x, int y, const z64& v) {
+          const c32 e(float(v.re - (x == y ? 1.0 : 0.0)), x == y ? 0.f : float(v.im));
+          emax = fmax(emax, double(abs2(e)));
+          E[(long long)x * p + y] = e;
+        },
+        smem);
+    emax = -block_min(-emax, red);
+    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+        n, p, p, [&](int r, int q) { return ccast<float>(Q[(long long)r * p + q]); },
+        [&](int q, int c) { return E[(long long)q * p + c]; },
+        [&](int r, int c, c32 v) { C[(long long)r * ldc + c] = v; }, smem, ts);
+    __syncthreads();
+    for (int r = warp; r < n; r += nwarp)
+      for (int c = lane; c < p; c += 32) {
+        const c32 d = C[(long long)r * ldc + c];
+        z64& q = Q[(long long)r * p + c];
+        q = z64(q.re - 0.5 * double(d.re), q.im - 0.5 * double(d.im));
+      }
+    if (!tc_ok && tid == 0) report(a.status, ST_ETIMEOUT, k, 0.0);
+    if (!(c2 <= 1e-17) || !(emax <= 1e-16)) {  // uniform (block reductions)
+      if (tid == 0) a.need[kw] = 1;
+      __syncthreads();
+      continue;
+    }
+    __syncthreads();
+    // lower edge: vectors of G's last gl columns
+    for (int e = tid; e < p * gl; e += nt) {
+      const int r = e / gl, b = e - r * gl;
+      XL[r * POLISH_G + b] = z64(double(r == p - gl + b), 0.0);
+    }
+    __syncthreads();
+    auto apply_g = [&]() {
+      for (int r = warp; r < p; r += nwarp)
+        for (int b = 0; b < gl; ++b) {
+          z64 acc(0.0, 0.0);
+          for (int q = lane; q < p; q += 32) cfma(acc, G[(long long)r * p + q], XL[q * POLISH_G + b]);
+          acc = warp_csum(acc);
+          if (lane == 0) YL[r * POLISH_G + b] = acc;
+        }
+      __syncthreads();
+    };
+    for (int it = 0; it < 3; ++it) {
+      apply_g();
+      for (int e = tid; e < p * gl; e += nt) {
+        const int r = e / gl, b = e - r * gl;
+        const double rho = G[(long long)(p - gl + b) * p + p - gl + b].re;
+        if (r < p - gl) {
+          const double dl = rho - G[(long long)r * p + r].re;
+          const double w = fabs(dl) > 0.1 * double(width) ? 1.0 / dl : 0.0;
+          const z64 res = YL[r * POLISH_G + b] - rho * XL[r * POLISH_G + b];
+          XL[r * POLISH_G + b] = XL[r * POLISH_G + b] + w * res;
+        }
+      }
+      __syncthreads();
+    }
+    polish_mgs(XL, p, gl, red);
+    apply_g();
+    // (the columns that G was formed with were orthonormal to E)
+    const double top = polish_ritz(XL, YL, p, gl, true, E + (long long)(p - gl) * p + p - gl, p, S, V, rot, red);
+    // upper edge: the corrected vectors, orthogonal to Q
+    for (int e = tid; e < n * g; e += nt) {
+      const int r = e / g, b = e - r * g;
+      const c32 x = X[(long long)r * nbt + p + b], c = C[(long long)r * ldc + p + b];
+      XU[r * POLISH_G + b] = z64(double(x.re) + double(c.re), double(x.im) + double(c.im));
+    }
+    __syncthreads();
+    for (int c = warp; c < p; c += nwarp)  // overlaps Q^dag x in XL
+      for (int b = 0; b < g; ++b) {
+        z64 acc(0.0, 0.0);
+        for (int r = lane; r < n; r += 32) cfma_conj(acc, Q[(long long)r * p + c], XU[r * POLISH_G + b]);
+        acc = warp_csum(acc);
+        if (lane == 0) XL[c * POLISH_G + b] = acc;
+      }
+    __syncthreads();
+    for (int r = warp; r < n; r += nwarp)
+      for (int b = 0; b < g; ++b) {
+        z64 acc(0.0, 0.0);
+        for (int c = lane; c < p; c += 32) cfma(acc, Q[(long long)r * p + c], XL[c * POLISH_G + b]);
+        acc = warp_csum(acc);
+        if (lane == 0) XU[r * POLISH_G + b] = XU[r * POLISH_G + b] - acc;
+      }
+    __syncthreads();
+    polish_mgs(XU, n, g, red);
+    polish_apply(a, He, n, g, [&](int q, int b) { return XU[q * POLISH_G + b]; }, YU);
+    __syncthreads();
+    const double bot = polish_ritz(XU, YU, n, g, false, static_cast<c32*>(nullptr), 0, S, V, rot, red);
+    if (tid == 0) {
+      const double gp = bot - top;
+      a.gap[k] = gp;
+      a.need[kw] = 0;
+      if (!(gp > a.gap_tol)) report(a.status, ST_EGAP, k, gp);
     }
     __syncthreads();
   }
@@ -1274,6 +1655,19 @@ cudaError_t launch_states_large(const LargeArgs& a, cudaStream_t s) {
   k_lg_refine<<<lg_grid(a.W), LG_THREADS, smr, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   lg_mark(a, "lg_refine");
+  if (a.polish) {
+    const size_t smp = std::max(std::max(reflect_wy_smem(), tc::SMEM), cg_smem<GemmPlainT<double>>());
+    static size_t cached_p32 = 0, cached_p64 = 0;
+    if (a.p <= 32) {
+      if ((e = set_smem_once(k_lg_polish<32>, smp, cached_p32)) != cudaSuccess) return e;
+      k_lg_polish<32><<<lg_grid(a.W), LG_THREADS, smp, s>>>(a);
+    } else {
+      if ((e = set_smem_once(k_lg_polish<64>, smp, cached_p64)) != cudaSuccess) return e;
+      k_lg_polish<64><<<lg_grid(a.W), LG_THREADS, smp, s>>>(a);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    lg_mark(a, "lg_polish");
+  }
   return cudaSuccess;
 }
 

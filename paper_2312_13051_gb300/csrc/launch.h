@@ -114,6 +114,7 @@ struct LargeArgs {
   long long k0, W;
   long long kstride;      // k-point of wave slot kw: k0 + kw * kstride (0 means 1)
   int mixed;
+  int polish;             // FP64 request from the FP32 solve (mixed = 1): one more correction, in FP64
   double gap_tol;
   // wave scratch
   void* A;                // W x n x n complex (T)
@@ -128,6 +129,9 @@ struct LargeArgs {
   z64* R64;               // W x n x p (mixed)
   c32* C32;               // W x n x p (mixed)
   z64* G64;               // W x p x p (mixed)
+  z64* H64;               // W x n_ent (polish): the FP64 entries
+  int* need;              // W: set by the polish where a k-point needs the FP64 solve; a plain
+                          // FP64 run (mixed = 0) with need set solves only those
   const int* row_ptr;     // n + 1: first entry of each row in the plan
   // outputs
   z64* U;                 // W x n x p (wave-relative)
@@ -145,6 +149,11 @@ struct LargeArgs {
   int no_refine;          // mixed path without a block to refine (p = 0)
   int subspace_only;      // only the span of the nvec vectors matters (parallel clusters)
 };
+
+// Levels that a band edge of the polish may hold within 1e-3 of the spectral radius.
+constexpr int POLISH_G = 8;
+// Largest n of the polish (its scratch and its FP32 start are measured up to here).
+constexpr int POLISH_N_MAX = 512;
 
 // Outputs of the batched eigensolve for one wave of the large path.
 struct EighScatterArgs {

@@ -509,6 +509,98 @@ bw::DevPlane dev_plane(const PlaneX& X) {
   return d;
 }
 
+// Scratch of the large-n solver per wave slot (every array a multiple of 256 bytes) and its
+// binding to one block.  An FP64 request up to POLISH_N_MAX bands runs the FP32 solve and
+// the FP64 polish, and the FP64 solve for the k-points that need it: the two use the block
+// one after the other, so the slot takes the larger of the two layouts.
+struct LargePlan {
+  int n = 0, p = 0, n_ent = 0;
+  bool mx = false, polish = false;
+  // FP32 (mixed) and FP64 layouts
+  size_t bytes_of(bool f32) const {
+    const size_t ts = f32 ? sizeof(float) : sizeof(double);
+    const size_t nval = f32 ? n : std::min(n, p + 1), nvec = f32 ? n : p, nb = nbt(f32);
+    size_t b = al256(size_t(n) * n * 2 * ts) + 2 * al256(size_t(n) * ts) + al256(size_t(n) * 2 * ts) +
+               al256(nval * ts) + al256(nvec * n * ts) + al256(nvec * 6 * n * ts);
+    if (f32) {
+      b += al256(n * nb * sizeof(bw::c32)) + al256(size_t(n_ent) * sizeof(z64)) + r64() + c32() + g64();
+      if (polish) b += al256(size_t(n_ent) * sizeof(z64));
+    }
+    return b;
+  }
+  int nbt(bool f32) const { return f32 ? std::min(n, p + (polish ? bw::POLISH_G : 1)) : p; }
+  size_t r64() const { return al256(size_t(n) * (p + (polish ? 4 * bw::POLISH_G : 0)) * sizeof(z64)); }
+  size_t c32() const { return al256(size_t(n) * (p + (polish ? bw::POLISH_G : 0)) * sizeof(bw::c32)); }
+  size_t g64() const { return al256(size_t(p) * p * sizeof(z64) + (polish ? (size_t(p) * p + 1) / 2 * sizeof(z64) : 0)); }
+  size_t bytes() const {
+    if (!polish) return bytes_of(mx);
+    return std::max(bytes_of(true), bytes_of(false)) + 256;  // and the slot's need flag
+  }
+  LargePlan(int n_, int p_, int n_ent_, bool mx_) : n(n_), p(p_), n_ent(n_ent_), mx(mx_) {
+    polish = !mx && p < n && n <= bw::POLISH_N_MAX;
+  }
+  // Without room for one slot of the larger layout beside `others` bytes, the FP64 solve alone.
+  void fit(size_t avail, size_t others) {
+    if (polish && bytes() + others > avail) polish = false;
+  }
+  void bind(bw::LargeArgs& lg, char* base, long long W, bool f32) const {
+    const size_t ts = f32 ? sizeof(float) : sizeof(double);
+    auto take = [&](size_t per) {
+      char* q = base;
+      base += size_t(W) * per;
+      return q;
+    };
+    lg.n = n;
+    lg.p = p;
+    lg.nval = f32 ? n : std::min(n, p + 1);
+    lg.nvec = f32 ? n : p;
+    lg.nbt = nbt(f32);
+    lg.mixed = f32;
+    lg.polish = f32 && polish;
+    lg.A = take(al256(size_t(n) * n * 2 * ts));
+    lg.dg = take(al256(size_t(n) * ts));
+    lg.od = take(al256(size_t(n) * ts));
+    lg.Dp = take(al256(size_t(n) * 2 * ts));
+    lg.lam = take(al256(size_t(lg.nval) * ts));
+    lg.Z = take(al256(size_t(lg.nvec) * n * ts));
+    lg.work = take(al256(size_t(lg.nvec) * 6 * n * ts));
+    if (f32) {
+      lg.X = take(al256(size_t(n) * lg.nbt * sizeof(bw::c32)));
+      lg.Hent = reinterpret_cast<z64*>(take(al256(size_t(n_ent) * sizeof(z64))));
+      lg.R64 = reinterpret_cast<z64*>(take(r64()));
+      lg.C32 = reinterpret_cast<bw::c32*>(take(c32()));
+      lg.G64 = reinterpret_cast<z64*>(take(g64()));
+      if (polish) lg.H64 = reinterpret_cast<z64*>(take(al256(size_t(n_ent) * sizeof(z64))));
+    }
+  }
+  // Both argument sets of a wave on the block at `base` (W slots): `lg` as the first (or
+  // only) solve, `fix` the FP64 solve of what the polish leaves (unused without it).
+  void bind_all(bw::LargeArgs& lg, bw::LargeArgs& fix, char* base, long long W) const {
+    fix = lg;
+    if (polish) {
+      int* need = reinterpret_cast<int*>(base + size_t(W) * (bytes() - 256));
+      bind(fix, base, W, false);
+      fix.need = need;
+      lg.need = need;
+    }
+    bind(lg, base, W, mx || polish);
+  }
+};
+
+// One wave on the arguments of LargePlan::bind_all.
+cudaError_t launch_large_wave(bw::LargeArgs& lg, bw::LargeArgs& fix, long long k0, long long W, z64* U,
+                              cudaStream_t s) {
+  lg.k0 = k0;
+  lg.W = W;
+  lg.U = U;
+  const cudaError_t e = bw::launch_states_large(lg, s);
+  if (e != cudaSuccess || !lg.polish) return e;
+  fix.k0 = k0;
+  fix.W = W;
+  fix.U = U;
+  return bw::launch_states_large(fix, s);
+}
+
 // Projected-spin split of waves of occupied blocks (Sec. IV) for n > 32: the
 // occupied-space operator S = U^dagger (sigma s U) of every k-point of a wave by one
 // sparse application and one batched GEMM, its FP64 eigen-decomposition on the
@@ -643,26 +735,17 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   const bool spin = op != nullptr;
   const int pl = spin ? p / 2 : p;  // columns the loop runs on
   const long long K = (long long)N * Nt;
-  const size_t ts = mx ? sizeof(float) : sizeof(double);
-  const int nval = mx ? n : std::min(n, p + 1), nvec = mx ? n : p;
-  const int nbt = mx ? std::min(n, p + 1) : p;
-  const size_t sz_A = al256(size_t(n) * n * 2 * ts), sz_v = al256(size_t(n) * ts),
-               sz_D = al256(size_t(n) * 2 * ts), sz_lam = al256(size_t(nval) * ts),
-               sz_Z = al256(size_t(nvec) * n * ts), sz_wk = al256(size_t(nvec) * 6 * n * ts),
-               sz_X = mx ? al256(size_t(n) * nbt * sizeof(bw::c32)) : 0,
-               sz_He = mx ? al256(size_t(P.n_ent) * sizeof(z64)) : 0,
-               sz_R = mx ? al256(size_t(n) * p * sizeof(z64)) : 0,
-               sz_C = mx ? al256(size_t(n) * p * sizeof(bw::c32)) : 0,
-               sz_G = mx ? al256(size_t(p) * p * sizeof(z64)) : 0;
+  LargePlan LP(n, p, P.n_ent, mx);
   // spin split, per wave slot: the occupied block and the split's scratch
   const size_t sp_U = spin ? al256(size_t(n) * p * sizeof(z64)) : 0;
-  const size_t per_k = sz_A + 2 * sz_v + sz_D + sz_lam + sz_Z + sz_wk + sz_X + sz_He + sz_R + sz_C +
-                       sz_G + sp_U + (spin ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
+  const size_t sp_k = sp_U + (spin ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
   const size_t bUk = size_t(n) * pl * sizeof(z64), bPk = size_t(pl) * pl * sizeof(z64);
   const size_t bEl = size_t(pl) * (2 * sizeof(z64) + sizeof(double) + sizeof(int)) + 8 * sizeof(double);
   const size_t per_loop = size_t(N) * (bUk + bPk) + 2 * bPk + bEl;
   size_t total = al256(blob.data.size()) + (spin ? 2 : 1) * al256(size_t(K) * sizeof(double)) + 48 * 256;
   const size_t avail = ctx->budget > total ? ctx->budget - total : 0;
+  LP.fit(avail, sp_k + per_loop);
+  const size_t per_k = LP.bytes() + sp_k;
   long long Wv = std::min<long long>(K, 2048);
   while (Wv > 1 && size_t(Wv) * per_k + per_loop > avail) Wv /= 2;
   const size_t left = avail > size_t(Wv) * per_k ? avail - size_t(Wv) * per_k : 0;
@@ -685,37 +768,18 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   int* e_ord = reinterpret_cast<int*>(carve(ctx, nl_max * size_t(pl) * sizeof(int)));
   double* e_ctl = reinterpret_cast<double*>(carve(ctx, nl_max * 8 * sizeof(double)));
 
-  bw::LargeArgs lg;
+  bw::LargeArgs lg, fix;
   std::memset(&lg, 0, sizeof(lg));
   lg.model = dev_model(P, dblob);
   lg.plane = dev_plane(PX);
-  lg.n = n;
-  lg.p = p;
-  lg.nval = nval;
-  lg.nvec = nvec;
-  lg.nbt = nbt;
-  lg.mixed = mx;
   lg.gap_tol = o.gap_tol;
   lg.row_ptr = reinterpret_cast<const int*>(dblob + P.o_rowptr);
   lg.gap = gap;
   lg.status = ctx->status;
-  lg.A = carve(ctx, Wv * sz_A);
-  lg.dg = carve(ctx, Wv * sz_v);
-  lg.od = carve(ctx, Wv * sz_v);
-  lg.Dp = carve(ctx, Wv * sz_D);
-  lg.lam = carve(ctx, Wv * sz_lam);
-  lg.Z = carve(ctx, Wv * sz_Z);
-  lg.work = carve(ctx, Wv * sz_wk);
-  if (mx) {
-    lg.X = carve(ctx, Wv * sz_X);
-    lg.Hent = reinterpret_cast<z64*>(carve(ctx, Wv * sz_He));
-    lg.R64 = reinterpret_cast<z64*>(carve(ctx, Wv * sz_R));
-    lg.C32 = reinterpret_cast<bw::c32*>(carve(ctx, Wv * sz_C));
-    lg.G64 = reinterpret_cast<z64*>(carve(ctx, Wv * sz_G));
-  }
   MarkHook hook{ctx, s};
   lg.mark = mark_hook;
   lg.mark_user = &hook;
+  LP.bind_all(lg, fix, reinterpret_cast<char*>(carve(ctx, Wv * LP.bytes())), Wv);
   // spin split of a wave: the wave's occupied blocks, then the sector states
   z64* Uw = nullptr;
   PsoSplit X;
@@ -732,10 +796,7 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
     const long long kb = (long long)i0 * N, Kb = (long long)nl * N;
     for (long long w0 = 0; w0 < Kb; w0 += Wv) {
       const long long Wn = std::min(Wv, Kb - w0);
-      lg.k0 = kb + w0;
-      lg.W = Wn;
-      lg.U = spin ? Uw : Ublk + w0 * sU;
-      BW_CUDA(bw::launch_states_large(lg, s), "large-n states kernels");
+      BW_CUDA(launch_large_wave(lg, fix, kb + w0, Wn, spin ? Uw : Ublk + w0 * sU, s), "large-n states kernels");
       if (!spin) continue;
       if ((st = pso_split_wave(ctx, X, Uw, Wn, kb + w0, Ublk + w0 * sU, s))) return st;
       prof_mark(ctx, s, "pso_split");
@@ -904,20 +965,11 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
   size_t total = al256(blob.data.size()) + bU + bGap + bM + bW + bNu + bPso + 2 * bLink + 4096;
   // large n: per-k-point scratch of the tridiagonal solver, processed in waves
   const bool mx = prec == BW_MIXED;
-  const size_t ts = mx ? sizeof(float) : sizeof(double);
-  const int nval = mx ? n : std::min(n, p + 1), nvec = mx ? n : p;
-  const int nbt = mx ? std::min(n, p + 1) : p;
-  const size_t sz_A = al256(size_t(n) * n * 2 * ts), sz_v = al256(size_t(n) * ts),
-               sz_D = al256(size_t(n) * 2 * ts), sz_lam = al256(size_t(nval) * ts),
-               sz_Z = al256(size_t(nvec) * n * ts), sz_wk = al256(size_t(nvec) * 6 * n * ts),
-               sz_X = mx ? al256(size_t(n) * nbt * sizeof(bw::c32)) : 0,
-               sz_He = mx ? al256(size_t(P.n_ent) * sizeof(z64)) : 0,
-               sz_R = mx ? al256(size_t(n) * p * sizeof(z64)) : 0,
-               sz_C = mx ? al256(size_t(n) * p * sizeof(bw::c32)) : 0,
-               sz_G = mx ? al256(size_t(p) * p * sizeof(z64)) : 0,
-               sz_Uf = spin ? al256(size_t(n) * p * sizeof(z64)) : 0;
-  const size_t per_k = sz_A + 2 * sz_v + sz_D + sz_lam + sz_Z + sz_wk + sz_X + sz_He + sz_R + sz_C +
-                       sz_G + sz_Uf + (spin && large ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
+  LargePlan LP(n, p, P.n_ent, mx);
+  const size_t sz_Uf = spin ? al256(size_t(n) * p * sizeof(z64)) : 0;
+  const size_t sp_k = sz_Uf + (spin && large ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
+  LP.fit(ctx->budget > total ? ctx->budget - total : 0, sp_k);
+  const size_t per_k = LP.bytes() + sp_k;
   long long Wv = 0;
   if (large) {
     const size_t avail = ctx->budget > total ? (ctx->budget - total) / 2 : 0;
@@ -990,49 +1042,29 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
   } else if (!large) {
     BW_CUDA(bw::launch_states_small(sa, p_eff, s), "states kernel");
   } else {
-    bw::LargeArgs lg;
+    bw::LargeArgs lg, fix;
     std::memset(&lg, 0, sizeof(lg));
     lg.model = sa.model;
     lg.plane = sa.plane;
-    lg.n = n;
-    lg.p = p;
-    lg.nval = nval;
-    lg.nvec = nvec;
-    lg.nbt = nbt;
-    lg.mixed = mx;
     lg.gap_tol = o.gap_tol;
     lg.row_ptr = reinterpret_cast<const int*>(dblob + P.o_rowptr);
     lg.gap = gap;
     lg.status = ctx->status;
-    lg.A = carve(ctx, Wv * sz_A);
-    lg.dg = carve(ctx, Wv * sz_v);
-    lg.od = carve(ctx, Wv * sz_v);
-    lg.Dp = carve(ctx, Wv * sz_D);
-    lg.lam = carve(ctx, Wv * sz_lam);
-    lg.Z = carve(ctx, Wv * sz_Z);
-    lg.work = carve(ctx, Wv * sz_wk);
-    if (mx) {
-      lg.X = carve(ctx, Wv * sz_X);
-      lg.Hent = reinterpret_cast<z64*>(carve(ctx, Wv * sz_He));
-      lg.R64 = reinterpret_cast<z64*>(carve(ctx, Wv * sz_R));
-      lg.C32 = reinterpret_cast<bw::c32*>(carve(ctx, Wv * sz_C));
-      lg.G64 = reinterpret_cast<z64*>(carve(ctx, Wv * sz_G));
-    }
+    char* lbase = reinterpret_cast<char*>(carve(ctx, Wv * LP.bytes()));
     z64* Ufull = reinterpret_cast<z64*>(carve(ctx, Wv * sz_Uf));
     PsoSplit X;
     MarkHook hook{ctx, s};
     lg.mark = mark_hook;
     lg.mark_user = &hook;
+    LP.bind_all(lg, fix, lbase, Wv);
     if (spin && (st = pso_split_setup(ctx, X, Wv, n, p, op, dblob, sign, o.pso_gap_tol, pso_evals, psog,
                                       &hook, s)))
       return st;
     X.median = o.pso_median;
     for (long long k0 = 0; k0 < K; k0 += Wv) {
-      lg.k0 = k0;
-      lg.W = std::min(Wv, K - k0);
       // the wave's occupied blocks go straight to U, or through the spin split
-      lg.U = spin ? Ufull : U + k0 * (long long)n * p;
-      BW_CUDA(bw::launch_states_large(lg, s), "large-n states kernels");
+      BW_CUDA(launch_large_wave(lg, fix, k0, std::min(Wv, K - k0), spin ? Ufull : U + k0 * (long long)n * p, s),
+              "large-n states kernels");
       if (spin) {
         if ((st = pso_split_wave(ctx, X, Ufull, lg.W, k0, U + k0 * (long long)n * p_eff, s))) return st;
         prof_mark(ctx, s, "pso_split");

@@ -259,7 +259,7 @@ __device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const
 // an error of (eps32 ||H|| / width)^2 in the vectors and its square in the Ritz values of
 // the cluster, taken after Cholesky-QR.  Y, HY: n x g scratch, G, Zg: g x g.
 __device__ double edge_energy(const z64* H, const c32* V, const int* ord, const double* lam, int n, int c0, int c1,
-                              bool want_max, z64* Y, z64* HY, z64* G, z64* Zg, JacRot<double>* rot, double* red,
+                              double width, bool want_max, z64* Y, z64* HY, z64* G, z64* Zg, JacRot<double>* rot, double* red,
                               int max_sweeps, int* ok, int* flag) {
   const int tid = threadIdx.x, nt = blockDim.x, g = c1 - c0 + 1;
   for (int e = tid; e < n * g; e += nt) {
@@ -274,7 +274,10 @@ __device__ double edge_energy(const z64* H, const c32* V, const int* ord, const 
     c32 acc(0.f, 0.f);
     if (j < c0 || j > c1) {
       for (int r = 0; r < n; ++r) cfma_conj(acc, V[r * n + ord[j]], ccast<float>(Y[r * g + b]));
-      acc = float(1.0 / (lam[ord[c0 + b]] - lam[ord[j]])) * acc;
+      // (a level just outside the cluster may come close to a far member of it; the edge
+      // itself is a width away)
+      const double dl = lam[ord[c0 + b]] - lam[ord[j]];
+      acc = fabs(dl) > 0.1 * width ? float(1.0 / dl) * acc : c32(0.f, 0.f);
     }
     HY[e] = ccast<double>(acc);
   }
@@ -336,9 +339,9 @@ __device__ bool refine_fp64(const z64* H, const c32* V, const int* ord, const do
     if (!ok || !(c2 < 1e-4)) return false;
   }
   if (!(c2 <= 1e-17)) return false;
-  const double top = edge_energy(H, V, ord, lam, n, c0, p - 1, true, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
+  const double top = edge_energy(H, V, ord, lam, n, c0, p - 1, width, true, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
   if (!ok) return false;
-  const double bot = edge_energy(H, V, ord, lam, n, p, c1, false, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
+  const double bot = edge_energy(H, V, ord, lam, n, p, c1, width, false, C, HQ, G, Zg, rot, red, max_sweeps, &ok, flag);
   gap = bot - top;
   return ok != 0;
 }

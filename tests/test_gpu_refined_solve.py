@@ -68,3 +68,45 @@ def test_gap_down_to_closing(lib, ctx, n, offset):
 def test_energy_scale_outside_fp32(lib, ctx, scale):
     for n, p in ((4, 2), (10, 4)):
         _check(lib, ctx, _scaled(I.random_hermitian_model(n, 5), scale, hop=0.03), I.Plane(7, 4), p)
+
+
+# ---- n > 32: the FP32 solve with the FP64 polish, the FP64 solve where it does not apply
+
+
+@pytest.mark.parametrize("n,p", [(33, 1), (33, 16), (40, 32), (41, 33), (63, 31), (64, 62), (97, 65)])
+def test_polished_states_and_gap(lib, ctx, n, p):
+    """Dense models: both column tiles (p <= 32 and beyond) and their remainders."""
+    _check(lib, ctx, _scaled(I.random_hermitian_model(n, 11 + n), 1.0, hop=0.03), I.Plane(6, 3), p)
+
+
+@pytest.mark.parametrize("copies", [9, 11])
+@pytest.mark.parametrize("split", [0.0, 1e-6, 2e-3])
+def test_polished_degenerate_edges(lib, ctx, copies, split):
+    """Sparse models whose band edges hold 2 to 22 levels: small clusters in the polish, larger
+    ones in the FP64 solve."""
+    parts = []
+    for c in range(copies):
+        m = I.bbh(0.5, 0.5)
+        parts.append(I.HoppingList(n=4, R=np.concatenate([m.R, np.zeros((4, 3), np.int32)]),
+                                   i=np.concatenate([m.i, np.arange(4)]), j=np.concatenate([m.j, np.arange(4)]),
+                                   t=np.concatenate([m.t, np.full(4, c * split * c + 0j)]), dim=m.dim))
+    _check(lib, ctx, I.direct_sum(parts), I.Plane(6, 3), 2 * copies)
+
+
+@pytest.mark.parametrize("offset", [1e-7, 1e-4, 1e-2])
+def test_polished_gap_down_to_closing(lib, ctx, offset):
+    m = I.random_hermitian_model(20, 3)
+    sh = I.HoppingList(n=20, R=np.concatenate([m.R, np.zeros((20, 3), np.int32)]),
+                       i=np.concatenate([m.i, np.arange(20)]), j=np.concatenate([m.j, np.arange(20)]),
+                       t=np.concatenate([m.t, np.full(20, offset + 0j)]), dim=m.dim)
+    _check(lib, ctx, I.direct_sum([m, sh]), I.Plane(6, 3), 1, phases=False)
+
+
+def test_polish_without_room_takes_the_fp64_solve(lib):
+    """A budget that holds the FP64 solve's slot (0.6 MiB) but not the polish's (1.6 MiB)."""
+    model = I.direct_sum([_scaled(I.random_hermitian_model(4, 5 + b), 1.0, hop=0.03) for b in range(50)])
+    small = lib.Context(0, mem_budget_bytes=5 << 18)
+    try:
+        _check(lib, small, model, I.Plane(3, 1), 1, phases=False)
+    finally:
+        small.close()
