@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256) k_zgemm(GemmArgs g) {
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) cfma(acc[x][y], av[x], bv[y]);
+        for (int y = 0; y < 4; ++y) cmac(acc[x][y], av[x], bv[y]);
     }
     __syncthreads();
   }
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k_zgemm(GemmArgs g) {
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
       const int gc = c0 + tx + 16 * y;
-      if (gc < g.n) C[(long long)gr * g.ldc + gc] = acc[x][y];
+      if (gc < g.n) C[(long long)gr * g.ldc + gc] = cfin(acc[x][y]);
     }
   }
 }
@@ -692,7 +692,8 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
     for (int col = c + 1 + gtid; work && col < p; col += gnt) {
       E w = A::zero();
 #pragma unroll 4
-      for (int r = c + 1; r < p; ++r) cfma_conj(w, vsh[r], A::ld(H + (long long)r * p + col));
+      for (int r = c + 1; r < p; ++r) cmac_conj(w, vsh[r], A::ld(H + (long long)r * p + col));
+      w = cfin(w);
 #pragma unroll 4
       for (int r = c + 1; r < p; ++r) {
         E* h = H + (long long)r * p + col;
@@ -706,7 +707,8 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
     for (int row = gwarp; work && row < p; row += gnwarp) {
       E* hr = H + (long long)row * p;
       E w = A::zero();
-      for (int k = c + 1 + lane; k < p; k += 32) cfma(w, A::ld(hr + k), vsh[k]);
+      for (int k = c + 1 + lane; k < p; k += 32) cmac(w, A::ld(hr + k), vsh[k]);
+      w = cfin(w);
       for (int o = 16; o > 0; o >>= 1) w = w + A::shfl_xor(w, o);
       for (int k = c + 1 + lane; k < p; k += 32) hr[k] = A::ld(hr + k) - R(2.0) * (w * conj(vsh[k]));
     }

@@ -106,9 +106,10 @@ __global__ void k_lg_build(LargeArgs a) {
         for (int h = md.ent_start[e]; h < md.ent_start[e + 1]; ++h) {
           const int r = md.hop_r[h];
           const float* t4 = md.hop_tdf + 4 * h;
-          acc = acc + cdf(df(t4[0], t4[1]), df(t4[2], t4[3])) *
-                          (r < nRs ? phd[r] : cdf_from(bloch_phase(f, md.Rv + 3 * r)));
+          cmac(acc, cdf(df(t4[0], t4[1]), df(t4[2], t4[3])),
+               r < nRs ? phd[r] : cdf_from(bloch_phase(f, md.Rv + 3 * r)));
         }
+        acc = cfin(acc);
         A[(long long)md.ent_row[e] * n + md.ent_col[e]] = cx<T>(T(acc.re.hi), T(acc.im.hi));
         c32* dst = reinterpret_cast<c32*>(a.Hent + kw * (long long)md.n_ent + e);
         dst[0] = c32(acc.re.hi, acc.im.hi);

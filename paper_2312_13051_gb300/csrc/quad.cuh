@@ -241,8 +241,8 @@ __device__ __forceinline__ c32 group_sum_c32(c32 v) {
 __device__ __forceinline__ cdf quad_matvec(const cdf (&Hr)[4], cdf x, int base) {
   cdf acc = cdf_zero();
 #pragma unroll 1
-  for (int q = 0; q < 4; ++q) cfma(acc, sel4(Hr, q), shfl_cdf(x, base + q));
-  return acc;
+  for (int q = 0; q < 4; ++q) cmac(acc, sel4(Hr, q), shfl_cdf(x, base + q));
+  return cfin(acc);
 }
 
 // First-order Lowdin step X <- X - X (X^dag X - I) / 2 for two vectors of the group,
@@ -255,7 +255,7 @@ __device__ __forceinline__ void lowdin2(cdf& X0, cdf& X1) {
   for (int t = 0; t < 3; ++t) {  // (0, 0), (0, 1), (1, 1)
     const cdf xa = t == 2 ? X1 : X0, xb = t == 0 ? X0 : X1;
     cdf g = cdf_zero();
-    cfma_conj(g, xa, xb);
+    cmac_conj(g, xa, xb);
     const df gre = group_sum_df(g.re) - df(t == 1 ? 0.f : 1.f), gim = group_sum_df(g.im);
     if (t == 0) e00 = gre.hi;
     if (t == 1) e01 = c32(gre.hi, gim.hi);
@@ -283,7 +283,7 @@ __device__ __forceinline__ void ritz2(const cdf (&Hr)[4], cdf X0, cdf X1, int ba
 #pragma unroll 1
   for (int t = 0; t < 3; ++t) {  // X0^dag h0, X1^dag h1, X0^dag h1
     cdf g = cdf_zero();
-    cfma_conj(g, t == 1 ? X1 : X0, t == 0 ? h0 : h1);
+    cmac_conj(g, t == 1 ? X1 : X0, t == 0 ? h0 : h1);
     const df gre = group_sum_df(g.re);
     if (t == 0) aa = gre;
     if (t == 1) dd = gre;
