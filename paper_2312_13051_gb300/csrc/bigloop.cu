@@ -50,13 +50,14 @@ __global__ void __launch_bounds__(256) k_zgemm(GemmArgs g) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int tiles_n = (g.n + GT - 1) / GT;
   const long long bl = g.b0 + blockIdx.y, b = g.kfirst + bl;
+  const long long bo = g.bin > 0 ? bl / g.bin : 0, bi = bl - bo * g.bin;  // two-level batch
   const long long ba = g.a_next_N > 0 ? (b / g.a_next_N) * g.a_next_N + (b % g.a_next_N + 1) % g.a_next_N
                        : g.a_mod > 0  ? (b + g.a_shift) % g.a_mod
                                       : b;
   const int r0 = (blockIdx.x / tiles_n) * GT, c0 = (blockIdx.x % tiles_n) * GT;
-  const E* A = reinterpret_cast<const E*>(g.A) + ba * g.sA;
-  const E* B = reinterpret_cast<const E*>(g.B) + b * g.sB;
-  E* C = reinterpret_cast<E*>(g.C) + bl * g.sC;
+  const E* A = reinterpret_cast<const E*>(g.A) + (g.bin > 0 ? bo * g.sAo + bi * g.sA : ba * g.sA);
+  const E* B = reinterpret_cast<const E*>(g.B) + (g.bin > 0 ? bo * g.sBo + bi * g.sB : b * g.sB);
+  E* C = reinterpret_cast<E*>(g.C) + (g.bin > 0 ? bo * g.sCo + bi * g.sC : bl * g.sC);
   E acc[4][4];
 #pragma unroll
   for (int x = 0; x < 4; ++x)
@@ -430,7 +431,8 @@ cudaError_t launch_iota(long long* off, int* idx, long long W, long long stride,
 // ---------------------------------------------------------------------------
 constexpr int GC_CTAS = 4, GC_W = 16, GC_THREADS = 256;
 constexpr int GC_WR = GC_W + 3, GC_WC = GC_W + 2;  // window rows, columns
-constexpr int GC_MIN_P = 128;                      // smaller p: k_geig_big
+constexpr int GC_MIN_P = 128;                      // FP64, smaller p: k_geig_big
+constexpr int GC_MIN_P_DF = 33;                    // double-float (the loops come here from p = 33 on)
 
 struct GcCtl {
   double mu[4];  // the shift, as the solver's element type (16 bytes)
@@ -871,7 +873,7 @@ static cudaError_t launch_geig_cluster(const BigEigArgs& a, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, k_geig_cluster<E>, a);
 }
 
-bool geig_df_eligible(int p) { return p >= GC_MIN_P; }
+bool geig_df_eligible(int p) { return p >= GC_MIN_P_DF; }
 
 cudaError_t launch_geig_big(const BigEigArgs& a, cudaStream_t s) {
   if (a.nl <= 0) return cudaSuccess;

@@ -104,11 +104,12 @@ constexpr size_t CG_SMEM = CG_K * CG_LD * (sizeof(SplitC) + sizeof(c32));  // th
 // C(m, c) = sum_k A(m, k) B(k, c) (the policy's product and accumulator) for m < M,
 // c < Ncol, k < K, computed by all blockDim.x == 256 threads of the CTA in 64 x TN output
 // tiles (thread (ty, tx) owns rows ty + 16 i and columns tx + 16 j; TN = 32 or 64).
+// kUpper: only the results with m <= c (a Hermitian product; the consumer mirrors them).
 // la(m, k) and lb(k, c) return the operands (out-of-range indices are never
 // requested); st(m, c, acc) consumes each result once.  A_K_CONTIG / B_C_CONTIG say
 // which index of the operand is contiguous in memory, so that the staging loads
 // are coalesced.  sm: cg_smem<Pol>() bytes.
-template <class Pol, bool A_K_CONTIG, bool B_C_CONTIG, int TN = CG_TILE, class LA, class LB, class ST>
+template <class Pol, bool A_K_CONTIG, bool B_C_CONTIG, int TN = CG_TILE, bool kUpper = false, class LA, class LB, class ST>
 __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned char* sm) {
   using TA = typename Pol::TA;
   using TB = typename Pol::TB;
@@ -117,6 +118,7 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += CG_TILE)
     for (int c0 = 0; c0 < Ncol; c0 += TN) {
+      if (kUpper && c0 + TN <= m0) continue;
       typename Pol::Acc acc[4][TN / 16];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -201,7 +203,8 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < TN / 16; ++j) Pol::mac(acc[i][j], av[i], bv[j]);
+            for (int j = 0; j < TN / 16; ++j)
+              if (!kUpper || m0 + 16 * i < c0 + 16 * (j + 1)) Pol::mac(acc[i][j], av[i], bv[j]);
         }
         __syncthreads();
       }
@@ -210,7 +213,7 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
 #pragma unroll
         for (int j = 0; j < TN / 16; ++j) {
           const int gm = m0 + ty + 16 * i, gc = c0 + tx + 16 * j;
-          if (gm < M && gc < Ncol) st(gm, gc, acc[i][j]);
+          if (gm < M && gc < Ncol && (!kUpper || gm <= gc)) st(gm, gc, acc[i][j]);
         }
     }
 }

@@ -1107,30 +1107,31 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
     tc_ok = tc_ok && cta_reflect_wy(A, n, C, p, p, true, work, ts);
     // E = Q^dag Q - I with Q = Q32 + C: Q32^dag Q32 - I compensated (the FP32 basis is
     // orthonormal to ~1e-7, so the difference needs the extra precision), then the
-    // small terms Q32^dag C + C^dag (Q32 + C) in FP32 as one GEMM over 2 n rows
-    cta_gemm<GemmGramComp, false, true>(
+    // small terms Q32^dag C + C^dag Q32 + C^dag C = D + D^dag, D = (Q32 + C / 2)^dag C, in FP32
+    cta_gemm<GemmGramComp, false, true, CG_TILE, true>(
         p, p, n, [&](int x, int r) { return X[(long long)r * nbt + x]; },
         [&](int r, int y) { return X[(long long)r * nbt + y]; },
         [&](int x, int y, const CDF& acc) {
           z64 v = acc.value();
-          if (x == y) v.re -= 1.0;
+          if (x == y) v = z64(v.re - 1.0, 0.0);
           E[(long long)x * p + y] = c32(float(v.re), float(v.im));
+          E[(long long)y * p + x] = c32(float(v.re), float(-v.im));
         },
         work);
+    c32* F = E + (long long)p * p;
     __syncthreads();
     tc_ok = tc_ok && cta_cgemm_tc<false, true>(
-        p, p, 2 * n,
-        [&](int x, int k) {
-          return conj(k < n ? X[(long long)k * nbt + x] : C[(long long)(k - n) * p + x]);
-        },
-        [&](int k, int y) {
-          return k < n ? C[(long long)k * p + y] : X[(long long)(k - n) * nbt + y] + C[(long long)(k - n) * p + y];
-        },
-        [&](int x, int y, c32 v) { E[(long long)x * p + y] = E[(long long)x * p + y] + v; }, work, ts);
+        p, p, n,
+        [&](int x, int r) { return conj(X[(long long)r * nbt + x] + 0.5f * C[(long long)r * p + x]); },
+        [&](int r, int y) { return C[(long long)r * p + y]; },
+        [&](int x, int y, c32 v) { F[(long long)x * p + y] = v; }, work, ts);
+    __syncthreads();
+    for (int x = warp; x < p; x += nwarp)
+      for (int y = lane; y < p; y += 32)
+        E[(long long)x * p + y] = E[(long long)x * p + y] + F[(long long)x * p + y] + conj(F[(long long)y * p + x]);
     __syncthreads();
     // second order of (I + E)^{-1/2}: F = E - 3/4 E^2 (E reaches ~3e-5 where inverse iteration
     // leaves neighbouring vectors short of orthogonal, and E^2 would stay as the error)
-    c32* F = E + (long long)p * p;
     tc_ok = tc_ok && cta_cgemm_tc<true, true>(
         p, p, p, [&](int x, int q) { return E[(long long)x * p + q]; },
         [&](int q, int y) { return E[(long long)q * p + y]; },
@@ -1337,10 +1338,14 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
       }
     }
     __syncthreads();
-    cta_gemm<GemmPlainT<double>, false, true, TN>(
+    cta_gemm<GemmPlainT<double>, false, true, TN, true>(
         p, p, n, [&](int x, int r) { return conj(Q[(long long)r * p + x]); },
         [&](int r, int y) { return R[(long long)r * ldr + y]; },
-        [&](int x, int y, const z64& v) { G[(long long)x * p + y] = x == y ? z64(v.re, 0.0) : v; }, smem);
+        [&](int x, int y, const z64& v) {
+          G[(long long)x * p + y] = x == y ? z64(v.re, 0.0) : v;
+          if (x != y) G[(long long)y * p + x] = conj(v);
+        },
+        smem);
     __syncthreads();
     cta_gemm<GemmPlainT<double>, true, true, TN>(
         n, p, p, [&](int r, int q) { return Q[(long long)r * p + q]; },
@@ -1440,13 +1445,14 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
     c2 = block_sum(c2, red);
     // E = Q^dag Q - I
     double emax = 0.0;
-    cta_gemm<GemmPlainT<double>, false, true, TN>(
+    cta_gemm<GemmPlainT<double>, false, true, TN, true>(
         p, p, n, [&](int x, int r) { return conj(Q[(long long)r * p + x]); },
         [&](int r, int y) { return Q[(long long)r * p + y]; },
         [&](int x, int y, const z64& v) {
           const c32 e(float(v.re - (x == y ? 1.0 : 0.0)), x == y ? 0.f : float(v.im));
           emax = fmax(emax, double(abs2(e)));
           E[(long long)x * p + y] = e;
+          E[(long long)y * p + x] = conj(e);
         },
         smem);
     emax = -block_min(-emax, red);

@@ -14,6 +14,10 @@ constexpr int SMALL_N_MAX = 32;
 constexpr int LARGE_N_MAX = 4096;
 // Largest p handled by the shared-memory loop kernels (Wilson matrix p x p).
 constexpr int LOOP_P_MAX = 64;
+// Mixed plain loops of more bands than this take the batched-GEMM loops: their products run
+// on every SM instead of one CTA per loop, and their eigenphases in double-float on a cluster
+// (p = 64, 27 loops of 31 points: 12.1 ms in one CTA per loop, see the loop stage).
+constexpr int LOOP_P_MAX_DF = 32;
 // Distinct translations whose phases are cached in shared memory per k-point.
 constexpr int PHASE_CACHE = 256;
 // Distinct translations the one-thread-per-k-point path keeps per thread.
@@ -192,6 +196,9 @@ struct GemmArgs {
   long long b0;           // first batch index of this launch (set by launch_zgemm)
   long long kfirst;       // absolute index of batch 0 for A and B (C stays relative)
   long long a_shift, a_mod;
+  // bin > 0: batch b = (b / bin, b % bin) at A + (b / bin) sAo + (b % bin) sA, B and C alike
+  long long bin;
+  long long sAo, sBo, sCo;
 };
 
 // Eigenphases of nl Wilson matrices W (p x p, stride sW), loops i0 .. i0+nl-1.

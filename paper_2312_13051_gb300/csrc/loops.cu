@@ -797,6 +797,104 @@ __global__ void k_loops_scan(LoopArgs a) {
   }
 }
 
+// Plain FP64 loops of one or two bands, a warp per loop: lane l multiplies the overlaps of a
+// run of consecutive points, the lanes' products are folded in order by shuffles, and the
+// eigenphases come in closed form.  The scan kernel above spends most of its time at block
+// barriers here (log N levels with a few scalar products each); it stays for nested loops,
+// which need every partial product.  Eq. 4, 24 x 24: see launch_loops.
+template <int PP>
+__global__ void k_loops_warp(LoopArgs a) {
+  const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= a.N_t) return;
+  const int n = a.n, N = a.N;
+  const long long k0 = (long long)i * N;
+  const z64* Ul = a.U + k0 * n * PP;
+  const int per = (N + 31) / 32, j0 = lane * per, j1 = min(N, j0 + per);
+  z64 W[PP][PP];
+#pragma unroll
+  for (int r = 0; r < PP; ++r)
+#pragma unroll
+    for (int c = 0; c < PP; ++c) W[r][c] = z64(double(r == c), 0.0);
+  for (int j = j0; j < j1; ++j) {
+    const z64* Uh = Ul + (long long)j * n * PP;
+    const z64* Un = Ul + (long long)(j + 1 == N ? 0 : j + 1) * n * PP;
+    z64 M[PP][PP];
+#pragma unroll
+    for (int r = 0; r < PP; ++r)
+#pragma unroll
+      for (int c = 0; c < PP; ++c) M[r][c] = z64(0.0, 0.0);
+#pragma unroll 4
+    for (int q = 0; q < n; ++q)
+#pragma unroll
+      for (int r = 0; r < PP; ++r)
+#pragma unroll
+        for (int c = 0; c < PP; ++c) cfma_conj(M[r][c], Un[q * PP + r], Uh[q * PP + c]);
+    z64 T[PP][PP];
+#pragma unroll
+    for (int r = 0; r < PP; ++r)
+#pragma unroll
+      for (int c = 0; c < PP; ++c) {
+        T[r][c] = z64(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < PP; ++q) cfma(T[r][c], M[r][q], W[q][c]);
+      }
+#pragma unroll
+    for (int r = 0; r < PP; ++r)
+#pragma unroll
+      for (int c = 0; c < PP; ++c) W[r][c] = T[r][c];
+  }
+  double g = INFINITY, gp = INFINITY;
+  for (int j = lane; j < N; j += 32) {
+    if (a.gap) g = fmin(g, a.gap[k0 + j]);
+    if (a.pso_gap) gp = fmin(gp, a.pso_gap[k0 + j]);
+  }
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    z64 B[PP][PP], T[PP][PP];
+    const bool take = (lane & (2 * o - 1)) == 0 && (lane + o) * per < N;
+#pragma unroll
+    for (int r = 0; r < PP; ++r)
+#pragma unroll
+      for (int c = 0; c < PP; ++c)
+        B[r][c] = z64(__shfl_down_sync(0xffffffffu, W[r][c].re, o), __shfl_down_sync(0xffffffffu, W[r][c].im, o));
+    if (take) {  // later points on the left
+#pragma unroll
+      for (int r = 0; r < PP; ++r)
+#pragma unroll
+        for (int c = 0; c < PP; ++c) {
+          T[r][c] = z64(0.0, 0.0);
+#pragma unroll
+          for (int q = 0; q < PP; ++q) cfma(T[r][c], B[r][q], W[q][c]);
+        }
+#pragma unroll
+      for (int r = 0; r < PP; ++r)
+#pragma unroll
+        for (int c = 0; c < PP; ++c) W[r][c] = T[r][c];
+    }
+    g = fmin(g, __shfl_xor_sync(0xffffffffu, g, o));
+    gp = fmin(gp, __shfl_xor_sync(0xffffffffu, gp, o));
+  }
+  if (lane == 0) {
+    if (a.min_gap) a.min_gap[i] = g;
+    if (a.min_pso_gap) a.min_pso_gap[i] = gp;
+  }
+  if constexpr (PP == 1) {
+    if (lane == 0) a.phases[i] = phase_of(W[0][0]);
+  } else {
+    z64 lam[2];
+    const z64 H[4] = {W[0][0], W[0][1], W[1][0], W[1][1]};
+    eig2_closed(H, 2, lam, nullptr, false);
+    const z64 l1(__shfl_sync(0xffffffffu, lam[1].re, 0), __shfl_sync(0xffffffffu, lam[1].im, 0));
+    const double t = phase_of(lane == 1 ? l1 : lam[0]);
+    const double t1 = __shfl_sync(0xffffffffu, t, 1);
+    if (lane == 0) {
+      const bool sw = rank_key(t1) < rank_key(t);
+      a.phases[2LL * i] = sw ? t1 : t;
+      a.phases[2LL * i + 1] = sw ? t : t1;
+    }
+  }
+}
+
 // Nested loop of one Wannier band at base point j: the loop matrix is the product
 // of the scalar overlaps w(i+1)^dagger w(i) (any order), taken by the CTA's first
 // warp straight from global memory; the other threads return at once.
@@ -1126,12 +1224,12 @@ __device__ __forceinline__ void loops_fused_body(const StatesArgs& sa, const Loo
 }
 
 template <bool kNested1>
-__global__ void __launch_bounds__(FUSED_THREADS) k_loops_fused_df(StatesArgs sa, LoopArgs a) {
+__global__ void __launch_bounds__(FUSED_THREADS, kNested1 ? 1 : 3) k_loops_fused_df(StatesArgs sa, LoopArgs a) {
   loops_fused_body<kNested1>(sa, a, nullptr, nullptr);
 }
 
 template <bool kNested1>
-__global__ void __launch_bounds__(FUSED_THREADS)
+__global__ void __launch_bounds__(FUSED_THREADS, kNested1 ? 1 : 3)
     k_loops_fused_df_inl(StatesArgs sa, LoopArgs a, const char* dbase, const __grid_constant__ FusedPlan plan) {
   loops_fused_body<kNested1>(sa, a, plan.bytes, dbase);
 }
@@ -1373,6 +1471,15 @@ cudaError_t launch_loops(const LoopArgs& a, cudaStream_t s) {
       cudaError_t e = set_smem_once(k_loops_scan<cdf>, Z.total, cached_df);
       if (e != cudaSuccess) return e;
       k_loops_scan<cdf><<<a.N_t, 128, Z.total, s>>>(a);
+      return cudaGetLastError();
+    }
+    if (a.p <= 2 && a.n <= 32 && !a.nested && !a.unitarise) {
+      // few loops: a CTA each, so that every SM takes part
+      const int warps = a.N_t < 4 * 152 ? 1 : 4, grid = (a.N_t + warps - 1) / warps;
+      if (a.p == 1)
+        k_loops_warp<1><<<grid, 32 * warps, 0, s>>>(a);
+      else
+        k_loops_warp<2><<<grid, 32 * warps, 0, s>>>(a);
       return cudaGetLastError();
     }
     static size_t cached_scan = 0;

@@ -217,8 +217,14 @@ __device__ __forceinline__ cdf tab_at_df(const cdf* lo, const cdf* hi, TabShape 
   return hi[m / t.B] * lo[m % t.B];
 }
 
-// Re(conj(x) y) with x exact in float, y double-float.
-__device__ __forceinline__ df re_conj_dot(c32 x, cdf y) { return df_fma(df(x.re), y.re, x.im * y.im); }
+// acc += a b with b exact in float (df_mac without the term in b.lo).
+__device__ __forceinline__ void df_mac(df& acc, df a, float b) {
+  const float p = a.hi * b;
+  const float e = fmaf(a.lo, b, fmaf(a.hi, b, -p));
+  const df s = df_two_sum(acc.hi, p);
+  acc.hi = s.hi;
+  acc.lo += s.lo + e;
+}
 
 __device__ __forceinline__ df group_sum_df(df v) {
   v = v + shfl_xor_df(v, 1);
@@ -237,75 +243,100 @@ __device__ __forceinline__ c32 group_sum_c32(c32 v) {
 // than unrolled code: it runs once per k-point on few warps per SM, where a long
 // straight-line body stalls on instruction fetch.
 
-// (H x)[l] for a double-float vector x held one entry per lane (x[q] in lane q).
-__device__ __forceinline__ cdf quad_matvec(const cdf (&Hr)[4], cdf x, int base) {
+// (H x)[l] for an FP32 vector x held one entry per lane (x[q] in lane q).
+__device__ __forceinline__ cdf quad_matvec(const cdf (&Hr)[4], c32 x, int base) {
   cdf acc = cdf_zero();
 #pragma unroll 1
-  for (int q = 0; q < 4; ++q) cmac(acc, sel4(Hr, q), shfl_cdf(x, base + q));
+  for (int q = 0; q < 4; ++q) {
+    const cdf h = sel4(Hr, q);
+    const c32 v = shfl_z(x, base + q);
+    df_mac(acc.re, h.re, v.re);
+    df_mac(acc.im, h.re, v.im);
+    df_mac(acc.re, h.im, -v.im);
+    df_mac(acc.im, h.im, v.re);
+  }
   return cfin(acc);
 }
 
-// First-order Lowdin step X <- X - X (X^dag X - I) / 2 for two vectors of the group,
-// the Gram matrix in double-float (its deviation E from I is ~1e-7, so the
-// correction X E / 2 itself is computed in FP32).
-__device__ __forceinline__ void lowdin2(cdf& X0, cdf& X1) {
-  float e00 = 0.f, e11 = 0.f;
-  c32 e01(0.f, 0.f);
+// An FP32 pair x0, x1 of the group with h_c = H x_c: the Ritz matrix g = x^dag h and the
+// deviation e = x^dag x - I (~1e-7, kept in FP32; with kDev) from double-float sums.
+struct QuadPair {
+  df g00, g11, gre, gim;
+  float e00, e11;
+  c32 e01;
+};
+template <bool kDev>
+__device__ __forceinline__ QuadPair quad_pair(c32 x0, c32 x1, cdf h0, cdf h1) {
+  QuadPair r;
+  r.e00 = r.e11 = 0.f;
+  r.e01 = c32(0.f, 0.f);
 #pragma unroll 1
   for (int t = 0; t < 3; ++t) {  // (0, 0), (0, 1), (1, 1)
-    const cdf xa = t == 2 ? X1 : X0, xb = t == 0 ? X0 : X1;
-    cdf g = cdf_zero();
-    cmac_conj(g, xa, xb);
-    const df gre = group_sum_df(g.re) - df(t == 1 ? 0.f : 1.f), gim = group_sum_df(g.im);
-    if (t == 0) e00 = gre.hi;
-    if (t == 1) e01 = c32(gre.hi, gim.hi);
-    if (t == 2) e11 = gre.hi;
-  }
-  const c32 x0(X0.re.hi, X0.im.hi), x1(X1.re.hi, X1.im.hi);
-  const c32 c0 = c32(x0.re * e00, x0.im * e00) + x1 * conj(e01);
-  const c32 c1 = x0 * e01 + c32(x1.re * e11, x1.im * e11);
-  X0 = cdf(X0.re + df(-0.5f * c0.re), X0.im + df(-0.5f * c0.im));
-  X1 = cdf(X1.re + df(-0.5f * c1.re), X1.im + df(-0.5f * c1.im));
-}
-
-// Eigenvalues lo <= hi of the 2 x 2 Hermitian Ritz matrix X^dag H X of two
-// orthonormal vectors: (a + d) / 2 -+ sqrt(((a - d) / 2)^2 + |b|^2), in double-float.
-__device__ __forceinline__ void ritz2(const cdf (&Hr)[4], cdf X0, cdf X1, int base, df& lo,
-                                      df& hi) {
-  cdf h0 = cdf_zero(), h1 = cdf_zero();
-#pragma unroll 1
-  for (int t = 0; t < 2; ++t) {
-    const cdf h = quad_matvec(Hr, t ? X1 : X0, base);
-    if (t == 0) h0 = h;
-    if (t == 1) h1 = h;
-  }
-  df aa(0.f), dd(0.f), bre(0.f), bim(0.f);
-#pragma unroll 1
-  for (int t = 0; t < 3; ++t) {  // X0^dag h0, X1^dag h1, X0^dag h1
-    cdf g = cdf_zero();
-    cmac_conj(g, t == 1 ? X1 : X0, t == 0 ? h0 : h1);
-    const df gre = group_sum_df(g.re);
-    if (t == 0) aa = gre;
-    if (t == 1) dd = gre;
-    if (t == 2) {
-      bre = gre;
-      bim = group_sum_df(g.im);
+    const c32 a = t == 2 ? x1 : x0, b = t == 0 ? x0 : x1;
+    const cdf h = t == 0 ? h0 : h1;
+    df gr(0.f), gi(0.f), er(0.f), ei(0.f);
+    df_mac(gr, h.re, a.re);
+    df_mac(gr, h.im, a.im);
+    gr = group_sum_df(gr);
+    if (t == 1) {
+      df_mac(gi, h.im, a.re);
+      df_mac(gi, h.re, -a.im);
+      r.gre = gr;
+      r.gim = group_sum_df(gi);
+    }
+    if (t == 0) r.g00 = gr;
+    if (t == 2) r.g11 = gr;
+    if constexpr (kDev) {
+      df_mac(er, df(b.re), a.re);
+      df_mac(er, df(b.im), a.im);
+      er = group_sum_df(er);
+      if (t == 1) {
+        df_mac(ei, df(b.im), a.re);
+        df_mac(ei, df(b.re), -a.im);
+        r.e01 = c32(er.hi, group_sum_df(ei).hi);
+      }
+      const float d = (er.hi - 1.f) + er.lo;
+      if (t == 0) r.e00 = d;
+      if (t == 2) r.e11 = d;
     }
   }
+  return r;
+}
+
+// e - 3/4 e^2 of a Hermitian 2 x 2 deviation: (I + e)^{-1/2} = I - (e - 3/4 e^2) / 2 to second
+// order (e^2 ~ 1e-13 would stay as the error otherwise).
+__device__ __forceinline__ void dev_second_order(float& e00, float& e11, c32& e01) {
+  const float q = abs2(e01), t = 1.f - 0.75f * (e00 + e11);
+  e00 -= 0.75f * fmaf(e00, e00, q);
+  e11 -= 0.75f * fmaf(e11, e11, q);
+  e01 = t * e01;
+}
+
+// Eigenvalues lo <= hi of the pair's 2 x 2 Ritz matrix in the orthonormalised basis,
+// g - (e g + g e) / 2 + s, s a small Hermitian correction (FP32):
+// (a + d) / 2 -+ sqrt(((a - d) / 2)^2 + |b|^2) in double-float.
+__device__ __forceinline__ void quad_pair_edges(QuadPair r, float s00, float s11, c32 s01, df& lo, df& hi) {
+  dev_second_order(r.e00, r.e11, r.e01);
+  const c32 g(r.gre.hi, r.gim.hi);
+  const float a = r.g00.hi, d = r.g11.hi, m = 0.5f * (a + d), x = g.re * r.e01.re + g.im * r.e01.im;
+  const df aa = r.g00 + df(s00 - r.e00 * a - x), dd = r.g11 + df(s11 - r.e11 * d - x);
+  const float eh = 0.5f * (r.e00 + r.e11);
+  const df bre = r.gre + df(s01.re - eh * g.re - m * r.e01.re), bim = r.gim + df(s01.im - eh * g.im - m * r.e01.im);
   const df mean = df(0.5f) * (aa + dd), half = df(0.5f) * (aa - dd);
-  const df r = df_sqrt(df_fma(half, half, df_fma(bre, bre, bim * bim)));
-  lo = mean - r;
-  hi = mean + r;
+  const df q = df_sqrt(df_fma(half, half, df_fma(bre, bre, bim * bim)));
+  lo = mean - q;
+  hi = mean + q;
 }
 
 // Occupied pair of a four-band H(k) given as double-float rows (lane l holds row
 // l): FP32 Jacobi on the float part of H, made exactly Hermitian; one Newton
 // correction of the two lowest FP32 vectors q_c in the FP32 eigenbasis with the
-// residual R = H q_c - q_c rho_c in double-float (q_c += z_a (z_a^dag R_c) /
-// (rho_c - lam_a) over the unoccupied z_a); one first-order Lowdin step; the gap
-// from the double-float Ritz values of the refined occupied pair and of the
-// re-orthonormalised unoccupied pair (accurate whatever the splitting inside each
-// pair).  Every lane of the warp must call it (warp shuffles).  Returns the Jacobi
+// residual R = H q_c - q_c rho_c in double-float (q_c += z_a C_ac, C_ac = z_a^dag R_c /
+// (rho_c - lam_a) over the unoccupied z_a); one second-order Lowdin step; the gap from
+// double-float Ritz values of the FP32 pairs with the second-order shifts
+// -+ C^dag (lam_a - rho_c) C (accurate whatever the splitting inside each pair).  Four
+// matrix-vector products in all: the refined pair needs none of its own.  Every lane of the
+// warp must call it (warp shuffles).  Returns the Jacobi
 // sweeps used (-1: no convergence); Q0, Q1 are row l of the occupied vectors.
 __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int base, int max_sweeps,
                                                 cdf& Q0, cdf& Q1, double& gap) {
@@ -325,43 +356,67 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
   float lam[4];
   int ord[4];
   quad_order(Ar, l, base, lam, ord);
-  Q0 = Q1 = cdf_zero();
+  const c32 q0 = sel4(Vr, ord[0]), q1 = sel4(Vr, ord[1]), z0 = sel4(Vr, ord[2]), z1 = sel4(Vr, ord[3]);
+  const float lz0 = sel4(lam, ord[2]), lz1 = sel4(lam, ord[3]);
+  cdf h[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) h[t] = cdf_zero();
 #pragma unroll 1
-  for (int c = 0; c < 2; ++c) {
-    const c32 q = sel4(Vr, ord[c]);
-    const cdf hq = quad_matvec(Hr, cdf_from(q), base);
-    const df rho = group_sum_df(re_conj_dot(q, hq));
-    const cdf R(hq.re - q.re * rho, hq.im - q.im * rho);
-    const c32 r32(R.re.hi, R.im.hi);
-    c32 upd(0.f, 0.f);
-#pragma unroll 1
-    for (int aa = 2; aa < 4; ++aa) {
-      const c32 z = sel4(Vr, ord[aa]);
-      const c32 d = group_sum_c32(conj(z) * r32);
-      const float den = rho.hi - sel4(lam, ord[aa]);
-      const c32 coef = den != 0.f ? c32(d.re / den, d.im / den) : c32(0.f, 0.f);
-      upd = upd + z * coef;
-    }
-    const cdf qn(df_two_sum(q.re, upd.re), df_two_sum(q.im, upd.im));
-    if (c == 0) Q0 = qn;
-    if (c == 1) Q1 = qn;
+  for (int t = 0; t < 4; ++t) {
+    const cdf v = quad_matvec(Hr, t == 0 ? q0 : (t == 1 ? q1 : (t == 2 ? z0 : z1)), base);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u == t) h[u] = v;
   }
-  const cdf Z0 = cdf_from(sel4(Vr, ord[2])), Z1 = cdf_from(sel4(Vr, ord[3]));
-  df occ_hi(0.f), un_lo(0.f);
+  QuadPair oc = quad_pair<false>(q0, q1, h[0], h[1]);
+  const QuadPair un = quad_pair<true>(z0, z1, h[2], h[3]);
+  // residuals and coefficients C[a][c]
+  auto resid = [](cdf hv, c32 q, df rho) {
+    return c32((hv.re - q.re * rho).hi, (hv.im - q.im * rho).hi);
+  };
+  const c32 r0 = resid(h[0], q0, oc.g00), r1 = resid(h[1], q1, oc.g11);
+  auto coef = [](c32 z, c32 r, float den) {
+    const c32 d = group_sum_c32(conj(z) * r);
+    return den != 0.f ? (1.f / den) * d : c32(0.f, 0.f);
+  };
+  const float d00 = oc.g00.hi - lz0, d01 = oc.g11.hi - lz0, d10 = oc.g00.hi - lz1, d11 = oc.g11.hi - lz1;
+  const c32 c00 = coef(z0, r0, d00), c01 = coef(z0, r1, d01), c10 = coef(z1, r0, d10), c11 = coef(z1, r1, d11);
+  const c32 u0 = z0 * c00 + z1 * c10, u1 = z0 * c01 + z1 * c11;
+  Q0 = cdf(df_two_sum(q0.re, u0.re), df_two_sum(q0.im, u0.im));
+  Q1 = cdf(df_two_sum(q1.re, u1.re), df_two_sum(q1.im, u1.im));
+  // Lowdin step: the deviation E of the corrected pair in double-float
+  {
+    float e00 = 0.f, e11 = 0.f;
+    c32 e01(0.f, 0.f);
 #pragma unroll 1
-  for (int t = 0; t < 2; ++t) {  // the occupied pair, then the unoccupied one
-    cdf X0 = t ? Z0 : Q0, X1 = t ? Z1 : Q1;
-    lowdin2(X0, X1);
-    df lo, hi;
-    ritz2(Hr, X0, X1, base, lo, hi);
-    if (t == 0) {
-      Q0 = X0;
-      Q1 = X1;
-      occ_hi = hi;
-    } else {
-      un_lo = lo;
+    for (int t = 0; t < 3; ++t) {  // (0, 0), (0, 1), (1, 1)
+      const cdf xa = t == 2 ? Q1 : Q0, xb = t == 0 ? Q0 : Q1;
+      cdf g = cdf_zero();
+      cmac_conj(g, xa, xb);
+      const df gre = group_sum_df(g.re);
+      const float d = (gre.hi - 1.f) + gre.lo;
+      if (t == 0) e00 = d;
+      if (t == 1) e01 = c32(gre.hi, group_sum_df(g.im).hi);
+      if (t == 2) e11 = d;
     }
+    // the FP32 pair's own deviation, for its Ritz matrix (up to cross terms of ~1e-13)
+    oc.e00 = e00 - abs2(c00) - abs2(c10);
+    oc.e11 = e11 - abs2(c01) - abs2(c11);
+    oc.e01 = e01 - conj(c00) * c01 - conj(c10) * c11;
+    dev_second_order(e00, e11, e01);
+    const c32 x0(Q0.re.hi, Q0.im.hi), x1(Q1.re.hi, Q1.im.hi);
+    const c32 f0 = e00 * x0 + x1 * conj(e01), f1 = x0 * e01 + e11 * x1;
+    Q0 = cdf(Q0.re + df(-0.5f * f0.re), Q0.im + df(-0.5f * f0.im));
+    Q1 = cdf(Q1.re + df(-0.5f * f1.re), Q1.im + df(-0.5f * f1.im));
   }
+  // second-order shifts of the Ritz matrices (level repulsion between the pairs)
+  df occ_lo, occ_hi, un_lo, un_hi;
+  const float m0 = 0.5f * (d00 + d01), m1 = 0.5f * (d10 + d11);
+  quad_pair_edges(oc, d00 * abs2(c00) + d10 * abs2(c10), d01 * abs2(c01) + d11 * abs2(c11),
+                  m0 * (conj(c00) * c01) + m1 * (conj(c10) * c11), occ_lo, occ_hi);
+  const float n0 = 0.5f * (d00 + d10), n1 = 0.5f * (d01 + d11);
+  quad_pair_edges(un, -(d00 * abs2(c00) + d01 * abs2(c01)), -(d10 * abs2(c10) + d11 * abs2(c11)),
+                  -(n0 * (c00 * conj(c10)) + n1 * (c01 * conj(c11))), un_lo, un_hi);
   gap = df_to_double(un_lo - occ_hi);
   return sweeps;
 }

@@ -751,7 +751,12 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   const size_t left = avail > size_t(Wv) * per_k ? avail - size_t(Wv) * per_k : 0;
   const int nl_max = int(std::min<long long>(Nt, std::max<long long>(1, (long long)(left / per_loop))));
   Wv = std::min<long long>(Wv, (long long)nl_max * N);
-  total += size_t(Wv) * per_k + size_t(nl_max) * per_loop;
+  // The ordered product as a tree of pairwise products (every SM busy from the first level on)
+  // needs room for half the overlaps; without it, as a chain.
+  const int n2 = (N + 1) / 2;
+  const size_t tree_extra = size_t(nl_max) * (n2 > 2 ? n2 - 2 : 0) * bPk;
+  const bool tree = N > 2 && size_t(Wv) * per_k + size_t(nl_max) * per_loop + tree_extra <= avail;
+  total += size_t(Wv) * per_k + size_t(nl_max) * per_loop + (tree ? tree_extra : 0);
   bw_status st;
   if ((st = reserve(ctx, total, s))) return st;
   char* dblob = carve(ctx, blob.data.size());
@@ -760,8 +765,12 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   if ((st = upload(ctx, blob, dblob, s))) return st;
   z64* Ublk = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * N * bUk));
   z64* Mblk = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * N * bPk));
-  z64* Wbuf[2];
-  for (auto& w : Wbuf) w = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * bPk));
+  z64* Wbuf[2] = {nullptr, nullptr};
+  z64* Thalf = nullptr;
+  if (tree)
+    Thalf = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * std::max(n2, 2) * bPk));
+  else
+    for (auto& w : Wbuf) w = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * bPk));
   z64* e_lam = reinterpret_cast<z64*>(carve(ctx, nl_max * size_t(pl) * sizeof(z64)));
   z64* e_vec = reinterpret_cast<z64*>(carve(ctx, nl_max * size_t(pl) * sizeof(z64)));
   double* e_th = reinterpret_cast<double*>(carve(ctx, nl_max * size_t(pl) * sizeof(double)));
@@ -818,17 +827,48 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
     // W = M_{N-1} ... M_0 for the nl loops at once
     const z64* Wcur = Mblk;  // M_0 of loop l at Mblk + l N pl^2
     long long sWcur = (long long)N * sP;
-    for (int j = 1; j < N; ++j) {
-      z64* Wout = Wbuf[j & 1];
-      std::memset(&g, 0, sizeof(g));
-      g.A = Mblk + (long long)j * sP; g.B = Wcur; g.C = Wout;
-      g.m = pl; g.n = pl; g.k = pl; g.opA = 0;
-      g.lda = pl; g.ldb = pl; g.ldc = pl;
-      g.sA = (long long)N * sP; g.sB = sWcur; g.sC = sP;
-      g.batch = nl;
-      BW_CUDA(bw::launch_zgemm(g, s, mx), "loop-product GEMM");
-      Wcur = Wout;
-      sWcur = sP;
+    if (tree) {
+      // level: cnt matrices per loop at stride sIn -> pairs M_{2j+1} M_{2j}, an odd last one
+      // carried over
+      z64* src = Mblk;
+      z64* dst = Thalf;
+      long long sIn = (long long)N * sP;
+      for (int cnt = N; cnt > 1;) {
+        const int half = cnt / 2, out = (cnt + 1) / 2;
+        const long long sOut = (long long)out * sP;
+        std::memset(&g, 0, sizeof(g));
+        g.A = src + sP; g.B = src; g.C = dst;
+        g.m = pl; g.n = pl; g.k = pl; g.opA = 0;
+        g.lda = pl; g.ldb = pl; g.ldc = pl;
+        g.bin = half;
+        g.sA = 2 * sP; g.sB = 2 * sP; g.sC = sP;
+        g.sAo = sIn; g.sBo = sIn; g.sCo = sOut;
+        g.batch = (long long)nl * half;
+        BW_CUDA(bw::launch_zgemm(g, s, mx), "loop-product GEMM");
+        if (cnt & 1)
+          BW_CUDA(cudaMemcpy2DAsync(dst + (long long)half * sP, size_t(sOut) * sizeof(z64),
+                                    src + (long long)(cnt - 1) * sP, size_t(sIn) * sizeof(z64),
+                                    size_t(sP) * sizeof(z64), size_t(nl), cudaMemcpyDeviceToDevice, s),
+                  "loop-product copy");
+        std::swap(src, dst);
+        sIn = sOut;
+        cnt = out;
+      }
+      Wcur = src;
+      sWcur = sIn;
+    } else {
+      for (int j = 1; j < N; ++j) {
+        z64* Wout = Wbuf[j & 1];
+        std::memset(&g, 0, sizeof(g));
+        g.A = Mblk + (long long)j * sP; g.B = Wcur; g.C = Wout;
+        g.m = pl; g.n = pl; g.k = pl; g.opA = 0;
+        g.lda = pl; g.ldb = pl; g.ldc = pl;
+        g.sA = (long long)N * sP; g.sB = sWcur; g.sC = sP;
+        g.batch = nl;
+        BW_CUDA(bw::launch_zgemm(g, s, mx), "loop-product GEMM");
+        Wcur = Wout;
+        sWcur = sP;
+      }
     }
     // the eigenphases in double-float as well when the cluster solver takes p; else W
     // back to FP64 (nl consecutive p x p matrices: sWcur = sP, or N sP = sP at N = 1)
@@ -912,7 +952,7 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
     return fail(ctx, BW_EINVAL, "nested loop supports p <= %d (p = %d)", bw::LOOP_P_MAX, p_eff);
   // many occupied bands: batched-GEMM loops (the spin-resolved one from p > 64 at
   // large n, where the split runs on the tridiagonal path)
-  const bool big = (kind == LoopKind::Plain && p_eff > bw::LOOP_P_MAX) ||
+  const bool big = (kind == LoopKind::Plain && p_eff > (prec == BW_MIXED ? bw::LOOP_P_MAX_DF : bw::LOOP_P_MAX)) ||
                    (kind == LoopKind::Spin && large && p > 64);
   const Opts o = resolve_opts(opts, P.tmax);
   if (o.unitarise && p_eff > 32) return fail(ctx, BW_EINVAL, "unitarise supports p <= 32");

@@ -13,7 +13,7 @@
 // the differences are exact in FP32, and 3 x 8 significant bits hold an FP32
 // significand), and every product keeps the eight terms a_i b_j with i + j <= 3
 // (smallest first); the one dropped term, a2 b2, is ~2^-48 relative.  The products of
-// bf16 values are exact.  Each chunk of 32 real terms is accumulated in TMEM in two
+// bf16 values are exact.  Each chunk of 64 real terms is accumulated in TMEM in two
 // accumulators, the seven cross products (smallest first) in one and a0 b0 alone in
 // the other, so that no small term is added into a full-size sum inside the tensor
 // core; the two are then added into FP32 registers.
@@ -22,7 +22,13 @@
 // holding its K range as consecutive 8-row x 16-byte core matrices (8 bf16 per row).  The
 // matrix descriptor's leading byte offset (LBO) is the distance between core matrices
 // adjacent along K (128 bytes), its stride byte offset (SBO) the distance between 8-row
-// groups (512 bytes: a chunk's 32 K values are four core matrices).
+// groups (1024 bytes: a chunk's 64 K values are eight core matrices).
+//
+// A thread stages eight consecutive inner indices of one row (or column), whose split
+// pieces are 16-byte core-matrix rows: conflict-free vector stores.  (Element by element, the
+// two-byte stores of a chunk serialised four ways and took longer than its MMAs; the chunk
+// of 16 complex indices then cost ~7000 clocks with two CTAs per SM.)  The next chunk's
+// operands are loaded into registers while the tensor core works.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -112,25 +118,38 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-// x = x0 + x1 + x2 in bf16 (round to nearest; each difference is exact in FP32).
-__device__ __forceinline__ void split3(float x, __nv_bfloat16 (&b)[3]) {
-  b[0] = __float2bfloat16_rn(x);
-  const float r1 = x - __bfloat162float(b[0]);
-  b[1] = __float2bfloat16_rn(r1);
-  b[2] = __float2bfloat16_rn(r1 - __bfloat162float(b[1]));
+// x = x0 + x1 + x2 in bf16 (round to nearest; each difference is exact in FP32) for eight
+// values: the three pieces as rows of eight bf16.
+__device__ __forceinline__ void split3x8(const float (&x)[8], uint4 (&out)[3]) {
+  uint32_t w[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float a = x[2 * i], b = x[2 * i + 1];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+      w[t][i] = *reinterpret_cast<const uint32_t*>(&h);
+      a -= __low2float(h);
+      b -= __high2float(h);
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 3; ++t) out[t] = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
 }
 
-// Byte offset of real element (row, k) of a tile with 32 bf16 values per row (4 core
-// matrices along K; SBO = 512).
-__device__ __forceinline__ int off16(int row, int k) {
-  return (row >> 3) * 512 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
+__device__ __forceinline__ uint4 neg8(uint4 v) {  // sign bits of eight bf16
+  return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
 }
 
 constexpr int TILE = 64;                  // complex rows / columns per output tile
-constexpr int KC = 16;                    // complex inner-dimension chunk (32 real)
-constexpr int A_BYTES = 128 * 32 * 2;     // one bf16 piece of the embedded A chunk (8 KB)
-constexpr int B_BYTES = 64 * 32 * 2;      // one bf16 piece of the embedded B chunk (4 KB)
-constexpr size_t SMEM = 3 * A_BYTES + 3 * B_BYTES;  // 36 KB (the epilogue reuses it)
+constexpr int KC = 32;                    // complex inner-dimension chunk (64 real)
+constexpr int ROW8 = 8 * 2 * KC * 2;      // bytes of a group of 8 rows (SBO)
+constexpr int A_BYTES = 128 * 2 * KC * 2; // one bf16 piece of the embedded A chunk (16 KB)
+constexpr int B_BYTES = 64 * 2 * KC * 2;  // one bf16 piece of the embedded B chunk (8 KB)
+constexpr size_t SMEM = 3 * A_BYTES + 3 * B_BYTES;  // 72 KB (the epilogue reuses it)
+
+// Byte offset of the 16-byte row (row, 8 oct .. 8 oct + 7) of a tile.
+__device__ __forceinline__ int off8(int row, int oct) { return (row >> 3) * ROW8 + oct * 128 + (row & 7) * 16; }
 constexpr uint32_t TMEM_COLS = 128;     // two 128 x 64 FP32 accumulators
 constexpr int WAIT_POLLS = 1 << 22;
 
@@ -181,53 +200,54 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
   const int row = 32 * (warp & 3) + lane, col0 = 32 * (warp >> 2);
   const uint32_t taddr = s.tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(col0);
   constexpr uint32_t IDESC = idesc_bf16(128, 64);
-  constexpr int PER = KC * TILE / 256;  // complex elements of each operand per thread per chunk
+  // this thread stages inner indices 8 oct .. 8 oct + 7 of row (of A) and column (of B) u
+  const int u = tid & 63, oct = tid >> 6;
+  static_assert(TILE == 64 && KC == 32, "one unit of each operand per thread");
   for (int m0 = 0; m0 < M; m0 += TILE)
     for (int c0 = 0; c0 < Ncol; c0 += TILE) {
       if (s.failed) return false;
       float acc[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) acc[j] = 0.f;
-      for (int k0 = 0; k0 < K; k0 += KC) {
+      c32 ra[8], rb[8];
+      auto fetch = [&](int k0) {
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const int e = tid + 256 * q;
-          int kk, mm;
-          if (A_K_CONTIG) {
-            mm = e / KC;
-            kk = e - mm * KC;
-          } else {
-            kk = e / TILE;
-            mm = e - kk * TILE;
-          }
-          const c32 a = (m0 + mm < M && k0 + kk < K) ? la(m0 + mm, k0 + kk) : c32(0.f, 0.f);
-          __nv_bfloat16 re[3], im[3];
-          split3(a.re, re);
-          split3(a.im, im);
+        for (int j = 0; j < 8; ++j) {
+          const int k = k0 + 8 * oct + j;
+          ra[j] = (m0 + u < M && k < K) ? la(m0 + u, k) : c32(0.f, 0.f);
+          rb[j] = (c0 + u < Ncol && k < K) ? lb(k, c0 + u) : c32(0.f, 0.f);
+        }
+      };
+      fetch(0);
+      for (int k0 = 0; k0 < K; k0 += KC) {
+        {
+          float x[8];
+          uint4 re[3], im[3];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = ra[j].re;
+          split3x8(x, re);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = ra[j].im;
+          split3x8(x, im);
 #pragma unroll
           for (int t = 0; t < 3; ++t) {
             unsigned char* P = Ap + t * A_BYTES;
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(mm, kk)) = re[t];
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(mm, KC + kk)) = __hneg(im[t]);
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(TILE + mm, kk)) = im[t];
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(TILE + mm, KC + kk)) = re[t];
+            *reinterpret_cast<uint4*>(P + off8(u, oct)) = re[t];
+            *reinterpret_cast<uint4*>(P + off8(u, KC / 8 + oct)) = neg8(im[t]);
+            *reinterpret_cast<uint4*>(P + off8(TILE + u, oct)) = im[t];
+            *reinterpret_cast<uint4*>(P + off8(TILE + u, KC / 8 + oct)) = re[t];
           }
-          int cc;
-          if (B_C_CONTIG) {
-            kk = e / TILE;
-            cc = e - kk * TILE;
-          } else {
-            cc = e / KC;
-            kk = e - cc * KC;
-          }
-          const c32 b = (c0 + cc < Ncol && k0 + kk < K) ? lb(k0 + kk, c0 + cc) : c32(0.f, 0.f);
-          split3(b.re, re);
-          split3(b.im, im);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = rb[j].re;
+          split3x8(x, re);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = rb[j].im;
+          split3x8(x, im);
 #pragma unroll
           for (int t = 0; t < 3; ++t) {
             unsigned char* P = Bp + t * B_BYTES;
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(cc, kk)) = re[t];
-            *reinterpret_cast<__nv_bfloat16*>(P + off16(cc, KC + kk)) = im[t];
+            *reinterpret_cast<uint4*>(P + off8(u, oct)) = re[t];
+            *reinterpret_cast<uint4*>(P + off8(u, KC / 8 + oct)) = im[t];
           }
         }
         fence_async_smem();
@@ -242,15 +262,16 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
 #pragma unroll
           for (int t = 0; t < 8; ++t)
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {  // 16 real K values (two core matrices) per MMA
+            for (int ks = 0; ks < 2 * KC / 16; ++ks) {  // 16 real K values (two core matrices) per MMA
               const uint32_t o = ks * 256;
               const bool big = t == 7;
-              mma_bf16(s.tmem + (big ? 64u : 0u), smem_desc(a0 + PI[t] * A_BYTES + o, 128, 512),
-                       smem_desc(b0 + PJ[t] * B_BYTES + o, 128, 512), IDESC,
+              mma_bf16(s.tmem + (big ? 64u : 0u), smem_desc(a0 + PI[t] * A_BYTES + o, 128, ROW8),
+                       smem_desc(b0 + PJ[t] * B_BYTES + o, 128, ROW8), IDESC,
                        (big ? ks : (ks | t)) ? 1u : 0u);
             }
           commit(s.mbar);
         }
+        if (k0 + KC < K) fetch(k0 + KC);
         // every thread waits for the chunk's MMAs before its shared memory is restaged
         const bool ok = mbar_wait(s.mbar, s.phase, WAIT_POLLS);
         s.phase ^= 1u;
@@ -260,9 +281,9 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
           return false;
         }
         // the chunk's partial sums into the FP32 register accumulators
-        float v[16], w[16];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+          float v[16], w[16];
           ld16(taddr + uint32_t(16 * h), v);
           ld16(taddr + 64u + uint32_t(16 * h), w);
 #pragma unroll

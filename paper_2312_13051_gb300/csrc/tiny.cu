@@ -100,7 +100,7 @@ __device__ __forceinline__ void sort_eig(const cx<T> (&A)[NN][NN], const cx<T> (
   }
 }
 
-constexpr int TINY_THREADS = 32;
+constexpr int TINY_THREADS = 128;
 // Above this many points a direction's phase table is split in two levels
 // (w^m = w^{B (m / B)} w^{m mod B}, B ~ sqrt(M)): each CTA fills its own tables, and past
 // about a hundred entries their sines and cosines (~45 FP64 instructions each) would cost
@@ -112,16 +112,6 @@ __host__ __device__ inline TabShape tab_shape(int M) {
   int B = 1;
   while (B * B < M) ++B;
   return {B, (M + B - 1) / B};
-}
-
-// Fills lo[0..B) and hi[0..H) with exp(i 2pi m / M).
-__device__ void fill_tab(z64* lo, z64* hi, int M, TabShape t) {
-  for (int m = threadIdx.x; m < t.B + t.H; m += blockDim.x) {
-    const long long e = m < t.B ? m : (long long)(m - t.B) * t.B;
-    double sn, cs;
-    sincospi(2.0 * double(e) / double(M), &sn, &cs);
-    *(m < t.B ? lo + m : hi + (m - t.B)) = z64(cs, sn);
-  }
 }
 
 __device__ __forceinline__ z64 tab_at(const z64* lo, const z64* hi, TabShape t, int m) {
@@ -199,25 +189,35 @@ __device__ __forceinline__ TinySmem tiny_tables(const StatesArgs& a, unsigned ch
       S.hr[h] = md.hop_r[h];
     }
   if (use_tab) {
-    fill_tab(S.tabN, S.tabN + tN.B, N, tN);
-    fill_tab(S.tabNt, S.tabNt + tT.B, Nt, tT);
-    for (int r = tid; r < nR; r += bd) {
-      const int* R = md.Rv + 3 * r;
+    // w_N^m, w_Nt^m (both levels) and the translations' factors at the origin: one loop, so
+    // that a CTA with a thread per entry evaluates sine and cosine (~40 dependent FP64
+    // operations) once
+    const int cN = tN.B + tN.H, cT = tT.B + tT.H;
+    for (int m = tid; m < cN + cT + nR; m += bd) {
       double x = 0.0;
-      long long l = 0, t = 0, sw = 0;
-      for (int d = 0; d < 3; ++d) {
-        x += a.plane.origin[d] * double(R[d]);
-        l += (long long)(a.plane.loop_dir[d]) * R[d];
-        t += (long long)(a.plane.trans_dir[d]) * R[d];
-        sw += (long long)a.plane.sweep[d] * R[d];
+      if (m < cN + cT) {
+        const int q = m < cN ? m : m - cN, M = m < cN ? N : Nt;
+        const TabShape t = m < cN ? tN : tT;
+        x = 2.0 * double(q < t.B ? (long long)q : (long long)(q - t.B) * t.B) / double(M);
+      } else {
+        const int r = m - cN - cT;
+        const int* R = md.Rv + 3 * r;
+        long long l = 0, t = 0, sw = 0;
+        for (int d = 0; d < 3; ++d) {
+          x += a.plane.origin[d] * double(R[d]);
+          l += (long long)(a.plane.loop_dir[d]) * R[d];
+          t += (long long)(a.plane.trans_dir[d]) * R[d];
+          sw += (long long)a.plane.sweep[d] * R[d];
+        }
+        x *= 2.0;
+        // exponents of w_N per loop step, and of w_Nt per transverse and per sweep step
+        S.lR[r] = pmod(l, N);
+        S.tR[r] = pmod(a.plane.N_s > 1 ? t * a.plane.N_s : t, Nt);
+        S.sR[r] = pmod(a.plane.N_s > 1 ? sw * a.plane.N_tp : 0, Nt);
       }
       double sn, cs;
-      sincospi(2.0 * x, &sn, &cs);
-      S.oph[r] = z64(cs, sn);
-      // exponents of w_N per loop step, and of w_Nt per transverse and per sweep step
-      S.lR[r] = pmod(l, N);
-      S.tR[r] = pmod(a.plane.N_s > 1 ? t * a.plane.N_s : t, Nt);
-      S.sR[r] = pmod(a.plane.N_s > 1 ? sw * a.plane.N_tp : 0, Nt);
+      sincospi(x, &sn, &cs);
+      S.tabN[m] = z64(cs, sn);  // tabN, tabNt and oph follow each other
     }
   }
   if (!plan) {
