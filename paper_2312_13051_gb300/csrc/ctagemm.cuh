@@ -204,7 +204,8 @@ __device__ void cta_gemm(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned c
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < TN / 16; ++j)
-              if (!kUpper || m0 + 16 * i < c0 + 16 * (j + 1)) Pol::mac(acc[i][j], av[i], bv[j]);
+              if (m0 + 16 * i < M && c0 + 16 * j < Ncol && (!kUpper || m0 + 16 * i < c0 + 16 * (j + 1)))
+                Pol::mac(acc[i][j], av[i], bv[j]);  // groups past a ragged edge cost as much as full ones
         }
         __syncthreads();
       }

@@ -25,7 +25,8 @@ constexpr int GEIG_NB = 8;
 struct GeigShared {
   double c[GEIG_NB];    // Givens of each sweep: G = [[c, s], [-conj(s), c]], c real
   z64 s[GEIG_NB];
-  z64 shift[GEIG_NB];
+  z64 shift;                 // of a single sweep
+  c32 shifts[GEIG_NB];       // of several
   c32 B[GEIG_NB * GEIG_NB];  // trailing block (shift selection)
   z64 mu;
   int l, hi, nb, active, fail;
@@ -106,18 +107,13 @@ __device__ __forceinline__ z64 geig_shift(z64 a, z64 b, z64 c, z64 d, int iter, 
   return (abs2(m1 - d) <= abs2(m2 - d)) ? m1 : m2;
 }
 
-// Shifts of nb simultaneous sweeps: the eigenvalues of the trailing nb x nb block of the
-// active window (last row hi) by single-shift QR in FP32 (a shift decides how fast the
+// Shifts of nb simultaneous sweeps: the eigenvalues of the trailing nb x nb block B (FP32,
+// Hessenberg) of the active window by single-shift QR (a shift decides how fast the
 // sweeps converge, not what they converge to), in the order in which they separate from
-// the bottom.  At its cap of sweeps the diagonal entries left over serve.  The first warp
-// calls it, all lanes.
-__device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, z64* shift) {
-  const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
-  for (int e = lane; e < nb * nb; e += 32) {
-    const int r = e / nb, c = e - r * nb;
-    B[e] = r <= c + 1 ? ccast<float>(H[(h0 + r) * ld + h0 + c]) : c32(0.f, 0.f);
-  }
-  __syncwarp();
+// the bottom.  At its cap of sweeps the diagonal entries left over serve.  One warp calls
+// it, all lanes; nb <= 32.
+__device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
+  const int lane = threadIdx.x & 31;
   int top = nb - 1, out = 0;
   for (int it = 0; it < 8 * GEIG_NB && top > 0; ++it) {
     // split point: the largest l whose subdiagonal entry is negligible
@@ -127,7 +123,7 @@ __device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb
     const unsigned m = __ballot_sync(0xffffffffu, small);
     const int l = m ? 31 - __clz(m) : 0;
     if (l == top) {
-      if (lane == 0) shift[out] = ccast<double>(B[top * nb + top]);
+      if (lane == 0) shift[out] = B[top * nb + top];
       ++out;
       --top;
       continue;
@@ -171,8 +167,18 @@ __device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb
       __syncwarp();
     }
   }
-  if (lane <= top) shift[out + lane] = ccast<double>(B[(top - lane) * nb + top - lane]);
+  if (lane <= top) shift[out + lane] = B[(top - lane) * nb + top - lane];
   __syncwarp();
+}
+
+__device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, c32* shift) {
+  const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
+  for (int e = lane; e < nb * nb; e += 32) {
+    const int r = e / nb, c = e - r * nb;
+    B[e] = r <= c + 1 ? ccast<float>(H[(h0 + r) * ld + h0 + c]) : c32(0.f, 0.f);
+  }
+  __syncwarp();
+  geig_block_shifts(B, nb, shift);
 }
 
 // Largest l in [1, hi] whose subdiagonal entry is negligible, or 0: the first warp
@@ -225,12 +231,20 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
       vec[r] = r == c + 1 ? z64(nv * v0m * ph.re, nv * v0m * ph.im) : nv * H[r * ld + c];
     if (tid == 0) sh->mu = -nx * ph;
     __syncthreads();
-    // left: H <- (I - 2 v v^dagger) H on rows c+1.., columns c+1.. (column c is set below)
-    for (int col = c + 1 + tid; col < p; col += nt) {
+    // left: H <- (I - 2 v v^dagger) H on rows c+1.., columns c+1.. (column c is set below);
+    // a warp takes eight columns, four lanes per column share its rows
+    for (int cb = c + 1 + 8 * warp; cb < p; cb += 8 * nwarp) {
+      const int col = cb + (lane & 7), r0 = c + 1 + (lane >> 3);
       z64 w(0.0, 0.0);
-      for (int r = c + 1; r < p; ++r) cfma_conj(w, vec[r], H[r * ld + col]);
-      const z64 w2 = 2.0 * w;
-      for (int r = c + 1; r < p; ++r) cfms(H[r * ld + col], vec[r], w2);
+      if (col < p)
+        for (int r = r0; r < p; r += 4) cfma_conj(w, vec[r], H[r * ld + col]);
+      for (int o = 8; o < 32; o <<= 1) {
+        w.re += __shfl_xor_sync(0xffffffffu, w.re, o);
+        w.im += __shfl_xor_sync(0xffffffffu, w.im, o);
+      }
+      w = 2.0 * w;
+      if (col < p)
+        for (int r = r0; r < p; r += 4) cfms(H[r * ld + col], vec[r], w);
     }
     __syncthreads();
     // right: H <- H (I - 2 v v^dagger) on columns c+1..; Z likewise
@@ -291,9 +305,9 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         // nothing deflates (exceptional shifts)
         nb = size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
         if (nb > 1) {
-          geig_shifts(H, ld, hi, nb, sh->B, sh->shift);
+          geig_shifts(H, ld, hi, nb, sh->B, sh->shifts);
         } else if (tid == 0) {
-          sh->shift[0] =
+          sh->shift =
               geig_shift(H[(hi - 1) * ld + hi - 1], H[(hi - 1) * ld + hi], H[hi * ld + hi - 1], H[hi * ld + hi],
                          iter, hi >= 2 ? zabs(H[(hi - 1) * ld + hi - 2]) : 0.0);
         }
@@ -328,7 +342,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         if (k >= l && k < hi) {
           z64 x, y;
           if (k == l) {
-            x = H[l * ld + l] - sh->shift[tid];
+            x = H[l * ld + l] - (nb > 1 ? ccast<double>(sh->shifts[tid]) : sh->shift);
             y = H[(l + 1) * ld + l];
           } else {
             x = H[k * ld + k - 1];
@@ -384,39 +398,42 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
   __shared__ double tmax[32];
   tn = -block_min(-tn, tmax);
   const double small = fmax(eps * tn, 1e-300);
-  // Decreasing k: column k of X = Z[:, 0..k] y_k only uses columns <= k of the
-  // original Z, which are untouched when columns are replaced from the right.
-  for (int k = p - 1; k >= 0; --k) {
-    if (tid == 0) {
-      const z64 lk = H[k * ld + k];
-      for (int r = k + 1; r < p; ++r) vec[r] = z64(0.0, 0.0);
-      vec[k] = z64(1.0, 0.0);
-      for (int r = k - 1; r >= 0; --r) {
-        z64 acc(0.0, 0.0);
-        for (int c = r + 1; c <= k; ++c) cfma(acc, H[r * ld + c], vec[c]);
-        z64 den = H[r * ld + r] - lk;
-        if (zabs(den) < small) den = z64(small, 0.0);
-        const double dd = abs2(den);
-        vec[r] = z64(-(acc.re * den.re + acc.im * den.im) / dd,
-                     -(acc.im * den.re - acc.re * den.im) / dd);
-      }
+  // One thread per eigenvector: y_k by back substitution, kept in row k left of the diagonal
+  // (free below T), y_k[k] = 1.  (One thread for all of them, a division and a chain of sums
+  // per entry, was a quarter of the solver at p = 12.)
+  for (int k = tid; k < p; k += nt) {
+    z64* y = H + k * ld;
+    const z64 lk = H[k * ld + k];
+    for (int r = k - 1; r >= 0; --r) {
+      z64 acc = H[r * ld + k];
+      for (int c = r + 1; c < k; ++c) cfma(acc, H[r * ld + c], y[c]);
+      z64 den = H[r * ld + r] - lk;
+      if (zabs(den) < small) den = z64(small, 0.0);
+      const double dd = abs2(den);
+      y[r] = z64(-(acc.re * den.re + acc.im * den.im) / dd, -(acc.im * den.re - acc.re * den.im) / dd);
     }
-    __syncthreads();
-    double nrm = 0.0;
-    z64 xr[4];
-    int cnt = 0;
-    for (int row = tid; row < p; row += nt, ++cnt) {
-      z64 acc(0.0, 0.0);
-      for (int c = 0; c <= k; ++c) cfma(acc, Z[row * ld + c], vec[c]);
-      if (cnt < 4) xr[cnt] = acc;
-      nrm += abs2(acc);
-    }
-    nrm = block_sum(nrm, tmax);
-    const double inv = 1.0 / sqrt(nrm);
-    cnt = 0;
-    for (int row = tid; row < p; row += nt, ++cnt) Z[row * ld + k] = inv * xr[cnt];
-    __syncthreads();
   }
+  __syncthreads();
+  // X = Z Y row by row, columns from the right: column k only uses columns <= k of the
+  // original row
+  for (int row = tid; row < p; row += nt) {
+    z64* z = Z + row * ld;
+    for (int k = p - 1; k >= 0; --k) {
+      const z64* y = H + k * ld;
+      z64 acc = z[k];
+      for (int c = 0; c < k; ++c) cfma(acc, z[c], y[c]);
+      z[k] = acc;
+    }
+  }
+  __syncthreads();
+  for (int k = warp; k < p; k += nwarp) {  // unit columns
+    double s2 = 0.0;
+    for (int r = lane; r < p; r += 32) s2 += abs2(Z[r * ld + k]);
+    for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    const double inv = 1.0 / sqrt(s2);
+    for (int r = lane; r < p; r += 32) Z[r * ld + k] = inv * Z[r * ld + k];
+  }
+  __syncthreads();
   return 0;
 }
 

@@ -189,6 +189,8 @@ struct GemmArgs {
   z64* C;
   int m, n, k;
   int opA;                // 0: A (m x k), 1: A^dagger (A stored k x m)
+  int lower;              // 1: a Hermitian result, only its lower triangle is read (entries above
+                          // the diagonal are left undefined)
   long long lda, ldb, ldc;
   long long sA, sB, sC;
   long long a_next_N;
@@ -201,6 +203,9 @@ struct GemmArgs {
   long long sAo, sBo, sCo;
 };
 
+// Scratch per loop of the eigenphase kernels: a vector, or a chunk's rotations.
+__host__ __device__ inline int geig_vec_len(int p) { return p > 64 ? p : 64; }
+
 // Eigenphases of nl Wilson matrices W (p x p, stride sW), loops i0 .. i0+nl-1.
 struct BigEigArgs {
   z64* W;
@@ -212,7 +217,7 @@ struct BigEigArgs {
   double* min_gap;        // N_t (optional)
   double* min_pso_gap;    // N_t (optional)
   z64* lam;               // nl x p scratch
-  z64* vec;               // nl x p scratch
+  z64* vec;               // nl x geig_vec_len(p) scratch
   double* th;             // nl x p scratch
   int* ord;               // nl x p scratch
   double* ctl;            // nl x 8 scratch (control block of the cluster solver)
