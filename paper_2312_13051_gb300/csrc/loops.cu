@@ -161,7 +161,8 @@ __global__ void __launch_bounds__(OVL_THREADS, 1) k_overlaps_df(LoopArgs a) {
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int v = 0; v < 4; ++v) cmac_conj(acc[u][v], an[u], ah[v]);
+          for (int v = 0; v < 4; ++v)
+            if (16 * u < p && 16 * v < p) cmac_conj(acc[u][v], an[u], ah[v]);
       }
       __syncthreads();
     }
@@ -184,7 +185,8 @@ struct LoopSmem {
 };
 
 // df: room for one overlap matrix in double-float (the mixed request's product)
-__host__ __device__ inline LoopSmem loop_layout(int p, bool df = false) {
+// tree: room for N overlap matrices and half as many products in double-float
+__host__ __device__ inline LoopSmem loop_layout(int p, bool df = false, int tree = 0) {
   auto al = [](size_t x) { return (x + 15) & ~size_t(15); };
   LoopSmem L;
   size_t o = 0;
@@ -192,7 +194,7 @@ __host__ __device__ inline LoopSmem loop_layout(int p, bool df = false) {
   // column (a row length of p would put p = 32 or 64 rows in one bank)
   L.X = o; o = al(o + size_t(p) * (p + 1) * sizeof(z64));
   L.Y = o; o = al(o + size_t(p) * (p + 1) * sizeof(z64));
-  L.Ms = o; o = al(o + (df ? size_t(p) * p * sizeof(cdf) : 0));
+  L.Ms = o; o = al(o + (df ? size_t(p) * p * sizeof(cdf) * (tree ? tree + (tree + 1) / 2 : 1) : 0));
   L.lam = o; o = al(o + size_t(p) * sizeof(z64));
   L.vec = o; o = al(o + size_t(p) * sizeof(z64));
   L.th = o; o = al(o + size_t(p) * sizeof(double));
@@ -204,11 +206,11 @@ __host__ __device__ inline LoopSmem loop_layout(int p, bool df = false) {
   return L;
 }
 
-__global__ void k_loops(LoopArgs a) {
+__global__ void k_loops(LoopArgs a, int tree) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = a.n, p = a.p, N = a.N, tid = threadIdx.x, nt = blockDim.x;
   const int m = a.nested ? a.m : 1;
-  const LoopSmem L = loop_layout(p, a.df_overlaps != 0);
+  const LoopSmem L = loop_layout(p, a.df_overlaps != 0, tree ? N : 0);
   z64* X = reinterpret_cast<z64*>(smem + L.X);
   z64* Y = reinterpret_cast<z64*>(smem + L.Y);
   z64* lam = reinterpret_cast<z64*>(smem + L.lam);
@@ -244,33 +246,62 @@ __global__ void k_loops(LoopArgs a) {
       cdf* Wd = reinterpret_cast<cdf*>(X);
       cdf* Td = reinterpret_cast<cdf*>(Y);
       cdf* Md = reinterpret_cast<cdf*>(smem + L.Ms);
-      for (int e = tid; e < p * p; e += nt) {
-        const int r = e / p, c = e - r * p;
-        Wd[e] = cdf(df(r == c ? 1.f : 0.f), df(0.f));
-      }
-      for (int j = 0; j < N; ++j) {
-        const z64* M = a.M + (k0 + j) * (long long)p * p;
-        for (int e = tid; e < p * p; e += nt) Md[e] = cdf_from(M[e]);
+      const int pp = p * p;
+      if (tree) {
+        // few loops of small matrices: every overlap in shared memory, pairwise products
+        // (M_{2j+1} M_{2j}, an odd last one carried over) level by level
+        cdf* src = Md;
+        cdf* dst = Md + N * pp;
+        const z64* M = a.M + k0 * (long long)pp;
+        for (int e = tid; e < N * pp; e += nt) src[e] = cdf_from(M[e]);
         __syncthreads();
-        for (int e0 = tid; e0 < p * p; e0 += 4 * nt) {
-          cdf acc[4];
-          int rr[4], cc[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int e = min(e0 + u * nt, p * p - 1);
-            rr[u] = e / p;
-            cc[u] = e - rr[u] * p;
-            acc[u] = cdf_zero();
+        for (int cnt = N; cnt > 1; cnt = (cnt + 1) / 2) {
+          for (int e = tid; e < (cnt + 1) / 2 * pp; e += nt) {
+            const int j = e / pp, rc = e - j * pp, r = rc / p, c = rc - r * p;
+            const cdf* B = src + 2 * j * pp;
+            if (2 * j + 1 == cnt) {
+              dst[e] = B[rc];
+              continue;
+            }
+            const cdf* A = B + pp + r * p;
+            cdf acc = cdf_zero();
+            for (int q = 0; q < p; ++q) cmac(acc, A[q], B[q * p + c]);
+            dst[e] = cfin(acc);
           }
-          for (int q = 0; q < p; ++q)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) cmac(acc[u], Md[rr[u] * p + q], Wd[q * p + cc[u]]);
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (e0 + u * nt < p * p) Td[e0 + u * nt] = cfin(acc[u]);
+          __syncthreads();
+          cdf* t = src; src = dst; dst = t;
         }
+        for (int e = tid; e < pp; e += nt) Wd[e] = src[e];
         __syncthreads();
-        cdf* t = Wd; Wd = Td; Td = t;
+      } else {
+        for (int e = tid; e < p * p; e += nt) {
+          const int r = e / p, c = e - r * p;
+          Wd[e] = cdf(df(r == c ? 1.f : 0.f), df(0.f));
+        }
+        for (int j = 0; j < N; ++j) {
+          const z64* M = a.M + (k0 + j) * (long long)p * p;
+          for (int e = tid; e < p * p; e += nt) Md[e] = cdf_from(M[e]);
+          __syncthreads();
+          for (int e0 = tid; e0 < p * p; e0 += 4 * nt) {
+            cdf acc[4];
+            int rr[4], cc[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int e = min(e0 + u * nt, p * p - 1);
+              rr[u] = e / p;
+              cc[u] = e - rr[u] * p;
+              acc[u] = cdf_zero();
+            }
+            for (int q = 0; q < p; ++q)
+#pragma unroll
+              for (int u = 0; u < 4; ++u) cmac(acc[u], Md[rr[u] * p + q], Wd[q * p + cc[u]]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (e0 + u * nt < p * p) Td[e0 + u * nt] = cfin(acc[u]);
+          }
+          __syncthreads();
+          cdf* t = Wd; Wd = Td; Td = t;
+        }
       }
       // back to FP64 in place for the eigen-decomposition
       z64* Wz = reinterpret_cast<z64*>(Wd);
@@ -458,7 +489,9 @@ cudaError_t launch_wannier(const LoopArgs& a, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // Nested loop per base point
 // ---------------------------------------------------------------------------
-__global__ void k_nested(LoopArgs a) {
+// all: room for every overlap of a base point; they are formed at once, and only their ordered
+// product is a chain.
+__global__ void k_nested(LoopArgs a, int all) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = a.n, m = a.m, Ns = n_planes(a), Nt = a.N_t / Ns, tid = threadIdx.x, nt = blockDim.x;
   const LoopSmem L = loop_layout(m);
@@ -478,7 +511,29 @@ __global__ void k_nested(LoopArgs a) {
     }
     __syncthreads();
     const z64* wj = a.w + ((long long)j * a.N_t + (long long)sp * Nt) * n * m;
-    for (int i = 0; i < Nt; ++i) {
+    if (all) {
+      for (int e = tid; e < Nt * m * m; e += nt) {
+        const int i = e / (m * m), rc = e - i * m * m, r = rc / m, c = rc - r * m;
+        const z64* wa = wj + (long long)i * n * m;
+        const z64* wb = wj + (long long)(i + 1 == Nt ? 0 : i + 1) * n * m;
+        z64 acc(0.0, 0.0);
+        for (int q = 0; q < n; ++q) cfma_conj(acc, wb[q * m + r], wa[q * m + c]);
+        Mt[e] = acc;
+      }
+      __syncthreads();
+      for (int i = 0; i < Nt; ++i) {
+        const z64* Mi = Mt + i * m * m;
+        for (int e = tid; e < m * m; e += nt) {
+          const int r = e / m, c = e - r * m;
+          z64 acc(0.0, 0.0);
+          for (int q = 0; q < m; ++q) cfma(acc, Mi[r * m + q], W[q * m + c]);
+          T[e] = acc;
+        }
+        __syncthreads();
+        z64* t = W; W = T; T = t;
+      }
+    }
+    for (int i = 0; i < Nt && !all; ++i) {
       const z64* wa = wj + (long long)i * n * m;
       const z64* wb = wj + (long long)(i + 1 == Nt ? 0 : i + 1) * n * m;
       for (int e = tid; e < m * m; e += nt) {
@@ -801,7 +856,8 @@ __global__ void k_loops_scan(LoopArgs a) {
 // run of consecutive points, the lanes' products are folded in order by shuffles, and the
 // eigenphases come in closed form.  The scan kernel above spends most of its time at block
 // barriers here (log N levels with a few scalar products each); it stays for nested loops,
-// which need every partial product.  Eq. 4, 24 x 24: see launch_loops.
+// which need every partial product.  Eq. 4, 24 x 24: 11.9 -> 9.9 us; spin-Hall 51 x 51 14.3 ->
+// 10.9 us.
 template <int PP>
 __global__ void k_loops_warp(LoopArgs a) {
   const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1493,11 +1549,16 @@ cudaError_t launch_loops(const LoopArgs& a, cudaStream_t s) {
   LoopArgs b = a;
   if (b.df_overlaps && loop_layout(b.p, true).total > size_t(227) * 1024)
     b.df_overlaps = 0;
-  const LoopSmem L = loop_layout(b.p, b.df_overlaps != 0);
+  // with a CTA per SM at most, the product as a tree where its matrices fit (p = 12, 31 loops of
+  // 31 points: the chain's 31 steps of one round trip and two barriers each took a quarter of
+  // the kernel)
+  int tree = b.df_overlaps && b.N > 2 && b.N_t <= 152;
+  if (tree && loop_layout(b.p, true, b.N).total > size_t(200) * 1024) tree = 0;
+  const LoopSmem L = loop_layout(b.p, b.df_overlaps != 0, tree ? b.N : 0);
   static size_t cached = 0;
   cudaError_t e = set_smem_once(k_loops, L.total, cached);
   if (e != cudaSuccess) return e;
-  k_loops<<<b.N_t, loop_threads(b.p), L.total, s>>>(b);
+  k_loops<<<b.N_t, tree ? 256 : loop_threads(b.p), L.total, s>>>(b, tree);
   return cudaGetLastError();
 }
 
@@ -1692,11 +1753,14 @@ cudaError_t launch_nested(const LoopArgs& a, cudaStream_t s) {
     return cudaGetLastError();
   }
   const LoopSmem L = loop_layout(a.m);
-  const size_t sm = L.total + size_t(a.m) * a.m * sizeof(z64);
+  // every overlap of a base point at once where they take little shared memory
+  const size_t mm = size_t(a.m) * a.m * sizeof(z64), every = mm * (a.N_t / n_planes(a));
+  const int all = every <= 48 * 1024;
+  const size_t sm = L.total + (all ? every : mm);
   static size_t cached = 0;
   cudaError_t e = set_smem_once(k_nested, sm, cached);
   if (e != cudaSuccess) return e;
-  k_nested<<<grid, loop_threads(a.m), sm, s>>>(a);
+  k_nested<<<grid, all ? 256 : loop_threads(a.m), sm, s>>>(a, all);
   return cudaGetLastError();
 }
 
