@@ -105,8 +105,10 @@ __global__ void k_lg_build(LargeArgs a) {
         cdf acc(df(0.f), df(0.f));
         for (int h = md.ent_start[e]; h < md.ent_start[e + 1]; ++h) {
           const int r = md.hop_r[h];
-          const float* t4 = md.hop_tdf + 4 * h;
-          cmac(acc, cdf(df(t4[0], t4[1]), df(t4[2], t4[3])),
+          // one 16-byte load: the entries of neighbouring threads lie n_R hoppings apart, so
+          // every load instruction touches a line per lane
+          const float4 t4 = reinterpret_cast<const float4*>(md.hop_tdf)[h];
+          cmac(acc, cdf(df(t4.x, t4.y), df(t4.z, t4.w)),
                r < nRs ? phd[r] : cdf_from(bloch_phase(f, md.Rv + 3 * r)));
         }
         acc = cfin(acc);
@@ -124,7 +126,8 @@ __global__ void k_lg_build(LargeArgs a) {
       z64 acc(0.0, 0.0);
       for (int h = md.ent_start[e]; h < md.ent_start[e + 1]; ++h) {
         const int r = md.hop_r[h];
-        cfma(acc, md.hop_t[h], r < nRs ? phs[r] : bloch_phase(f, md.Rv + 3 * r));
+        const double2 t = reinterpret_cast<const double2*>(md.hop_t)[h];
+        cfma(acc, z64(t.x, t.y), r < nRs ? phs[r] : bloch_phase(f, md.Rv + 3 * r));
       }
       A[(long long)md.ent_row[e] * n + md.ent_col[e]] = ccast<T>(acc);
       if (a.Hent) {  // FP64 entry as an unevaluated sum of two floats (hi, lo)
@@ -273,69 +276,48 @@ __global__ void k_lg_tridiag(LargeArgs a) {
 // result does not depend on scheduling.
 // ---------------------------------------------------------------------------
 
-// Turns xs[c+1..n) (column c below the diagonal) into the unit reflector u with
-// (I - 2 u u^dag) x = alpha e_1 and returns alpha; u = 0 when nothing lies below the
-// subdiagonal.  Block-wide.
 // Block-wide sum in the working precision (FP32 for the mixed solve: GB300's FP64
 // pipe is ~70x narrower, and these per-step reductions would otherwise cost as much
-// as the sweep over the matrix).
+// as the sweep over the matrix), with one barrier: the caller's next use of `red` comes
+// after another one.
 template <typename T>
-__device__ __forceinline__ T block_sum_t(T v, double* red) {
+__device__ __forceinline__ T block_sum_1(T v, T* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  T* r = reinterpret_cast<T*>(red);
-  const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) r[w] = v;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   T s = T(0);
-  for (int k = 0; k < nw; ++k) s += r[k];
-  __syncthreads();
+  for (int k = 0; k < int(blockDim.x >> 5); ++k) s += red[k];
   return s;
 }
 
-// Turns xs[c+1..n) (column c below the diagonal) into the unit reflector u with
-// (I - 2 u u^dag) x = alpha e_1 and returns alpha; u = 0 when nothing lies below the
-// subdiagonal.  Block-wide, in the working precision T.
+// The reflector of a column x with leading entry x0 and |x|^2 - |x0|^2 = tail: (I - 2 u u^dag) x =
+// alpha e_1 with u = inv (x - alpha e_1), u_0 = inv v0; u = 0 and alpha = x0 when nothing
+// lies below the leading entry.
 template <typename T>
-__device__ cx<T> lg_reflector(cx<T>* xs, int c, int n, double* red) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  T s = T(0);
-  for (int r = c + 1 + tid; r < n; r += nt) s += abs2(xs[r]);
-  s = block_sum_t(s, red);
-  const cx<T> x0 = xs[c + 1];
-  const T ax0 = sqrt(abs2(x0)), tail = s - ax0 * ax0;
-  __syncthreads();
-  if (!(tail > T(0))) {
-    for (int r = c + 1 + tid; r < n; r += nt) xs[r] = cx<T>(T(0), T(0));
-    __syncthreads();
-    return x0;
+struct LgReflector {
+  cx<T> alpha, v0;
+  T inv;
+  __device__ LgReflector(cx<T> x0, T tail) : alpha(x0), v0(T(0), T(0)), inv(T(0)) {
+    if (!(tail > T(0))) return;
+    const T ax2 = abs2(x0), ax0 = sqrt(ax2), nx = sqrt(ax2 + tail);
+    const cx<T> ph = ax0 > T(0) ? cx<T>(x0.re / ax0, x0.im / ax0) : cx<T>(T(1), T(0));
+    const T v0m = ax0 + nx;
+    inv = T(1) / sqrt(v0m * v0m + tail);
+    v0 = v0m * ph;
+    alpha = -nx * ph;
   }
-  const T nx = sqrt(s);
-  const T phr = ax0 > T(0) ? x0.re / ax0 : T(1), phi = ax0 > T(0) ? x0.im / ax0 : T(0);
-  const T v0m = ax0 + nx;
-  const T inv = T(1) / sqrt(v0m * v0m + tail);
-  for (int r = c + 1 + tid; r < n; r += nt) {
-    const cx<T> v = r == c + 1 ? cx<T>(phr * v0m, phi * v0m) : xs[r];
-    xs[r] = inv * v;
-  }
-  __syncthreads();
-  return cx<T>(-phr * nx, -phi * nx);
-}
+};
 
 // Rows and columns lo..n-1 of the lower triangle: with upd, A <- A - 2 (u w^dag + w u^dag);
-// then pa = A u2 (pw: per-warp accumulators, stride n).  A warp takes RW rows at a
+// then A u2 into pw (per-warp accumulators, stride n).  A warp takes RW rows at a
 // time (r, r + nwarp, ...) and walks their columns together, so that RW loads per
-// lane are in flight even when the rows are short.  Ends with pa complete.
-template <typename T>
-__device__ void lg_hpass(cx<T>* A, int n, int lo, bool upd, const cx<T>* u, const cx<T>* w,
-                         const cx<T>* u2, cx<T>* pw, cx<T>* pa) {
+// lane are in flight even when the rows are short.  Row r is read at src(r)[q] and, with upd
+// or kCopy, written to dst(r)[q].  The caller zeroes pw before and sums it over warps after.
+template <typename T, bool kCopy, class SR, class DR>
+__device__ void lg_hpass(SR src, DR dst, int n, int lo, bool upd, const cx<T>* u, const cx<T>* w,
+                         const cx<T>* u2, cx<T>* pw) {
   constexpr int RW = sizeof(T) == 4 ? 8 : 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int e = threadIdx.x; e < nwarp * (n - lo); e += blockDim.x) {
-    const int ww = e / (n - lo), q = lo + (e - ww * (n - lo));
-    pw[ww * n + q] = cx<T>(T(0), T(0));
-  }
-  __syncthreads();
   cx<T>* acc_w = pw + warp * n;
   const cx<T> zero(T(0), T(0));
   for (int r0 = lo + warp; r0 < n; r0 += RW * nwarp) {
@@ -347,8 +329,8 @@ __device__ void lg_hpass(cx<T>* A, int n, int lo, bool upd, const cx<T>* u, cons
       rr[i] = r0 + i * nwarp;
       const bool ok = rr[i] < n;
       if (ok) rmax = rr[i];
-      ur[i] = ok && upd ? u[rr[i]] : zero;
-      wr[i] = ok && upd ? w[rr[i]] : zero;
+      ur[i] = ok && upd ? T(2) * u[rr[i]] : zero;
+      wr[i] = ok && upd ? T(2) * w[rr[i]] : zero;
       u2r[i] = ok ? u2[rr[i]] : zero;
       acc[i] = zero;
       if (!ok) rr[i] = -1;
@@ -357,7 +339,7 @@ __device__ void lg_hpass(cx<T>* A, int n, int lo, bool upd, const cx<T>* u, cons
       cx<T> v[RW];
 #pragma unroll
       for (int i = 0; i < RW; ++i)
-        v[i] = q <= rr[i] ? A[(long long)rr[i] * n + q] : zero;
+        v[i] = q <= rr[i] ? src(rr[i])[q] : zero;
       const cx<T> wq = upd ? w[q] : zero, uq = upd ? u[q] : zero, u2q = u2[q];
       cx<T> tq = zero;
 #pragma unroll
@@ -365,12 +347,24 @@ __device__ void lg_hpass(cx<T>* A, int n, int lo, bool upd, const cx<T>* u, cons
         if (q > rr[i]) continue;
         cx<T> x = v[i];
         if (upd) {
-          x = x - T(2) * (ur[i] * conj(wq) + wr[i] * conj(uq));
+          // FP64: eight fused operations.  FP32, where latency counts: the two products side by
+          // side (n = 400, 256 k-points: 12.1 ms against 15.2 with the fused chain)
+          if constexpr (sizeof(T) == 8) {
+            cfms(x, ur[i], conj(wq));
+            cfms(x, wr[i], conj(uq));
+          } else {
+            x = x - (ur[i] * conj(wq) + wr[i] * conj(uq));
+          }
           if (q == rr[i]) x.im = T(0);
-          A[(long long)rr[i] * n + q] = x;
         }
+        if (upd || kCopy) dst(rr[i])[q] = x;
         cfma(acc[i], x, u2q);
-        if (q < rr[i]) tq = tq + conj(x) * u2r[i];
+        if (q < rr[i]) {
+          if constexpr (sizeof(T) == 8)
+            cfma_conj(tq, x, u2r[i]);
+          else
+            tq = tq + conj(x) * u2r[i];
+        }
       }
       acc_w[q] = acc_w[q] + tq;
     }
@@ -382,79 +376,111 @@ __device__ void lg_hpass(cx<T>* A, int n, int lo, bool upd, const cx<T>* u, cons
     }
     __syncwarp();
   }
-  __syncthreads();
-  for (int q = lo + threadIdx.x; q < n; q += blockDim.x) {
-    cx<T> t(T(0), T(0));
-    for (int ww = 0; ww < nwarp; ++ww) t = t + pw[ww * n + q];
-    pa[q] = t;
-  }
-  __syncthreads();
 }
 
-// w = p - (u^dag p) u on lo..n-1 (p in pa).
-template <typename T>
-__device__ void lg_make_w(const cx<T>* u, const cx<T>* pa, cx<T>* w, int lo, int n, double* red) {
-  T kr = T(0);
-  for (int r = lo + threadIdx.x; r < n; r += blockDim.x) kr += u[r].re * pa[r].re + u[r].im * pa[r].im;
-  kr = block_sum_t(kr, red);
-  for (int r = lo + threadIdx.x; r < n; r += blockDim.x) w[r] = pa[r] - kr * u[r];
-  __syncthreads();
-}
-
-template <typename T>
+// kShared: the matrix is held in shared memory (packed lower triangle) from the first sweep on.
+// A step has five block barriers: the column with its norm, the reflector, the sweep, p = A u
+// with u^dag p, and w.
+template <typename T, bool kShared>
 __global__ void __launch_bounds__(512) k_lg_tridiag_h(LargeArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
+  const int n = a.n, tid = threadIdx.x, nt = blockDim.x, nwarp = nt >> 5;
   cx<T>* u = reinterpret_cast<cx<T>*>(smem);  // reflector of the current step
   cx<T>* w = u + n;
   cx<T>* u2 = w + n;                          // reflector of the next step
   cx<T>* pa = u2 + n;                         // A u2
   cx<T>* al = pa + n;                         // complex subdiagonal
   cx<T>* pw = al + n;                         // (blockDim / 32) x n per-warp accumulators
-  double* red = reinterpret_cast<double*>(pw + (nt >> 5) * n);
+  T* red = reinterpret_cast<T*>(pw + nwarp * n);  // two buffers of 16 partial sums, x0
+  cx<T>* x0s = reinterpret_cast<cx<T>*>(red + 32);
+  cx<T>* tri = reinterpret_cast<cx<T>*>(reinterpret_cast<double*>(red) + 64);
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
     if (std::is_same<T, double>::value && a.need && !a.need[kw]) continue;
     cx<T>* A = reinterpret_cast<cx<T>*>(a.A) + kw * (long long)n * n;
     T* dg = reinterpret_cast<T*>(a.dg) + kw * n;
     T* od = reinterpret_cast<T*>(a.od) + kw * n;
     cx<T>* Dp = reinterpret_cast<cx<T>*>(a.Dp) + kw * n;
+    auto grow = [&](int r) { return A + (long long)r * n; };
+    auto trow = [&](int r) { return kShared ? tri + r * (r + 1) / 2 : grow(r); };
+    // the column in u2[lo..n) with the partial sum s of its tail becomes the reflector, which
+    // also goes to column lo - 1 of A
+    auto reflect = [&](T s, int lo) {
+      s = block_sum_1(s, red);
+      const LgReflector<T> f(*x0s, s);
+      if (tid == 0) al[lo - 1] = f.alpha;
+      for (int r = lo + tid; r < n; r += nt) {
+        const cx<T> v = f.inv * (r == lo ? f.v0 : u2[r]);
+        u2[r] = v;
+        grow(r)[lo - 1] = v;
+      }
+      __syncthreads();
+    };
+    // after a sweep: pa = A u2, w = pa - (u2^dag pa) u2; u2 becomes u
+    auto finish = [&](int lo) {
+      __syncthreads();
+      T kr = T(0);
+      for (int q = lo + tid; q < n; q += nt) {
+        cx<T> t(T(0), T(0));
+        for (int k = 0; k < nwarp; ++k) {
+          t = t + pw[k * n + q];
+          pw[k * n + q] = cx<T>(T(0), T(0));
+        }
+        pa[q] = t;
+        kr += u2[q].re * t.re + u2[q].im * t.im;
+      }
+      kr = block_sum_1(kr, red + 16);
+      for (int q = lo + tid; q < n; q += nt) w[q] = pa[q] - kr * u2[q];
+      cx<T>* t = u;
+      u = u2;
+      u2 = t;
+      __syncthreads();
+    };
     // step 0: reflector of column 0 and p = A22 u
-    for (int r = 1 + tid; r < n; r += nt) u[r] = A[(long long)r * n];
-    __syncthreads();
-    cx<T> alpha = lg_reflector(u, 0, n, red);
-    if (tid == 0) {
-      al[0] = alpha;
-      dg[0] = A[0].re;
+    for (int e = tid; e < nwarp * n; e += nt) pw[e] = cx<T>(T(0), T(0));
+    T s = T(0);
+    for (int r = 1 + tid; r < n; r += nt) {
+      const cx<T> x = A[(long long)r * n];
+      u2[r] = x;
+      if (r == 1)
+        *x0s = x;
+      else
+        s += abs2(x);
     }
-    for (int r = 1 + tid; r < n; r += nt) A[(long long)r * n] = u[r];
-    __syncthreads();
-    lg_hpass<T>(A, n, 1, false, nullptr, nullptr, u, pw, pa);
-    lg_make_w(u, pa, w, 1, n, red);
+    if (tid == 0) dg[0] = A[0].re;
+    reflect(s, 1);
+    lg_hpass<T, kShared>(grow, trow, n, 1, false, nullptr, nullptr, u2, pw);
+    finish(1);
+    if (n == 2 && tid == 0) dg[1] = trow(1)[1].re;
     for (int c = 0; c + 2 < n; ++c) {
       // column c+1 of A - 2 (u w^dag + w u^dag), rows c+1..n-1
-      const cx<T> uc = u[c + 1], wc = w[c + 1];
-      for (int r = c + 1 + tid; r < n; r += nt)
-        u2[r] = A[(long long)r * n + c + 1] - T(2) * (u[r] * conj(wc) + w[r] * conj(uc));
-      __syncthreads();
-      if (tid == 0) dg[c + 1] = u2[c + 1].re;
+      const cx<T> uc = T(2) * conj(u[c + 1]), wc = T(2) * conj(w[c + 1]);
+      s = T(0);
+      for (int r = c + 1 + tid; r < n; r += nt) {
+        cx<T> x = trow(r)[c + 1];
+        cfms(x, u[r], wc);
+        cfms(x, w[r], uc);
+        u2[r] = x;
+        if (r == c + 1)
+          dg[c + 1] = x.re;
+        else if (r == c + 2)
+          *x0s = x;
+        else
+          s += abs2(x);
+      }
       if (c + 3 == n) {  // last 2 x 2 block: its subdiagonal and diagonal, no reflector
+        __syncthreads();
         if (tid == 0) {
           al[n - 2] = u2[n - 1];
           const cx<T> un = u[n - 1], wn = w[n - 1];
-          dg[n - 1] = A[(long long)(n - 1) * n + n - 1].re - T(4) * (un.re * wn.re + un.im * wn.im);
+          dg[n - 1] = trow(n - 1)[n - 1].re - T(4) * (un.re * wn.re + un.im * wn.im);
           A[(long long)(n - 1) * n + n - 2] = cx<T>(T(0), T(0));
         }
         __syncthreads();
         break;
       }
-      alpha = lg_reflector(u2, c + 1, n, red);
-      if (tid == 0) al[c + 1] = alpha;
-      for (int r = c + 2 + tid; r < n; r += nt) A[(long long)r * n + c + 1] = u2[r];
-      __syncthreads();
-      lg_hpass<T>(A, n, c + 2, true, u, w, u2, pw, pa);
-      lg_make_w(u2, pa, w, c + 2, n, red);
-      for (int r = c + 2 + tid; r < n; r += nt) u[r] = u2[r];
-      __syncthreads();
+      reflect(s, c + 2);
+      lg_hpass<T, false>(trow, trow, n, c + 2, true, u, w, u2, pw);
+      finish(c + 2);
     }
     // unit phases of the subdiagonal, then their prefix products (serial: cheap)
     for (int c = tid; c + 1 < n; c += nt) {
@@ -1578,12 +1604,23 @@ cudaError_t lg_common(const LargeArgs& a, cudaStream_t s) {
   const int fit = fixed < lim ? int(std::min<size_t>(16, (lim - fixed) / vec_b)) : 0;
   const int want = a.W >= 4 * 152 ? 4 : (a.W >= 2 * 152 ? 8 : 16);
   const int warps = std::min(fit, want);
-  if (warps >= 4) {
+  // The matrix in shared memory where two CTAs of 8 warps or more fit an SM with it: every
+  // column then sweeps it at shared-memory instead of L2 rates (with the five-barrier step:
+  // n = 124, 256 k-points 4.9 -> 2.9 ms with the FP64 spin eigensolves; n = 127, 289 k-points
+  // 1.12 -> 0.63).  One CTA per SM
+  // with most of a larger matrix was slower than four on L2 (n = 256, 837 k-points: 11.2 ->
+  // 14.0 ms): each step is a dozen dependent barriers that only other CTAs can hide.
+  const size_t sm_s = fixed + 8 * vec_b + size_t(a.n) * (a.n + 1) / 2 * sizeof(cx<T>);
+  static size_t cached_h = 0, cached_s = 0;
+  if (sm_s + 1024 <= (size_t(227) << 10) / 2) {
+    if ((e = set_smem_once(k_lg_tridiag_h<T, true>, sm_s, cached_s)) != cudaSuccess) return e;
+    const long long per_sm = std::min<long long>(4, (227 << 10) / (long long)(sm_s + 1024));
+    k_lg_tridiag_h<T, true><<<int(std::min<long long>(a.W, 152LL * per_sm)), 256, sm_s, s>>>(a);
+  } else if (warps >= 4) {
     const size_t sm_h = fixed + size_t(warps) * vec_b;
-    static size_t cached_h = 0;
-    if ((e = set_smem_once(k_lg_tridiag_h<T>, sm_h, cached_h)) != cudaSuccess) return e;
+    if ((e = set_smem_once(k_lg_tridiag_h<T, false>, sm_h, cached_h)) != cudaSuccess) return e;
     const long long ctas = std::min<long long>(a.W, 152LL * (16 / warps));
-    k_lg_tridiag_h<T><<<int(ctas), 32 * warps, sm_h, s>>>(a);
+    k_lg_tridiag_h<T, false><<<int(ctas), 32 * warps, sm_h, s>>>(a);
   } else {
     const size_t sm_tri = 3 * size_t(a.n) * sizeof(cx<T>) + 64 * sizeof(double);
     static size_t cached = 0;

@@ -110,3 +110,19 @@ def test_polish_without_room_takes_the_fp64_solve(lib):
         _check(lib, small, model, I.Plane(3, 1), 1, phases=False)
     finally:
         small.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_spin_split_of_two_bands_at_large_n(lib, ctx, precision):
+    """n = 36, p = 2: the projected spin operator is 2 x 2, the smallest matrix of the
+    tridiagonal eigensolver.  Two spin blocks, one shifted by less than the gap."""
+    m = _scaled(I.random_hermitian_model(18, 8), 1.0, hop=0.03)
+    up = I.HoppingList(n=18, R=np.concatenate([m.R, np.zeros((18, 3), np.int32)]),
+                       i=np.concatenate([m.i, np.arange(18)]), j=np.concatenate([m.j, np.arange(18)]),
+                       t=np.concatenate([m.t, np.full(18, 0.02 + 0j)]), dim=m.dim)
+    model, S = I.direct_sum([m, up]), np.diag(np.repeat([1.0, -1.0], 18))
+    plane = I.Plane(6, 3)
+    ref, rpso, _, _ = oracle.spin_resolved_wilson_loop(model, plane, 2, S, -1)
+    ph, pso, _, _ = lib.spin_resolved_wilson_loop(model, plane, 2, S, -1, precision=precision, ctx=ctx)
+    assert circ_err_rows(ph.cpu().numpy(), ref) <= (1e-10 if precision == "fp64" else 1e-6)
+    assert np.abs(pso.cpu().numpy() - rpso).max() <= 1e-9
