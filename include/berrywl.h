@@ -58,7 +58,7 @@ typedef enum {
 } bw_status;
 
 typedef enum {
-  BW_FP64 = 0,      /* FP64 accuracy throughout (n <= 32: an FP32 eigenbasis may seed
+  BW_FP64 = 0,      /* FP64 accuracy throughout (n <= 512: an FP32 eigenbasis may seed
                        the states, which FP64 corrections then bring to rounding)  */
   BW_MIXED = 1      /* eigensolve in FP32, occupied block refined in FP64          */
 } bw_precision;

@@ -16,7 +16,7 @@ constexpr int LARGE_N_MAX = 4096;
 constexpr int LOOP_P_MAX = 64;
 // Mixed plain loops of more bands than this take the batched-GEMM loops: their products run
 // on every SM instead of one CTA per loop, and their eigenphases in double-float on a cluster
-// (p = 64, 27 loops of 31 points: 12.1 ms in one CTA per loop, see the loop stage).
+// (p = 64, 27 loops of 31 points: products and eigenphases 12.1 -> 8.0 ms).
 constexpr int LOOP_P_MAX_DF = 32;
 // Distinct translations whose phases are cached in shared memory per k-point.
 constexpr int PHASE_CACHE = 256;
@@ -290,8 +290,13 @@ cudaError_t launch_z2(const double* phases, int Nt, int p, double* mid, double* 
                       int* nu, DevStatus* status, cudaStream_t s);
 
 cudaError_t launch_build_hk(const BuildArgs& a, cudaStream_t s);
-cudaError_t launch_states_small(const StatesArgs& a, int p_out, cudaStream_t s);
-cudaError_t launch_states_tiny(const StatesArgs& a, int p_out, cudaStream_t s, bool* handled);
+// plan_host (optional, states_plan_inline() must hold): the plan as for launch_loops_fused_df.
+cudaError_t launch_states_small(const StatesArgs& a, int p_out, cudaStream_t s, const void* plan_host = nullptr,
+                                size_t plan_bytes = 0, const void* plan_dev = nullptr);
+cudaError_t launch_states_tiny(const StatesArgs& a, int p_out, cudaStream_t s, bool* handled,
+                               const void* plan_host = nullptr, size_t plan_bytes = 0, const void* plan_dev = nullptr);
+// The few-band kernels take this problem (and can carry its plan as a parameter).
+bool states_plan_inline(const StatesArgs& a, int p_out);
 // True when the mixed-precision double-float states kernel (n = 4) can serve the
 // problem; with want_df set it writes U as complex double-float.
 bool states_df_eligible(const StatesArgs& a, int p_out);
@@ -316,7 +321,10 @@ bool loops_fused_eligible(const LoopArgs& a, const DevModel& md);
 // plan_host (optional, at most FUSED_PLAN_BYTES): the hopping-list plan whose device
 // copy sa.model / sa.row_ptr point into at plan_dev; the launch then carries the plan
 // as a kernel parameter and nothing needs to be copied to plan_dev.
-constexpr int FUSED_PLAN_BYTES = 2048;
+// 6 KB: the four-band models with a full on-site term and a spin operator.  (Kernel parameters
+// hold up to 32 KB.)  A copy ahead of the kernels costs its own node, and the next call waits
+// on the host until the staging buffer is free.
+constexpr int FUSED_PLAN_BYTES = 6144;
 struct alignas(16) FusedPlan {
   unsigned char bytes[FUSED_PLAN_BYTES];
 };

@@ -1307,8 +1307,8 @@ cudaError_t launch_loops_fused_df(const StatesArgs& sa, const LoopArgs& a, cudaS
   FusedPlan fp;  // the kernel parameter (copied at launch)
   const char* dbase = static_cast<const char*>(plan_dev);
   if (inl) {
-    std::memset(fp.bytes, 0, sizeof(fp.bytes));
     std::memcpy(fp.bytes, plan_host, plan_bytes);
+    std::memset(fp.bytes + plan_bytes, 0, sizeof(fp.bytes) - plan_bytes);
   }
   const ScanSmem Z = scan_layout(a.N, 2, a.nested ? a.N * 2 * a.m : 1);
   const FusedSmem F = fused_layout(Z, a.N, sa.model.n_R, sa.model.n_ent, sa.model.n_hop);

@@ -713,14 +713,16 @@ bw_status pso_split_wave(bw_ctx* ctx, PsoSplit& X, const z64* Uw, long long Wn, 
   return BW_OK;
 }
 
-// Wilson loop with many occupied bands (p > LOOP_P_MAX, n > SMALL_N_MAX).  The
-// Wilson matrix no longer fits in shared memory, so the loop runs as batched GEMMs
+// Wilson loop with many occupied bands (p > LOOP_P_MAX, or LOOP_P_MAX_DF in the mixed request;
+// n > SMALL_N_MAX).  The Wilson matrix no longer fits in shared memory, or one CTA per loop
+// would leave most of the chip idle, so the loop runs as batched GEMMs
 // (FP64, or double-float on the FP32 pipe in the mixed request):
 // for a block of nl loops (their k-points are contiguous, k = i N + j) the states are
 // solved in waves of up to 2048 k-points, one GEMM forms every overlap
-// M_j = U(k_{j+1})^dagger U(k_j) of the block (closing on U(k_0), Eq. 2), N - 1 GEMMs
-// form W = M_{N-1} ... M_0 for all loops of the block at once, and one CTA per loop
-// takes the eigenphases.  Memory per loop: N n x p states, N + 2 p x p matrices;
+// M_j = U(k_{j+1})^dagger U(k_j) of the block (closing on U(k_0), Eq. 2), log2 N levels of
+// pairwise GEMMs (or a chain of N - 1, where the scratch is short) form W = M_{N-1} ... M_0 for
+// all loops of the block at once, and one CTA or cluster per loop takes the eigenphases.
+// Memory per loop: N n x p states, 3/2 N (N + 2 for the chain) p x p matrices;
 // the solver's per-k-point scratch is per wave.  The block shrinks to fit the budget.
 // With a spin operator (Sec. IV) each wave also forms S = U^dagger (sigma s U) by
 // one sparse application and one GEMM, diagonalises it in FP64 on the tridiagonal
@@ -1074,14 +1076,16 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
     fused = use_df && bw::loops_fused_eligible(q, sa.model);
   }
   sa.want_df = use_df ? 1 : 0;
-  // a small plan rides along as a parameter of the fused kernel (no copy to dblob)
-  const bool plan_inline = fused && blob.data.size() <= sizeof(bw::FusedPlan);
+  // a small plan rides along as a parameter of the fused or few-band kernel (no copy to dblob)
+  const bool plan_inline = blob.data.size() <= sizeof(bw::FusedPlan) &&
+                           (fused || (!large && bw::states_plan_inline(sa, p_eff)));
   if (!plan_inline && (st = upload(ctx, blob, dblob, s))) return st;
   prof_start(ctx, s);
   if (fused) {
     // states are solved inside the loop kernel below
   } else if (!large) {
-    BW_CUDA(bw::launch_states_small(sa, p_eff, s), "states kernel");
+    BW_CUDA(bw::launch_states_small(sa, p_eff, s, plan_inline ? blob.data.data() : nullptr, blob.data.size(), dblob),
+            "states kernel");
   } else {
     bw::LargeArgs lg, fix;
     std::memset(&lg, 0, sizeof(lg));

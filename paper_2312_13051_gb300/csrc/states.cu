@@ -627,10 +627,11 @@ static cudaError_t states_impl(const StatesArgs& a, int p_out, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_states_small(const StatesArgs& a, int p_out, cudaStream_t s) {
+cudaError_t launch_states_small(const StatesArgs& a, int p_out, cudaStream_t s, const void* plan_host,
+                                size_t plan_bytes, const void* plan_dev) {
   if (a.K <= 0) return cudaSuccess;
   bool handled = false;
-  const cudaError_t e = launch_states_tiny(a, p_out, s, &handled);
+  const cudaError_t e = launch_states_tiny(a, p_out, s, &handled, plan_host, plan_bytes, plan_dev);
   if (handled || e != cudaSuccess) return e;
   return states_impl(a, p_out, s);
 }

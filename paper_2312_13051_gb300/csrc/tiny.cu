@@ -10,6 +10,9 @@
 // with w_M = exp(i 2pi / M) tabulated once per CTA (in two levels for long grids).
 #include <float.h>
 
+#include <cstring>
+#include <type_traits>
+
 #include "launch.h"
 #include "quad.cuh"
 
@@ -296,9 +299,27 @@ __device__ __forceinline__ int tiny_sector(const StatesArgs& a, long long k, con
   return a.sign < 0 ? 0 : PP / 2;
 }
 
+// The plan arrays in the kernel's parameter copy of the plan instead of at dbase.
+__device__ __forceinline__ void tiny_relocate(StatesArgs& a, const unsigned char* inl, const char* dbase) {
+  auto at = [&](auto*& p) {
+    if (p) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(inl + (reinterpret_cast<const char*>(p) - dbase));
+  };
+  at(a.model.Rv);
+  at(a.model.ent_row);
+  at(a.model.ent_col);
+  at(a.model.ent_start);
+  at(a.model.hop_r);
+  at(a.model.hop_t);
+  if (a.op.nnz > 0) {
+    at(a.op.row);
+    at(a.op.col);
+    at(a.op.val);
+  }
+}
+
 // n = 2: one thread per k-point, eigenvalues and states in closed form.
 template <int PP>
-__global__ void __launch_bounds__(TINY_THREADS) k_states_two(StatesArgs a, int use_tab) {
+__device__ __forceinline__ void states_two(const StatesArgs& a, int use_tab) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int eb[4], ee[4];
   const int tid = threadIdx.x, bd = blockDim.x;
@@ -649,7 +670,7 @@ __device__ __forceinline__ bool quad_refined(const z64 (&Hr)[4], int l, int base
 // The mixed-precision request takes it as well where the double-float kernel below does not
 // apply.
 template <int PP>
-__global__ void __launch_bounds__(QUAD_THREADS) k_states_quad(StatesArgs a, int use_tab) {
+__device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int eb[16], ee[16];
   constexpr int KPB = QUAD_THREADS / 4;
@@ -750,6 +771,27 @@ __global__ void __launch_bounds__(QUAD_THREADS) k_states_quad(StatesArgs a, int 
   z64* out = a.U + k * 4LL * PP + l * PP;
 #pragma unroll
   for (int c = 0; c < PP; ++c) out[c] = Q[c];
+}
+
+template <int PP>
+__global__ void __launch_bounds__(TINY_THREADS) k_states_two(StatesArgs a, int use_tab) {
+  states_two<PP>(a, use_tab);
+}
+template <int PP>
+__global__ void __launch_bounds__(TINY_THREADS)
+    k_states_two_inl(StatesArgs a, int use_tab, const char* dbase, const __grid_constant__ FusedPlan plan) {
+  tiny_relocate(a, plan.bytes, dbase);
+  states_two<PP>(a, use_tab);
+}
+template <int PP>
+__global__ void __launch_bounds__(QUAD_THREADS) k_states_quad(StatesArgs a, int use_tab) {
+  states_quad<PP>(a, use_tab);
+}
+template <int PP>
+__global__ void __launch_bounds__(QUAD_THREADS)
+    k_states_quad_inl(StatesArgs a, int use_tab, const char* dbase, const __grid_constant__ FusedPlan plan) {
+  tiny_relocate(a, plan.bytes, dbase);
+  states_quad<PP>(a, use_tab);
 }
 
 // ---------------------------------------------------------------------------
@@ -864,21 +906,37 @@ cudaError_t quad_df_launch(const StatesArgs& a, size_t smem, cudaStream_t s) {
 }
 
 template <int PP>
-cudaError_t quad_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape tT, cudaStream_t s) {
+cudaError_t quad_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape tT, cudaStream_t s,
+                        const FusedPlan* plan, const char* dbase) {
   constexpr int KPB = QUAD_THREADS / 4;
   const size_t smem = tiny_smem_bytes(a.model.n_R, a.model.n_hop, KPB, use_tab, tN, tT);
+  cudaError_t e;
+  if (plan) {
+    static size_t cached_i = 0;
+    if ((e = set_smem_once(k_states_quad_inl<PP>, smem, cached_i)) != cudaSuccess) return e;
+    k_states_quad_inl<PP><<<int((a.K + KPB - 1) / KPB), QUAD_THREADS, smem, s>>>(a, use_tab, dbase, *plan);
+    return cudaGetLastError();
+  }
   static size_t cached = 0;
-  cudaError_t e = set_smem_once(k_states_quad<PP>, smem, cached);
+  e = set_smem_once(k_states_quad<PP>, smem, cached);
   if (e != cudaSuccess) return e;
   k_states_quad<PP><<<int((a.K + KPB - 1) / KPB), QUAD_THREADS, smem, s>>>(a, use_tab);
   return cudaGetLastError();
 }
 
 template <int PP>
-cudaError_t two_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape tT, cudaStream_t s) {
+cudaError_t two_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape tT, cudaStream_t s,
+                        const FusedPlan* plan, const char* dbase) {
   const size_t smem = tiny_smem_bytes(a.model.n_R, a.model.n_hop, TINY_THREADS, use_tab, tN, tT);
+  cudaError_t e;
+  if (plan) {
+    static size_t cached_i = 0;
+    if ((e = set_smem_once(k_states_two_inl<PP>, smem, cached_i)) != cudaSuccess) return e;
+    k_states_two_inl<PP><<<int((a.K + TINY_THREADS - 1) / TINY_THREADS), TINY_THREADS, smem, s>>>(a, use_tab, dbase, *plan);
+    return cudaGetLastError();
+  }
   static size_t cached = 0;
-  cudaError_t e = set_smem_once(k_states_two<PP>, smem, cached);
+  e = set_smem_once(k_states_two<PP>, smem, cached);
   if (e != cudaSuccess) return e;
   k_states_two<PP><<<int((a.K + TINY_THREADS - 1) / TINY_THREADS), TINY_THREADS, smem, s>>>(a, use_tab);
   return cudaGetLastError();
@@ -897,13 +955,30 @@ bool states_df_eligible(const StatesArgs& a, int p_out) {
   return quad_df_smem(a.model.n_R, a.plane.N, a.plane.N_t) <= 48 * 1024;
 }
 
+bool tiny_takes(const StatesArgs& a, int p_out) {
+  const int n = a.model.n, p = a.p;
+  if (!(n == 2 || n == 4) || p < 1 || p > n || a.model.n_R > TINY_R_MAX || a.K <= 0) return false;
+  return !(a.op.nnz > 0 && (p % 2 || p_out != p / 2));
+}
+
+bool states_plan_inline(const StatesArgs& a, int p_out) { return !a.want_df && tiny_takes(a, p_out); }
+
 // Few-band path: n in {2, 4}, at most TINY_R_MAX distinct translations.  Sets
 // *handled = false (and launches nothing) when the problem is outside it.
-cudaError_t launch_states_tiny(const StatesArgs& a, int p_out, cudaStream_t s, bool* handled) {
+cudaError_t launch_states_tiny(const StatesArgs& a, int p_out, cudaStream_t s, bool* handled, const void* plan_host,
+                               size_t plan_bytes, const void* plan_dev) {
   *handled = false;
   const int n = a.model.n, p = a.p;
-  if (!(n == 2 || n == 4) || p < 1 || p > n || a.model.n_R > TINY_R_MAX || a.K <= 0) return cudaSuccess;
-  if (a.op.nnz > 0 && (p % 2 || p_out != p / 2)) return cudaSuccess;
+  if (!tiny_takes(a, p_out)) return plan_host ? cudaErrorInvalidValue : cudaSuccess;
+  if (plan_host && (a.want_df || plan_bytes > sizeof(FusedPlan))) return cudaErrorInvalidValue;
+  FusedPlan plan;  // the kernel parameter (copied at launch)
+  const FusedPlan* fp = nullptr;
+  const char* dbase = static_cast<const char*>(plan_dev);
+  if (plan_host) {
+    std::memcpy(plan.bytes, plan_host, plan_bytes);
+    std::memset(plan.bytes + plan_bytes, 0, sizeof(plan.bytes) - plan_bytes);
+    fp = &plan;
+  }
   const int N = a.plane.N, Nt = a.plane.N_t;
   bool integer_plane = a.f == nullptr;
   for (int d = 0; d < 3; ++d)
@@ -914,12 +989,12 @@ cudaError_t launch_states_tiny(const StatesArgs& a, int p_out, cudaStream_t s, b
   *handled = true;
   if (a.want_df)  // the caller checked states_df_eligible()
     return quad_df_launch<2>(a, quad_df_smem(a.model.n_R, N, Nt), s);
-  if (n == 2) return p == 1 ? two_launch<1>(a, use_tab, tN, tT, s) : two_launch<2>(a, use_tab, tN, tT, s);
+  if (n == 2) return p == 1 ? two_launch<1>(a, use_tab, tN, tT, s, fp, dbase) : two_launch<2>(a, use_tab, tN, tT, s, fp, dbase);
   switch (p) {
-    case 1: return quad_launch<1>(a, use_tab, tN, tT, s);
-    case 2: return quad_launch<2>(a, use_tab, tN, tT, s);
-    case 3: return quad_launch<3>(a, use_tab, tN, tT, s);
-    default: return quad_launch<4>(a, use_tab, tN, tT, s);
+    case 1: return quad_launch<1>(a, use_tab, tN, tT, s, fp, dbase);
+    case 2: return quad_launch<2>(a, use_tab, tN, tT, s, fp, dbase);
+    case 3: return quad_launch<3>(a, use_tab, tN, tT, s, fp, dbase);
+    default: return quad_launch<4>(a, use_tab, tN, tT, s, fp, dbase);
   }
 }
 
