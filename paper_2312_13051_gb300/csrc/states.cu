@@ -177,16 +177,25 @@ __device__ bool ritz(const z64* H, z64* Q, z64* HQ, z64* C, z64* G, z64* Zg, dou
 // of the order of the FP32 error and enters the correction at second order), then
 // Cholesky-QR.  An error e of the subspace becomes about e^2.  Returns |C|_F^2; *ok = 0
 // when the Cholesky factorisation broke down.
+// kLow: the products with V in FP32.  They carry the correction, which only has to be right
+// relative to its own size: 6e-8 |C|, removed by the next step or, in the last one (|C| <=
+// 3e-9), below rounding.  With V converted to FP64 they were more than half of the step's FP64
+// work (two conversions and four operations per term on a pipe of one warp instruction per ~19
+// clocks).
+template <bool kLow>
 __device__ double newton_step(const z64* H, const c32* V, const int* ord, const double* lam, int n, int p, z64* Q,
                               z64* HQ, z64* C, z64* G, double* red, int* ok, int* flag) {
   const int tid = threadIdx.x, nt = blockDim.x;
   mm(H, Q, HQ, n, n, p);
-  // G = Q^dagger H Q, then R = H Q - Q G (full G)
+  // G = Q^dagger H Q (upper triangle mirrored), then R = H Q - Q G
   for (int e = tid; e < p * p; e += nt) {
     const int a = e / p, b = e - a * p;
+    if (b < a) continue;
     z64 acc(0.0, 0.0);
     for (int r = 0; r < n; ++r) cfma_conj(acc, Q[r * p + a], HQ[r * p + b]);
+    if (a == b) acc.im = 0.0;
     G[e] = acc;
+    if (a != b) G[b * p + a] = conj(acc);
   }
   __syncthreads();
   for (int e = tid; e < n * p; e += nt) {
@@ -198,20 +207,44 @@ __device__ double newton_step(const z64* H, const c32* V, const int* ord, const 
   __syncthreads();
   const int nu = n - p;
   double c2 = 0.0;
-  for (int e = tid; e < nu * p; e += nt) {
-    const int a = e / p, i = e - a * p;
-    const int col = ord[p + a];
-    z64 acc(0.0, 0.0);
-    for (int r = 0; r < n; ++r) cfma_conj(acc, ccast<double>(V[r * n + col]), C[r * p + i]);
-    HQ[e] = (1.0 / (G[i * p + i].re - lam[col])) * acc;  // correction coefficients
-    c2 += abs2(HQ[e]);
-  }
-  __syncthreads();
-  for (int e = tid; e < n * p; e += nt) {
-    const int r = e / p, i = e - r * p;
-    z64 acc = Q[e];
-    for (int a = 0; a < nu; ++a) cfma(acc, ccast<double>(V[r * n + ord[p + a]]), HQ[a * p + i]);
-    Q[e] = acc;
+  if constexpr (kLow) {
+    c32* Cf = reinterpret_cast<c32*>(HQ);  // the residual, then the coefficients behind it
+    c32* Kf = Cf + n * p;
+    for (int e = tid; e < n * p; e += nt) Cf[e] = ccast<float>(C[e]);
+    __syncthreads();
+    float s2 = 0.f;
+    for (int e = tid; e < nu * p; e += nt) {
+      const int a = e / p, i = e - a * p, col = ord[p + a];
+      c32 acc(0.f, 0.f);
+      for (int r = 0; r < n; ++r) cfma_conj(acc, V[r * n + col], Cf[r * p + i]);
+      acc = (1.f / float(G[i * p + i].re - lam[col])) * acc;
+      Kf[e] = acc;
+      s2 += abs2(acc);
+    }
+    c2 = double(s2);
+    __syncthreads();
+    for (int e = tid; e < n * p; e += nt) {
+      const int r = e / p, i = e - r * p;
+      c32 acc(0.f, 0.f);
+      for (int a = 0; a < nu; ++a) cfma(acc, V[r * n + ord[p + a]], Kf[a * p + i]);
+      Q[e] = Q[e] + ccast<double>(acc);
+    }
+  } else {
+    for (int e = tid; e < nu * p; e += nt) {
+      const int a = e / p, i = e - a * p;
+      const int col = ord[p + a];
+      z64 acc(0.0, 0.0);
+      for (int r = 0; r < n; ++r) cfma_conj(acc, ccast<double>(V[r * n + col]), C[r * p + i]);
+      HQ[e] = (1.0 / (G[i * p + i].re - lam[col])) * acc;  // correction coefficients
+      c2 += abs2(HQ[e]);
+    }
+    __syncthreads();
+    for (int e = tid; e < n * p; e += nt) {
+      const int r = e / p, i = e - r * p;
+      z64 acc = Q[e];
+      for (int a = 0; a < nu; ++a) cfma(acc, ccast<double>(V[r * n + ord[p + a]]), HQ[a * p + i]);
+      Q[e] = acc;
+    }
   }
   __syncthreads();
   if (!cholqr(Q, G, n, p, flag)) *ok = 0;
@@ -227,7 +260,7 @@ __device__ double refine_mixed(const z64* H, const c32* V, const int* ord, const
                                int n, int p, z64* Q, z64* HQ, z64* C, z64* G, double* red, int* ok, int* flag) {
   const int tid = threadIdx.x, nt = blockDim.x;
   *ok = cholqr(Q, G, n, p, flag) ? 1 : 0;
-  if (p < n) newton_step(H, V, ord, lam, n, p, Q, HQ, C, G, red, ok, flag);
+  if (p < n) newton_step<false>(H, V, ord, lam, n, p, Q, HQ, C, G, red, ok, flag);
   // gap from FP64 Rayleigh quotients of the FP32 vectors p-1 and p
   double gap = INFINITY;
   if (p < n) {
@@ -335,7 +368,7 @@ __device__ bool refine_fp64(const z64* H, const c32* V, const int* ord, const do
   if (p - c0 > p || c1 - p + 1 > p) return false;
   double c2 = 1.0;
   for (int it = 0; it < 4 && !(c2 <= 1e-17); ++it) {
-    c2 = newton_step(H, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
+    c2 = newton_step<true>(H, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
     if (!ok || !(c2 < 1e-4)) return false;
   }
   if (!(c2 <= 1e-17)) return false;
