@@ -554,6 +554,7 @@ __device__ __forceinline__ bool quad_refined(const z64 (&Hr)[4], int l, int base
   }
   const float lmin = sel4(lam, ord[0]), lmax = sel4(lam, ord[3]);
   ok = ok && lu[0] - sel4(lam, ord[PP - 1]) > 1e-3f * fmaxf(fabsf(lmin), fabsf(lmax));
+  if (__all_sync(0xffffffffu, !ok)) return false;
   {
     c32 E[PP][PP];
     quad_dev<PP>(Q, E, l, base);
@@ -773,6 +774,59 @@ __device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
   for (int c = 0; c < PP; ++c) out[c] = Q[c];
 }
 
+// n = 4 on large grids when H has entries that are identically zero (the models' own sparse
+// forms): one thread per k-point, FP64 Jacobi, whose rotations of zero entries are skipped.
+// There the sweeps take fewer FP64 instructions than the refined solve (BBH, 230 400 k-points:
+// 0.68 ms against 0.93; spin-Hall, 60 000: 0.16 against 0.24), with a full matrix more (BBH with
+// an on-site term: 1.98 against 1.22 ms); on small grids four lanes per k-point win either way.
+constexpr int FOUR_THREADS = 32;
+
+template <int PP>
+__device__ __forceinline__ void states_four(const StatesArgs& a, int use_tab) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int eb[16], ee[16];
+  const int tid = threadIdx.x, bd = blockDim.x;
+  const TinySmem T = tiny_tables<4>(a, smem, bd, use_tab != 0, eb, ee);
+  const long long k = (long long)blockIdx.x * bd + tid;
+  if (k >= a.K) return;
+  tiny_phases(a, T, k, tid, bd, use_tab != 0, 0, 1);
+  z64 A[4][4], V[4][4], Vs[4][4];
+  double lam[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = r; c < 4; ++c) {
+      A[r][c] = tiny_entry(T, eb[4 * r + c], ee[4 * r + c], tid, bd);
+      if (r == c)
+        A[r][r].im = 0.0;
+      else
+        A[c][r] = conj(A[r][c]);
+    }
+  const bool ok = jac_serial<4, double>(A, V, a.max_sweeps) >= 0;
+  sort_eig<4, double>(A, V, Vs, lam);
+  double gap = INFINITY;
+  if constexpr (PP < 4) gap = lam[PP] - lam[PP - 1];
+  a.gap[k] = gap;
+  if (!ok) report(a.status, ST_ENOCONV, k, 0.0);
+  if (!(gap > a.gap_tol)) report(a.status, ST_EGAP, k, gap);
+  z64* out = a.U + k * 4LL * PP;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < PP; ++c) out[r * PP + c] = Vs[r][c];
+}
+
+template <int PP>
+__global__ void __launch_bounds__(FOUR_THREADS) k_states_four(StatesArgs a, int use_tab) {
+  states_four<PP>(a, use_tab);
+}
+template <int PP>
+__global__ void __launch_bounds__(FOUR_THREADS)
+    k_states_four_inl(StatesArgs a, int use_tab, const char* dbase, const __grid_constant__ FusedPlan plan) {
+  tiny_relocate(a, plan.bytes, dbase);
+  states_four<PP>(a, use_tab);
+}
+
 template <int PP>
 __global__ void __launch_bounds__(TINY_THREADS) k_states_two(StatesArgs a, int use_tab) {
   states_two<PP>(a, use_tab);
@@ -909,8 +963,22 @@ template <int PP>
 cudaError_t quad_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape tT, cudaStream_t s,
                         const FusedPlan* plan, const char* dbase) {
   constexpr int KPB = QUAD_THREADS / 4;
-  const size_t smem = tiny_smem_bytes(a.model.n_R, a.model.n_hop, KPB, use_tab, tN, tT);
   cudaError_t e;
+  if (a.model.n_ent < 16 && a.op.nnz == 0 && a.K > 8192) {
+    const size_t sm = tiny_smem_bytes(a.model.n_R, a.model.n_hop, FOUR_THREADS, use_tab, tN, tT);
+    const int grid = int((a.K + FOUR_THREADS - 1) / FOUR_THREADS);
+    if (plan) {
+      static size_t cached_fi = 0;
+      if ((e = set_smem_once(k_states_four_inl<PP>, sm, cached_fi)) != cudaSuccess) return e;
+      k_states_four_inl<PP><<<grid, FOUR_THREADS, sm, s>>>(a, use_tab, dbase, *plan);
+    } else {
+      static size_t cached_f = 0;
+      if ((e = set_smem_once(k_states_four<PP>, sm, cached_f)) != cudaSuccess) return e;
+      k_states_four<PP><<<grid, FOUR_THREADS, sm, s>>>(a, use_tab);
+    }
+    return cudaGetLastError();
+  }
+  const size_t smem = tiny_smem_bytes(a.model.n_R, a.model.n_hop, KPB, use_tab, tN, tT);
   if (plan) {
     static size_t cached_i = 0;
     if ((e = set_smem_once(k_states_quad_inl<PP>, smem, cached_i)) != cudaSuccess) return e;

@@ -126,3 +126,17 @@ def test_spin_split_of_two_bands_at_large_n(lib, ctx, precision):
     ph, pso, _, _ = lib.spin_resolved_wilson_loop(model, plane, 2, S, -1, precision=precision, ctx=ctx)
     assert circ_err_rows(ph.cpu().numpy(), ref) <= (1e-10 if precision == "fp64" else 1e-6)
     assert np.abs(pso.cpu().numpy() - rpso).max() <= 1e-9
+
+
+@pytest.mark.parametrize("p", [1, 2, 3])
+def test_sparse_four_band_model_on_a_large_grid(lib, ctx, p):
+    """n = 4 with entries that are identically zero, past 8192 k-points: one thread per k-point;
+    row 0 against the oracle and the small grid of the same row against the large one."""
+    t = I.bbh(0.5, 0.7)
+    on = I.HoppingList(n=4, R=np.concatenate([t.R, np.zeros((4, 3), np.int32)]), i=np.concatenate([t.i, np.arange(4)]),
+                       j=np.concatenate([t.j, np.arange(4)]),
+                       t=np.concatenate([t.t, np.array([0.0, 0.3, 0.7, 1.1]) + 0j]), dim=t.dim)
+    ph, gap = lib.wilson_loop(on, I.Plane(11, 751), p, precision="fp64", ctx=ctx, gap_tol=0.0)
+    ref, rgap = oracle.wilson_loop(on, I.Plane(11, 1), p, gap_tol=0.0)
+    assert abs(float(gap[0]) - rgap[0]) <= 8 * 4 * EPS * 4.0
+    assert circ_err_rows(ph[:1].cpu().numpy(), ref) <= 1e-10
