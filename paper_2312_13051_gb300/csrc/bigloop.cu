@@ -436,8 +436,8 @@ cudaError_t launch_iota(long long* off, int* idx, long long W, long long stride,
 
 // ---------------------------------------------------------------------------
 // Eigenphases of large Wilson matrices on a cluster of GC_CTAS CTAs per loop: the
-// same arithmetic as k_geig_big (Householder-Hessenberg, single-shift QR with the
-// same shifts, rotations and deflation tests), organised so that one SM does not
+// same steps as k_geig_big (Householder-Hessenberg, several QR sweeps at once with the
+// shifts, rotations and deflation tests of geig.cuh), organised so that one SM does not
 // wait on one thread:
 //  - Hessenberg: every CTA forms the Householder vector in its shared memory (same
 //    data, same order, same bits); the left update is split over the columns, the
@@ -517,7 +517,14 @@ struct GcA<z64> {
   __device__ static R abs(z64 a) { return zabs(a); }
   __device__ static R sqrt_(R x) { return sqrt(x); }
   __device__ static R inv_sqrt(R x) { return 1.0 / sqrt(x); }
-  __device__ static R div(R x, R y) { return x / y; }
+  __device__ static bool squares_underflow(R) { return false; }
+  __device__ static float cmax(z64 a) { return float(fmax(fabs(a.re), fabs(a.im))); }
+  __device__ static z64 scl(z64 a, float) { return a; }
+  // |x| and x / |x| (1 for x = 0)
+  __device__ static void polar(z64 x, R& ax, z64& ph) {
+    ax = zabs(x);
+    ph = ax > 0.0 ? z64(x.re / ax, x.im / ax) : one();
+  }
   __device__ static bool positive(R x) { return x > 0.0; }
   __device__ static R bsum(R v, double* red) { return block_sum(v, red); }
   __device__ static z64 shfl_xor(z64 v, int o) {
@@ -531,7 +538,8 @@ struct GcA<z64> {
   }
   __device__ static void rot(z64 x, z64 y, R& c, z64& sr) { givens(x, y, c, sr); }
   __device__ static double phase(z64 z) { return atan2(z.im, z.re); }
-  __device__ static c32 low(z64 z) { return ccast<float>(z); }
+  __device__ static z64 wide(z64 z) { return z; }
+  __device__ static z64 narrow(z64 z) { return z; }
 };
 template <>
 struct GcA<cdf> {
@@ -544,7 +552,22 @@ struct GcA<cdf> {
   __device__ static R abs(cdf a) { return df_sqrt(abs2(a)); }
   __device__ static R sqrt_(R x) { return df_sqrt(x); }
   __device__ static R inv_sqrt(R x) { return gc_rsqrt(x); }
-  __device__ static R div(R x, R y) { return df_div(x, y); }
+  // a column whose squares lose bits below the FP32 range (|x| < 1e-11) is scaled first: with
+  // its norm off by those bits the reflector would not be unitary
+  __device__ static bool squares_underflow(R nrm2) { return !(nrm2.hi > 1e-22f); }
+  __device__ static float cmax(cdf a) { return cmax_hi(a); }
+  __device__ static cdf scl(cdf a, float s) { return cscale(a, s); }
+  __device__ static void polar(cdf x, R& ax, cdf& ph) {
+    const float m = cmax_hi(x);
+    ax = df(0.f);
+    ph = one();
+    if (!(m > 1e-36f)) return;
+    const float sc = pow2_inv(m), us = 1.f / sc;
+    x = cscale(x, sc);
+    const df a = abs(x);
+    ph = cdf(df_div(x.re, a), df_div(x.im, a));
+    ax = df(a.hi * us, a.lo * us);
+  }
   __device__ static bool positive(R x) { return x.hi > 0.f; }
   __device__ static R bsum(R v, double* red) { return block_sum_df(v, reinterpret_cast<df*>(red)); }
   __device__ static cdf shfl_xor(cdf v, int o) { return cdf(shfl_xor_df(v.re, o), shfl_xor_df(v.im, o)); }
@@ -568,7 +591,7 @@ struct GcA<cdf> {
   __device__ static cdf shift(cdf a, cdf b, cdf c, cdf d, int iter, cdf h2, bool has_h2) {
     float m = fmaxf(fmaxf(cmax_hi(a), cmax_hi(b)), fmaxf(cmax_hi(c), cmax_hi(d)));
     if (has_h2) m = fmaxf(m, cmax_hi(h2));
-    if (!(m > 0.f) || !(m < INFINITY)) return d;
+    if (!(m > 1e-36f) || !(m < INFINITY)) return d;
     const float sc = pow2_inv(m), us = 1.f / sc;
     a = cscale(a, sc);
     b = cscale(b, sc);
@@ -583,10 +606,13 @@ struct GcA<cdf> {
     const cdf m1 = d + half - sq, m2 = d + half + sq;
     return cscale(df_gt(abs2(m1 - d), abs2(m2 - d)) ? m2 : m1, us);
   }
-  // computed on x, y scaled by a power of two (c and s do not depend on the scale)
+  // computed on x, y scaled by a power of two (c and s do not depend on the scale); where
+  // both are below 1e-36 (which the deflation test takes for zero, and whose scale may be
+  // outside FP32) the rotation is the identity: the caller sets y's entry to zero.  Sweeps
+  // that follow each other meet such pairs where an earlier one has just converged
   __device__ static void rot(cdf x, cdf y, R& c, cdf& sr) {
     const float m = fmaxf(cmax_hi(x), cmax_hi(y));
-    if (!(m > 0.f)) {
+    if (!(m > 1e-36f)) {
       c = df(1.f);
       sr = cdf_zero();
       return;
@@ -612,7 +638,8 @@ struct GcA<cdf> {
     sr = ir * (ux * conj(y));
   }
   __device__ static double phase(cdf z) { return df_phase(z); }
-  __device__ static c32 low(cdf z) { return c32(z.re.hi, z.im.hi); }
+  __device__ static z64 wide(cdf z) { return cdf_to_z64(z); }
+  __device__ static cdf narrow(z64 z) { return cdf_from(z); }
 };
 
 // geig_split_point with L1-bypassing loads, for the first warp.
@@ -728,20 +755,34 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
   if (rank == 0 && tid == 0) ctl->fail = 0;  // read by CTA 0 alone, at the end
   // --- Householder reduction to Hessenberg form
   for (int c = 0; c + 2 < p; ++c) {
-    R nrm2 = R(0.0);
-    for (int r = c + 1 + tid; r < p; r += nt) nrm2 = nrm2 + abs2(A::ld(H + (long long)r * p + c));
-    nrm2 = A::bsum(nrm2, red);
-    const E x0 = A::ld(H + (long long)(c + 1) * p + c);
+    float sc = 1.f;  // power of two on the column
+    auto entry = [&](int r) { return A::scl(A::ld(H + (long long)r * p + c), sc); };
+    auto norm2 = [&]() {
+      R t = R(0.0);
+      for (int r = c + 1 + tid; r < p; r += nt) t = t + abs2(entry(r));
+      return A::bsum(t, red);
+    };
+    R nrm2 = norm2();
+    if (A::squares_underflow(nrm2)) {
+      float m = 0.f;
+      for (int r = c + 1 + tid; r < p; r += nt) m = fmaxf(m, A::cmax(entry(r)));
+      m = float(-block_min(-double(m), red));
+      sc = m > 1e-36f ? pow2_inv(m) : 0.f;
+      nrm2 = norm2();
+    }
+    const E x0 = entry(c + 1);
     const R tail = nrm2 - abs2(x0);
     // a column already reduced is skipped; the barriers below run regardless, so the
     // CTAs of the cluster pass the same barriers whatever the data
     const bool work = A::positive(tail);
-    const R nx = A::sqrt_(nrm2), ax0 = A::abs(x0);
-    const E ph = A::positive(ax0) ? E(A::div(x0.re, ax0), A::div(x0.im, ax0)) : A::one();
+    const R nx = A::sqrt_(nrm2);
+    R ax0;
+    E ph;
+    A::polar(x0, ax0, ph);
     const R v0m = ax0 + nx, nv = work ? A::inv_sqrt(v0m * v0m + tail) : R(0.0);
     if (work)
       for (int r = c + 1 + tid; r < p; r += nt)
-        vsh[r] = r == c + 1 ? E(nv * v0m * ph.re, nv * v0m * ph.im) : nv * A::ld(H + (long long)r * p + c);
+        vsh[r] = r == c + 1 ? E(nv * v0m * ph.re, nv * v0m * ph.im) : nv * entry(r);
     __syncthreads();
     // left: H <- (I - 2 v v^dagger) H on rows c+1.., the cluster's columns c+1..; a warp takes
     // eight columns, four lanes per column share its rows (a thread per column left four
@@ -767,7 +808,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
     }
     cluster.sync();
     if (work && rank == 0)  // column c (every CTA has read it)
-      for (int r = c + 1 + tid; r < p; r += nt) H[(long long)r * p + c] = r == c + 1 ? (-nx) * ph : A::zero();
+      for (int r = c + 1 + tid; r < p; r += nt) H[(long long)r * p + c] = r == c + 1 ? A::scl((-nx) * ph, 1.f / sc) : A::zero();
     // right: H <- H (I - 2 v v^dagger) on columns c+1.., one warp per row of the cluster
     for (int row = gwarp; work && row < p; row += gnwarp) {
       E* hr = H + (long long)row * p;
@@ -804,15 +845,15 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
         const int size = hi - l + 1;
         nb = size < 8 || (iter > 0 && iter % 12 == 0) ? 1 : min(GC_NB, size / 4);
         if (nb > 1) {
-          const int h0 = hi - nb + 1;
-          for (int e = lane; e < nb * nb; e += 32) {
-            const int r = e / nb, c = e - r * nb;
-            blk[e] = r <= c + 1 ? A::low(A::ld(H + (long long)(h0 + r) * p + h0 + c)) : c32(0.f, 0.f);
+          const E* Hb = H + (long long)(hi - nb + 1) * (p + 1);
+          const double up = geig_shifts([&](int r, int c) { return A::wide(A::ld(Hb + (long long)r * p + c)); }, nb, blk, bsh);
+          if (up > 0.0) {
+            if (lane < nb) shift[lane] = A::narrow(up * ccast<double>(bsh[lane]));
+          } else {
+            nb = 1;
           }
-          __syncwarp();
-          geig_block_shifts(blk, nb, bsh);
-          if (lane < nb) shift[lane] = E(R(bsh[lane].re), R(bsh[lane].im));
-        } else {
+        }
+        if (nb == 1) {
           const E mu = A::shift(A::ld(H + (long long)(hi - 1) * p + hi - 1), A::ld(H + (long long)(hi - 1) * p + hi),
                                 A::ld(H + (long long)hi * p + hi - 1), A::ld(H + (long long)hi * p + hi), iter,
                                 hi >= 2 ? A::ld(H + (long long)(hi - 1) * p + hi - 2) : A::zero(), hi >= 2);

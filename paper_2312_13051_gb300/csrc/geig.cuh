@@ -25,9 +25,9 @@ constexpr int GEIG_NB = 8;
 struct GeigShared {
   double c[GEIG_NB];    // Givens of each sweep: G = [[c, s], [-conj(s), c]], c real
   z64 s[GEIG_NB];
-  z64 shift;                 // of a single sweep
-  c32 shifts[GEIG_NB];       // of several
-  c32 B[GEIG_NB * GEIG_NB];  // trailing block (shift selection)
+  z64 shift[GEIG_NB];        // of each sweep
+  c32 low[GEIG_NB];          // the same in FP32, scaled (shift selection)
+  c32 B[GEIG_NB * GEIG_NB];  // trailing block
   z64 mu;
   int l, hi, nb, active, fail;
 };
@@ -107,19 +107,31 @@ __device__ __forceinline__ z64 geig_shift(z64 a, z64 b, z64 c, z64 d, int iter, 
   return (abs2(m1 - d) <= abs2(m2 - d)) ? m1 : m2;
 }
 
+// 2^-e with 2^e <= m < 2^(e+1), from the exponent bits (m finite, below 2^127; subnormal m and
+// zero give 2^127): a scaling without rounding that brings m into [1, 2).
+__device__ __forceinline__ float geig_unit(float m) {
+  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+}
+__device__ __forceinline__ float geig_max(c32 a, c32 b) {
+  return fmaxf(fmaxf(fabsf(a.re), fabsf(a.im)), fmaxf(fabsf(b.re), fabsf(b.im)));
+}
+__device__ __forceinline__ float geig_abs1(c32 a) { return fabsf(a.re) + fabsf(a.im); }
+
 // Shifts of nb simultaneous sweeps: the eigenvalues of the trailing nb x nb block B (FP32,
-// Hessenberg) of the active window by single-shift QR (a shift decides how fast the
-// sweeps converge, not what they converge to), in the order in which they separate from
-// the bottom.  At its cap of sweeps the diagonal entries left over serve.  One warp calls
-// it, all lanes; nb <= 32.
+// Hessenberg, entries at most 2) of the active window by single-shift QR (a shift decides how
+// fast the sweeps converge, not what they converge to), in the order in which they separate
+// from the bottom.  At its cap of sweeps the diagonal entries left over serve.  The block of
+// a nearly singular Wilson matrix spans the whole FP32 range, so nothing below squares an
+// entry or takes the reciprocal of one without scaling it by a power of two first: every
+// shift is finite.  One warp calls it, all lanes; nb <= 32.
 __device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
   const int lane = threadIdx.x & 31;
   int top = nb - 1, out = 0;
   for (int it = 0; it < 8 * GEIG_NB && top > 0; ++it) {
     // split point: the largest l whose subdiagonal entry is negligible
     const bool small = lane >= 1 && lane <= top &&
-                       abs2(B[lane * nb + lane - 1]) <=
-                           1e-12f * (abs2(B[lane * nb + lane]) + abs2(B[(lane - 1) * nb + lane - 1]));
+                       geig_abs1(B[lane * nb + lane - 1]) <=
+                           1e-6f * (geig_abs1(B[lane * nb + lane]) + geig_abs1(B[(lane - 1) * nb + lane - 1]));
     const unsigned m = __ballot_sync(0xffffffffu, small);
     const int l = m ? 31 - __clz(m) : 0;
     if (l == top) {
@@ -130,37 +142,52 @@ __device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
     }
     // Wilkinson shift: the eigenvalue of the last 2 x 2 block [[a, b], [c, d]] closest to d,
     // d - b c / (g +- sqrt(g^2 + b c)) with g = (a - d) / 2 and the larger denominator
-    const c32 a = B[(top - 1) * nb + top - 1], d = B[top * nb + top];
-    const c32 bc = B[(top - 1) * nb + top] * B[top * nb + top - 1], g = 0.5f * (a - d), q = g * g + bc;
-    const float aq = sqrtf(abs2(q)), sr = sqrtf(fmaxf(0.5f * (aq + fabsf(q.re)), 1e-38f));
-    c32 sq = q.re >= 0.f ? c32(sr, 0.5f * q.im / sr) : c32(0.5f * fabsf(q.im) / sr, copysignf(sr, q.im));
+    c32 a = B[(top - 1) * nb + top - 1], b = B[(top - 1) * nb + top], c = B[top * nb + top - 1], d = B[top * nb + top];
+    const float u2 = geig_unit(fmaxf(geig_max(a, b), geig_max(c, d)));
+    a = u2 * a;
+    b = u2 * b;
+    c = u2 * c;
+    const c32 bc = b * c, g = 0.5f * (a - u2 * d), q = g * g + bc;
+    const float sr = sqrtf(0.5f * (hypotf(q.re, q.im) + fabsf(q.re)));
+    c32 sq(0.f, 0.f);
+    if (sr > 0.f)
+      sq = q.re >= 0.f ? c32(sr, 0.5f * q.im / sr) : c32(0.5f * fabsf(q.im) / sr, copysignf(sr, q.im));
     if (g.re * sq.re + g.im * sq.im < 0.f) sq = -sq;
     const c32 den = g + sq;
     const float d2 = abs2(den);
-    const c32 mu = d2 > 0.f ? d - (1.f / d2) * (bc * conj(den)) : d;
+    const c32 mu = d2 > 1e-30f ? d - (1.f / u2) * ((1.f / d2) * (bc * conj(den))) : d;
     for (int k = l; k < top; ++k) {
-      const c32 x = k == l ? B[l * nb + l] - mu : B[k * nb + k - 1];
-      const c32 y = k == l ? B[(l + 1) * nb + l] : B[(k + 1) * nb + k - 1];
-      const float ax2 = abs2(x), r2 = ax2 + abs2(y);
-      float c = 1.f;
+      c32 x = k == l ? B[l * nb + l] - mu : B[k * nb + k - 1];
+      c32 y = k == l ? B[(l + 1) * nb + l] : B[(k + 1) * nb + k - 1];
+      const float m1 = geig_max(x, y);
+      float cr = 1.f;
       c32 s(0.f, 0.f);
-      if (r2 > 0.f) {
-        const float ir = rsqrtf(r2), iax = ax2 > 0.f ? rsqrtf(ax2) : 0.f;
-        c = ax2 * iax * ir;
-        s = ax2 > 0.f ? (ir * iax) * (x * conj(y)) : ir * conj(y);
+      if (m1 > 0.f) {
+        const float u1 = geig_unit(m1);
+        x = u1 * x;
+        y = u1 * y;
+        const float ax2 = abs2(x), ir = rsqrtf(ax2 + abs2(y));
+        if (ax2 > 1e-30f) {
+          const float iax = rsqrtf(ax2);
+          cr = ax2 * iax * ir;
+          s = (iax * x) * conj(ir * y);
+        } else {
+          cr = 0.f;
+          s = ir * conj(y);
+        }
       }
       __syncwarp();
       const int cb = k > l ? k - 1 : l;
       if (lane >= cb && lane <= top) {
         const c32 u = B[k * nb + lane], v = B[(k + 1) * nb + lane];
-        B[k * nb + lane] = c * u + s * v;
-        B[(k + 1) * nb + lane] = c * v - conj(s) * u;
+        B[k * nb + lane] = cr * u + s * v;
+        B[(k + 1) * nb + lane] = cr * v - conj(s) * u;
       }
       __syncwarp();
       if (lane >= l && lane <= min(k + 2, top)) {
         const c32 u = B[lane * nb + k], v = B[lane * nb + k + 1];
-        B[lane * nb + k] = c * u + v * conj(s);
-        B[lane * nb + k + 1] = c * v - u * s;
+        B[lane * nb + k] = cr * u + v * conj(s);
+        B[lane * nb + k + 1] = cr * v - u * s;
       }
       __syncwarp();
       if (lane == 0 && k > l) B[(k + 1) * nb + k - 1] = c32(0.f, 0.f);
@@ -171,14 +198,30 @@ __device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
   __syncwarp();
 }
 
-__device__ __forceinline__ void geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, c32* shift) {
-  const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
+// The same from the trailing block at(r, c) of the matrix itself (FP64, r <= c + 1): scaled by a
+// power of two to FP32, its entries below 2; returns the power that the shifts are to be
+// multiplied by, or 0 when a shift is not finite (the matrix itself is not).
+template <class At>
+__device__ __forceinline__ double geig_shifts(At at, int nb, c32* B, c32* shift) {
+  const int lane = threadIdx.x & 31;
+  unsigned top = 0;  // leading word of the largest magnitude
   for (int e = lane; e < nb * nb; e += 32) {
     const int r = e / nb, c = e - r * nb;
-    B[e] = r <= c + 1 ? ccast<float>(H[(h0 + r) * ld + h0 + c]) : c32(0.f, 0.f);
+    if (r > c + 1) continue;
+    const z64 v = at(r, c);
+    top = max(top, max(unsigned(__double2hiint(fabs(v.re))), unsigned(__double2hiint(fabs(v.im)))));
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  const int ex = min(max(int(top >> 20), 1), 2045);
+  const double down = __hiloint2double((2046 - ex) << 20, 0);
+  for (int e = lane; e < nb * nb; e += 32) {
+    const int r = e / nb, c = e - r * nb;
+    B[e] = r <= c + 1 ? ccast<float>(down * at(r, c)) : c32(0.f, 0.f);
   }
   __syncwarp();
   geig_block_shifts(B, nb, shift);
+  const bool ok = lane >= nb || (isfinite(shift[lane].re) && isfinite(shift[lane].im));
+  return __all_sync(0xffffffffu, ok) ? __hiloint2double(ex << 20, 0) : 0.0;
 }
 
 // Largest l in [1, hi] whose subdiagonal entry is negligible, or 0: the first warp
@@ -305,9 +348,16 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         // nothing deflates (exceptional shifts)
         nb = size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
         if (nb > 1) {
-          geig_shifts(H, ld, hi, nb, sh->B, sh->shifts);
-        } else if (tid == 0) {
-          sh->shift =
+          const z64* Hb = H + (hi - nb + 1) * (ld + 1);
+          const double up = geig_shifts([&](int r, int c) { return Hb[r * ld + c]; }, nb, sh->B, sh->low);
+          if (up > 0.0) {
+            if (tid < nb) sh->shift[tid] = up * ccast<double>(sh->low[tid]);
+          } else {
+            nb = 1;
+          }
+        }
+        if (nb == 1 && tid == 0) {
+          sh->shift[0] =
               geig_shift(H[(hi - 1) * ld + hi - 1], H[(hi - 1) * ld + hi], H[hi * ld + hi - 1], H[hi * ld + hi],
                          iter, hi >= 2 ? zabs(H[(hi - 1) * ld + hi - 2]) : 0.0);
         }
@@ -342,7 +392,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         if (k >= l && k < hi) {
           z64 x, y;
           if (k == l) {
-            x = H[l * ld + l] - (nb > 1 ? ccast<double>(sh->shifts[tid]) : sh->shift);
+            x = H[l * ld + l] - sh->shift[tid];
             y = H[(l + 1) * ld + l];
           } else {
             x = H[k * ld + k - 1];
