@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(256) k_geig_big(BigEigArgs a) {
     }
     z64* W = a.W + (long long)l * a.sW;
     z64* lam = a.lam + (long long)l * p;
-    z64* vec = a.vec + (long long)l * geig_vec_len(p);
+    z64* vec = a.vec + (long long)l * p;
     double* th = a.th + (long long)l * p;
     int* ord = a.ord + (long long)l * p;
     const int rc = geig(W, nullptr, p, p, false, lam, vec, &sh);
@@ -435,35 +435,35 @@ cudaError_t launch_iota(long long* off, int* idx, long long W, long long stride,
 }
 
 // ---------------------------------------------------------------------------
-// Eigenphases of large Wilson matrices on a cluster of GC_CTAS CTAs per loop: the
-// same steps as k_geig_big (Householder-Hessenberg, several QR sweeps at once with the
-// shifts, rotations and deflation tests of geig.cuh), organised so that one SM does not
-// wait on one thread:
+// Eigenphases of large Wilson matrices on a cluster of GC_CTAS CTAs per loop
+// (Householder-Hessenberg, single-shift QR with the 2 x 2 shifts, rotations and deflation
+// tests of geig.cuh), organised so that one SM does not wait on one thread:
 //  - Hessenberg: every CTA forms the Householder vector in its shared memory (same
 //    data, same order, same bits); the left update is split over the columns, the
 //    right update over the rows of the cluster; two cluster barriers per column.
-//  - Up to GC_NB QR sweeps at once, two rows apart (geig.cuh), in chunks of GC_W steps: two
-//    warps of CTA 0 chase the bulges through the window of rows and columns that the
-//    chunk's rotations touch, in shared memory, and publish the rotations; then every
-//    thread of the cluster applies the chunk's row rotations to one column right of the
-//    window, or its column rotations to one row above it, in order.  Right of the window
-//    only the chunk's row rotations act and above it only its column rotations, so every
-//    entry receives its rotations in the sequential order.  A step is a chain of ~20
-//    dependent operations whatever the number of sweeps, and a chunk ends with a cluster
-//    barrier, so the sweeps share both.
+//  - QR sweep in chunks of GC_W rotations: the first warp of CTA 0 chases the bulge
+//    through the window rows [k0-1, kend+1] x columns [k0-1, kend] (kend = k0 + GC_W)
+//    in shared memory and publishes the rotations; then every thread of the cluster
+//    applies the chunk's row rotations to one column right of the window, or its
+//    column rotations to one row above it, in order.  Right of the window only the
+//    chunk's row rotations act and above it only its column rotations, so every
+//    entry receives its rotations in the sequential order.
+//  - One sweep at a time, with the shift in the solver's own precision: four sweeps that
+//    share the chunks, with the shifts of an FP32 block, take 20.5 instead of 21.5 ms at
+//    p = 200, but their subdiagonals end just below the deflation test instead of far below
+//    it, and the double-float phases of p = 144 lost a digit (median 4.7e-12 rad from FP64
+//    against 7e-13, worst 1e-10).
 //  - The matrix lives in global memory and other SMs of the cluster write it: every
 //    read bypasses L1 (ld.global.cg); the cluster barriers order the accesses.
 // ---------------------------------------------------------------------------
-constexpr int GC_CTAS = 4, GC_NB = 4, GC_W = 8, GC_THREADS = 256;
-constexpr int GC_K = GC_W + 2 * (GC_NB - 1);       // rows that start a rotation of a chunk
-constexpr int GC_WR = GC_K + 3, GC_WC = GC_K + 2;  // window rows, columns
-constexpr int GC_ROT = 2 * GC_W * GC_NB;           // a chunk's rotations: (c, s) per step and sweep
-constexpr int GC_CHASE = 64;                       // threads of the chase
+constexpr int GC_CTAS = 4, GC_W = 16, GC_THREADS = 256;
+constexpr int GC_WR = GC_W + 3, GC_WC = GC_W + 2;  // window rows, columns
 constexpr int GC_MIN_P = 128;                      // FP64, smaller p: k_geig_big
 constexpr int GC_MIN_P_DF = 33;                    // double-float (the loops come here from p = 33 on)
 
 struct GcCtl {
-  int active, l, hi, fail, nb;  // active: sweeps are to be run
+  double mu[4];  // the shift, as the solver's element type (16 bytes)
+  int active, l, hi, fail;
 };
 
 // Block-wide double-float sum (`red` holds >= blockDim.x / 32 df).
@@ -538,8 +538,6 @@ struct GcA<z64> {
   }
   __device__ static void rot(z64 x, z64 y, R& c, z64& sr) { givens(x, y, c, sr); }
   __device__ static double phase(z64 z) { return atan2(z.im, z.re); }
-  __device__ static z64 wide(z64 z) { return z; }
-  __device__ static z64 narrow(z64 z) { return z; }
 };
 template <>
 struct GcA<cdf> {
@@ -608,8 +606,7 @@ struct GcA<cdf> {
   }
   // computed on x, y scaled by a power of two (c and s do not depend on the scale); where
   // both are below 1e-36 (which the deflation test takes for zero, and whose scale may be
-  // outside FP32) the rotation is the identity: the caller sets y's entry to zero.  Sweeps
-  // that follow each other meet such pairs where an earlier one has just converged
+  // outside FP32) the rotation is the identity: the caller sets y's entry to zero
   __device__ static void rot(cdf x, cdf y, R& c, cdf& sr) {
     const float m = fmaxf(cmax_hi(x), cmax_hi(y));
     if (!(m > 1e-36f)) {
@@ -638,8 +635,6 @@ struct GcA<cdf> {
     sr = ir * (ux * conj(y));
   }
   __device__ static double phase(cdf z) { return df_phase(z); }
-  __device__ static z64 wide(cdf z) { return cdf_to_z64(z); }
-  __device__ static cdf narrow(z64 z) { return cdf_from(z); }
 };
 
 // geig_split_point with L1-bypassing loads, for the first warp.
@@ -659,72 +654,50 @@ __device__ __forceinline__ int gc_split_point(const E* H, int p, int hi) {
   return 0;
 }
 
-__device__ __forceinline__ void gc_chase_sync() { asm volatile("bar.sync 1, %0;" ::"n"(GC_CHASE) : "memory"); }
-
-// Rows of a chunk of steps T0 .. T1-1 (sweep b at row k = l + T - 2 b): the rotations start on
-// rows kmin .. kmax, the window is [rlo, rhi] x [rlo, chi].
-struct GcChunk {
-  int kmin, kmax, rlo, rhi, chi;
-  __device__ GcChunk(int l, int hi, int T0, int T1, int nb) {
-    kmin = max(l, l + T0 - 2 * (nb - 1));
-    kmax = min(hi - 1, l + T1 - 1);
-    rlo = max(l, kmin - 1);
-    rhi = min(kmax + 2, hi);
-    chi = min(kmax + 1, hi);
-  }
-};
-
-// The chase of a chunk on the window (the first GC_CHASE threads of CTA 0); rs: its rotations.
+// The bulge chase of rotations k0 .. kend-1 on the window (first warp of CTA 0).
 template <typename E>
-__device__ void gc_chase(E* H, int p, int l, int hi, int T0, int T1, int nb, const E* shift, E* win, E* rs) {
+__device__ void gc_chase(E* H, int p, int l, int hi, int k0, int kend, E mu, E* win, E* rot) {
   using A = GcA<E>;
   using R = typename A::R;
-  const int tid = threadIdx.x;
-  const GcChunk w(l, hi, T0, T1, nb);
-  const int nr = w.rhi - w.rlo + 1, nc = w.chi - w.rlo + 1;
-  for (int e = tid; e < nr * nc; e += GC_CHASE) {
+  const int lane = threadIdx.x & 31;
+  const int rlo = k0 > l ? k0 - 1 : l, rhi = min(kend + 1, hi), clo = rlo, chi = kend;
+  const int nr = rhi - rlo + 1, nc = chi - clo + 1;
+  for (int e = lane; e < nr * nc; e += 32) {
     const int r = e / nc, c = e - r * nc;
-    win[r * GC_WC + c] = A::ld(H + (long long)(w.rlo + r) * p + w.rlo + c);
+    win[r * GC_WC + c] = A::ld(H + (long long)(rlo + r) * p + clo + c);
   }
-  gc_chase_sync();
-#define GCW(r, c) win[((r) - w.rlo) * GC_WC + ((c) - w.rlo)]
-  for (int T = T0; T < T1; ++T) {
-    E* rt = rs + 2 * GC_NB * (T - T0);
-    if (tid < nb) {
-      const int k = l + T - 2 * tid;
-      if (k >= l && k < hi) {
-        const E x = k == l ? GCW(l, l) - shift[tid] : GCW(k, k - 1);
-        const E y = k == l ? GCW(l + 1, l) : GCW(k + 1, k - 1);
-        R c;
-        E sr;
-        A::rot(x, y, c, sr);
-        rt[2 * tid] = E(c, R(0.0));
-        rt[2 * tid + 1] = sr;
-      }
-    }
-    gc_chase_sync();
-    for (int e = tid; e < nb * GC_WC; e += GC_CHASE) {
-      const int b = e / GC_WC, k = l + T - 2 * b, col = w.rlo + (e - b * GC_WC);
-      if (k < l || k >= hi || col > w.chi || col < (k > l ? k - 1 : l)) continue;
-      const R c = rt[2 * b].re;
-      const E sr = rt[2 * b + 1], xv = GCW(k, col), yv = GCW(k + 1, col);
+  __syncwarp();
+#define GCW(r, c) win[((r) - rlo) * GC_WC + ((c) - clo)]
+  for (int k = k0; k < kend; ++k) {
+    const E x = k == l ? GCW(l, l) - mu : GCW(k, k - 1);
+    const E y = k == l ? GCW(l + 1, l) : GCW(k + 1, k - 1);
+    R c;
+    E sr;
+    A::rot(x, y, c, sr);  // every lane, same values
+    const int cb = k > l ? k - 1 : l;
+    for (int col = cb + lane; col <= chi; col += 32) {
+      const E xv = GCW(k, col), yv = GCW(k + 1, col);
       GCW(k, col) = c * xv + sr * yv;
-      GCW(k + 1, col) = k > l && col == k - 1 ? A::zero() : c * yv - conj(sr) * xv;
+      GCW(k + 1, col) = c * yv - conj(sr) * xv;
     }
-    gc_chase_sync();
-    for (int e = tid; e < nb * GC_WR; e += GC_CHASE) {
-      const int b = e / GC_WR, k = l + T - 2 * b, row = w.rlo + (e - b * GC_WR);
-      if (k < l || k >= hi || row > min(k + 2, hi)) continue;
-      const R c = rt[2 * b].re;
-      const E sr = rt[2 * b + 1], xv = GCW(row, k), yv = GCW(row, k + 1);
+    __syncwarp();
+    if (lane == 0 && k > l) GCW(k + 1, k - 1) = A::zero();
+    __syncwarp();
+    const int re = min(k + 2, hi);
+    for (int row = rlo + lane; row <= re; row += 32) {
+      const E xv = GCW(row, k), yv = GCW(row, k + 1);
       GCW(row, k) = c * xv + yv * conj(sr);
       GCW(row, k + 1) = c * yv - xv * sr;
     }
-    gc_chase_sync();
+    __syncwarp();
+    if (lane == 0) {
+      rot[2 * (k - k0)] = E(c, R(0.0));
+      rot[2 * (k - k0) + 1] = sr;
+    }
   }
-  for (int e = tid; e < nr * nc; e += GC_CHASE) {
+  for (int e = lane; e < nr * nc; e += 32) {
     const int r = e / nc, c = e - r * nc;
-    H[(long long)(w.rlo + r) * p + w.rlo + c] = win[r * GC_WC + c];
+    H[(long long)(rlo + r) * p + clo + c] = win[r * GC_WC + c];
   }
 #undef GCW
 }
@@ -739,9 +712,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
   const int p = a.p, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   E* vsh = reinterpret_cast<E*>(gsm);  // p: Householder vector
   E* win = vsh + p;                    // GC_WR x GC_WC window (CTA 0)
-  E* rsh = win + GC_WR * GC_WC;        // GC_ROT: the chunk's rotations
-  __shared__ __align__(16) E shift[GC_NB];  // CTA 0
-  __shared__ c32 blk[GC_NB * GC_NB], bsh[GC_NB];
+  E* rsh = win + GC_WR * GC_WC;        // 2 GC_W: the chunk's rotations
   __shared__ double red[32];
   const int rank = int(cluster.block_rank());
   const int lp = blockIdx.x / GC_CTAS;  // the cluster's loop: every CTA of it runs every
@@ -750,7 +721,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
   const int nwarp = nt >> 5, gwarp = rank * nwarp + warp, gnwarp = GC_CTAS * nwarp;
   E* H = reinterpret_cast<E*>(a.W) + (long long)lp * a.sW;
   E* lam = reinterpret_cast<E*>(a.lam) + (long long)lp * p;
-  E* rot = reinterpret_cast<E*>(a.vec) + (long long)lp * geig_vec_len(p);
+  E* rot = reinterpret_cast<E*>(a.vec) + (long long)lp * p;
   GcCtl* ctl = reinterpret_cast<GcCtl*>(a.ctl + 8LL * lp);
   if (rank == 0 && tid == 0) ctl->fail = 0;  // read by CTA 0 alone, at the end
   // --- Householder reduction to Hessenberg form
@@ -825,7 +796,8 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
   const int cap = 120 * p + 120;
   while (true) {
     if (rank == 0 && warp == 0) {
-      int hi = hi_s, l = 0, nb = 0, fail = 0;
+      int hi = hi_s, l = 0, active = 0, fail = 0;
+      E mu = A::zero();
       while (hi >= 0) {
         if (hi == 0) {
           if (lane == 0) lam[0] = A::ld(H);
@@ -841,37 +813,24 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
           iter = 0;
           continue;
         }
+        mu = A::shift(A::ld(H + (long long)(hi - 1) * p + hi - 1), A::ld(H + (long long)(hi - 1) * p + hi),
+                      A::ld(H + (long long)hi * p + hi - 1), A::ld(H + (long long)hi * p + hi), iter,
+                      hi >= 2 ? A::ld(H + (long long)(hi - 1) * p + hi - 2) : A::zero(), hi >= 2);
         l = sl;
-        const int size = hi - l + 1;
-        nb = size < 8 || (iter > 0 && iter % 12 == 0) ? 1 : min(GC_NB, size / 4);
-        if (nb > 1) {
-          const E* Hb = H + (long long)(hi - nb + 1) * (p + 1);
-          const double up = geig_shifts([&](int r, int c) { return A::wide(A::ld(Hb + (long long)r * p + c)); }, nb, blk, bsh);
-          if (up > 0.0) {
-            if (lane < nb) shift[lane] = A::narrow(up * ccast<double>(bsh[lane]));
-          } else {
-            nb = 1;
-          }
-        }
-        if (nb == 1) {
-          const E mu = A::shift(A::ld(H + (long long)(hi - 1) * p + hi - 1), A::ld(H + (long long)(hi - 1) * p + hi),
-                                A::ld(H + (long long)hi * p + hi - 1), A::ld(H + (long long)hi * p + hi), iter,
-                                hi >= 2 ? A::ld(H + (long long)(hi - 1) * p + hi - 2) : A::zero(), hi >= 2);
-          if (lane == 0) shift[0] = mu;
-        }
+        active = 1;
         break;
       }
       ++iter;
-      total += nb;
+      ++total;
       if (total > cap) {
         fail = 1;
-        nb = 0;
+        active = 0;
         hi = -1;
       }
       hi_s = hi;
       if (lane == 0) {
-        ctl->active = nb > 0;
-        ctl->nb = nb;
+        *reinterpret_cast<E*>(ctl->mu) = mu;
+        ctl->active = active;
         ctl->l = l;
         ctl->hi = hi;
         if (fail) ctl->fail = 1;
@@ -880,52 +839,56 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
     cluster.sync();
     const int active = __ldcg(&ctl->active);
     if (!active) break;  // the same value in every CTA of the cluster
-    const int l = __ldcg(&ctl->l), hi = __ldcg(&ctl->hi), nb = __ldcg(&ctl->nb);
-    const int steps = hi - l + 2 * (nb - 1);
-    for (int T0 = 0; T0 < steps; T0 += GC_W) {
-      const int T1 = min(T0 + GC_W, steps), nk = T1 - T0;
-      const GcChunk w(l, hi, T0, T1, nb);
-      if (rank == 0 && tid < GC_CHASE) {
-        gc_chase(H, p, l, hi, T0, T1, nb, shift, win, rsh);
-        for (int e = tid; e < 2 * GC_NB * nk; e += GC_CHASE) rot[e] = rsh[e];
-      }
+    const int l = __ldcg(&ctl->l), hi = __ldcg(&ctl->hi);
+    const E mu = A::ld(reinterpret_cast<const E*>(ctl->mu));
+    for (int k0 = l; k0 < hi; k0 += GC_W) {
+      const int kend = min(k0 + GC_W, hi), nk = kend - k0;
+      const int rlo = k0 > l ? k0 - 1 : l, chi = kend;
+      if (rank == 0 && warp == 0) gc_chase(H, p, l, hi, k0, kend, mu, win, rot);
       cluster.sync();
-      if (rank != 0) {
-        for (int e = tid; e < 2 * GC_NB * nk; e += nt) rsh[e] = A::ld(rot + e);
-      }
+      for (int e = tid; e < 2 * nk; e += nt) rsh[e] = A::ld(rot + e);
       __syncthreads();
-      // right of the window: its rows of columns chi+1 .. hi, row rotations in order; above
-      // it: its columns of rows l .. rlo-1, column rotations in order.  Entry q of v is row
-      // (column) base + q, so that rotation (t, b) acts on fixed entries
-      const int nA = hi - w.chi, nB = w.rlo - l, base = l + T0 - 2 * (GC_NB - 1);
-      const int q0 = w.kmin - base, q1 = min(w.kmax + 1, hi) - base;
+      // right of the window: rows k0 .. kend of columns chi+1 .. hi, row rotations in
+      // order; above it: columns k0 .. kend of rows l .. rlo-1, column rotations in order
+      const int nA = hi - chi, nB = rlo - l;
       for (int t = gtid; t < nA + nB; t += gnt) {
-        const bool right = t < nA;
-        E* h = right ? H + (long long)base * p + w.chi + 1 + t : H + (long long)(l + t - nA) * p + base;
-        const long long inc = right ? p : 1;
-        E v[GC_K + 1];
+        if (t < nA) {
+          E* hc = H + (long long)k0 * p + chi + 1 + t;
+          E v[GC_W + 1];
 #pragma unroll
-        for (int q = 0; q <= GC_K; ++q)
-          if (q >= q0 && q <= q1) v[q] = A::ld(h + q * inc);
+          for (int q = 0; q <= GC_W; ++q)
+            if (q <= nk) v[q] = A::ld(hc + (long long)q * p);
 #pragma unroll
-        for (int s = 0; s < GC_W; ++s) {
-          if (s >= nk) break;
+          for (int q = 0; q < GC_W; ++q)
+            if (q < nk) {
+              const R c = rsh[2 * q].re;
+              const E sr = rsh[2 * q + 1];
+              const E x = v[q], y = v[q + 1];
+              v[q] = c * x + sr * y;
+              v[q + 1] = c * y - conj(sr) * x;
+            }
 #pragma unroll
-          for (int b = 0; b < GC_NB; ++b) {
-            const int k = l + T0 + s - 2 * b;
-            if (b >= nb || k < l || k >= hi) continue;
-            const int q = s + 2 * (GC_NB - 1) - 2 * b;
-            const R c = rsh[2 * (GC_NB * s + b)].re;
-            // rows: x' = c x + s y, y' = c y - conj(s) x; columns: with conj(s)
-            const E sr = right ? rsh[2 * (GC_NB * s + b) + 1] : conj(rsh[2 * (GC_NB * s + b) + 1]);
-            const E x = v[q], y = v[q + 1];
-            v[q] = c * x + sr * y;
-            v[q + 1] = c * y - conj(sr) * x;
-          }
+          for (int q = 0; q <= GC_W; ++q)
+            if (q <= nk) hc[(long long)q * p] = v[q];
+        } else {
+          E* hr = H + (long long)(l + t - nA) * p + k0;
+          E v[GC_W + 1];
+#pragma unroll
+          for (int q = 0; q <= GC_W; ++q)
+            if (q <= nk) v[q] = A::ld(hr + q);
+#pragma unroll
+          for (int q = 0; q < GC_W; ++q)
+            if (q < nk) {
+              const R c = rsh[2 * q].re;
+              const E sr = rsh[2 * q + 1];
+              const E x = v[q], y = v[q + 1];
+              v[q] = c * x + y * conj(sr);
+              v[q + 1] = c * y - x * sr;
+            }
+#pragma unroll
+          for (int q = 0; q <= GC_W; ++q)
+            if (q <= nk) hr[q] = v[q];
         }
-#pragma unroll
-        for (int q = 0; q <= GC_K; ++q)
-          if (q >= q0 && q <= q1) h[q * inc] = v[q];
       }
       cluster.sync();
     }
@@ -966,7 +929,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
 
 template <typename E>
 static cudaError_t launch_geig_cluster(const BigEigArgs& a, cudaStream_t s) {
-  const size_t smem = (size_t(a.p) + GC_WR * GC_WC + GC_ROT) * sizeof(E);
+  const size_t smem = (size_t(a.p) + GC_WR * GC_WC + 2 * GC_W) * sizeof(E);
   static size_t cached = 0;
   cudaError_t e = set_smem_once(k_geig_cluster<E>, smem, cached);
   if (e != cudaSuccess) return e;

@@ -198,17 +198,16 @@ __device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
   __syncwarp();
 }
 
-// The same from the trailing block at(r, c) of the matrix itself (FP64, r <= c + 1): scaled by a
+// The same from the trailing block of the matrix itself (rows hi - nb + 1 .. hi): scaled by a
 // power of two to FP32, its entries below 2; returns the power that the shifts are to be
 // multiplied by, or 0 when a shift is not finite (the matrix itself is not).
-template <class At>
-__device__ __forceinline__ double geig_shifts(At at, int nb, c32* B, c32* shift) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ double geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, c32* shift) {
+  const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
   unsigned top = 0;  // leading word of the largest magnitude
   for (int e = lane; e < nb * nb; e += 32) {
     const int r = e / nb, c = e - r * nb;
     if (r > c + 1) continue;
-    const z64 v = at(r, c);
+    const z64 v = H[(h0 + r) * ld + h0 + c];
     top = max(top, max(unsigned(__double2hiint(fabs(v.re))), unsigned(__double2hiint(fabs(v.im)))));
   }
   top = __reduce_max_sync(0xffffffffu, top);
@@ -216,7 +215,7 @@ __device__ __forceinline__ double geig_shifts(At at, int nb, c32* B, c32* shift)
   const double down = __hiloint2double((2046 - ex) << 20, 0);
   for (int e = lane; e < nb * nb; e += 32) {
     const int r = e / nb, c = e - r * nb;
-    B[e] = r <= c + 1 ? ccast<float>(down * at(r, c)) : c32(0.f, 0.f);
+    B[e] = r <= c + 1 ? ccast<float>(down * H[(h0 + r) * ld + h0 + c]) : c32(0.f, 0.f);
   }
   __syncwarp();
   geig_block_shifts(B, nb, shift);
@@ -348,8 +347,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         // nothing deflates (exceptional shifts)
         nb = size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
         if (nb > 1) {
-          const z64* Hb = H + (hi - nb + 1) * (ld + 1);
-          const double up = geig_shifts([&](int r, int c) { return Hb[r * ld + c]; }, nb, sh->B, sh->low);
+          const double up = geig_shifts(H, ld, hi, nb, sh->B, sh->low);
           if (up > 0.0) {
             if (tid < nb) sh->shift[tid] = up * ccast<double>(sh->low[tid]);
           } else {

@@ -203,9 +203,6 @@ struct GemmArgs {
   long long sAo, sBo, sCo;
 };
 
-// Scratch per loop of the eigenphase kernels: a vector, or a chunk's rotations.
-__host__ __device__ inline int geig_vec_len(int p) { return p > 64 ? p : 64; }
-
 // Eigenphases of nl Wilson matrices W (p x p, stride sW), loops i0 .. i0+nl-1.
 struct BigEigArgs {
   z64* W;
@@ -217,7 +214,7 @@ struct BigEigArgs {
   double* min_gap;        // N_t (optional)
   double* min_pso_gap;    // N_t (optional)
   z64* lam;               // nl x p scratch
-  z64* vec;               // nl x geig_vec_len(p) scratch
+  z64* vec;               // nl x p scratch
   double* th;             // nl x p scratch
   int* ord;               // nl x p scratch
   double* ctl;            // nl x 8 scratch (control block of the cluster solver)

@@ -743,7 +743,7 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   const size_t sp_U = spin ? al256(size_t(n) * p * sizeof(z64)) : 0;
   const size_t sp_k = sp_U + (spin ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
   const size_t bUk = size_t(n) * pl * sizeof(z64), bPk = size_t(pl) * pl * sizeof(z64);
-  const size_t bEl = size_t(pl) * (sizeof(z64) + sizeof(double) + sizeof(int)) + bw::geig_vec_len(pl) * sizeof(z64) + 8 * sizeof(double);
+  const size_t bEl = size_t(pl) * (2 * sizeof(z64) + sizeof(double) + sizeof(int)) + 8 * sizeof(double);
   const size_t per_loop = size_t(N) * (bUk + bPk) + 2 * bPk + bEl;
   size_t total = al256(blob.data.size()) + (spin ? 2 : 1) * al256(size_t(K) * sizeof(double)) + 48 * 256;
   const size_t avail = ctx->budget > total ? ctx->budget - total : 0;
@@ -775,7 +775,7 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   else
     for (auto& w : Wbuf) w = reinterpret_cast<z64*>(carve(ctx, size_t(nl_max) * bPk));
   z64* e_lam = reinterpret_cast<z64*>(carve(ctx, nl_max * size_t(pl) * sizeof(z64)));
-  z64* e_vec = reinterpret_cast<z64*>(carve(ctx, nl_max * size_t(bw::geig_vec_len(pl)) * sizeof(z64)));
+  z64* e_vec = reinterpret_cast<z64*>(carve(ctx, nl_max * size_t(pl) * sizeof(z64)));
   double* e_th = reinterpret_cast<double*>(carve(ctx, nl_max * size_t(pl) * sizeof(double)));
   int* e_ord = reinterpret_cast<int*>(carve(ctx, nl_max * size_t(pl) * sizeof(int)));
   double* e_ctl = reinterpret_cast<double*>(carve(ctx, nl_max * 8 * sizeof(double)));
