@@ -458,8 +458,7 @@ cudaError_t launch_iota(long long* off, int* idx, long long W, long long stride,
 // ---------------------------------------------------------------------------
 constexpr int GC_CTAS = 4, GC_W = 16, GC_THREADS = 256;
 constexpr int GC_WR = GC_W + 3, GC_WC = GC_W + 2;  // window rows, columns
-constexpr int GC_MIN_P = 128;                      // FP64, smaller p: k_geig_big
-constexpr int GC_MIN_P_DF = 33;                    // double-float (the loops come here from p = 33 on)
+constexpr int GC_MIN_P = 128;                      // smaller p: k_geig_big, in FP64 in either request
 
 struct GcCtl {
   double mu[4];  // the shift, as the solver's element type (16 bytes)
@@ -948,7 +947,7 @@ static cudaError_t launch_geig_cluster(const BigEigArgs& a, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, k_geig_cluster<E>, a);
 }
 
-bool geig_df_eligible(int p) { return p >= GC_MIN_P_DF; }
+bool geig_df_eligible(int p) { return p >= GC_MIN_P; }
 
 cudaError_t launch_geig_big(const BigEigArgs& a, cudaStream_t s) {
   if (a.nl <= 0) return cudaSuccess;

@@ -14,9 +14,9 @@ constexpr int SMALL_N_MAX = 32;
 constexpr int LARGE_N_MAX = 4096;
 // Largest p handled by the shared-memory loop kernels (Wilson matrix p x p).
 constexpr int LOOP_P_MAX = 64;
-// Mixed plain loops of more bands than this take the batched-GEMM loops: their products run
-// on every SM instead of one CTA per loop, and their eigenphases in double-float on a cluster
-// (p = 64, 27 loops of 31 points: products and eigenphases 12.1 -> 8.0 ms).
+// Mixed plain loops of more bands than this take the batched-GEMM loops: their products run on
+// every SM instead of one CTA per loop (p = 64, 27 loops of 31 points: overlaps, products and
+// FP64 eigenphases 13.9 -> 12.6 ms; p = 40: 6.3 -> 6.3).
 constexpr int LOOP_P_MAX_DF = 32;
 // Distinct translations whose phases are cached in shared memory per k-point.
 constexpr int PHASE_CACHE = 256;

@@ -37,3 +37,13 @@ def test_mixed_phases_at_double_float_rounding(lib, ctx, copies, seed):
     ph, _ = lib.wilson_loop(model, plane, p, precision="mixed", ctx=ctx)
     ref, _ = oracle.wilson_loop(model, plane, p)
     assert circ_err_rows(ph.cpu().numpy(), ref) <= plane.N * p * 2.0 ** -47
+
+
+@pytest.mark.parametrize("copies", [17, 63, 64])
+def test_mixed_phases_at_the_solvers_limits(lib, ctx, copies):
+    # p = 34 (the first beyond one CTA per loop) and 126: FP64 eigenphases; 128: double-float
+    model = coupled_copies(copies, 3)
+    plane, p = I.Plane(9, 3, origin=(0.013, 0.021, 0.0)), 2 * copies
+    ph, _ = lib.wilson_loop(model, plane, p, precision="mixed", ctx=ctx)
+    ref, _ = oracle.wilson_loop(model, plane, p)
+    assert circ_err_rows(ph.cpu().numpy(), ref) <= plane.N * p * 2.0 ** -47
