@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256, 2) k_zgemm(GemmArgs g) {
       for (int x = 0; x < 4; ++x)
 #pragma unroll
         for (int y = 0; y < 4; ++y)
-          if (x < nx && y < ny && y <= x + diag) cmac(acc[x][y], av[x], bv[y]);
+          if (x < nx && y < ny && y <= x + diag) cfma(acc[x][y], av[x], bv[y]);
     }
     __syncthreads();
   }
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256, 2) k_zgemm(GemmArgs g) {
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
       const int gc = c0 + tx + 16 * y;
-      if (gc < g.n) C[(long long)gr * g.ldc + gc] = cfin(acc[x][y]);
+      if (gc < g.n) C[(long long)gr * g.ldc + gc] = acc[x][y];
     }
   }
 }
@@ -762,9 +762,8 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
       E w = A::zero();
       if (col < p) {
 #pragma unroll 8
-        for (int r = r0; r < p; r += 4) cmac_conj(w, vsh[r], A::ld(H + (long long)r * p + col));
+        for (int r = r0; r < p; r += 4) cfma_conj(w, vsh[r], A::ld(H + (long long)r * p + col));
       }
-      w = cfin(w);
       w = w + A::shfl_xor(w, 8);
       w = w + A::shfl_xor(w, 16);
       w = R(2.0) * w;
@@ -783,8 +782,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_geig_cluster(BigEigArgs a) {
     for (int row = gwarp; work && row < p; row += gnwarp) {
       E* hr = H + (long long)row * p;
       E w = A::zero();
-      for (int k = c + 1 + lane; k < p; k += 32) cmac(w, A::ld(hr + k), vsh[k]);
-      w = cfin(w);
+      for (int k = c + 1 + lane; k < p; k += 32) cfma(w, A::ld(hr + k), vsh[k]);
       for (int o = 16; o > 0; o >>= 1) w = w + A::shfl_xor(w, o);
       for (int k = c + 1 + lane; k < p; k += 32) hr[k] = A::ld(hr + k) - R(2.0) * (w * conj(vsh[k]));
     }

@@ -108,10 +108,9 @@ __global__ void k_lg_build(LargeArgs a) {
           // one 16-byte load: the entries of neighbouring threads lie n_R hoppings apart, so
           // every load instruction touches a line per lane
           const float4 t4 = reinterpret_cast<const float4*>(md.hop_tdf)[h];
-          cmac(acc, cdf(df(t4.x, t4.y), df(t4.z, t4.w)),
+          cfma(acc, cdf(df(t4.x, t4.y), df(t4.z, t4.w)),
                r < nRs ? phd[r] : cdf_from(bloch_phase(f, md.Rv + 3 * r)));
         }
-        acc = cfin(acc);
         A[(long long)md.ent_row[e] * n + md.ent_col[e]] = cx<T>(T(acc.re.hi), T(acc.im.hi));
         c32* dst = reinterpret_cast<c32*>(a.Hent + kw * (long long)md.n_ent + e);
         dst[0] = c32(acc.re.hi, acc.im.hi);

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(OVL_THREADS, 1) k_overlaps_df(LoopArgs a) {
         for (int u = 0; u < 4; ++u)
 #pragma unroll
           for (int v = 0; v < 4; ++v)
-            if (16 * u < p && 16 * v < p) cmac_conj(acc[u][v], an[u], ah[v]);
+            if (16 * u < p && 16 * v < p) cfma_conj(acc[u][v], an[u], ah[v]);
       }
       __syncthreads();
     }
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(OVL_THREADS, 1) k_overlaps_df(LoopArgs a) {
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int r = ty + 16 * u, c = tx + 16 * v;
-        if (r < p && c < p) M[r * p + c] = cdf_to_z64(cfin(acc[u][v]));
+        if (r < p && c < p) M[r * p + c] = cdf_to_z64(acc[u][v]);
       }
   }
 }
@@ -265,8 +265,8 @@ __global__ void k_loops(LoopArgs a, int tree) {
             }
             const cdf* A = B + pp + r * p;
             cdf acc = cdf_zero();
-            for (int q = 0; q < p; ++q) cmac(acc, A[q], B[q * p + c]);
-            dst[e] = cfin(acc);
+            for (int q = 0; q < p; ++q) cfma(acc, A[q], B[q * p + c]);
+            dst[e] = acc;
           }
           __syncthreads();
           cdf* t = src; src = dst; dst = t;
@@ -294,10 +294,10 @@ __global__ void k_loops(LoopArgs a, int tree) {
             }
             for (int q = 0; q < p; ++q)
 #pragma unroll
-              for (int u = 0; u < 4; ++u) cmac(acc[u], Md[rr[u] * p + q], Wd[q * p + cc[u]]);
+              for (int u = 0; u < 4; ++u) cfma(acc[u], Md[rr[u] * p + q], Wd[q * p + cc[u]]);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              if (e0 + u * nt < p * p) Td[e0 + u * nt] = cfin(acc[u]);
+              if (e0 + u * nt < p * p) Td[e0 + u * nt] = acc[u];
           }
           __syncthreads();
           cdf* t = Wd; Wd = Td; Td = t;
@@ -620,8 +620,8 @@ __device__ E* prefix_products(E* S, E* T, int L, int q) {
         const E* A = S + j * qq;
         const E* B = S + (j - d) * qq;
         E acc = Arith<E>::zero();
-        for (int k = 0; k < q; ++k) cmac(acc, A[r * q + k], B[k * q + c]);
-        T[e] = cfin(acc);
+        for (int k = 0; k < q; ++k) cfma(acc, A[r * q + k], B[k * q + c]);
+        T[e] = acc;
       }
     }
     __syncthreads();
@@ -744,8 +744,8 @@ __device__ void scan_one_loop(const LoopArgs& a, int i, const E* Ul, const doubl
         const E* Uh = Ul + jj * (long long)n * p;
         const E* Un = Ul + (jj + 1 == N ? 0 : jj + 1) * (long long)n * p;
         E acc = A::zero();
-        for (int q = 0; q < n; ++q) cmac_conj(acc, Un[q * p + r], Uh[q * p + c]);
-        S[e] = cfin(acc);
+        for (int q = 0; q < n; ++q) cfma_conj(acc, Un[q * p + r], Uh[q * p + c]);
+        S[e] = acc;
       }
     }
     __syncthreads();
@@ -807,16 +807,14 @@ __device__ void scan_one_loop(const LoopArgs& a, int i, const E* Ul, const doubl
             acc = Ye[r * p + col];
           } else {
             const E* P = Pf + (size_t)(j - 1) * pp;
-            for (int q = 0; q < p; ++q) cmac(acc, P[r * p + q], Ye[q * p + col]);
-            acc = cfin(acc);
+            for (int q = 0; q < p; ++q) cfma(acc, P[r * p + q], Ye[q * p + col]);
           }
           nu[r * m + c] = acc;
         }
       for (int c = 0; c < m; ++c) {
         for (int c2 = 0; c2 < c; ++c2) {
           E d = A::zero();
-          for (int r = 0; r < p; ++r) cmac_conj(d, nu[r * m + c2], nu[r * m + c]);
-          d = cfin(d);
+          for (int r = 0; r < p; ++r) cfma_conj(d, nu[r * m + c2], nu[r * m + c]);
           for (int r = 0; r < p; ++r) nu[r * m + c] = nu[r * m + c] - nu[r * m + c2] * d;
         }
         typename A::R s = abs2(nu[c]);
@@ -832,8 +830,7 @@ __device__ void scan_one_loop(const LoopArgs& a, int i, const E* Ul, const doubl
       const E* Uk = Ul + j * (long long)n * p;
       const E* nu = Nu + (size_t)j * p * m;
       E acc = A::zero();
-      for (int q = 0; q < p; ++q) cmac(acc, Uk[r * p + q], nu[q * m + c]);
-      acc = cfin(acc);
+      for (int q = 0; q < p; ++q) cfma(acc, Uk[r * p + q], nu[q * m + c]);
       wg[((long long)j * a.N_t + i) * n * m + rc2] = acc;
     }
     __syncthreads();
@@ -966,8 +963,8 @@ __device__ void nested_base_m1(const LoopArgs& a, int b) {
     const E* wa = wj + (size_t)i * n;
     const E* wb = wj + (size_t)(i + 1 == Nt ? 0 : i + 1) * n;
     E acc = A::zero();
-    for (int q = 0; q < n; ++q) cmac_conj(acc, wb[q], wa[q]);
-    prod = prod * cfin(acc);
+    for (int q = 0; q < n; ++q) cfma_conj(acc, wb[q], wa[q]);
+    prod = prod * acc;
   }
   for (int o = 16; o > 0; o >>= 1) prod = prod * A::shfl_xor(prod, o);
   if (tid == 0) a.nested_out[b] = phase_E(prod);
@@ -1045,17 +1042,16 @@ __device__ void pair_loop_df(const LoopArgs& a, int i, const cdf* Us, const doub
   const int jn = jj + 1 == N ? 0 : jj + 1;
   cdf x = cdf_zero();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) cmac_conj(x, Us[(jn * 4 + q) * 2 + r], Us[(jj * 4 + q) * 2 + c]);
-  x = cfin(x);
+  for (int q = 0; q < 4; ++q) cfma_conj(x, Us[(jn * 4 + q) * 2 + r], Us[(jj * 4 + q) * 2 + c]);
   // x <- x y over the groups of the warp: y from the group d earlier
   auto step = [&](cdf& v, int src4, bool take) {
     const cdf a0 = shfl_cdf(v, g4 + 2 * r), a1 = shfl_cdf(v, g4 + 2 * r + 1);
     const cdf b0 = shfl_cdf(v, src4 + c), b1 = shfl_cdf(v, src4 + 2 + c);
     if (take) {
       cdf y = cdf_zero();
-      cmac(y, a0, b0);
-      cmac(y, a1, b1);
-      v = cfin(y);
+      cfma(y, a0, b0);
+      cfma(y, a1, b1);
+      v = y;
     }
   };
 #pragma unroll 1
@@ -1073,9 +1069,9 @@ __device__ void pair_loop_df(const LoopArgs& a, int i, const cdf* Us, const doub
     const cdf a0 = shfl_cdf(x, g4 + 2 * r), a1 = shfl_cdf(x, g4 + 2 * r + 1);
     const cdf* E = Tw + eoff + 4 * (warp - 1);
     cdf y = cdf_zero();
-    cmac(y, a0, E[c]);
-    cmac(y, a1, E[2 + c]);
-    x = cfin(y);
+    cfma(y, a0, E[c]);
+    cfma(y, a1, E[2 + c]);
+    x = y;
   }
   if (active) Ps[4 * j + l] = x;
   __syncthreads();
@@ -1122,9 +1118,8 @@ __device__ void pair_loop_df(const LoopArgs& a, int i, const cdf* Us, const doub
   cdf nu = Ye[c * 2 + col];
   if (jj > 0) {
     nu = cdf_zero();
-    cmac(nu, Ps[4 * (jj - 1) + 2 * c], Ye[col]);
-    cmac(nu, Ps[4 * (jj - 1) + 2 * c + 1], Ye[2 + col]);
-    nu = cfin(nu);
+    cfma(nu, Ps[4 * (jj - 1) + 2 * c], Ye[col]);
+    cfma(nu, Ps[4 * (jj - 1) + 2 * c + 1], Ye[2 + col]);
   }
   const cdf nu_o = shfl_cdf(nu, lane ^ 1);
   const df s = c == 0 ? abs2(nu) + abs2(nu_o) : abs2(nu_o) + abs2(nu);
@@ -1133,9 +1128,9 @@ __device__ void pair_loop_df(const LoopArgs& a, int i, const cdf* Us, const doub
   // Wannier state w(j, i) = U(k_j) nu_j, row l on lane l
   const cdf n0 = shfl_cdf(nu, g4), n1 = shfl_cdf(nu, g4 + 1);
   cdf wv = cdf_zero();
-  cmac(wv, Q0, n0);
-  cmac(wv, Q1, n1);
-  if (active) reinterpret_cast<cdf*>(a.w)[((long long)j * a.N_t + i) * 4 + l] = cfin(wv);
+  cfma(wv, Q0, n0);
+  cfma(wv, Q1, n1);
+  if (active) reinterpret_cast<cdf*>(a.w)[((long long)j * a.N_t + i) * 4 + l] = wv;
 }
 
 // The plan arrays as the kernel reads them: in global memory, or (inl != NULL) in the
@@ -1159,7 +1154,7 @@ __device__ __forceinline__ void nested_base_m1_cta(const LoopArgs& a, int b, cdf
   for (int i0 = 0; i0 < Nt; i0 += FUSED_THREADS / 4) {
     const int i = i0 + (tid >> 2), q = tid & 3;
     cdf z = cdf_zero();
-    if (i < Nt) cmac_conj(z, wj[(size_t)(i + 1 == Nt ? 0 : i + 1) * 4 + q], wj[(size_t)i * 4 + q]);
+    if (i < Nt) cfma_conj(z, wj[(size_t)(i + 1 == Nt ? 0 : i + 1) * 4 + q], wj[(size_t)i * 4 + q]);
     z = z + Arith<cdf>::shfl_xor(z, 1);
     z = z + Arith<cdf>::shfl_xor(z, 2);
     if (!(i < Nt)) z = one;
@@ -1240,9 +1235,8 @@ __device__ __forceinline__ void loops_fused_body(const StatesArgs& sa, const Loo
       cdf acc = cdf_zero();
       for (int h = s_ent[e]; h < s_ent[e + 1]; ++h) {
         const float4 t4 = s_ht[h];
-        cmac(acc, cdf(df(t4.x, t4.y), df(t4.z, t4.w)), cache[s_hr[h] * KPB + kl]);
+        cfma(acc, cdf(df(t4.x, t4.y), df(t4.z, t4.w)), cache[s_hr[h] * KPB + kl]);
       }
-      acc = cfin(acc);
       const int col = s_col[e];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -1450,8 +1444,8 @@ __global__ void k_nested_scan(LoopArgs a) {
       const E* wa = Wn + (size_t)i * nm;
       const E* wb = Wn + (size_t)(i + 1 == Nt ? 0 : i + 1) * nm;
       E acc = A::zero();
-      for (int q = 0; q < n; ++q) cmac_conj(acc, wb[q * m + r], wa[q * m + c]);
-      S[e] = cfin(acc);
+      for (int q = 0; q < n; ++q) cfma_conj(acc, wb[q * m + r], wa[q * m + c]);
+      S[e] = acc;
     }
     __syncthreads();
     E* Pf = prefix_products(S, T, Nt, m);

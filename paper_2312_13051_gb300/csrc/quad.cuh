@@ -217,13 +217,12 @@ __device__ __forceinline__ cdf tab_at_df(const cdf* lo, const cdf* hi, TabShape 
   return hi[m / t.B] * lo[m % t.B];
 }
 
-// acc += a b with b exact in float (df_mac without the term in b.lo).
-__device__ __forceinline__ void df_mac(df& acc, df a, float b) {
-  const float p = a.hi * b;
-  const float e = fmaf(a.lo, b, fmaf(a.hi, b, -p));
-  const df s = df_two_sum(acc.hi, p);
-  acc.hi = s.hi;
-  acc.lo += s.lo + e;
+// acc += a b + c d with b and d exact in float (df_mac2 without the terms in their low parts).
+__device__ __forceinline__ void df_mac2(df& acc, df a, float b, df c, float d) {
+  const float p = a.hi * b, q = c.hi * d;
+  const float e = fmaf(a.lo, b, fmaf(a.hi, b, -p)), f = fmaf(c.lo, d, fmaf(c.hi, d, -q));
+  const df s = df_two_sum(p, q), t = df_two_sum(acc.hi, s.hi);
+  acc = df_two_sum(t.hi, (s.lo + t.lo) + ((e + f) + acc.lo));
 }
 
 __device__ __forceinline__ df group_sum_df(df v) {
@@ -250,12 +249,10 @@ __device__ __forceinline__ cdf quad_matvec(const cdf (&Hr)[4], c32 x, int base) 
   for (int q = 0; q < 4; ++q) {
     const cdf h = sel4(Hr, q);
     const c32 v = shfl_z(x, base + q);
-    df_mac(acc.re, h.re, v.re);
-    df_mac(acc.im, h.re, v.im);
-    df_mac(acc.re, h.im, -v.im);
-    df_mac(acc.im, h.im, v.re);
+    df_mac2(acc.re, h.re, v.re, h.im, -v.im);
+    df_mac2(acc.im, h.re, v.im, h.im, v.re);
   }
-  return cfin(acc);
+  return acc;
 }
 
 // An FP32 pair x0, x1 of the group with h_c = H x_c: the Ritz matrix g = x^dag h and the
@@ -275,24 +272,20 @@ __device__ __forceinline__ QuadPair quad_pair(c32 x0, c32 x1, cdf h0, cdf h1) {
     const c32 a = t == 2 ? x1 : x0, b = t == 0 ? x0 : x1;
     const cdf h = t == 0 ? h0 : h1;
     df gr(0.f), gi(0.f), er(0.f), ei(0.f);
-    df_mac(gr, h.re, a.re);
-    df_mac(gr, h.im, a.im);
+    df_mac2(gr, h.re, a.re, h.im, a.im);
     gr = group_sum_df(gr);
     if (t == 1) {
-      df_mac(gi, h.im, a.re);
-      df_mac(gi, h.re, -a.im);
+      df_mac2(gi, h.im, a.re, h.re, -a.im);
       r.gre = gr;
       r.gim = group_sum_df(gi);
     }
     if (t == 0) r.g00 = gr;
     if (t == 2) r.g11 = gr;
     if constexpr (kDev) {
-      df_mac(er, df(b.re), a.re);
-      df_mac(er, df(b.im), a.im);
+      df_mac2(er, df(b.re), a.re, df(b.im), a.im);
       er = group_sum_df(er);
       if (t == 1) {
-        df_mac(ei, df(b.im), a.re);
-        df_mac(ei, df(b.re), -a.im);
+        df_mac2(ei, df(b.im), a.re, df(b.re), -a.im);
         r.e01 = c32(er.hi, group_sum_df(ei).hi);
       }
       const float d = (er.hi - 1.f) + er.lo;
@@ -392,7 +385,7 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
     for (int t = 0; t < 3; ++t) {  // (0, 0), (0, 1), (1, 1)
       const cdf xa = t == 2 ? Q1 : Q0, xb = t == 0 ? Q0 : Q1;
       cdf g = cdf_zero();
-      cmac_conj(g, xa, xb);
+      cfma_conj(g, xa, xb);
       const df gre = group_sum_df(g.re);
       const float d = (gre.hi - 1.f) + gre.lo;
       if (t == 0) e00 = d;

@@ -927,9 +927,8 @@ __global__ void __launch_bounds__(QUAD_THREADS) k_states_quad_df(StatesArgs a) {
     cdf acc = cdf_zero();
     for (int h = md.ent_start[e]; h < md.ent_start[e + 1]; ++h) {
       const float* t4 = md.hop_tdf + 4 * h;
-      cmac(acc, cdf(df(t4[0], t4[1]), df(t4[2], t4[3])), cache[md.hop_r[h] * KPB + kl]);
+      cfma(acc, cdf(df(t4[0], t4[1]), df(t4[2], t4[3])), cache[md.hop_r[h] * KPB + kl]);
     }
-    acc = cfin(acc);
     const int col = md.ent_col[e];
 #pragma unroll
     for (int c = 0; c < 4; ++c)
