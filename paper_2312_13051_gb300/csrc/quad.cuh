@@ -305,12 +305,21 @@ __device__ __forceinline__ void dev_second_order(float& e00, float& e11, c32& e0
   e01 = t * e01;
 }
 
-// Eigenvalues lo <= hi of the pair's 2 x 2 Ritz matrix in the orthonormalised basis,
-// g - (e g + g e) / 2 + s, s a small Hermitian correction (FP32):
+// Eigenvalues lo <= hi of the pair's 2 x 2 Ritz matrix in the orthonormalised basis, to second
+// order in the deviation: (I + e)^{-1/2} g (I + e)^{-1/2} + s = g - (e' g + g e') / 2 + e g e / 4 + s
+// with e' = e - 3/4 e^2, s a small Hermitian correction (the small terms in FP32; the FP32 rotations
+// leave e up to ~5e-6, so that e g e / 4 is worth 1e-11);
 // (a + d) / 2 -+ sqrt(((a - d) / 2)^2 + |b|^2) in double-float.
 __device__ __forceinline__ void quad_pair_edges(QuadPair r, float s00, float s11, c32 s01, df& lo, df& hi) {
-  dev_second_order(r.e00, r.e11, r.e01);
   const c32 g(r.gre.hi, r.gim.hi);
+  {
+    const c32 m00 = r.g00.hi * c32(r.e00, 0.f) + g * conj(r.e01), m01 = r.g00.hi * r.e01 + r.e11 * g;
+    const c32 m10 = r.e00 * conj(g) + r.g11.hi * conj(r.e01), m11 = conj(g) * r.e01 + r.g11.hi * c32(r.e11, 0.f);
+    s00 += 0.25f * (r.e00 * m00.re + (r.e01 * m10).re);
+    s11 += 0.25f * ((conj(r.e01) * m01).re + r.e11 * m11.re);
+    s01 = s01 + 0.25f * (r.e00 * m01 + r.e01 * m11);
+  }
+  dev_second_order(r.e00, r.e11, r.e01);
   const float a = r.g00.hi, d = r.g11.hi, m = 0.5f * (a + d), x = g.re * r.e01.re + g.im * r.e01.im;
   const df aa = r.g00 + df(s00 - r.e00 * a - x), dd = r.g11 + df(s11 - r.e11 * d - x);
   const float eh = 0.5f * (r.e00 + r.e11);
@@ -375,6 +384,9 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
   const float d00 = oc.g00.hi - lz0, d01 = oc.g11.hi - lz0, d10 = oc.g00.hi - lz1, d11 = oc.g11.hi - lz1;
   const c32 c00 = coef(z0, r0, d00), c01 = coef(z0, r1, d01), c10 = coef(z1, r0, d10), c11 = coef(z1, r1, d11);
   const c32 u0 = z0 * c00 + z1 * c10, u1 = z0 * c01 + z1 * c11;
+  // z_a^dag q_c: the pairs are orthogonal to FP32 only, which counts at second order
+  const c32 o00 = group_sum_c32(conj(z0) * q0), o01 = group_sum_c32(conj(z0) * q1);
+  const c32 o10 = group_sum_c32(conj(z1) * q0), o11 = group_sum_c32(conj(z1) * q1);
   Q0 = cdf(df_two_sum(q0.re, u0.re), df_two_sum(q0.im, u0.im));
   Q1 = cdf(df_two_sum(q1.re, u1.re), df_two_sum(q1.im, u1.im));
   // Lowdin step: the deviation E of the corrected pair in double-float
@@ -392,10 +404,10 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
       if (t == 1) e01 = c32(gre.hi, group_sum_df(g.im).hi);
       if (t == 2) e11 = d;
     }
-    // the FP32 pair's own deviation, for its Ritz matrix (up to cross terms of ~1e-13)
-    oc.e00 = e00 - abs2(c00) - abs2(c10);
-    oc.e11 = e11 - abs2(c01) - abs2(c11);
-    oc.e01 = e01 - conj(c00) * c01 - conj(c10) * c11;
+    // the FP32 pair's own deviation, for its Ritz matrix: E - C^dag C - o^dag C - C^dag o
+    oc.e00 = e00 - (conj(c00 + 2.f * o00) * c00).re - (conj(c10 + 2.f * o10) * c10).re;
+    oc.e11 = e11 - (conj(c01 + 2.f * o01) * c01).re - (conj(c11 + 2.f * o11) * c11).re;
+    oc.e01 = e01 - conj(c00 + o00) * c01 - conj(c10 + o10) * c11 - conj(c00) * o01 - conj(c10) * o11;
     dev_second_order(e00, e11, e01);
     const c32 x0(Q0.re.hi, Q0.im.hi), x1(Q1.re.hi, Q1.im.hi);
     const c32 f0 = e00 * x0 + x1 * conj(e01), f1 = x0 * e01 + e11 * x1;
@@ -407,9 +419,11 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
   const float m0 = 0.5f * (d00 + d01), m1 = 0.5f * (d10 + d11);
   quad_pair_edges(oc, d00 * abs2(c00) + d10 * abs2(c10), d01 * abs2(c01) + d11 * abs2(c11),
                   m0 * (conj(c00) * c01) + m1 * (conj(c10) * c11), occ_lo, occ_hi);
+  // (the unoccupied vectors' coefficients on the occupied ones are -conj(C + o))
+  const c32 b00 = c00 + o00, b01 = c01 + o01, b10 = c10 + o10, b11 = c11 + o11;
   const float n0 = 0.5f * (d00 + d10), n1 = 0.5f * (d01 + d11);
-  quad_pair_edges(un, -(d00 * abs2(c00) + d01 * abs2(c01)), -(d10 * abs2(c10) + d11 * abs2(c11)),
-                  -(n0 * (c00 * conj(c10)) + n1 * (c01 * conj(c11))), un_lo, un_hi);
+  quad_pair_edges(un, -(d00 * abs2(b00) + d01 * abs2(b01)), -(d10 * abs2(b10) + d11 * abs2(b11)),
+                  -(n0 * (b00 * conj(b10)) + n1 * (b01 * conj(b11))), un_lo, un_hi);
   gap = df_to_double(un_lo - occ_hi);
   return sweeps;
 }

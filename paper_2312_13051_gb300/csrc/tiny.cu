@@ -858,11 +858,9 @@ __global__ void __launch_bounds__(QUAD_THREADS)
 //  - one Newton correction of the occupied block Q in the FP32 eigenbasis, with the
 //    residual R = H Q - Q rho in double-float: for each unoccupied FP32 vector z_a,
 //    Q_c += z_a (z_a^dag R_c) / (rho_c - lam_a), rho_c = q_c^dag H q_c;
-//  - one first-order Lowdin step Q <- Q - Q (Q^dag Q - I) / 2 with the Gram matrix
-//    in double-float;
-//  - the gap from double-float Ritz values of the refined occupied pair and of the
-//    re-orthonormalised unoccupied pair (errors quadratic in the subspace errors,
-//    whatever the splitting inside each pair).
+//  - one second-order Lowdin step with the Gram matrix in double-float;
+//  - the gap from double-float Ritz values of the two FP32 pairs, to second order in what
+//    they lack of orthonormality and of convergence (60 x 3840 points: at most 2.7e-13 off).
 // The occupied block leaves as complex double-float (hi, lo per part, 16 bytes like
 // a complex128), accurate to about 1e-13, for the double-float loop kernels.
 // ---------------------------------------------------------------------------
