@@ -530,7 +530,7 @@ struct GcA<z64> {
     return z64(__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o));
   }
   __device__ static bool negligible(z64 h11, z64 h12, z64 h21, z64 h22) {
-    return geig_negligible_v(h11, h12, h21, h22, 2.220446049250313e-16);
+    return geig_negligible_v(h11, h12, h21, h22, 2.220446049250313e-16, true);
   }
   __device__ static z64 shift(z64 a, z64 b, z64 c, z64 d, int iter, z64 h2, bool has_h2) {
     return geig_shift(a, b, c, d, iter, has_h2 ? zabs(h2) : 0.0);

@@ -21,6 +21,7 @@ namespace bw {
 // included, 19.5 -> 12.9 ms; p = 32 FP64, 17 loops, 5.1 -> 3.5 ms; p = 12 with vectors 1.46 ->
 // 1.16 ms.  A step at p = 64 takes ~7000 clocks: 2100 the rotations, the rest FP64 throughput.
 constexpr int GEIG_NB = 8;
+constexpr int GEIG_STALL = 30;  // rounds without a deflation after which the product test decides too
 
 struct GeigShared {
   double c[GEIG_NB];    // Givens of each sweep: G = [[c, s], [-conj(s), c]], c real
@@ -59,16 +60,22 @@ __device__ __forceinline__ void givens(z64 x, z64 y, double& c, z64& s) {
 }
 
 // Whether the subdiagonal entry H[l][l-1] is negligible: against the neighbouring
-// diagonal entries, or by the product test of Ahues and Tisseur (its product with
-// the superdiagonal small against the local separation of the diagonal entries).
+// diagonal entries, or with `product` also by the product test of Ahues and Tisseur (its
+// product with the superdiagonal small against the local separation of the diagonal entries).
 // Magnitudes are |re| + |im| (within a factor sqrt(2) of the modulus, a hypot each otherwise).
+// The product test lets go of entries far above rounding where the superdiagonal one is
+// small.  That is right for the 2 x 2 block, but several sweeps at once leave many such entries
+// inside a matrix that has not converged, where what is dropped couples to everything right of
+// the superdiagonal: phases of weakly coupled bands lost two digits (p = 32 to 80, FP64: up to
+// 8e-13 rad from FP64, without it 8e-15, at the same speed).  So those sweeps use it only where nothing
+// else has deflated for GEIG_STALL rounds; the cluster solver, one sweep at a time, always.
 __device__ __forceinline__ double zabs1(z64 a) { return fabs(a.re) + fabs(a.im); }
 
-__device__ __forceinline__ bool geig_negligible_v(z64 h11, z64 h12, z64 h21, z64 h22, double eps) {
+__device__ __forceinline__ bool geig_negligible_v(z64 h11, z64 h12, z64 h21, z64 h22, double eps, bool product) {
   const double sub = zabs1(h21);
   const double dia = zabs1(h22) + zabs1(h11);
   bool small = sub <= eps * dia || sub < 1e-300;
-  if (!small && sub <= dia) {
+  if (product && !small && sub <= dia) {
     const double x = zabs1(h12);
     const double ab = fmax(sub, x), ba = fmin(sub, x);
     const double y = zabs1(h11 - h22);
@@ -79,9 +86,9 @@ __device__ __forceinline__ bool geig_negligible_v(z64 h11, z64 h12, z64 h21, z64
   return small;
 }
 
-__device__ __forceinline__ bool geig_negligible(const z64* H, int ld, int l, double eps) {
+__device__ __forceinline__ bool geig_negligible(const z64* H, int ld, int l, double eps, bool product) {
   return geig_negligible_v(H[(l - 1) * ld + l - 1], H[(l - 1) * ld + l], H[l * ld + l - 1],
-                           H[l * ld + l], eps);
+                           H[l * ld + l], eps, product);
 }
 
 // Shift of a QR sweep from the trailing 2 x 2 [[a, b], [c, d]] of the active window:
@@ -225,11 +232,11 @@ __device__ __forceinline__ double geig_shifts(const z64* H, int ld, int hi, int 
 
 // Largest l in [1, hi] whose subdiagonal entry is negligible, or 0: the first warp
 // tests 32 subdiagonals at a time from hi down.  Every lane of the warp calls it.
-__device__ __forceinline__ int geig_split_point(const z64* H, int ld, int hi, double eps) {
+__device__ __forceinline__ int geig_split_point(const z64* H, int ld, int hi, double eps, bool product) {
   const int lane = threadIdx.x & 31;
   for (int base = hi; base >= 1; base -= 32) {
     const int l = base - lane;
-    const bool f = l >= 1 && geig_negligible(H, ld, l, eps);
+    const bool f = l >= 1 && geig_negligible(H, ld, l, eps, product);
     const unsigned m = __ballot_sync(0xffffffffu, f);
     if (m) return base - (__ffs(m) - 1);
   }
@@ -239,7 +246,7 @@ __device__ __forceinline__ int geig_split_point(const z64* H, int ld, int hi, do
 // Eigen-decomposition of H (p x p, leading dimension ld), destroyed on output.
 // lam[p] receives the eigenvalues.  With want_vec, Z (p x p) receives the right
 // eigenvectors as unit-norm columns; vec scratch needs p z64.  Returns 0, or -1
-// when the QR iteration cap (120 p sweeps) is reached.
+// when the QR iteration cap (120 p + 120 rounds of sweeps) is reached.
 __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* lam, z64* vec,
                     GeigShared* sh) {
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -333,7 +340,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
           hi = -1;
           break;
         }
-        l = geig_split_point(H, ld, hi, eps);
+        l = geig_split_point(H, ld, hi, eps, iter >= GEIG_STALL);
         __syncwarp();
         if (tid == 0 && l > 0) H[l * ld + l - 1] = z64(0.0, 0.0);
         if (l == hi) {
@@ -362,7 +369,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
         break;
       }
       ++iter;
-      total += nb;
+      ++total;
       if (tid == 0) {
         sh->hi = hi;
         sh->l = l;

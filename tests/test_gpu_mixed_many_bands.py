@@ -47,3 +47,15 @@ def test_mixed_phases_at_the_solvers_limits(lib, ctx, copies):
     ph, _ = lib.wilson_loop(model, plane, p, precision="mixed", ctx=ctx)
     ref, _ = oracle.wilson_loop(model, plane, p)
     assert circ_err_rows(ph.cpu().numpy(), ref) <= plane.N * p * 2.0 ** -47
+
+
+@pytest.mark.parametrize("copies,seed", [(16, 6), (24, 1), (24, 3), (40, 1), (40, 7)])
+def test_fp64_phases_at_rounding(lib, ctx, copies, seed):
+    # the same in FP64: units of 2^-52 from N p independent roundings, with a factor of eight
+    # (8 sqrt(N p) 2^-52).  With a weak coupling many entries next to the diagonal of the
+    # Hessenberg matrix are small at once
+    model = coupled_copies(copies, seed, eps=1e-4)
+    plane, p = I.Plane(16, 24, origin=(0.013, 0.021, 0.0)), 2 * copies
+    ph, _ = lib.wilson_loop(model, plane, p, precision="fp64", ctx=ctx)
+    ref, _ = oracle.wilson_loop(model, plane, p)
+    assert circ_err_rows(ph.cpu().numpy(), ref) <= 8 * np.sqrt(plane.N * p) * 2.0 ** -52
