@@ -857,7 +857,9 @@ __global__ void k_loops_scan(LoopArgs a) {
 // 10.9 us.
 template <int PP>
 __global__ void k_loops_warp(LoopArgs a) {
-  const int lane = threadIdx.x & 31, i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  // (the thread index of a grid of 2^27 loops and more passes 32 bits)
+  const long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= a.N_t) return;
   const int n = a.n, N = a.N;
   const long long k0 = (long long)i * N;
