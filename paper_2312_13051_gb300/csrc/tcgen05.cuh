@@ -13,10 +13,11 @@
 // the differences are exact in FP32, and 3 x 8 significant bits hold an FP32
 // significand), and every product keeps the eight terms a_i b_j with i + j <= 3
 // (smallest first); the one dropped term, a2 b2, is ~2^-48 relative.  The products of
-// bf16 values are exact.  Each chunk of 64 real terms is accumulated in TMEM in two
+// bf16 values are exact.  Each half of a chunk, 32 real terms, is accumulated in TMEM in two
 // accumulators, the seven cross products (smallest first) in one and a0 b0 alone in
 // the other, so that no small term is added into a full-size sum inside the tensor
-// core; the two are then added into FP32 registers.
+// core; the two are then added into FP32 registers.  (One pair of accumulators for the 64
+// terms of a chunk would sum twice as many terms in the tensor core's own rounding.)
 //
 // Shared-memory layout of a tile (no swizzle, K-major): rows in groups of 8, each group
 // holding its K range as consecutive 8-row x 16-byte core matrices (8 bf16 per row).  The
@@ -150,7 +151,7 @@ constexpr size_t SMEM = 3 * A_BYTES + 3 * B_BYTES;  // 72 KB (the epilogue reuse
 
 // Byte offset of the 16-byte row (row, 8 oct .. 8 oct + 7) of a tile.
 __device__ __forceinline__ int off8(int row, int oct) { return (row >> 3) * ROW8 + oct * 128 + (row & 7) * 16; }
-constexpr uint32_t TMEM_COLS = 128;     // two 128 x 64 FP32 accumulators
+constexpr uint32_t TMEM_COLS = 256;     // four 128 x 64 FP32 accumulators (two CTAs fill an SM's TMEM)
 constexpr int WAIT_POLLS = 1 << 22;
 
 // Per-CTA state: the TMEM base, the MMA-completion barrier and its phase, and whether a
@@ -256,7 +257,8 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
         fence_after();
         if (tid == 0) {
           // pieces (i, j) with i + j <= 3: the seven cross products, smallest first, into
-          // the first accumulator; a0 b0 alone into the second (columns 64 ..)
+          // the first accumulator of a half; a0 b0 alone into the second (64 columns on).
+          // Half h holds inner indices 16 h .. 16 h + 15: real K values 16 h .. and KC + 16 h ..
           constexpr int PI[8] = {1, 2, 0, 1, 2, 0, 1, 0}, PJ[8] = {2, 1, 2, 1, 0, 1, 0, 0};
           const uint32_t a0 = smem_u32(Ap), b0 = smem_u32(Bp);
 #pragma unroll
@@ -264,10 +266,9 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
 #pragma unroll
             for (int ks = 0; ks < 2 * KC / 16; ++ks) {  // 16 real K values (two core matrices) per MMA
               const uint32_t o = ks * 256;
-              const bool big = t == 7;
-              mma_bf16(s.tmem + (big ? 64u : 0u), smem_desc(a0 + PI[t] * A_BYTES + o, 128, ROW8),
-                       smem_desc(b0 + PJ[t] * B_BYTES + o, 128, ROW8), IDESC,
-                       (big ? ks : (ks | t)) ? 1u : 0u);
+              const bool big = t == 7, first = ks < 2 && (big || t == 0);
+              mma_bf16(s.tmem + 128u * (ks & 1) + (big ? 64u : 0u), smem_desc(a0 + PI[t] * A_BYTES + o, 128, ROW8),
+                       smem_desc(b0 + PJ[t] * B_BYTES + o, 128, ROW8), IDESC, first ? 0u : 1u);
             }
           commit(s.mbar);
         }
@@ -282,12 +283,13 @@ __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsign
         }
         // the chunk's partial sums into the FP32 register accumulators
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int q = 0; q < 4; ++q) {  // half q / 2 of the chunk, columns 16 (q % 2) ..
+          const int h = q >> 1, c = 16 * (q & 1);
           float v[16], w[16];
-          ld16(taddr + uint32_t(16 * h), v);
-          ld16(taddr + 64u + uint32_t(16 * h), w);
+          ld16(taddr + uint32_t(128 * h + c), v);
+          ld16(taddr + uint32_t(128 * h + 64 + c), w);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) acc[16 * h + j] += w[j] + v[j];
+          for (int j = 0; j < 16; ++j) acc[c + j] += w[j] + v[j];
         }
         fence_before();
         __syncthreads();  // TMEM read before the next chunk's first MMA overwrites it
