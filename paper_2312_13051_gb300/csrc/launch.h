@@ -45,7 +45,13 @@ struct StatesArgs {
   double* pso_gap;      // K (optional)
   DevStatus* status;
   int want_df;          // write U as complex double-float (states_df_eligible() holds)
+  int rotations;        // n = 4: Jacobi rotations that H(k) takes at generic points (0: not known)
 };
+
+// n = 4, more k-points than this, H(k) diagonal after this many Jacobi rotations: one thread per
+// k-point (k_states_four).
+constexpr long long FOUR_MIN_K = 12288;
+constexpr int FOUR_MAX_ROT = 8;
 
 struct EighArgs {
   const z64* H;               // packed

@@ -299,6 +299,30 @@ __device__ __forceinline__ int tiny_sector(const StatesArgs& a, long long k, con
   return a.sign < 0 ? 0 : PP / 2;
 }
 
+// Columns v of the sector in the occupied basis from the projected spin operator S (Hermitian,
+// overwritten), with the checks and outputs of tiny_sector.
+template <int PP>
+__device__ __forceinline__ void tiny_sector_columns(const StatesArgs& a, long long k, z64 (&S)[PP][PP], bool write,
+                                                    z64 (&v)[PP][PP / 2]) {
+  double mu[PP];
+  if constexpr (PP == 2) {
+    z64 v0, v1;
+    eig2_herm(S[0][0].re, S[1][1].re, S[0][1], mu[0], mu[1], v0, v1);
+    const bool up = tiny_sector<2>(a, k, mu, true, write) != 0;
+    v[0][0] = up ? -conj(v1) : v0;
+    v[1][0] = up ? conj(v0) : v1;
+  } else {
+    z64 SV[PP][PP], SVs[PP][PP];
+    const bool okp = jac_serial<PP, double>(S, SV, a.max_sweeps) >= 0;
+    sort_eig<PP, double>(S, SV, SVs, mu);
+    const bool up = tiny_sector<PP>(a, k, mu, okp, write) != 0;
+#pragma unroll
+    for (int q = 0; q < PP; ++q)
+#pragma unroll
+      for (int c = 0; c < PP / 2; ++c) v[q][c] = up ? SVs[q][c + PP / 2] : SVs[q][c];
+  }
+}
+
 // The plan arrays in the kernel's parameter copy of the plan instead of at dbase.
 __device__ __forceinline__ void tiny_relocate(StatesArgs& a, const unsigned char* inl, const char* dbase) {
   auto at = [&](auto*& p) {
@@ -738,24 +762,8 @@ __device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
         for (int c = 0; c < PP; ++c) cfma(sQ[c], v, shfl_z(Q[c], base + col));
       }
       quad_gram<PP>(Q, sQ, S, l, base);
-      double mu[PP];
-      z64 v[PP][PP / 2];  // sector columns
-      if constexpr (PP == 2) {
-        z64 v0, v1;
-        eig2_herm(S[0][0].re, S[1][1].re, S[0][1], mu[0], mu[1], v0, v1);
-        const bool up = tiny_sector<2>(a, k, mu, true, write) != 0;
-        v[0][0] = up ? -conj(v1) : v0;
-        v[1][0] = up ? conj(v0) : v1;
-      } else {
-        z64 SV[PP][PP], SVs[PP][PP];
-        const bool okp = jac_serial<PP, double>(S, SV, a.max_sweeps) >= 0;
-        sort_eig<PP, double>(S, SV, SVs, mu);
-        const bool up = tiny_sector<PP>(a, k, mu, okp, write) != 0;
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-#pragma unroll
-          for (int c = 0; c < PP / 2; ++c) v[q][c] = up ? SVs[q][c + PP / 2] : SVs[q][c];
-      }
+      z64 v[PP][PP / 2];
+      tiny_sector_columns<PP>(a, k, S, write, v);
       if (!active) return;
       z64* out = a.U + k * 4LL * (PP / 2) + l * (PP / 2);
 #pragma unroll
@@ -774,11 +782,16 @@ __device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
   for (int c = 0; c < PP; ++c) out[c] = Q[c];
 }
 
-// n = 4 on large grids when H has entries that are identically zero (the models' own sparse
-// forms): one thread per k-point, FP64 Jacobi, whose rotations of zero entries are skipped.
-// There the sweeps take fewer FP64 instructions than the refined solve (BBH, 230 400 k-points:
-// 0.68 ms against 0.93; spin-Hall, 60 000: 0.16 against 0.24), with a full matrix more (BBH with
-// an on-site term: 1.98 against 1.22 ms); on small grids four lanes per k-point win either way.
+// n = 4 on large grids when H(k) is diagonal after a few rotations (the models with symmetry;
+// four_band_rotations counts them): one thread per k-point, FP64 Jacobi, whose rotations of
+// zero entries are skipped.  There the sweeps take fewer FP64 instructions than the refined
+// solve, 20 rotations take twice as many, and below ~13 000 points four lanes per k-point finish
+// before one thread's chain does.  States kernel, one thread / four lanes, us:
+//   BBH (5 rotations)       9000 points 61 / 43, 18 000 65 / 78, 90 000 264 / 344, 230 400 635 / 866
+//   spin-Hall (2), spin     9000 49 / 51, 18 000 53 / 92, 90 000 192 / 412, 230 400 463 / 1038
+//   Eq. 9 (5)               18 000 72 / 82, 230 400 676 / 926
+//   BBH + diagonal (22)     18 000 184 / 82, 230 400 1830 / 892 (as any other pattern of 8 to 16
+//                           entries that does not end early)
 constexpr int FOUR_THREADS = 32;
 
 template <int PP>
@@ -809,6 +822,57 @@ __device__ __forceinline__ void states_four(const StatesArgs& a, int use_tab) {
   a.gap[k] = gap;
   if (!ok) report(a.status, ST_ENOCONV, k, 0.0);
   if (!(gap > a.gap_tol)) report(a.status, ST_EGAP, k, gap);
+  if (a.op.nnz > 0) {
+    if constexpr (PP % 2 == 0) {
+      // projected spin operator restricted to the occupied space (Sec. IV)
+      z64 S[PP][PP];
+#pragma unroll
+      for (int x = 0; x < PP; ++x)
+#pragma unroll
+        for (int y = 0; y < PP; ++y) S[x][y] = z64(0.0, 0.0);
+      for (int q = 0; q < a.op.nnz; ++q) {
+        const int row = a.op.row[q], col = a.op.col[q];
+        const z64 v = a.op.val[q];
+        z64 qa[PP], qb[PP];
+#pragma unroll
+        for (int c = 0; c < PP; ++c) {
+          qa[c] = qb[c] = z64(0.0, 0.0);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            if (r == row) qa[c] = Vs[r][c];
+            if (r == col) qb[c] = Vs[r][c];
+          }
+          qb[c] = v * qb[c];
+        }
+#pragma unroll
+        for (int x = 0; x < PP; ++x)
+#pragma unroll
+          for (int y = 0; y < PP; ++y) cfma_conj(S[x][y], qa[x], qb[y]);
+      }
+#pragma unroll
+      for (int x = 0; x < PP; ++x) {
+        S[x][x].im = 0.0;
+#pragma unroll
+        for (int y = x + 1; y < PP; ++y) {
+          S[x][y] = 0.5 * (S[x][y] + conj(S[y][x]));
+          S[y][x] = conj(S[x][y]);
+        }
+      }
+      z64 v[PP][PP / 2];
+      tiny_sector_columns<PP>(a, k, S, true, v);
+      z64* out = a.U + k * 4LL * (PP / 2);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < PP / 2; ++c) {
+          z64 acc(0.0, 0.0);
+#pragma unroll
+          for (int q = 0; q < PP; ++q) cfma(acc, Vs[r][q], v[q][c]);
+          out[r * (PP / 2) + c] = acc;
+        }
+    }
+    return;
+  }
   z64* out = a.U + k * 4LL * PP;
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -961,7 +1025,7 @@ cudaError_t quad_launch(const StatesArgs& a, bool use_tab, TabShape tN, TabShape
                         const FusedPlan* plan, const char* dbase) {
   constexpr int KPB = QUAD_THREADS / 4;
   cudaError_t e;
-  if (a.model.n_ent < 16 && a.op.nnz == 0 && a.K > 8192) {
+  if (a.rotations > 0 && a.rotations <= FOUR_MAX_ROT && a.K > FOUR_MIN_K) {
     const size_t sm = tiny_smem_bytes(a.model.n_R, a.model.n_hop, FOUR_THREADS, use_tab, tN, tT);
     const int grid = int((a.K + FOUR_THREADS - 1) / FOUR_THREADS);
     if (plan) {
