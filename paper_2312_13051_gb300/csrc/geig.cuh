@@ -60,22 +60,24 @@ __device__ __forceinline__ void givens(z64 x, z64 y, double& c, z64& s) {
 }
 
 // Whether the subdiagonal entry H[l][l-1] is negligible: against the neighbouring
-// diagonal entries, or with `product` also by the product test of Ahues and Tisseur (its
-// product with the superdiagonal small against the local separation of the diagonal entries).
+// diagonal entries, or by the product test of Ahues and Tisseur (its product with the
+// superdiagonal small against the local separation of the diagonal entries).
 // Magnitudes are |re| + |im| (within a factor sqrt(2) of the modulus, a hypot each otherwise).
-// The product test lets go of entries far above rounding where the superdiagonal one is
+// The product test can let go of entries far above rounding where the superdiagonal one is
 // small.  That is right for the 2 x 2 block, but several sweeps at once leave many such entries
 // inside a matrix that has not converged, where what is dropped couples to everything right of
 // the superdiagonal: phases of weakly coupled bands lost two digits (p = 32 to 80, FP64: up to
-// 8e-13 rad from FP64, without it 8e-15, at the same speed).  So those sweeps use it only where nothing
-// else has deflated for GEIG_STALL rounds; the cluster solver, one sweep at a time, always.
+// 8e-13 rad from FP64, without it 1e-14).  So those sweeps use it for entries up to 64 roundings
+// (`product` false), what a block of equal eigenvalues, whose off-diagonal entries are rounding
+// themselves, needs in order to fall apart; any entry only after GEIG_STALL rounds without a
+// deflation.  The cluster solver, one sweep at a time, uses it for any entry.
 __device__ __forceinline__ double zabs1(z64 a) { return fabs(a.re) + fabs(a.im); }
 
 __device__ __forceinline__ bool geig_negligible_v(z64 h11, z64 h12, z64 h21, z64 h22, double eps, bool product) {
   const double sub = zabs1(h21);
   const double dia = zabs1(h22) + zabs1(h11);
   bool small = sub <= eps * dia || sub < 1e-300;
-  if (product && !small && sub <= dia) {
+  if (!small && sub <= (product ? 1.0 : 64.0 * eps) * dia) {
     const double x = zabs1(h12);
     const double ab = fmax(sub, x), ba = fmin(sub, x);
     const double y = zabs1(h11 - h22);
@@ -207,8 +209,10 @@ __device__ __forceinline__ void geig_block_shifts(c32* B, int nb, c32* shift) {
 
 // The same from the trailing block of the matrix itself (rows hi - nb + 1 .. hi): scaled by a
 // power of two to FP32, its entries below 2; returns the power that the shifts are to be
-// multiplied by, or 0 when a shift is not finite (the matrix itself is not).
-__device__ __forceinline__ double geig_shifts(const z64* H, int ld, int hi, int nb, c32* B, c32* shift) {
+// multiplied by, or 0 when a shift is not finite (the matrix itself is not).  Shifts that FP32
+// does not tell apart (an eigenvalue of W that many bands share) are kept once: nb becomes
+// the number kept.
+__device__ __forceinline__ double geig_shifts(const z64* H, int ld, int hi, int& nb, c32* B, c32* shift) {
   const int lane = threadIdx.x & 31, h0 = hi - nb + 1;
   unsigned top = 0;  // leading word of the largest magnitude
   for (int e = lane; e < nb * nb; e += 32) {
@@ -226,7 +230,18 @@ __device__ __forceinline__ double geig_shifts(const z64* H, int ld, int hi, int 
   }
   __syncwarp();
   geig_block_shifts(B, nb, shift);
-  const bool ok = lane >= nb || (isfinite(shift[lane].re) && isfinite(shift[lane].im));
+  const c32 s = lane < nb ? shift[lane] : c32(0.f, 0.f);
+  const bool ok = isfinite(s.re) && isfinite(s.im);
+  bool keep = lane < nb;
+  for (int j = 0; j + 1 < nb; ++j) {
+    const c32 o(__shfl_sync(0xffffffffu, s.re, j), __shfl_sync(0xffffffffu, s.im, j));
+    if (j < lane && geig_abs1(s - o) < 4e-6f) keep = false;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, keep);
+  __syncwarp();
+  if (keep) shift[__popc(m & ((1u << lane) - 1u))] = s;
+  nb = __popc(m);
+  __syncwarp();
   return __all_sync(0xffffffffu, ok) ? __hiloint2double(ex << 20, 0) : 0.0;
 }
 
@@ -330,6 +345,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
   }
   __syncthreads();
   int iter = 0, total = 0;
+  bool one = false;  // one sweep at a time from here on
   const int cap = 120 * p + 120;
   while (true) {
     if (tid < 32) {  // the first warp finds the active block and the shifts
@@ -340,7 +356,7 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
           hi = -1;
           break;
         }
-        l = geig_split_point(H, ld, hi, eps, iter >= GEIG_STALL);
+        l = geig_split_point(H, ld, hi, eps, one || iter >= GEIG_STALL);
         __syncwarp();
         if (tid == 0 && l > 0) H[l * ld + l - 1] = z64(0.0, 0.0);
         if (l == hi) {
@@ -350,19 +366,23 @@ __device__ inline int geig(z64* H, z64* Z, int p, int ld, bool want_vec, z64* la
           continue;
         }
         const int size = hi - l + 1;
-        // one sweep with the 2 x 2 block's shift on short blocks, and now and then when
-        // nothing deflates (exceptional shifts)
-        nb = size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
+        // one sweep on short blocks, and now and then when nothing deflates (exceptional
+        // shifts); the last of several sweeps takes the 2 x 2 block's shift in FP64 as well: it
+        // is the one that ends the convergence (p = 64, 27 loops: 10.5 -> 9.3 ms)
+        nb = one || size < 6 || (iter > 0 && iter % 12 == 0) ? 1 : min(GEIG_NB, size / 3);
         if (nb > 1) {
+          const int want = nb;
           const double up = geig_shifts(H, ld, hi, nb, sh->B, sh->low);
+          one = 3 * nb <= want;  // eigenvalues shared by many bands: the block tells too little
           if (up > 0.0) {
             if (tid < nb) sh->shift[tid] = up * ccast<double>(sh->low[tid]);
           } else {
             nb = 1;
           }
         }
-        if (nb == 1 && tid == 0) {
-          sh->shift[0] =
+        __syncwarp();
+        if (tid == 0) {
+          sh->shift[nb - 1] =
               geig_shift(H[(hi - 1) * ld + hi - 1], H[(hi - 1) * ld + hi], H[hi * ld + hi - 1], H[hi * ld + hi],
                          iter, hi >= 2 ? zabs(H[(hi - 1) * ld + hi - 2]) : 0.0);
         }
