@@ -47,18 +47,28 @@ __device__ __forceinline__ void rr_pair(int r, int k, int np, int& p, int& q) {
 // Diagonalises A (n x n, leading dimension ld) in place and accumulates V = prod J.
 // On return A's diagonal holds the eigenvalues (unsorted).  rot: >= n/2+1 JacRot
 // slots; red: >= 32 doubles.  Returns the number of sweeps, or -1 without
-// convergence after max_sweeps.  Every thread of the block must call it.
+// convergence after max_sweeps.  turned (shared memory, optional) receives the number of
+// rotations.  Every thread of the block must call it.
 template <typename T>
 __device__ int jacobi_eigh(cx<T>* A, cx<T>* V, int n, int ld, int max_sweeps, JacRot<T>* rot,
-                           double* red) {
+                           double* red, int* turned = nullptr) {
   const int tid = threadIdx.x, nt = blockDim.x;
+  int count = 0;
+  auto done = [&](int result) {
+    if (turned) {
+      const double all = block_sum(double(count), red);
+      if (tid == 0) *turned = int(all);
+      __syncthreads();
+    }
+    return result;
+  };
   for (int e = tid; e < n * n; e += nt) {
     const int r = e / n, c = e - r * n;
     V[r * ld + c] = cx<T>(T(r == c), T(0));
   }
   if (n == 1) {
     __syncthreads();
-    return 0;
+    return done(0);
   }
   const int np = (n + 1) & ~1, npairs = np >> 1;
   // ||A||_F (invariant under the rotations)
@@ -77,7 +87,7 @@ __device__ int jacobi_eigh(cx<T>* A, cx<T>* V, int n, int ld, int max_sweeps, Ja
       if (r != c) off += double(abs2(A[r * ld + c]));
     }
     off = block_sum(off, red);
-    if (sqrt(off) <= tol || fro == 0.0) return sweep;
+    if (sqrt(off) <= tol || fro == 0.0) return done(sweep);
     if (sweep == max_sweeps) break;
     if (tid == 0) s_rotated = 0;
     __syncthreads();
@@ -100,6 +110,7 @@ __device__ int jacobi_eigh(cx<T>* A, cx<T>* V, int n, int ld, int max_sweeps, Ja
           const T b2 = abs2(b), e4 = T(4) * eps_of<T>();
           if (b2 > e4 * e4 * fabs(a) * fabs(d) && b2 > T(0)) {
             s_rotated = 1;
+            ++count;
             T ab, t, c, s;  // s = sin / |b|
             if constexpr (sizeof(T) == 4) {
               // hardware reciprocal roots with a Newton step for what keeps the rotation
@@ -173,9 +184,9 @@ __device__ int jacobi_eigh(cx<T>* A, cx<T>* V, int n, int ld, int max_sweeps, Ja
       }
       __syncthreads();
     }
-    if (!s_rotated) return sweep + 1;
+    if (!s_rotated) return done(sweep + 1);
   }
-  return -1;
+  return done(-1);
 }
 
 // Sort key that puts NaN after every number, so that ranks always form a

@@ -128,6 +128,7 @@ __global__ void k_lg_build(LargeArgs a) {
         const double2 t = reinterpret_cast<const double2*>(md.hop_t)[h];
         cfma(acc, z64(t.x, t.y), r < nRs ? phs[r] : bloch_phase(f, md.Rv + 3 * r));
       }
+      if (a.polish) acc = a.scale * acc;
       A[(long long)md.ent_row[e] * n + md.ent_col[e]] = ccast<T>(acc);
       if (a.Hent) {  // FP64 entry as an unevaluated sum of two floats (hi, lo)
         c32 hi, lo;
@@ -810,6 +811,13 @@ __device__ void tri_normalise(int n, const Strided<T>& W, long long t, T* Zc, in
   }
 }
 
+// What a stage after the eigenvalues skips: the FP32 ones the k-points that the polish cannot
+// take, the FP64 ones the others.
+template <typename T>
+__device__ __forceinline__ bool lg_skip(const LargeArgs& a, long long kw) {
+  return a.need && (a.need[kw] != 0) == (sizeof(T) == 4);
+}
+
 constexpr int INVIT_WINDOW_N = 512, INVIT_ITS = 3;
 
 template <typename T>
@@ -818,7 +826,7 @@ __global__ void k_lg_invit(LargeArgs a) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= NT) return;
   const long long kw = t / a.nvec;
-  if (std::is_same<T, double>::value && a.need && !a.need[kw]) return;
+  if (lg_skip<T>(a, kw)) return;
   const int idx = int(t - kw * a.nvec), n = a.n, nv = a.nvec;
   const T* dg = reinterpret_cast<const T*>(a.dg) + kw * n;
   const T* od = reinterpret_cast<const T*>(a.od) + kw * n;
@@ -937,6 +945,27 @@ __device__ __forceinline__ int polish_lower(const float* lam, int n, int p) {
   return p - c;
 }
 
+// Which k-points the polish can take, from the FP32 eigenvalues: energies in range, a gap of 1e-3
+// of the spectral radius, band edges of at most POLISH_G levels.  Told before the eigenvectors,
+// so that a k-point left to the FP64 solve costs the FP32 reduction and bisection only.
+// Where that is a quarter of the wave or more, the whole wave is left to it: the two solves are
+// chains of the same length whatever the number of their k-points, and would follow each other.
+// One CTA.
+__global__ void __launch_bounds__(256) k_lg_polish_need(LargeArgs a) {
+  __shared__ double red[32];
+  double left = 0.0;
+  for (long long kw = threadIdx.x; kw < a.W; kw += blockDim.x) {
+    const float* lam = reinterpret_cast<const float*>(a.lam) + kw * a.nval;
+    const float width = polish_width(lam, a.n), nrm = 1e3f * width;
+    const bool fit = nrm > 1e-8f && nrm < 1e12f && lam[a.p] - lam[a.p - 1] > width &&
+                     polish_upper(lam, a.n, a.p) <= POLISH_G && polish_lower(lam, a.n, a.p) <= POLISH_G;
+    a.need[kw] = fit ? 0 : 1;
+    left += fit ? 0.0 : 1.0;
+  }
+  if (4.0 * block_sum(left, red) < double(a.W)) return;
+  for (long long kw = threadIdx.x; kw < a.W; kw += blockDim.x) a.need[kw] = 1;
+}
+
 // ---------------------------------------------------------------------------
 // Stage 5: back-transform x = Q D z for the first ncol eigenvectors, Q = P_0 ... P_{n-3}:
 // X = D Z, then X <- P_c X for c = n-3 down to 0 (P_c = I - 2 u_c u_c^dagger): one
@@ -955,7 +984,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_backtransform(LargeArgs a, cx<To>
   if constexpr (kTc) ts = tc::setup(&tmem_slot, &tc_bar);
   const int n = a.n, tid = threadIdx.x, nt = blockDim.x;
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
-    if (!kTc && a.need && !a.need[kw]) continue;
+    if (lg_skip<T>(a, kw)) continue;
     const cx<T>* A = reinterpret_cast<const cx<T>*>(a.A) + kw * (long long)n * n;
     const cx<T>* Dp = reinterpret_cast<const cx<T>*>(a.Dp) + kw * n;
     const T* Z = reinterpret_cast<const T*>(a.Z) + kw * (long long)a.nvec * n;
@@ -1048,6 +1077,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
   __shared__ __align__(8) uint64_t tc_bar;
   tc::State ts = tc::setup(&tmem_slot, &tc_bar);      // plain FP32 products: tensor cores
   for (long long kw = blockIdx.x; kw < a.W; kw += gridDim.x) {
+    if (lg_skip<float>(a, kw)) continue;
     const long long k = a.k0 + kw * (a.kstride > 0 ? a.kstride : 1);
     const c32* A = reinterpret_cast<const c32*>(a.A) + kw * (long long)n * n;
     const c32* Dp = reinterpret_cast<const c32*>(a.Dp) + kw * n;
@@ -1338,14 +1368,9 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
     c32* C = a.C32 + kw * (long long)n * ldc;          // corrections: occupied, then upper edge
     z64* G = a.G64 + kw * ((long long)p * p + ((long long)p * p + 1) / 2);  // Q^dag H Q
     c32* E = reinterpret_cast<c32*>(G + (long long)p * p);  // Q^dag Q - I
-    const float width = polish_width(lam, n), nrm = 1e3f * width;
+    if (a.need[kw]) continue;  // uniform over the CTA
+    const float width = polish_width(lam, n);
     const int g = polish_upper(lam, n, p), gl = polish_lower(lam, n, p);
-    const bool fit = nrm > 1e-8f && nrm < 1e12f && lam[p] - lam[p - 1] > width && g <= POLISH_G && gl <= POLISH_G &&
-                     p + g <= nbt;
-    if (!fit) {  // uniform over the CTA
-      if (tid == 0) a.need[kw] = 1;
-      continue;
-    }
     // R = H Q
     if (md.n_ent == n * n) {
       cta_gemm<GemmPlainT<double>, true, true, TN>(
@@ -1561,9 +1586,8 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
     __syncthreads();
     const double bot = polish_ritz(XU, YU, n, g, false, static_cast<c32*>(nullptr), 0, S, V, rot, red);
     if (tid == 0) {
-      const double gp = bot - top;
+      const double gp = (bot - top) / a.scale;
       a.gap[k] = gp;
-      a.need[kw] = 0;
       if (!(gp > a.gap_tol)) report(a.status, ST_EGAP, k, gp);
     }
     __syncthreads();
@@ -1634,6 +1658,10 @@ cudaError_t lg_common(const LargeArgs& a, cudaStream_t s) {
   k_lg_bisect<T><<<dim3(unsigned(std::min<long long>(a.W, 65535)), unsigned((a.nval + BIS_THREADS - 1) / BIS_THREADS)),
                    BIS_THREADS, sm_b, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (sizeof(T) == 4 && a.polish) {
+    k_lg_polish_need<<<1, 256, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   lg_mark(a, "lg_bisect");
   const long long ni = a.W * a.nvec;
   if (ni > 0) {

@@ -46,6 +46,8 @@ struct StatesArgs {
   DevStatus* status;
   int want_df;          // write U as complex double-float (states_df_eligible() holds)
   int rotations;        // n = 4: Jacobi rotations that H(k) takes at generic points (0: not known)
+  double scale;         // power of two on H for FP64 requests that start from an FP32 solve (the
+                        // gap is divided by it): energies of any unit fit FP32
 };
 
 // n = 4, more k-points than this, H(k) diagonal after this many Jacobi rotations: one thread per
@@ -125,6 +127,7 @@ struct LargeArgs {
   long long kstride;      // k-point of wave slot kw: k0 + kw * kstride (0 means 1)
   int mixed;
   int polish;             // FP64 request from the FP32 solve (mixed = 1): one more correction, in FP64
+  double scale;           // polish: power of two on H (the gap is divided by it)
   double gap_tol;
   // wave scratch
   void* A;                // W x n x n complex (T)
@@ -140,8 +143,9 @@ struct LargeArgs {
   c32* C32;               // W x n x p (mixed)
   z64* G64;               // W x p x p (mixed)
   z64* H64;               // W x n_ent (polish): the FP64 entries
-  int* need;              // W: set by the polish where a k-point needs the FP64 solve; a plain
-                          // FP64 run (mixed = 0) with need set solves only those
+  int* need;              // W: set after the FP32 eigenvalues (the later FP32 stages skip those) or by
+                          // the polish where a k-point needs the FP64 solve; a plain FP64 run
+                          // (mixed = 0) with need set solves only those
   const int* row_ptr;     // n + 1: first entry of each row in the plan
   // outputs
   z64* U;                 // W x n x p (wave-relative)

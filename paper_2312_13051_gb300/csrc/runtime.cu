@@ -640,6 +640,11 @@ struct LargePlan {
   }
 };
 
+// The power of two that brings the largest hopping into [1, 2).
+double unit_scale(double tmax) {
+  return tmax > 0.0 ? std::ldexp(1.0, -std::max(-1000, std::min(1000, std::ilogb(tmax)))) : 1.0;
+}
+
 // One wave on the arguments of LargePlan::bind_all.
 cudaError_t launch_large_wave(bw::LargeArgs& lg, bw::LargeArgs& fix, long long k0, long long W, z64* U,
                               cudaStream_t s) {
@@ -837,6 +842,7 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
   std::memset(&lg, 0, sizeof(lg));
   lg.model = dev_model(P, dblob);
   lg.plane = dev_plane(PX);
+  lg.scale = unit_scale(P.tmax);
   lg.gap_tol = o.gap_tol;
   lg.row_ptr = reinterpret_cast<const int*>(dblob + P.o_rowptr);
   lg.gap = gap;
@@ -1096,6 +1102,7 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
   sa.mixed = prec == BW_MIXED;
   sa.max_sweeps = o.max_sweeps;
   sa.rotations = P.rotations;
+  sa.scale = unit_scale(P.tmax);
   sa.gap_tol = o.gap_tol;
   sa.op.nnz = 0;
   if (spin) {
@@ -1145,6 +1152,7 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
     std::memset(&lg, 0, sizeof(lg));
     lg.model = sa.model;
     lg.plane = sa.plane;
+    lg.scale = sa.scale;
     lg.gap_tol = o.gap_tol;
     lg.row_ptr = reinterpret_cast<const int*>(dblob + P.o_rowptr);
     lg.gap = gap;
@@ -1858,6 +1866,7 @@ bw_status noalloc_run(bw_ctx* ctx, const bw_model* model, const bw_plane* plane,
   sa.mixed = prec == BW_MIXED;
   sa.max_sweeps = o.max_sweeps;
   sa.rotations = P.rotations;
+  sa.scale = unit_scale(P.tmax);
   sa.gap_tol = o.gap_tol;
   sa.U = U;
   sa.gap = gap;

@@ -350,6 +350,10 @@ __device__ double edge_energy(const z64* H, const c32* V, const int* ord, const 
 // the FP64 Jacobi sweeps (~7 n^3 complex multiply-adds each) by ~13 n^2 p FP64 ones, which
 // the FP64 pipe was busy with (n = 32, p = 8, 441 k-points with the spin split: 4.40 ms
 // before, 1.65 ms now).
+// (Where the FP32 solve took fewer than n^2 / 4 rotations, of the ~2.5 n^2 of a full matrix, the
+// caller solves in FP64 at once: uncoupled blocks keep most entries at zero, and ~36 n FP64
+// operations per rotation are then fewer than the corrections' ~12 n^3.  Five uncoupled
+// copies of a four-band model, n = 20, 256 k-points: whole call 441 -> 257 us.)
 // Returns false, and the caller solves in FP64, where this does not apply: a gap below
 // 1e-3 of the spectral radius, H outside the FP32 range, more than p levels (the scratch)
 // within that distance of a band edge, corrections that do not converge.
@@ -520,11 +524,13 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
         cfma(acc, md.hop_t[h], ph);
       }
       const int at = md.ent_row[e] * n + md.ent_col[e];
+      if (!mixed) acc = a.scale * acc;
       A[at] = ccast<float>(acc);
       H64[at] = acc;
     }
     __syncthreads();
-    int sw = jacobi_eigh<float>(A, V, n, n, a.max_sweeps, rot, red);
+    int sw = jacobi_eigh<float>(A, V, n, n, a.max_sweeps, rot, red, flag + 1);
+    const int turned = flag[1];
     sort_diag<float>(A, n, n, ord);
     for (int c = tid; c < n; c += nt) lam[c] = double(A[c * n + c].re);
     for (int e = tid; e < n * p; e += nt) {
@@ -536,7 +542,7 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
     int ok = 1;
     if (mixed) {
       gap = refine_mixed(H64, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
-    } else if (sw < 0 ||
+    } else if (sw < 0 || 4 * turned < n * n ||
                !refine_fp64(H64, V, ord, lam, n, p, Q, HQ, C, G, Zg, rot64, red, a.max_sweeps, flag, gap)) {
       // FP64 Jacobi, in place on H
       __syncthreads();
@@ -550,6 +556,7 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
       __syncthreads();
       gap = p < n ? lam[ord[p]] - lam[ord[p - 1]] : INFINITY;
     }
+    if (!mixed) gap /= a.scale;
     if (tid == 0) {
       a.gap[k] = gap;
       if (sw < 0 || !ok) report(a.status, ST_ENOCONV, k, 0.0);

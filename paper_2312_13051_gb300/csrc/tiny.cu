@@ -721,7 +721,7 @@ __device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
     const z64 s3 = conj(shfl_z(s1, base + c3)), t2 = shfl_z(s2, base + (l & 1));
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      Hr[c] = c == l ? z64(dg, 0.0) : (c == c1 ? s1 : (c == c3 ? s3 : (l < 2 ? t2 : conj(t2))));
+      Hr[c] = a.scale * (c == l ? z64(dg, 0.0) : (c == c1 ? s1 : (c == c3 ? s3 : (l < 2 ? t2 : conj(t2)))));
   }
   z64 Q[PP];
   double gap = INFINITY;
@@ -743,6 +743,7 @@ __device__ __forceinline__ void states_quad(const StatesArgs& a, int use_tab) {
       if constexpr (PP < 4) gap = sel4(lam, ord[PP]) - sel4(lam, ord[PP - 1]);
     }
   }
+  gap /= a.scale;
   const bool write = active && l == 0;
   if (write) {
     a.gap[k] = gap;
