@@ -1070,14 +1070,15 @@ bw_status run_loop(bw_ctx* ctx, LoopKind kind, const bw_model* model, const bw_p
   LargePlan LP(n, p, P.n_ent, mx);
   const size_t sz_Uf = spin ? al256(size_t(n) * p * sizeof(z64)) : 0;
   const size_t sp_k = sz_Uf + (spin && large ? pso_split_bytes(n, p, pso_evals != nullptr) : 0);
-  LP.fit(ctx->budget > total ? ctx->budget - total : 0, sp_k);
+  const size_t wave_pad = 16 * 256;  // alignment of a wave's arrays
+  LP.fit(ctx->budget > total ? ctx->budget - total : 0, sp_k + wave_pad);
   const size_t per_k = LP.bytes() + sp_k;
   long long Wv = 0;
   if (large) {
     const size_t avail = ctx->budget > total ? (ctx->budget - total) / 2 : 0;
     Wv = std::min<long long>(K, std::max<long long>(1, (long long)(avail / per_k)));
     Wv = std::min<long long>(Wv, 2048);
-    total += size_t(Wv) * per_k + 16 * 256;
+    total += size_t(Wv) * per_k + wave_pad;
   }
   begin_call(ctx, s);
   if ((st = reserve(ctx, total, s))) return st;
