@@ -428,22 +428,45 @@ def _eig_frac(fl, st, peak):
     return (fl["lg_tridiag"] + fl["lg_backtransform"]) / (ms * 1e-3) / 1e12 / peak
 
 
-def manyband_stage_flops(n, p, N, Nt, nnz_groups, mixed, n_ent=None):
+def stage_pipe(stage, mixed, polished, p):
+    """The pipe ("fp32" or "fp64") that an n > 32 stage runs on.  The eigensolve stages run in
+    FP32 in the mixed request and in an FP64 request that starts from an FP32 solve
+    (polished: the call has an lg_polish stage, whose own products are FP64); overlaps, loop
+    products and, from 128 bands on, eigenphases of the mixed request are double-float on
+    the FP32 pipe."""
+    if stage == "lg_polish":
+        return "fp64"
+    if stage.startswith("lg_"):
+        return "fp32" if mixed or polished else "fp64"
+    if stage == "eigenphases" and p < 128:
+        return "fp64"
+    return "fp32" if mixed else "fp64"
+
+
+PIPE_SOURCE = {"fp32": "measured cuBLAS SGEMM 8192^3, TF32 off (the FP32 pipe the stage runs on)",
+               "fp64": "measured cuBLAS DGEMM 4096^3 (FP64 pipe)"}
+
+
+def manyband_stage_flops(n, p, N, Nt, nnz_groups, mixed, n_ent=None, polished=False):
     """Algorithmic flops of each stage of the n > 32 Wilson-loop call over K = N Nt
     k-points (complex multiply-add = 8 flops): Bloch sum 8 per hopping group,
     Householder tridiagonalisation 16/3 n^3, back-transform of nbt vectors 8 n^2 nbt,
     refinement 8 n_ent p (H Q from the n_ent assembled entries of H) + 16 n (n - p) p +
-    16 n p^2 (mixed only), overlaps 8 n p^2, loop products 8 p^3 per step plus ~10 p^3
-    for the eigenphases of each loop; bisection and inverse iteration are O(n p)."""
+    16 n p^2 (mixed, and polished FP64 requests), the polish's FP64 products 8 n_ent p +
+    16 n p^2 (H Q, Q^dag H Q and the Gram matrix by half, Q G), overlaps 8 n p^2, loop
+    products 8 p^3 per step plus ~10 p^3 for the eigenphases of each loop; bisection and
+    inverse iteration are O(n p)."""
     n_ent = n * n if n_ent is None else n_ent
     K = N * Nt
-    nbt = min(n, p + 1) if mixed else p
+    nbt = min(n, p + 1) if mixed or polished else p
     # keys: the stage names the library's per-kernel timing marks carry
     fl = {"lg_tridiag": K * 16.0 / 3.0 * n ** 3, "lg_backtransform": K * 8.0 * n * n * nbt,
           "overlaps": K * 8.0 * n * p * p, "loops": Nt * (N * 8.0 * p ** 3 + 10.0 * p ** 3),
           "lg_build": K * 8.0 * nnz_groups}
-    if mixed:
+    if mixed or polished:
         fl["lg_refine"] = K * (8.0 * n_ent * p + 16.0 * n * (n - p) * p + 16.0 * n * p * p)
+    if polished:
+        fl["lg_polish"] = K * (8.0 * n_ent * p + 16.0 * n * p * p)
     return fl
 
 
@@ -711,11 +734,16 @@ def run_ours(args):
             r = mb_res[prec]
             ms = r["total_ms"] / r["steps"]
             st = r["stages"]
+            polished = "lg_polish" in st
             fl = manyband_stage_flops(mb.model.n, mb.p, mb.plane.N, mb.plane.N_t, nnz_groups,
-                                      prec == "mixed", n_ent)
+                                      prec == "mixed", n_ent, polished)
+            if "eigenphases" in st:         # a stage of its own
+                fl["eigenphases"] = mb.plane.N_t * 10.0 * mb.p ** 3
+                fl["loops"] -= fl["eigenphases"]
             d = max((k for k in st if k in fl), key=st.get)
             ach = fl[d] / (st[d] * 1e-3) / 1e12
-            pk_ = peaks["fp32"] if prec == "mixed" else peaks["fp64"]
+            pipe = stage_pipe(d, prec == "mixed", polished, mb.p)
+            pk_ = peaks[pipe]
             blk[prec] = {"value": weak_scaling_value(Km, r["steps"], world,
                                                      reduce_max(r["total_ms"] / 1e3, dev)),
                          "ms_per_call": ms, "dtype": "f32+df32" if prec == "mixed" else "f64",
@@ -724,11 +752,9 @@ def run_ours(args):
                          "roofline": {"kernel": d, "bound": "alu", "achieved": ach, "peak": pk_,
                                       "unit": "TFLOP/s", "frac": ach / pk_,
                                       "algorithmic_flops_per_call": fl[d],
-                                      "peak_source": ("measured cuBLAS SGEMM 8192^3, TF32 off (the "
-                                                      "FP32 pipe the mixed stages run on)"
-                                                      if prec == "mixed" else
-                                                      "measured cuBLAS DGEMM 4096^3 (FP64 pipe)"),
-                                      "eigensolve_frac": _eig_frac(fl, st, pk_)}}
+                                      "peak_source": PIPE_SOURCE[pipe],
+                                      "eigensolve_frac": _eig_frac(
+                                          fl, st, peaks[stage_pipe("lg_tridiag", prec == "mixed", polished, mb.p)])}}
             if "phase_err_rad" in r:
                 blk[prec]["phase_err_rad_sampled_row"] = r["phase_err_rad"]
         for kind in ("spin_mixed", "nested_mixed"):
@@ -753,16 +779,14 @@ def run_ours(args):
                 r = sc_res[(Ls, prec)]
                 calls = len(r["per_call"])
                 st = {k: v / calls for k, v in r["stages"].items()}
-                fl = manyband_stage_flops(n_, p_, 16, 16, groups, prec == "mixed", n_ent)
+                polished = "lg_polish" in st
+                fl = manyband_stage_flops(n_, p_, 16, 16, groups, prec == "mixed", n_ent, polished)
                 fl["loops"] = 16 * 15 * 8.0 * p_ ** 3       # N - 1 products of p x p per loop
                 fl["eigenphases"] = 16 * 10.0 * p_ ** 3    # Hessenberg + QR per loop
                 d = max((k for k in st if k in fl), key=st.get)
                 ach = fl[d] / (st[d] * 1e-3) / 1e12
-                fp32_stage = prec == "mixed" and d.startswith("lg_")
-                pk_ = peaks["fp32"] if fp32_stage else peaks["fp64"]
-                src = ("measured cuBLAS SGEMM (FP32 pipe)" if fp32_stage else
-                       "measured cuBLAS DGEMM: FP64-grade arithmetic, computed in double-float on "
-                       "the FP32 pipe" if prec == "mixed" else "measured cuBLAS DGEMM (FP64 pipe)")
+                pipe = stage_pipe(d, prec == "mixed", polished, p_)
+                pk_ = peaks[pipe]
                 sub[prec] = {"value": Kc * calls / (r["total_ms"] * 1e-3), "unit": UNIT,
                              "ms_per_call": r["total_ms"] / calls,
                              "per_call_ms": [round(x, 2) for x in r["per_call"]],
@@ -771,7 +795,7 @@ def run_ours(args):
                              "roofline": {"kernel": d, "bound": "alu", "achieved": ach, "peak": pk_,
                                           "unit": "TFLOP/s", "frac": ach / pk_,
                                           "algorithmic_flops_per_call": fl[d],
-                                          "peak_source": src}}
+                                          "peak_source": PIPE_SOURCE[pipe]}}
             cpu = sc_res.get((Ls, "cpu"))
             if cpu:
                 sub["cpu_baseline"] = {"value": cpu["k_points"] / cpu["seconds"], "unit": UNIT,
