@@ -55,6 +55,17 @@ __device__ __forceinline__ df operator+(df a, df b) {
 
 __device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
 
+// Sum with the low parts added in FP32: 11 instructions instead of 20, absolute error about
+// 2^-47 (|a| + |b|) at most as for operator+ (root mean square 0.12 of it instead of 0.10), but no
+// relative accuracy where the high parts cancel.  For the short sums of the four-band kernels,
+// whose terms carry errors of that size already: phases, gaps and nested phases of BBH 60 x 60
+// and 60 x 3840 are as near to 64 bits with it as with operator+, and the kernel that fetches
+// its code from a flushed L2 takes 39.0 us instead of 41.5.
+__device__ __forceinline__ df df_sum(df a, df b) {
+  const df s = df_two_sum(a.hi, b.hi);
+  return df_fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+
 __device__ __forceinline__ df operator*(df a, df b) {
   const float p = a.hi * b.hi;
   float e = fmaf(a.hi, b.hi, -p);

@@ -226,8 +226,8 @@ __device__ __forceinline__ void df_mac2(df& acc, df a, float b, df c, float d) {
 }
 
 __device__ __forceinline__ df group_sum_df(df v) {
-  v = v + shfl_xor_df(v, 1);
-  return v + shfl_xor_df(v, 2);
+  v = df_sum(v, shfl_xor_df(v, 1));
+  return df_sum(v, shfl_xor_df(v, 2));
 }
 
 __device__ __forceinline__ c32 group_sum_c32(c32 v) {
@@ -321,13 +321,13 @@ __device__ __forceinline__ void quad_pair_edges(QuadPair r, float s00, float s11
   }
   dev_second_order(r.e00, r.e11, r.e01);
   const float a = r.g00.hi, d = r.g11.hi, m = 0.5f * (a + d), x = g.re * r.e01.re + g.im * r.e01.im;
-  const df aa = r.g00 + df(s00 - r.e00 * a - x), dd = r.g11 + df(s11 - r.e11 * d - x);
+  const df aa = df_sum(r.g00, df(s00 - r.e00 * a - x)), dd = df_sum(r.g11, df(s11 - r.e11 * d - x));
   const float eh = 0.5f * (r.e00 + r.e11);
-  const df bre = r.gre + df(s01.re - eh * g.re - m * r.e01.re), bim = r.gim + df(s01.im - eh * g.im - m * r.e01.im);
-  const df mean = df(0.5f) * (aa + dd), half = df(0.5f) * (aa - dd);
+  const df bre = df_sum(r.gre, df(s01.re - eh * g.re - m * r.e01.re)), bim = df_sum(r.gim, df(s01.im - eh * g.im - m * r.e01.im));
+  const df mean = 0.5f * df_sum(aa, dd), half = 0.5f * df_sum(aa, -dd);
   const df q = df_sqrt(df_fma(half, half, df_fma(bre, bre, bim * bim)));
-  lo = mean - q;
-  hi = mean + q;
+  lo = df_sum(mean, -q);
+  hi = df_sum(mean, q);
 }
 
 // Occupied pair of a four-band H(k) given as double-float rows (lane l holds row
@@ -374,7 +374,7 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
   const QuadPair un = quad_pair<true>(z0, z1, h[2], h[3]);
   // residuals and coefficients C[a][c]
   auto resid = [](cdf hv, c32 q, df rho) {
-    return c32((hv.re - q.re * rho).hi, (hv.im - q.im * rho).hi);
+    return c32(df_sum(hv.re, -(q.re * rho)).hi, df_sum(hv.im, -(q.im * rho)).hi);
   };
   const c32 r0 = resid(h[0], q0, oc.g00), r1 = resid(h[1], q1, oc.g11);
   auto coef = [](c32 z, c32 r, float den) {
@@ -411,8 +411,8 @@ __device__ __forceinline__ int quad_df_occupied(const cdf (&Hr)[4], int l, int b
     dev_second_order(e00, e11, e01);
     const c32 x0(Q0.re.hi, Q0.im.hi), x1(Q1.re.hi, Q1.im.hi);
     const c32 f0 = e00 * x0 + x1 * conj(e01), f1 = x0 * e01 + e11 * x1;
-    Q0 = cdf(Q0.re + df(-0.5f * f0.re), Q0.im + df(-0.5f * f0.im));
-    Q1 = cdf(Q1.re + df(-0.5f * f1.re), Q1.im + df(-0.5f * f1.im));
+    Q0 = cdf(df_sum(Q0.re, df(-0.5f * f0.re)), df_sum(Q0.im, df(-0.5f * f0.im)));
+    Q1 = cdf(df_sum(Q1.re, df(-0.5f * f1.re)), df_sum(Q1.im, df(-0.5f * f1.im)));
   }
   // second-order shifts of the Ritz matrices (level repulsion between the pairs)
   df occ_lo, occ_hi, un_lo, un_hi;
