@@ -168,6 +168,25 @@ cudaError_t launch_convert_cdf(z64* x, long long count, bool to_cdf, cudaStream_
   return cudaGetLastError();
 }
 
+// dst[l sd + e] = src[l ss + e], e < count, l < nl: one matrix of every loop, at whole-loop
+// strides.  A kernel and not a 2-D copy, whose pitch may not exceed 2^31 - 1 bytes (p = 1024 with
+// 129 k-points per loop has 2.2 GB).
+__global__ void k_copy_strided(z64* dst, long long sd, const z64* src, long long ss, long long count, long long nl) {
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nl * count; e += step) {
+    const long long l = e / count, q = e - l * count;
+    dst[l * sd + q] = src[l * ss + q];
+  }
+}
+
+cudaError_t launch_copy_strided(z64* dst, long long sd, const z64* src, long long ss, long long count, long long nl,
+                                cudaStream_t s) {
+  if (count <= 0 || nl <= 0) return cudaSuccess;
+  const long long blocks = std::min<long long>((nl * count + 255) / 256, 152LL * 16);
+  k_copy_strided<<<unsigned(blocks), 256, 0, s>>>(dst, sd, src, ss, count, nl);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // Phase of a determinant (the link variables of the plaquette Berry flux for p > 64).
 // Right-looking LU with partial pivoting of one p x p matrix per CTA in global memory:

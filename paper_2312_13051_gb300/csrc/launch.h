@@ -257,6 +257,9 @@ cudaError_t launch_iota(long long* off, int* idx, long long W, long long stride,
 cudaError_t launch_zgemm(const GemmArgs& g, cudaStream_t s, bool df = false);
 // In place, count elements: complex FP64 -> complex double-float (to_cdf) or back.
 cudaError_t launch_convert_cdf(z64* x, long long count, bool to_cdf, cudaStream_t s);
+// dst[l sd + e] = src[l ss + e] for e < count, l < nl
+cudaError_t launch_copy_strided(z64* dst, long long sd, const z64* src, long long ss, long long count, long long nl,
+                                cudaStream_t s);
 cudaError_t launch_geig_big(const BigEigArgs& a, cudaStream_t s);
 
 // Launches every stage of the large-n solver for one wave.

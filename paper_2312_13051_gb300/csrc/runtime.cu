@@ -908,9 +908,7 @@ bw_status run_big_loop(bw_ctx* ctx, const HostPlan& P, const Blob& blob, const P
         g.batch = (long long)nl * half;
         BW_CUDA(bw::launch_zgemm(g, s, mx), "loop-product GEMM");
         if (cnt & 1)
-          BW_CUDA(cudaMemcpy2DAsync(dst + (long long)half * sP, size_t(sOut) * sizeof(z64),
-                                    src + (long long)(cnt - 1) * sP, size_t(sIn) * sizeof(z64),
-                                    size_t(sP) * sizeof(z64), size_t(nl), cudaMemcpyDeviceToDevice, s),
+          BW_CUDA(bw::launch_copy_strided(dst + (long long)half * sP, sOut, src + (long long)(cnt - 1) * sP, sIn, sP, nl, s),
                   "loop-product copy");
         std::swap(src, dst);
         sIn = sOut;
