@@ -17,9 +17,10 @@ namespace bw {
 // Sweeps in flight.  A rotation is a chain of ~20 dependent FP64 operations (64 clocks each
 // on GB300) and three block barriers, whatever the number of entries it moves, so the sweeps
 // of several shifts share the steps: NB sweeps over an active block of s rows take
-// s + 2 NB steps instead of NB s.  Measured (one CTA per loop): p = 64, 27 loops, product
-// included, 19.5 -> 12.9 ms; p = 32 FP64, 17 loops, 5.1 -> 3.5 ms; p = 12 with vectors 1.46 ->
-// 1.16 ms.  A step at p = 64 takes ~7000 clocks: 2100 the rotations, the rest FP64 throughput.
+// s + 2 NB steps instead of NB s.  Measured (one CTA per loop, product included; one sweep at a
+// time, now): p = 64 FP64, 27 loops, 32.4, 17.0 ms; p = 32 FP64, 17 loops, 5.5, 3.0 ms; p = 12
+// with vectors, 31 loops, 1.56, 0.81 ms.  A step at p = 64 takes ~7000 clocks: 2100 the rotations,
+// the rest FP64 throughput.
 constexpr int GEIG_NB = 8;
 constexpr int GEIG_STALL = 30;  // rounds without a deflation after which the product test decides too
 

@@ -1260,8 +1260,10 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
 // their cluster, made orthogonal to Q, by their Ritz values (error of the vectors
 // (1e-6 ||H|| / width)^2, of the values its square).
 // A k-point is left to the FP64 solve (need = 1) where this is not enough: a gap or an
-// isolation of the edge clusters below 1e-3 of the spectral radius, |C|^2 above 1e-17 (its
-// square is the error that stays), entries outside the FP32 range.
+// isolation of the edge clusters below 1e-3 of the spectral radius, told after the bisection
+// (k_lg_polish_need), or |C| above 3e-9 here.  The FP32 basis is not renewed, so that |C| times
+// its error e0 stays: at that bound 2e-16 ||H|| / gap for e0 ~ 6e-8 ||H|| / gap, the forward
+// error of an FP64 solve.  H is scaled by a power of two, its unit does not matter.
 //
 // FP64 products bound it: four n p^2 (three of them on a sparse H) of the ~16/3 n^3 + 4 n^2 p
 // that the FP64 tridiagonal solve takes, as tiled GEMMs instead of matrix-vector products.

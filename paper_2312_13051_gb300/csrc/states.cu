@@ -175,8 +175,9 @@ __device__ bool ritz(const z64* H, z64* Q, z64* HQ, z64* C, z64* G, z64* Zg, dou
 //   Q <- Q + V_u C,  C[a][i] = (V_u^dagger R)[a][i] / (G_ii - lam_{p+a}),
 // with the FP64 residual R = H Q - Q G, G = Q^dagger H Q (its off-diagonal part is
 // of the order of the FP32 error and enters the correction at second order), then
-// Cholesky-QR.  An error e of the subspace becomes about e^2.  Returns |C|_F^2; *ok = 0
-// when the Cholesky factorisation broke down.
+// Cholesky-QR.  An error e of the subspace becomes about e (e + e0), e0 the error of V; the first
+// step, from V itself, squares it.  Returns |C|_F^2; *ok = 0 when the Cholesky factorisation
+// broke down.
 // kLow: the products with V in FP32.  They carry the correction, which only has to be right
 // relative to its own size: 6e-8 |C|, removed by the next step or, in the last one (|C| <=
 // 3e-9), below rounding.  With V converted to FP64 they were more than half of the step's FP64
@@ -344,12 +345,15 @@ __device__ double edge_energy(const z64* H, const c32* V, const int* ord, const 
   return e0;
 }
 
-// FP64 request from an FP32 eigenbasis V of H: the occupied block Q by Newton corrections,
-// repeated until the square of the last one is below rounding (|C|_F^2 <= 1e-17: two, when
-// the FP32 start is good to 1e-4), and the direct gap from the two band edges.  Replaces
-// the FP64 Jacobi sweeps (~7 n^3 complex multiply-adds each) by ~13 n^2 p FP64 ones, which
-// the FP64 pipe was busy with (n = 32, p = 8, 441 k-points with the spin split: 4.40 ms
-// before, 1.65 ms now).
+// FP64 request from an FP32 eigenbasis V of H: the occupied block Q by corrections, and the
+// direct gap from the two band edges.  V and its eigenvalues stay as they are (a chord
+// iteration): the first correction takes V's error e0 ~ 6e-8 ||H|| / gap to its square, each
+// further one multiplies the error by about e0.  It ends at |C|_F <= 3e-9 (two corrections where
+// e0 < 1e-4), which leaves |C| e0 <= 2e-16 ||H|| / gap, the forward error of an FP64 eigensolver;
+// FP64 phases at gaps of 1.5e-3 - 2e-2 of the spectral radius: 4e-16 - 2e-15 rad from a 34-digit
+// reference, the FP64 Jacobi's 2e-16 - 1.6e-14.  Replaces the FP64 Jacobi sweeps (~7 n^3 complex
+// multiply-adds each) by ~13 n^2 p FP64 ones, which the FP64 pipe was busy with (n = 32, p = 8,
+// 441 k-points with the spin split, whole call: 4.5 ms before, 0.93 ms now).
 // (Where the FP32 solve took fewer than n^2 / 4 rotations, of the ~2.5 n^2 of a full matrix, the
 // caller solves in FP64 at once: uncoupled blocks keep most entries at zero, and ~36 n FP64
 // operations per rotation are then fewer than the corrections' ~12 n^3.  Five uncoupled

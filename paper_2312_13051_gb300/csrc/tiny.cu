@@ -535,12 +535,14 @@ __device__ __forceinline__ double herm_edge(z64 (&G)[KK][KK], bool want_max) {
 
 // Occupied block (the lowest PP < 4 states; Q: row l) and direct gap of the group's H to FP64
 // accuracy without an FP64 eigensolve: FP32 Jacobi gives a start with an error of
-// ~1e-7 ||H|| / gap, and each Newton correction squares it,
+// e0 ~ 1e-7 ||H|| / gap; the first correction squares it, and each further one, in the same FP32
+// vectors, multiplies it by about e0,
 //   Q <- Q + Z C,  C[a][c] = z_a^dag (H Q - Q G)_c / (G_cc - lam_a),  G = Q^dag H Q,
 // (z_a, lam_a the unoccupied FP32 pairs).  The products that decide the accuracy (H Q, G,
 // the residual, the Gram matrices) are FP64; C and the correction, which only have to be
-// right relative to their own small size, are FP32.  Two corrections reach rounding: the
-// loop ends when |C|^2 <= 1e-17, so that the square of the last correction is below it.
+// right relative to their own small size, are FP32.  Two corrections are the rule: the loop ends
+// when |C| <= 3e-9, which leaves |C| e0 <= 3e-16 ||H|| / gap, the forward error of an FP64
+// eigensolver.
 // The gap comes from the FP64 Ritz values of Q and of its orthogonal complement.
 // Every lane of the warp must call it.  Returns false for a group where the method does not
 // apply (the caller solves it in FP64): a gap below 1e-3 of the spectral radius, H outside
