@@ -345,7 +345,7 @@ __device__ inline bool cta_reflect_wy(const c32* A, int n, c32* X, int ncol, lon
       return r > b0 + i ? A[(long long)r * n + b0 + i] : C(0.f, 0.f);
     };
     // Gram matrix V^dag V
-    if (!cta_cgemm_tc<false, true>(
+    if (!cta_cgemm_tc(
             bs, bs, rows, [&](int i, int q) { return conj(v(r0 + q, i)); },
             [&](int q, int i) { return v(r0 + q, i); },
             [&](int i, int j, const C& g) { Tm[i * RW_NB + j] = g; }, gsm, ts))
@@ -367,7 +367,7 @@ __device__ inline bool cta_reflect_wy(const c32* A, int n, c32* X, int ncol, lon
     for (int c0 = 0; c0 < ncol; c0 += RW_CW) {
       const int cw = min(RW_CW, ncol - c0);
       // W = V^dag X[:, c0 : c0 + cw]
-      if (!cta_cgemm_tc<false, true>(
+      if (!cta_cgemm_tc(
               bs, cw, rows, [&](int i, int q) { return conj(v(r0 + q, i)); },
               [&](int q, int c) { return X[(long long)(r0 + q) * ldx + c0 + c]; },
               [&](int i, int c, const C& w) { W[i * RW_CW + c] = w; }, gsm, ts))
@@ -391,7 +391,7 @@ __device__ inline bool cta_reflect_wy(const c32* A, int n, c32* X, int ncol, lon
       }
       __syncthreads();
       // X[:, chunk] <- X[:, chunk] - V W (rows r0 .. n-1)
-      if (!cta_cgemm_tc<true, true>(
+      if (!cta_cgemm_tc(
               rows, cw, bs, [&](int q, int i) { return v(r0 + q, i); },
               [&](int i, int c) { return W[i * RW_CW + c]; },
               [&](int q, int c, const C& y) {

@@ -1145,7 +1145,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
     const int nu = n - p;
     const int nvec = a.nvec;
     // coef[ua][c] = (Z_u^T C)[ua][c] / (rho_c - lam_{p+ua})
-    tc_ok = tc_ok && cta_cgemm_tc<false, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         nu, p, n, [&](int ua, int r) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
         [&](int r, int c) { return C[(long long)r * p + c]; },
         [&](int ua, int c, c32 v) {
@@ -1154,7 +1154,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
         work, ts);
     __syncthreads();
     // update = Q_h D Z_u coef
-    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         n, p, nu, [&](int r, int ua) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
         [&](int ua, int c) { return coef[(long long)ua * p + c]; },
         [&](int r, int c, c32 v) { C[(long long)r * p + c] = Dp[r] * v; }, work, ts);
@@ -1175,7 +1175,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
         work);
     c32* F = E + (long long)p * p;
     __syncthreads();
-    tc_ok = tc_ok && cta_cgemm_tc<false, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         p, p, n,
         [&](int x, int r) { return conj(X[(long long)r * nbt + x] + 0.5f * C[(long long)r * p + x]); },
         [&](int r, int y) { return C[(long long)r * p + y]; },
@@ -1187,13 +1187,13 @@ __global__ void __launch_bounds__(256, 2) k_lg_refine(LargeArgs a) {
     __syncthreads();
     // second order of (I + E)^{-1/2}: F = E - 3/4 E^2 (E reaches ~3e-5 where inverse iteration
     // leaves neighbouring vectors short of orthogonal, and E^2 would stay as the error)
-    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         p, p, p, [&](int x, int q) { return E[(long long)x * p + q]; },
         [&](int q, int y) { return E[(long long)q * p + y]; },
         [&](int x, int y, c32 v) { F[(long long)x * p + y] = E[(long long)x * p + y] - 0.75f * v; }, work, ts);
     __syncthreads();
     // Q = (Q32 + C) - (Q32 + C) F / 2, the correction in FP32
-    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         n, p, p, [&](int r, int q) { return X[(long long)r * nbt + q] + C[(long long)r * p + q]; },
         [&](int q, int c) { return F[(long long)q * p + c]; },
         [&](int r, int c, c32 v) {
@@ -1440,7 +1440,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
     c32* coef = reinterpret_cast<c32*>(YL + (long long)n * POLISH_G);  // (n - p) x p, then n x POLISH_G
     c32* coefx = reinterpret_cast<c32*>(XL);
     const int nu = n - p;
-    tc_ok = tc_ok && cta_cgemm_tc<false, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         nu, p, n, [&](int ua, int r) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
         [&](int r, int c) { return C[(long long)r * ldc + c]; },
         [&](int ua, int c, c32 v) {
@@ -1466,7 +1466,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
     }
     __syncthreads();
     // C = Q_h D Z coef
-    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         n, p, nu, [&](int r, int ua) { return c32(Z[(long long)r * nvec + p + ua], 0.f); },
         [&](int ua, int c) { return coef[(long long)ua * p + c]; },
         [&](int r, int c, c32 v) { C[(long long)r * ldc + c] = Dp[r] * v; }, smem, ts);
@@ -1508,7 +1508,7 @@ __global__ void __launch_bounds__(256, 2) k_lg_polish(LargeArgs a) {
         },
         smem);
     emax = -block_min(-emax, red);
-    tc_ok = tc_ok && cta_cgemm_tc<true, true>(
+    tc_ok = tc_ok && cta_cgemm_tc(
         n, p, p, [&](int r, int q) { return ccast<float>(Q[(long long)r * p + q]); },
         [&](int q, int c) { return E[(long long)q * p + c]; },
         [&](int r, int c, c32 v) { C[(long long)r * ldc + c] = v; }, smem, ts);

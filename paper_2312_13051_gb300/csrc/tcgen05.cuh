@@ -188,7 +188,7 @@ __device__ inline void teardown(const State& s) {
 // blockDim.x == 256 threads call it; sm holds tc::SMEM bytes, 16-byte aligned.  Returns
 // false (and produces no outputs from then on) when an MMA did not complete within the
 // bounded wait.
-template <bool A_K_CONTIG, bool B_C_CONTIG, class LA, class LB, class ST>
+template <class LA, class LB, class ST>
 __device__ bool cta_cgemm_tc(int M, int Ncol, int K, LA la, LB lb, ST st, unsigned char* sm, tc::State& s) {
   using namespace tc;
   unsigned char* Ap = sm;                    // pieces 0, 1, 2 of the embedded A chunk
