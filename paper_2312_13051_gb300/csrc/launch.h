@@ -45,7 +45,7 @@ struct StatesArgs {
   double* pso_gap;      // K (optional)
   DevStatus* status;
   int want_df;          // write U as complex double-float (states_df_eligible() holds)
-  int rotations;        // n = 4: Jacobi rotations that H(k) takes at generic points (0: not known)
+  int rotations;        // Jacobi rotations that H(k) takes at generic points (0: not known)
   double scale;         // power of two on H for FP64 requests that start from an FP32 solve (the
                         // gap is divided by it): energies of any unit fit FP32
 };

@@ -100,53 +100,76 @@ struct HostPlan {
   std::vector<int> Rv, ent_row, ent_col, ent_start, hop_r, row_ptr;
   std::vector<z64> hop_t;
   double tmax = 0.0;
-  int rotations = 0;  // n = 4: see four_band_rotations
+  int rotations = 0;  // n = 4, and uncoupled blocks up to n = 32: see jacobi_rotations
   size_t o_Rv, o_row, o_col, o_start, o_r, o_t, o_tdf, o_rowptr;
 };
 
-// Rotations of a cyclic Jacobi solve of the four-band H(k) at two generic points (the larger
-// count).  Models with symmetry keep entries at zero and turn by 45 degrees: the quadrupole
-// insulator, Eq. 9 and the (block-diagonal) spin-Hall model end after 2 to 6, any other
-// Hamiltonian takes 16 to 25, whichever of its entries vanish.
-int four_band_rotations(const HostPlan& P) {
+// True when H(k) falls apart into uncoupled blocks at every k: the entries off the diagonal do
+// not join all orbitals.
+bool uncoupled(const HostPlan& P) {
+  std::vector<int> up(P.n);
+  for (int i = 0; i < P.n; ++i) up[i] = i;
+  auto root = [&](int i) {
+    while (up[i] != i) i = up[i] = up[up[i]];
+    return i;
+  };
+  int parts = P.n;
+  for (int e = 0; e < P.n_ent; ++e) {
+    const int a = root(P.ent_row[e]), b = root(P.ent_col[e]);
+    if (a != b) {
+      up[a] = b;
+      --parts;
+    }
+  }
+  return parts > 1;
+}
+
+// Rotations of a cyclic Jacobi solve of H(k) at two generic points (the larger count; beyond four
+// bands counted up to n^2 / 4 only).  Models with symmetry keep entries at zero and turn by 45
+// degrees: the quadrupole insulator, Eq. 9 and the (block-diagonal) spin-Hall model end after 2
+// to 6, any other four-band Hamiltonian takes 16 to 25, whichever of its entries vanish.  Copies
+// take the sum of theirs.
+int jacobi_rotations(const HostPlan& P) {
   const double at[2][3] = {{0.137, 0.291, 0.413}, {0.619, 0.083, 0.777}};
+  const int n = P.n, enough = n == 4 ? 1 << 30 : n * n / 4 + 1;
+  std::vector<std::complex<double>> M(size_t(n) * n);
+  auto A = [&](int r, int c) -> std::complex<double>& { return M[size_t(r) * n + c]; };
   int most = 0;
   for (const auto& f : at) {
-    std::complex<double> A[4][4] = {};
+    std::fill(M.begin(), M.end(), 0.0);
     for (int e = 0; e < P.n_ent; ++e)
       for (int h = P.ent_start[e]; h < P.ent_start[e + 1]; ++h) {
         const int* R = P.Rv.data() + 3 * P.hop_r[h];
-        A[P.ent_row[e]][P.ent_col[e]] += std::complex<double>(P.hop_t[h].re, P.hop_t[h].im) *
+        A(P.ent_row[e], P.ent_col[e]) += std::complex<double>(P.hop_t[h].re, P.hop_t[h].im) *
                                          std::polar(1.0, 2.0 * M_PI * (f[0] * R[0] + f[1] * R[1] + f[2] * R[2]));
       }
     double top = 0.0;
-    for (auto& row : A)
-      for (auto& x : row) top = std::max(top, std::abs(x));
+    for (auto& x : M) top = std::max(top, std::abs(x));
     int count = 0;
     bool turned = top > 0.0;
-    for (int sweep = 0; turned && sweep < 12; ++sweep) {
+    for (int sweep = 0; turned && sweep < 12 && count < enough; ++sweep) {
       turned = false;
-      for (int p = 0; p < 4; ++p)
-        for (int q = p + 1; q < 4; ++q) {
-          const double ab = std::abs(A[p][q]), a = A[p][p].real(), d = A[q][q].real();
-          if (!(ab > 1e-14 * top)) continue;
+      for (int p = 0; p < n; ++p)
+        for (int q = p + 1; q < n; ++q) {
+          const double ab = std::abs(A(p, q)), a = A(p, p).real(), d = A(q, q).real();
+          if (!(ab > 1e-14 * top) || count >= enough) continue;
           turned = true;
           ++count;
           const double tau = (d - a) / (2.0 * ab);
           const double t = (tau >= 0.0 ? 1.0 : -1.0) / (std::fabs(tau) + std::sqrt(1.0 + tau * tau));
           const double c = 1.0 / std::sqrt(1.0 + t * t);
-          const std::complex<double> s = t * c / ab * A[p][q];
-          for (int k = 0; k < 4; ++k) {
-            const std::complex<double> x = A[p][k], y = A[q][k];
-            A[p][k] = c * x - s * y;
-            A[q][k] = std::conj(s) * x + c * y;
+          const std::complex<double> s = t * c / ab * A(p, q);
+          for (int k = 0; k < n; ++k) {
+            const std::complex<double> x = A(p, k), y = A(q, k);
+            A(p, k) = c * x - s * y;
+            A(q, k) = std::conj(s) * x + c * y;
           }
-          for (int k = 0; k < 4; ++k) {
-            const std::complex<double> x = A[k][p], y = A[k][q];
-            A[k][p] = c * x - y * std::conj(s);
-            A[k][q] = x * s + c * y;
+          for (int k = 0; k < n; ++k) {
+            const std::complex<double> x = A(k, p), y = A(k, q);
+            A(k, p) = c * x - y * std::conj(s);
+            A(k, q) = x * s + c * y;
           }
-          A[p][q] = A[q][p] = 0.0;
+          A(p, q) = A(q, p) = 0.0;
         }
     }
     most = std::max(most, count);
@@ -242,7 +265,7 @@ bw_status make_plan(bw_ctx* ctx, const bw_model* m, HostPlan& P) {
   P.row_ptr.assign(n + 1, 0);
   for (int e = 0; e < P.n_ent; ++e) P.row_ptr[P.ent_row[e] + 1]++;
   for (int r = 0; r < n; ++r) P.row_ptr[r + 1] += P.row_ptr[r];
-  if (n == 4) P.rotations = four_band_rotations(P);
+  if (n == 4 || (n > 4 && n <= bw::SMALL_N_MAX && uncoupled(P))) P.rotations = jacobi_rotations(P);
   return BW_OK;
 }
 

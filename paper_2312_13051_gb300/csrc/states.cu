@@ -357,7 +357,8 @@ __device__ double edge_energy(const z64* H, const c32* V, const int* ord, const 
 // (Where the FP32 solve took fewer than n^2 / 4 rotations, of the ~2.5 n^2 of a full matrix, the
 // caller solves in FP64 at once: uncoupled blocks keep most entries at zero, and ~36 n FP64
 // operations per rotation are then fewer than the corrections' ~12 n^3.  Five uncoupled
-// copies of a four-band model, n = 20, 256 k-points: whole call 441 -> 257 us.)
+// copies of a four-band model, n = 20, 256 k-points: whole call 441 -> 257 us.  Uncoupled blocks
+// are known from the hopping list, and the plan's count spares them the FP32 solve as well.)
 // Returns false, and the caller solves in FP64, where this does not apply: a gap below
 // 1e-3 of the spectral radius, H outside the FP32 range, more than p levels (the scratch)
 // within that distance of a band edge, corrections that do not converge.
@@ -533,20 +534,24 @@ __global__ void k_states_small(StatesArgs a, int p_out) {
       H64[at] = acc;
     }
     __syncthreads();
-    int sw = jacobi_eigh<float>(A, V, n, n, a.max_sweeps, rot, red, flag + 1);
-    const int turned = flag[1];
-    sort_diag<float>(A, n, n, ord);
-    for (int c = tid; c < n; c += nt) lam[c] = double(A[c * n + c].re);
-    for (int e = tid; e < n * p; e += nt) {
-      const int r = e / p, c = e - r * p;
-      Q[e] = ccast<double>(V[r * n + ord[c]]);
+    int sw = -1, turned = a.rotations;
+    const bool few = !mixed && a.rotations > 0 && 4 * a.rotations < n * n;
+    if (!few) {
+      sw = jacobi_eigh<float>(A, V, n, n, a.max_sweeps, rot, red, flag + 1);
+      turned = flag[1];
+      sort_diag<float>(A, n, n, ord);
+      for (int c = tid; c < n; c += nt) lam[c] = double(A[c * n + c].re);
+      for (int e = tid; e < n * p; e += nt) {
+        const int r = e / p, c = e - r * p;
+        Q[e] = ccast<double>(V[r * n + ord[c]]);
+      }
+      __syncthreads();
     }
-    __syncthreads();
     double gap;
     int ok = 1;
     if (mixed) {
       gap = refine_mixed(H64, V, ord, lam, n, p, Q, HQ, C, G, red, &ok, flag);
-    } else if (sw < 0 || 4 * turned < n * n ||
+    } else if (few || sw < 0 || 4 * turned < n * n ||
                !refine_fp64(H64, V, ord, lam, n, p, Q, HQ, C, G, Zg, rot64, red, a.max_sweeps, flag, gap)) {
       // FP64 Jacobi, in place on H
       __syncthreads();
